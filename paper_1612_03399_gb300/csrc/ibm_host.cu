@@ -556,6 +556,94 @@ cudaError_t launch_step_marker(ibm_ctx* c, const float* x, const float* v, const
                     true, true, true, true, clear, after_clear && !c->timing);
 }
 
+// Nodes that the marker kernel stages for one patch at rest (its row map,
+// restated on the host): per (y, z) row of the 4x4x4 windows of the centroids
+// (and, with `probe`, of the probe ends) the touched x-range in groups of 4
+// nodes, and the number of rows; -1 nodes when the patch has more rows than any
+// table holds.
+struct PatchNodes {
+  long long nodes, rows;
+};
+PatchNodes patch_nodes(const ibm_ctx* c, const ibm_body_desc& B, const HostTopo& T, int4 ch,
+                       bool probe) {
+  const Grid& g = c->grid;
+  const double h[3] = {c->gdesc.L[0] / g.n[0], c->gdesc.L[1] / g.n[1], c->gdesc.L[2] / g.n[2]};
+  std::vector<long long> win;   // lower corner of every window
+  long long lo[3] = {INT64_MAX, INT64_MAX, INT64_MAX}, hi[3] = {INT64_MIN, INT64_MIN, INT64_MIN};
+  for (int q = ch.y; q < ch.y + ch.z; ++q) {
+    const int32_t* tr = &T.tri[3 * (size_t)T.mface[q]];
+    const double *a = B.rest + 3 * (size_t)tr[0], *b = B.rest + 3 * (size_t)tr[1],
+                 *e = B.rest + 3 * (size_t)tr[2];
+    const D3 n = dcross({b[0] - a[0], b[1] - a[1], b[2] - a[2]},
+                        {e[0] - a[0], e[1] - a[1], e[2] - a[2]});
+    const double ln = dnorm(n), nn[3] = {n.x / ln, n.y / ln, n.z / ln};
+    for (int s = 0; s < (probe ? (B.closed ? 2 : 3) : 1); ++s) {
+      const double len = s == 0 ? 0.0 : (s == 1 ? 1.0 : -1.0) * (double)c->sc.probe_h;
+      for (int d = 0; d < 3; ++d) {
+        const double t = std::floor(((a[d] + b[d] + e[d]) / 3.0 + len * nn[d]) / h[d]);
+        if (!(std::fabs(t) < 1e15)) return {-1, 0};
+        const long long f = (long long)t;
+        win.push_back(f - 1);
+        lo[d] = std::min(lo[d], f - 1);
+        hi[d] = std::max(hi[d], f + 2);
+      }
+    }
+  }
+  const long long sy = hi[1] - lo[1] + 3, sz = hi[2] - lo[2] + 3;   // one generous row per side
+  if (sy > kTableRows || sz > kTableRows || sy * sz > kTableRows) return {-1, sy * sz};
+  std::vector<long long> x0(sy * sz, INT64_MAX), x1(sy * sz, INT64_MIN);
+  for (size_t w = 0; w < win.size(); w += 3)
+    for (int k = 0; k < 4; ++k)
+      for (int j = 0; j < 4; ++j) {
+        const size_t r = (size_t)((win[w + 2] - lo[2] + k) * sy + win[w + 1] - lo[1] + j);
+        x0[r] = std::min(x0[r], win[w]);
+        x1[r] = std::max(x1[r], win[w] + 3);
+      }
+  long long N = 0;
+  for (size_t r = 0; r < x0.size(); ++r)
+    if (x0[r] <= x1[r]) N += ((x1[r] >> 2) - (x0[r] >> 2) + 1) * 4;
+  return {N, sy * sz};
+}
+
+// The launch shapes of the marker kernels, from up to 64 patches spread over
+// the order of their areas (the largest among them).  A patch that does not
+// fit takes the global path, at about 4.4 times the time of a staged one;
+// against two buffers, one buffer measured the same with the spread in the
+// kernel and 1.05 .. 1.08 without, 16 warps per SM 1.2 .. 1.3, and where there is
+// at most one block per SM the warps per SM do not matter.  The shape with the
+// least expected time is taken; a tenth of the nodes and rows is kept for the
+// bodies' motion.
+void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
+                          const std::vector<HostTopo>& topos, const std::vector<int>& body_topo,
+                          const std::vector<int4>& chunks, const std::vector<float>& area, int n_sm) {
+  const int n = (int)chunks.size(), m = std::min(n, 64), MT = c->marker_patch;
+  std::vector<int> order(n);
+  for (int k = 0; k < n; ++k) order[k] = k;
+  std::sort(order.begin(), order.end(), [&](int p, int q) { return area[p] < area[q]; });
+  for (int probe = 0; probe < 2; ++probe) {
+    int unfit[kMarkerShapes] = {};
+    for (int s = 0; s < m; ++s) {
+      const int k = order[m == 1 ? n - 1 : (int)((long long)s * (n - 1) / (m - 1))];
+      const int b = chunks[k].x;
+      const PatchNodes P = patch_nodes(c, bodies[b], topos[body_topo[b]], chunks[k], probe != 0);
+      for (int q = 0; q < kMarkerShapes; ++q) {
+        const MarkerShape M = marker_shape(q, MT, probe != 0);
+        if (P.nodes < 0 || P.nodes + P.nodes / 10 > M.nodes || P.rows + P.rows / 10 > M.rows)
+          ++unfit[q];
+      }
+    }
+    const bool few = n <= n_sm;
+    const double rel[kMarkerShapes] = {1.0, 1.05, few ? 1.05 : 1.25, few ? 1.0 : 2.2};
+    int best = 0;
+    double cost[kMarkerShapes];
+    for (int q = 0; q < kMarkerShapes; ++q) {
+      cost[q] = rel[q] * (1.0 + 3.4 * unfit[q] / m);
+      if (cost[q] < cost[best]) best = q;
+    }
+    c->mshape[probe] = marker_shape(best, MT, probe != 0);
+  }
+}
+
 void make_consts(ibm_ctx* c) {
   const ibm_params& p = c->prm;
   ibm::Grid& g = c->grid;
@@ -572,6 +660,11 @@ void make_consts(ibm_ctx* c) {
   c->sc.mu = (float)p.mu;
   c->sc.probe_h = (float)(p.probe_h > 0 ? p.probe_h : (h[0] + h[1] + h[2]) / 3.0);
   c->sc.kappa = (float)(1.0 / ((1.5 * alpha) * (1.5 * alpha)));
+  const double kappa = 1.0 / ((1.5 * alpha) * (1.5 * alpha));
+  c->sc.mk.z = (float)(2.0 * kappa / std::log(2.0));
+  c->sc.mk.ek = (float)std::exp(-kappa);
+  c->sc.mk.hk = (float)(0.5 / kappa);
+  for (int d = 0; d < 3; ++d) c->sc.kg[d] = (float)(2.0 * kappa / h[d]);
   c->sc.cl_scale = (float)(((h[0] + h[1] + h[2]) / 3.0) / (h[0] * h[1] * h[2]));
   c->sc.forward_euler = p.forward_euler ? 1 : 0;
   const char* st = std::getenv("IBM_TEST_STARVE_TX");
@@ -705,6 +798,7 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     }
     std::vector<uint8_t> clamp(V, 0);
     std::vector<int4> chunks;
+    std::vector<float> chunk_area;   // rest area of each marker patch
     std::vector<int2> work;
     std::vector<float> frest;        // force-kernel rest data per work item, patch order
     std::vector<int64_t> wrest;
@@ -827,8 +921,12 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
       R.chunk_off = (int32_t)chunks.size();
       const int nch = (int)T.mbound.size() - 1;
       R.n_chunk = nch;
-      for (int k = 0; k < nch; ++k)
+      for (int k = 0; k < nch; ++k) {
         chunks.push_back(make_int4(b, T.mbound[k], T.mbound[k + 1] - T.mbound[k], k));
+        double area = 0.0;
+        for (int q = T.mbound[k]; q < T.mbound[k + 1]; ++q) area += a0[T.mface[q]];
+        chunk_area.push_back((float)area);
+      }
       R.work_off = (int32_t)work.size();
       for (int q = 0; q < (int)T.patch.size(); ++q) {
         work.push_back(make_int2(b, q));
@@ -943,6 +1041,9 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     check_cuda(set_adjoint_smem_limit(c->adjoint_smem), "cudaFuncSetAttribute");
     check_cuda(set_marker_smem_limit(), "cudaFuncSetAttribute");
     c->vec4 = (grid->n[0] % 4 == 0) ? 1 : 0;
+    int n_sm = 0;
+    check_cuda(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device), "attr");
+    choose_marker_shapes(c, bodies, topos, body_topo, chunks, chunk_area, n_sm);
 
     DeviceTables& d = c->d;
     d.body = upload(c, c->h_body);
@@ -1020,9 +1121,8 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
       t.state = zeros<int32_t>(c, 8);
       t.mlist = zeros<int32_t>(c, (size_t)std::max<long long>(c->max_pairs, 1));
       t.rec = zeros<float4>(c, 2 * (size_t)F);
-      int per_sm = 0, n_sm = 0;
+      int per_sm = 0;
       check_cuda(tile_spread_occupancy(&per_sm), "occupancy");
-      check_cuda(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device), "attr");
       c->tile_grid = std::max(1, per_sm) * std::max(1, n_sm);
       check_cuda(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking), "cudaStreamCreate");
       check_cuda(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming), "cudaEventCreate");
@@ -1428,7 +1528,7 @@ extern "C" ibm_status ibm_flow_step(ibm_flow* fl, ibm_ctx* c, const float* x, co
       int2* rm = zeros<int2>(c, (size_t)kMaxRows * nc);
       int4* bx = zeros<int4>(c, 2 * nc);
       float4* fa = zeros<float4>(c, (size_t)2 * kMT * nc);
-      c->fc_tab = zeros<int32_t>(c, (size_t)kCacheWords * nc);   // set last: marks all four
+      c->fc_tab = zeros<int32_t>(c, (size_t)cache_words(c->mshape[0]) * nc);   // set last: marks all four
       c->fc_face = fa;
       c->fc_boxes = bx;
       c->fc_rowmap = rm;

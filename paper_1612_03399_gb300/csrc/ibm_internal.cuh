@@ -96,10 +96,19 @@ struct Grid {
   float h[3], invh[3];
 };
 
+// constants of the closed-form MLS factors (kappa = 1 / (1.5 alpha)^2)
+struct MlsK {
+  float z;               // 2 kappa log2(e): exponent of the weight ratios per cell of offset
+  float ek;              // e^-kappa
+  float hk;              // 1 / (2 kappa)
+};
+
 // scalars of one call
 struct StepConsts {
   float dt, inv_dt, mu, probe_h;
   float kappa;           // 1 / (1.5 alpha)^2: W = exp(-kappa * (delta in cells)^2) per direction
+  MlsK mk;
+  float kg[3];           // 2 kappa / h: gradients of the closed form to gradients per length
   float cl_scale;        // (hx + hy + hz) / 3 / (hx hy hz): c_l = A_l * cl_scale
   int32_t forward_euler;
   int32_t starve_tx;     // bytes announced to the bulk-copy barriers beyond the copies: 0 in
@@ -238,34 +247,55 @@ struct DeviceTables {
   int32_t* err = nullptr;       // device error word
 };
 
-// marker-kernel dynamic shared memory: row tables (5 int arrays of kMaxRows;
-// per staged float4 group its global offset and its row id), then two
-// staging buffers of kMaxNodes words (velocity components, double-buffered;
-// then the fixed-point spread accumulators of two force components)
-constexpr int kMaxRows = 4 * kMT;                                  // (y, z) rows per patch
-constexpr int kMaxNodes = 35 * kMT;                                // staged nodes per buffer
-// (the staged-row-start array has kMaxRows + 4 entries, so every array
-// starts on a 16-byte boundary)
-constexpr int kRowTableBytes =
-    ((4 * (5 * kMaxRows + 4) + 4 * (kMaxNodes / 4) + 2 * (kMaxNodes / 4)) + 15) / 16 * 16;
+// marker-kernel dynamic shared memory: per (y, z) row the byte offset of its
+// staged start minus 4 x its first x, and its first group (16 bits); per
+// staged float4 group its global offset; a bit per group that received a
+// nonzero spread; then one or two staging buffers (velocity components, and in
+// place of a component once it is used its fixed-point spread accumulators),
+// and the probe kernels' per-thread values.  While the rows are being found,
+// the first buffer holds their x-ranges.
+constexpr int kMaxRows = 4 * kMT;      // rows of a patch's footprint record
+__host__ __device__ constexpr int marker_mask_words(int nodes) {
+  return ((nodes / 4 + 31) / 32 + 4) & ~3;
+}
+constexpr int kOwn = 19;               // per-thread values of the probe kernels
+// Launch shape of a marker kernel: (y, z) rows of its table, staged nodes of a
+// buffer, staging buffers
+struct MarkerShape {
+  int rows, nodes, buffers;
+};
+__host__ __device__ constexpr int marker_smem_bytes(int MT, MarkerShape m, bool probe) {
+  return 4 * m.rows + 2 * (m.rows + 8) + 4 * marker_mask_words(m.nodes) + 4 * (m.nodes / 4) +
+         4 * m.buffers * m.nodes + (probe ? 4 * kOwn * MT : 0);
+}
+// The shapes a launch may take: 24 warps per SM (three 256-face or six
+// 128-face blocks, 75 KB and 37 KB each) with two buffers; with one buffer (the
+// next component's copies then start only when the current one is used up);
+// 16 warps per SM; or 8 warps per SM
+constexpr int kMarkerShapes = 4;
+__host__ __device__ constexpr MarkerShape marker_shape(int k, int MT, bool probe) {
+  return k == 0   ? MarkerShape{4 * MT, (probe ? 21 : 29) * MT, 2}
+         : k == 1 ? MarkerShape{4 * MT, (probe ? 38 : 52) * MT, 1}
+         : k == 2 ? MarkerShape{6 * MT, (probe ? 64 : 80) * MT, 1}
+                  : MarkerShape{6 * MT, (probe ? 84 : 92) * MT, 2};
+}
+__host__ __device__ constexpr int marker_smem_max(int MT, bool probe) {
+  return marker_smem_bytes(MT, marker_shape(3, MT, probe), probe);
+}
+static_assert(marker_smem_max(kMT, true) <= 226 * 1024 && marker_smem_max(kMT, false) <= 226 * 1024,
+              "a marker block's shared memory");
+constexpr int kTableRows = marker_shape(3, kMT, false).rows;     // of the largest shape
 // Per-chunk cache of the coupled forcing launch (the markers stay at x^n for
 // the three substeps of a coupled step): a 16-word header (x, y, z lo, x, y,
-// z size, staged nodes, fits), then three row arrays (kMaxRows words each:
-// staged offset - x0, row length, staged start), the groups' global offsets
-// (kMaxNodes / 4 words) and their row ids (kMaxNodes / 4 16-bit ids)
-constexpr int kCacheWords = 16 + 3 * kMaxRows + kMaxNodes / 4 + kMaxNodes / 8;
-constexpr int kMarkerSmemBytes = kRowTableBytes + 8 * kMaxNodes;
-// the same sizes for a marker patch of MT faces (kMaxRows, kMaxNodes and the
-// cache layout are those of the largest patch, kMT)
-__host__ __device__ constexpr int marker_rows(int MT) { return 4 * MT; }
-__host__ __device__ constexpr int marker_nodes(int MT) { return 35 * MT; }
-__host__ __device__ constexpr int marker_row_table_bytes(int MT) {
-  return ((4 * (5 * marker_rows(MT) + 4) + 6 * (marker_nodes(MT) / 4)) + 15) / 16 * 16;
+// z size, staged nodes, fits), the row offsets (a word per row of the table),
+// the rows' first groups (rows + 8 16-bit values) and the groups' global offsets
+__host__ __device__ constexpr int cache_groups_at(MarkerShape m) { return 16 + m.rows; }
+__host__ __device__ constexpr int cache_offsets_at(MarkerShape m) {
+  return cache_groups_at(m) + (m.rows + 8) / 2;
 }
-__host__ __device__ constexpr int marker_smem_bytes(int MT) {
-  return marker_row_table_bytes(MT) + 8 * marker_nodes(MT);
+__host__ __device__ constexpr int cache_words(MarkerShape m) {
+  return cache_offsets_at(m) + m.nodes / 4;
 }
-static_assert(marker_smem_bytes(kMT) == kMarkerSmemBytes, "marker layout");
 
 // elementwise combinations of [3][V] arrays for the strong-coupling integrator
 constexpr int kLinCombMax = 6;
@@ -306,10 +336,13 @@ __device__ __forceinline__ float2 body_coef(const BodyDev& B, unsigned long long
 struct ibm_ctx {
   int device = 0;
   int marker_patch = ibm::kMT;      // faces per marker-kernel block: 128 or 256
+  // launch shapes of the marker kernels without and with probes (chosen at
+  // creation from the rest meshes)
+  ibm::MarkerShape mshape[2] = {};
   // coupled forcing (allocated by the first ibm_flow_step with this context):
   // the per-chunk tables and per-face geometry of substep 0, and the forcing's
   // own footprint record for the clears between substeps
-  int32_t* fc_tab = nullptr;        // [n_chunks][kCacheWords]
+  int32_t* fc_tab = nullptr;        // [n_chunks][cache_words(mshape[0])]
   float4* fc_face = nullptr;        // [n_chunks][kMT][2] (centroid in cells, area), (V^b, ok)
   int4* fc_boxes = nullptr;         // [n_chunks][2]
   int2* fc_rowmap = nullptr;        // [n_chunks][kMaxRows]

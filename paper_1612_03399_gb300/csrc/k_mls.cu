@@ -6,27 +6,31 @@
 // recursive coordinate bisection of the rest mesh), one thread per face.
 // The block builds a ROW MAP of its grid footprint: for every (y, z) row of
 // the nodes its 3x3x3 supports (centroids and probe ends) touch, the x-range
-// touched, padded to whole groups of 4 nodes (float4-aligned when the grid
-// allows).  The velocity components are staged in shared memory with
-// asynchronous copies, two buffers in flight, and interpolated and
-// differentiated from there.  The spread then accumulates one force component
-// at a time in exact fixed point (32-bit shared atomics on two words, a
-// power-of-two scale per block and component) and flushes it with float4
-// global atomics; the rows that received a nonzero spread are recorded so the
-// next step's clear zeroes exactly those.  A patch whose footprint does not
-// fit takes the direct global path (scalar loads and float atomics) and
-// records its bounding box.
+// touched in whole groups of 4 nodes (float4-aligned when the grid allows),
+// found with one shared bit mask per row.  The velocity components are staged
+// in shared memory one after the other with asynchronous copies, differentiated
+// and interpolated from there, and each component's marker forces are spread as
+// soon as they are known, in place of the staged component: exact fixed point
+// (32-bit shared atomics, a power-of-two scale per block and component),
+// flushed with float4 global atomics.  The rows that received a nonzero spread
+// are recorded so the next step's clear zeroes exactly those.  A patch whose
+// footprint does not fit takes the direct global path (scalar loads and float
+// atomics) and records its bounding box.
 //
-// MLS with the linear basis and a weight that factorises over directions
-// (W = prod_d exp(-kappa delta_d^2), delta in cells) has an exact closed-form
-// solution of the 4x4 moment system: with per-direction normalised weights
-// a_d(s) = w_d(s)/S_d, mean mu_d and variance s2_d of the node offsets,
-//   phi(sx,sy,sz) = a_x a_y a_z (1 - beta_x - beta_y - beta_z),
-//   beta_d(s) = mu_d (delta_d(s) - mu_d) / s2_d.
-// Writing b_d = a_d beta_d, phi = a_x a_y a_z - b_x a_y a_z - a_x b_y a_z
-// - a_x a_y b_z, so value and full derivative are short tensor contractions of
-// the 27 node values.  Partition of unity holds exactly, so c_l reduces to
-// A_l (hx+hy+hz)/3 / (hx hy hz) on the uniform grid.
+// What bounds it: instruction issue and the shared-memory pipe (162 loads and
+// 81 atomics per face at about three conflicting words each), at the number
+// of warps that registers and shared memory allow; not HBM (20 % busy).
+// Hence the closed form in central moments (mls_closed_form.cuh; 20 % fewer
+// instructions), the spread right after the interpolation (its factors are
+// computed once), and 24 warps per SM: 80 registers, for which the probe
+// kernels keep what a component needs once or twice per thread in shared
+// memory.  Kept in local memory instead it cost more than the 24 warps gave:
+// next to 220 KB of shared memory little L1 is left for it.  Measured, this
+// kernel alone (us; before: 128 registers, 16 warps, spread after all three
+// components): whole step 437 -> 354 for 1000 drops (1.28 M faces) on 512^3,
+// 151 -> 117 for 460 k faces of uneven bodies, 147 -> 114 for a membrane of
+// 377 k faces; interpolation and spread 232 -> 170 and probes with body sums
+// 233 -> 162 for the 1000 drops on 256^3.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
@@ -41,35 +45,47 @@ namespace {
 // The global-memory path of a marker block whose footprint does not fit its
 // shared memory (rare): out of line, so that it does not crowd the
 // instruction cache of the staged path it sits beside.
-__device__ __noinline__ float value_global(const float* f, Grid g, int c0, int c1, int c2, DirW X,
-                                          DirW Y, DirW Z) {
-  const int c[3] = {c0, c1, c2};
-  return mls_value(f, GlobalRows{g}.at(c), X, Y, Z);
+// (body cell G: read again here, so that it is not kept for this path)
+__device__ __forceinline__ GlobalRows global_rows(const Grid& g, const BodyDev* b) {
+  return GlobalRows{g, {b->G[0], b->G[1], b->G[2]}};
 }
-__device__ __noinline__ float3 gradient_global(const float* f, Grid g, ProbeW P, float sgn) {
-  float gr[3] = {0.f, 0.f, 0.f};
-  P.add_gradient(f, GlobalRows{g}, g.invh, sgn, gr);
+__device__ __noinline__ float value_global(const float* f, Grid g, const BodyDev* b, int c0, int c1,
+                                          int c2, DirW X, DirW Y, DirW Z) {
+  const int c[3] = {c0, c1, c2};
+  return mls_value(f, global_rows(g, b).at(c), X, Y, Z);
+}
+__device__ __noinline__ float3 gradient_global(const float* f, Grid g, const BodyDev* b, ProbeW P) {
+  float gr[3];
+  mls_grad(f, global_rows(g, b).at(P.cc), P.X, P.Y, P.Z, gr);
   return make_float3(gr[0], gr[1], gr[2]);
 }
-__device__ __noinline__ void spread_global(float* f, Grid g, int c0, int c1, int c2, DirW X,
-                                           DirW Y, DirW Z, float coef) {
+__device__ __noinline__ void spread_global(float* f, Grid g, const BodyDev* b, int c0, int c1,
+                                           int c2, DirW X, DirW Y, DirW Z, float coef) {
   const int c[3] = {c0, c1, c2};
-  mls_spread(f, GlobalRows{g}.at(c), X, Y, Z, coef);
+  mls_spread(f, global_rows(g, b).at(c), X, Y, Z, coef);
 }
 
+// sum over the warp of 64-bit integers, as three 32-bit reductions (24, 24
+// and 16 bits: 32 addends cannot overflow the unsigned words)
+__device__ __forceinline__ long long warp_sum_i64(long long q) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)q & 0xffffffu);
+  const unsigned mid = __reduce_add_sync(0xffffffffu, (unsigned)(q >> 24) & 0xffffffu);
+  const int hi = __reduce_add_sync(0xffffffffu, (int)(q >> 48));
+  return (long long)lo + ((long long)mid << 24) + ((long long)hi << 48);
+}
 
 // REC (record mode): instead of spreading, write each marker's spread record
 // (centroid in cells, c_l F) and count it under the tiles of the tile-owned
 // spread, with the tile's largest |c_l F| per component
 template <int MT, bool MEASURE, bool INTERP, bool PROBE, bool SPREAD, bool REC>
-__global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
+__global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
     DeviceTables T, Grid g, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ v, const float* __restrict__ u, const float* __restrict__ vv,
     const float* __restrict__ w, const float* __restrict__ pr, const float* __restrict__ accel,
     float* __restrict__ U, float* __restrict__ Fm, const float* __restrict__ Fm_in,
     float* __restrict__ Fext, float* __restrict__ fx, float* __restrict__ fy,
-    float* __restrict__ fz, int record, int vec4, TileDev td, int tmode, float phi_bound_all,
-    int cache, int* __restrict__ cache_tab, float4* __restrict__ cache_face) {
+    float* __restrict__ fz, int record, int vec4, TileDev td, float phi_bound_all,
+    int cache, int* __restrict__ cache_tab, float4* __restrict__ cache_face, MarkerShape shape) {
   constexpr bool FIELD = INTERP || PROBE || SPREAD;
   // the coupled forcing launch (interpolation and spread at the centroids)
   // may save its face geometry and row tables (cache 1) and, in the later
@@ -78,24 +94,31 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
   const bool load = CACHEABLE && cache == 2;
   const bool save = CACHEABLE && cache == 1;
   constexpr bool VEL = INTERP || PROBE;
-  constexpr bool ROWMAP = VEL || (SPREAD && !REC);
+  constexpr bool FLUSH = SPREAD && !REC;      // spreads into the fields
+  constexpr bool ROWMAP = VEL || FLUSH;
   extern __shared__ __align__(16) unsigned char dyn[];
-  constexpr int MR = marker_rows(MT), MN = marker_nodes(MT);   // (y, z) rows, staged nodes
-  int* s_xmin = reinterpret_cast<int*>(dyn);   // [MR]  then: staged offset - x0
-  int* s_xmax = s_xmin + MR;                   // [MR]  then: row length
-  int* s_off = s_xmax + MR;                    // [MR + 4] staged row start
-  int* s_nzlo = s_off + MR + 4;                // [MR] first / last group of the row
-  int* s_nzhi = s_nzlo + MR;                   //   that received a nonzero spread
-  int* s_gofs = s_nzhi + MR;                   // [MN/4] global offset of each group
-  unsigned short* s_grow = reinterpret_cast<unsigned short*>(s_gofs + MN / 4);  // row ids
-  float* bufA = reinterpret_cast<float*>(dyn + marker_row_table_bytes(MT));
-  float* bufB = bufA + MN;
+  const int MR = shape.rows, mn = shape.nodes;  // (y, z) rows, staged nodes of a buffer
+  int* s_off4 = reinterpret_cast<int*>(dyn);   // [MR] 4 (staged start of the row - its first x)
+  unsigned short* s_grp = reinterpret_cast<unsigned short*>(s_off4 + MR);   // [MR + 1] first group
+  unsigned* s_mask = reinterpret_cast<unsigned*>(s_grp + MR + 8);    // a bit per group: nonzero
+  int* s_gofs = reinterpret_cast<int*>(s_mask + marker_mask_words(mn));   // [mn/4] global offsets
+  float* bufA = reinterpret_cast<float*>(s_gofs + mn / 4);
+  const bool dbl = shape.buffers == 2;         // two staging buffers
+  float* bufB = bufA + mn;
+  // probe kernels keep per-thread values that a component needs once or twice
+  // here, not in registers: probe end(s), normal, centroid velocity, a.n
+  float* s_own = bufA + shape.buffers * mn + threadIdx.x;      // [kOwn][MT]
+  unsigned* s_xbits = reinterpret_cast<unsigned*>(bufA);   // [MR] x-intervals each row touches,
+                                                           //  while the rows are found
   __shared__ int s_lo[3], s_hi[3];
   __shared__ int s_N;
   __shared__ int s_warp[MT / 32];
-  __shared__ int s_bmax[3];
+  __shared__ unsigned s_bmax[3];
   __shared__ __align__(8) unsigned long long s_bar;
   __shared__ unsigned long long s_q[2][MT / 32];   // per-warp fixed-point body sums
+  // what the end of the block needs again: body, its cell G, closed, patch
+  // record, faces
+  __shared__ int s_hdr[8];
 
   // a force kernel launched after this one may start once every block of
   // this grid runs (it waits for this grid's results before using them)
@@ -103,27 +126,35 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
   const int4 ch = T.chunks[blockIdx.x];  // body, face-list offset, count, chunk index in body
   const BodyDev B = T.body[ch.x];
   const TopoDev topo = T.topo[B.topo];
+  const int lane = threadIdx.x & 31;
   const bool active = threadIdx.x < ch.z;
+  if (threadIdx.x == 0) {
+    s_hdr[0] = ch.x;
+    s_hdr[1] = B.G[0];
+    s_hdr[2] = B.G[1];
+    s_hdr[3] = B.G[2];
+    s_hdr[4] = B.closed;
+    s_hdr[5] = B.chunk_off + ch.w;
+    s_hdr[6] = ch.z;
+  }
   if (FIELD && threadIdx.x < 3) {
     s_lo[threadIdx.x] = INT_MAX;
     s_hi[threadIdx.x] = INT_MIN;
-    s_bmax[threadIdx.x] = 0;
+    s_bmax[threadIdx.x] = 0u;
   }
   if (ROWMAP && !load) {
-    // every row's x-range and nonzero range start empty; done first, so that
-    // the stores overlap the geometry loads (the barriers of the bounding-box
-    // reduction make them visible)
-    for (int r = threadIdx.x; r < MR; r += blockDim.x) {
-      s_xmin[r] = INT_MAX;
-      s_xmax[r] = INT_MIN;
-      s_nzlo[r] = INT_MAX;
-      s_nzhi[r] = INT_MIN;
-    }
+    // every row starts empty; done first, so that the stores overlap the
+    // geometry loads (the barriers of the bounding-box reduction make them
+    // visible)
+    for (int q = threadIdx.x; q < MR / 4; q += MT)
+      reinterpret_cast<uint4*>(s_xbits)[q] = make_uint4(0u, 0u, 0u, 0u);
   }
+  if (FLUSH)
+    for (int r = threadIdx.x; r < marker_mask_words(mn); r += MT) s_mask[r] = 0u;
   float Af = 0.f, Vf = 0.f;
   float nrm[3] = {0.f, 0.f, 0.f}, area = 0.f;
   float tc[3] = {0.f, 0.f, 0.f}, tp[3] = {0.f, 0.f, 0.f}, tm[3] = {0.f, 0.f, 0.f};
-  float vb[3] = {0.f, 0.f, 0.f};     // centroid velocity (interpolation) or marker force
+  float vb[3] = {0.f, 0.f, 0.f};     // centroid velocity, or the given marker force; then F
   float am[3] = {0.f, 0.f, 0.f};     // marker acceleration
   bool ok = false;
   int gf = 0;
@@ -196,6 +227,21 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
       }
       if (!ok) atomicOr(T.err, ERR_NONFINITE);
     }
+    if (PROBE) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        s_own[d * MT] = tp[d];
+        s_own[(3 + d) * MT] = tm[d];
+        s_own[(6 + d) * MT] = nrm[d];
+        s_own[(9 + d) * MT] = vb[d];
+      }
+      s_own[12 * MT] = am[0] * nrm[0] + am[1] * nrm[1] + am[2] * nrm[2];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        s_own[(13 + d) * MT] = tc[d];
+        s_own[(16 + d) * MT] = 0.f;      // (G + G^T) n
+      }
+    }
     if (save) {
       cache_face[2 * ((size_t)blockIdx.x * kMT + threadIdx.x)] = make_float4(tc[0], tc[1], tc[2], area);
       cache_face[2 * ((size_t)blockIdx.x * kMT + threadIdx.x) + 1] =
@@ -206,7 +252,8 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
   // ---- per-body area and volume: exact fixed-point sums -------------------
   // q = rint(value * 2^e) per face (2^e from the rest value), summed per warp
   // and added with 64-bit integer atomics: the body's sum does not depend on
-  // the order of the additions
+  // the order of the additions.  The atomics follow the wait for the launch
+  // before this one (a footprint clear zeroes the sums).
   if (MEASURE) {
     long long qa = 0, qv = 0;
     if (active) {
@@ -218,14 +265,9 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
         atomicOr(T.err, ERR_NONFINITE);
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      qa += __shfl_xor_sync(0xffffffffu, qa, o);
-      qv += __shfl_xor_sync(0xffffffffu, qv, o);
-    }
-    // added to the body's sums after the wait below (a footprint clear
-    // launched before this kernel zeroes them)
-    if ((threadIdx.x & 31) == 0) {
+    qa = warp_sum_i64(qa);
+    qv = warp_sum_i64(qv);
+    if (lane == 0) {
       s_q[0][threadIdx.x >> 5] = (unsigned long long)qa;
       s_q[1][threadIdx.x >> 5] = (unsigned long long)qv;
     }
@@ -240,8 +282,8 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
   int N = 0;
   if (ROWMAP && load) {
     // the tables of substep 0 of this coupled step: header, then one bulk
-    // copy per row array and one for the group -> row table
-    const int* hd = cache_tab + (size_t)blockIdx.x * kCacheWords;
+    // copy per table
+    const int* hd = cache_tab + (size_t)blockIdx.x * cache_words(shape);
     xlo = hd[0];
     ylo = hd[1];
     zlo = hd[2];
@@ -254,22 +296,14 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
     if (threadIdx.x == 0) {
       mbar_init(&s_bar, 1);
       const unsigned rb = 4u * (unsigned)pad4(nrows);
+      const unsigned gb = fit ? 2u * (unsigned)((nrows + 1 + 7) & ~7) : 0u;
       const unsigned ob = fit ? 4u * (unsigned)pad4(N / 4) : 0u;
-      const unsigned gb = fit ? 2u * (unsigned)((N / 4 + 7) & ~7) : 0u;
-      mbar_arrive_tx(&s_bar, 3u * rb + ob + gb + (unsigned)sc.starve_tx);
+      mbar_arrive_tx(&s_bar, rb + gb + ob + (unsigned)sc.starve_tx);
       if (fit) {
-        const int* src = hd + 16;
-        bulk_load(s_xmin, src, rb, &s_bar);
-        bulk_load(s_xmax, src + kMaxRows, rb, &s_bar);
-        bulk_load(s_off, src + 2 * kMaxRows, rb, &s_bar);
-        bulk_load(s_gofs, src + 3 * kMaxRows, ob, &s_bar);
-        bulk_load(s_grow, src + 3 * kMaxRows + kMaxNodes / 4, gb, &s_bar);
+        bulk_load(s_off4, hd + 16, rb, &s_bar);
+        bulk_load(s_grp, hd + cache_groups_at(shape), gb, &s_bar);
+        bulk_load(s_gofs, hd + cache_offsets_at(shape), ob, &s_bar);
       }
-      s_off[MR] = N;
-    }
-    for (int r = threadIdx.x; r < nrows; r += blockDim.x) {
-      s_nzlo[r] = INT_MAX;
-      s_nzhi[r] = INT_MIN;
     }
     __syncthreads();   // barrier initialised
     if (!__syncthreads_and(mbar_wait(&s_bar, kCopyWaitClocks))) {
@@ -292,7 +326,7 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
         const float(&t)[3] = l == 0 ? tc : (l == 1 ? tp : tm);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const int f0 = B.G[d] + (int)floorf(t[d]);
+          const int f0 = (int)floorf(t[d]);   // relative to the body's cell
           mlo[d] = min(mlo[d], f0 - 2);    // generous: every support lies in f0-1 .. f0+2
           mhi[d] = max(mhi[d], f0 + 3);
         }
@@ -300,14 +334,11 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
     }
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        mlo[d] = min(mlo[d], __shfl_xor_sync(0xffffffffu, mlo[d], o));
-        mhi[d] = max(mhi[d], __shfl_xor_sync(0xffffffffu, mhi[d], o));
-      }
+      mlo[d] = __reduce_min_sync(0xffffffffu, mlo[d]);
+      mhi[d] = __reduce_max_sync(0xffffffffu, mhi[d]);
     }
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         atomicMin(&s_lo[d], mlo[d]);
@@ -324,6 +355,12 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
     const long long nrows = (long long)sy * sz;
     const bool rows_ok = nrows > 0 && nrows <= MR && sx <= 30000;
     if (rows_ok) {
+      // a row's touched x in a 32-bit mask, one bit per interval of 4 nodes
+      // (aligned to float4 in global memory when the grid allows vector
+      // access; 4 x 2^k nodes where the patch is longer than 32 of them)
+      const int xb = vec4 ? ((B.G[0] + xlo) & ~3) - B.G[0] : xlo;
+      int ks = 2;
+      while (((xlo + sx - 1 - xb) >> ks) >= 32) ++ks;
       if (mine) {
         // every component's support at a point with f = floor(tau) lies in
         // the 4x4x4 window f - 1 .. f + 2 (the nearest-node choice is exact
@@ -332,90 +369,85 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
         for (int l = 0; l < 3; ++l) {
           if ((l == 1 && !PROBE) || (l == 2 && !two)) continue;
           const float(&t)[3] = l == 0 ? tc : (l == 1 ? tp : tm);
-          const int fx0 = B.G[0] + (int)floorf(t[0]) - 1;
-          const int r0 = (B.G[1] + (int)floorf(t[1]) - 1 - ylo) +
-                         sy * (B.G[2] + (int)floorf(t[2]) - 1 - zlo);
+          const int fx0 = (int)floorf(t[0]) - 1 - xb;
+          const int r0 = ((int)floorf(t[1]) - 1 - ylo) + sy * ((int)floorf(t[2]) - 1 - zlo);
+          const unsigned bits = (1u << (fx0 >> ks)) | (1u << ((fx0 + 3) >> ks));
 #pragma unroll
           for (int k = 0; k < 4; ++k)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              atomicMin(&s_xmin[r0 + j + sy * k], fx0);
-              atomicMax(&s_xmax[r0 + j + sy * k], fx0 + 3);
-            }
+            for (int j = 0; j < 4; ++j) atomicOr(&s_xbits[r0 + j + sy * k], bits);
         }
       }
       __syncthreads();
-      // row lengths in whole groups of 4 nodes (aligned to float4 in global
-      // memory when the grid allows vector access) and their exclusive scan;
-      // thread t owns rows 4t .. 4t + 3 here
-      int len[4], st[4], run = 0;
+      // row lengths in whole groups of 4 nodes and their exclusive scan, four
+      // rows per thread and pass (rows past nrows stay empty)
+      int carry = 0;
+#pragma unroll 1
+      for (int p0 = 0; p0 < (int)nrows; p0 += 4 * MT) {
+        const int q4 = p0 / 4 + threadIdx.x;
+        const bool in = q4 < MR / 4;
+        int len[4], st[4], run = 0;
+        {
+          const uint4 m4 = in ? reinterpret_cast<const uint4*>(s_xbits)[q4] : make_uint4(0, 0, 0, 0);
+          const unsigned m[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int r = 4 * threadIdx.x + q;
-        int L = 0, a = 0;
-        if (r < (int)nrows && s_xmin[r] <= s_xmax[r]) {
-          a = s_xmin[r];
-          int b = s_xmax[r] + 1;
-          if (vec4) {
-            a &= ~3;             // floor to a multiple of 4 (two's complement)
-            b = (b + 3) & ~3;
-          } else {
-            b = a + ((b - a + 3) & ~3);
+          for (int q = 0; q < 4; ++q) {
+            const int f = __ffs(m[q]) - 1, l = 31 - __clz(m[q]);   // -1, -1 when empty
+            st[q] = xb + (f << ks);
+            len[q] = m[q] ? (l - f + 1) << ks : 0;
+            run += len[q];
           }
-          L = b - a;
         }
-        len[q] = L;
-        st[q] = a;
-        run += L;
-      }
-      // block exclusive scan of run
-      int incl = run;
+        int incl = run;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if ((threadIdx.x & 31) >= o) incl += t;
-      }
-      if ((threadIdx.x & 31) == 31) s_warp[threadIdx.x >> 5] = incl;
-      __syncthreads();
-      int base = 0;
-      for (int k = 0; k < (int)(threadIdx.x >> 5); ++k) base += s_warp[k];
-      int pos = base + incl - run;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int r = 4 * threadIdx.x + q;
-        if (r < MR) {
-          s_off[r] = pos;
-          s_xmax[r] = len[q];
-          s_xmin[r] = st[q];
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, incl, o);
+          if (lane >= o) incl += t;
         }
-        pos += len[q];
+        if (lane == 31) s_warp[threadIdx.x >> 5] = incl;
+        __syncthreads();
+        int pos = carry + incl - run;
+#pragma unroll
+        for (int k = 0; k < MT / 32; ++k) {
+          const int t = s_warp[k];
+          if (k < (int)(threadIdx.x >> 5)) pos += t;
+          carry += t;
+        }
+        if (in) {
+          int o4[4];
+          unsigned short gr[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            o4[q] = 4 * (pos - st[q]);
+            gr[q] = (unsigned short)min(pos / 4, 65535);
+            pos += len[q];
+          }
+          reinterpret_cast<int4*>(s_off4)[q4] = make_int4(o4[0], o4[1], o4[2], o4[3]);
+          reinterpret_cast<ushort4*>(s_grp)[q4] = make_ushort4(gr[0], gr[1], gr[2], gr[3]);
+          if (4 * q4 + 4 >= (int)nrows && 4 * q4 < (int)nrows)   // the end of the last row
+            s_grp[4 * q4 + 4] = (unsigned short)min(pos / 4, 65535);
+        }
+        if (p0 + 4 * MT < (int)nrows) __syncthreads();   // the warp sums are used again
       }
-      if (threadIdx.x == blockDim.x - 1) {
-        s_N = pos;
-        s_off[MR] = pos;
-      }
+      if (threadIdx.x == 0) s_N = carry;
       __syncthreads();
       N = s_N;
-      fit = N <= MN;
-      // per row, strided over the whole block: group -> row ids, global row
-      // offset, wrapped first x and staged offset - x0 (row r is (y, z) =
-      // (r % sy, r / sy), followed incrementally)
-      {
+      fit = N <= mn;
+      // the groups' global offsets, rows strided over the whole block (row r
+      // is (y, z) = (r % sy, r / sy), followed incrementally)
+      if (fit) {
         int yy = (int)threadIdx.x % sy, zz = (int)threadIdx.x / sy;
-        const int dy = (int)blockDim.x % sy, dz = (int)blockDim.x / sy;
-        for (int r = threadIdx.x; r < (int)nrows; r += blockDim.x) {
-          const int L = s_xmax[r];
-          if (L > 0) {
-            const int p0 = s_off[r], a = s_xmin[r];
-            const int base = (wrap(zlo + zz, g.n[2]) * g.n[1] + wrap(ylo + yy, g.n[1])) * g.n[0];
-            const int x0w = wrap(a, g.n[0]);
-            // groups past MN / 4 only occur when the block does not fit
-            const int q1 = min((p0 + L) / 4, MN / 4);
-            for (int k = p0 / 4; k < q1; ++k) {
-              s_grow[k] = (unsigned short)r;
-              s_gofs[k] = base + wrap_pos(x0w + 4 * (k - p0 / 4), g.n[0]);
+        const int dy = MT % sy, dz = MT / sy;
+        for (int r = threadIdx.x; r < (int)nrows; r += MT) {
+          const int k0 = s_grp[r], k1 = s_grp[r + 1];
+          if (k1 > k0) {
+            const int base = (wrap(B.G[2] + zlo + zz, g.n[2]) * g.n[1] +
+                              wrap(B.G[1] + ylo + yy, g.n[1])) * g.n[0];
+            int xg = wrap(B.G[0] + k0 * 4 - (s_off4[r] >> 2), g.n[0]);
+            for (int k = k0; k < k1; ++k) {
+              s_gofs[k] = base + xg;
+              xg = wrap_pos(xg + 4, g.n[0]);
             }
-            s_xmin[r] = p0 - a;
           }
           yy += dy;
           zz += dz;
@@ -429,7 +461,7 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
     if (!fit && threadIdx.x == 0) atomicAdd(T.stats, 1);
     __syncthreads();
     if (save) {
-      int* hd = cache_tab + (size_t)blockIdx.x * kCacheWords;
+      int* hd = cache_tab + (size_t)blockIdx.x * cache_words(shape);
       if (threadIdx.x == 0) {
         hd[0] = xlo;
         hd[1] = ylo;
@@ -442,39 +474,39 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
       }
       if (fit) {
         int* dst = hd + 16;
-        for (int r = threadIdx.x; r < sy * sz; r += blockDim.x) {
-          dst[r] = s_xmin[r];
-          dst[kMaxRows + r] = s_xmax[r];
-          dst[2 * kMaxRows + r] = s_off[r];
+        unsigned short* gg = reinterpret_cast<unsigned short*>(hd + cache_groups_at(shape));
+        for (int r = threadIdx.x; r <= sy * sz; r += MT) {
+          if (r < sy * sz) dst[r] = s_off4[r];
+          gg[r] = s_grp[r];
         }
-        unsigned short* gg = reinterpret_cast<unsigned short*>(dst + 3 * kMaxRows + kMaxNodes / 4);
-        for (int q = threadIdx.x; q < N / 4; q += blockDim.x) {
-          dst[3 * kMaxRows + q] = s_gofs[q];
-          gg[q] = s_grow[q];
-        }
+        dst = hd + cache_offsets_at(shape);
+        for (int q = threadIdx.x; q < N / 4; q += MT) dst[q] = s_gofs[q];
       }
     }
   }
   const RowTable RT{s_gofs, g.n[0], vec4};
-  const StagedRows SR{s_xmin, ylo, zlo, sy};
+  const StagedRows SR{dyn, -(ylo + sy * zlo), sy};
+  const int ofsA = (int)(reinterpret_cast<unsigned char*>(bufA) - dyn);
   const int ngroups = fit ? N / 4 : 0;
 
-  // ---- velocity: interpolation at the centroid, gradient at the probes -----
-  // The three components are staged in two buffers (u -> A, v -> B, w -> A),
-  // the copies of the next component in flight while the current one is used.
-  // Traction t = (G + G^T) n: component i yields (G n)_i and adds n_i G_i. to
-  // G^T n.
-  float Fl[3] = {vb[0], vb[1], vb[2]};   // marker force per component
-  if (VEL) {
-    float tGn[3] = {0.f, 0.f, 0.f}, tGTn[3] = {0.f, 0.f, 0.f};
-    // with a pressure field it is staged as a fourth component (u -> A,
-    // v -> B, w -> A, p -> B); the jump P = p+ - p- (open) or p (closed)
+  // ---- the components, one after the other ---------------------------------
+  // Velocity: interpolation at the centroid, gradient at the probes.  The
+  // components are staged in two buffers (u -> A, v -> B, w -> A, and with a
+  // pressure field p -> B), the next one's copies in flight while the current
+  // one is used.  Traction t = (G + G^T) n: component i yields (G n)_i and
+  // adds n_i G_i. to G^T n; the pressure jump P = p+ - p- (open) or p (closed).
+  // Spread: a component's marker forces are spread as soon as they are known,
+  // with the factors of the interpolation, in exact fixed point (one 32-bit
+  // word per staged node) in place of the component's staged velocity, and
+  // flushed with float4 global atomics.
+  if (FIELD && (VEL || FLUSH)) {
     const bool press = PROBE && pr != nullptr;
     float Pj = 0.f;
-    if (fit) {
-      stage_async(bufA, u, RT, ngroups);
+    const float cl = area * sc.cl_scale;
+    if (VEL && fit) {
+      stage_async<MT>(bufA, u, RT, ngroups);
       cp_async_commit();
-      stage_async(bufB, vv, RT, ngroups);
+      if (dbl) stage_async<MT>(bufB, vv, RT, ngroups);
       cp_async_commit();
     }
     // the components in a loop, not unrolled: the unrolled kernel measured
@@ -482,115 +514,193 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
 #pragma unroll 1
     for (int comp = 0; comp < (press ? 4 : 3); ++comp) {
       const float* velc = comp == 0 ? u : (comp == 1 ? vv : (comp == 2 ? w : pr));
-      const float* buf = (comp & 1) ? bufB : bufA;
-      // the centroid's factors first: their arithmetic overlaps the copies
-      // still in flight (the probe's as well would not fit in registers)
-      DirW CX, CY, CZ;
-      int ccC[3];
-      if (INTERP && mine && comp < 3) {
-        float t3[3];
-        locate(tc, comp, B.G, ccC, t3);
-        dir_weights(t3[0], sc.kappa, CX);
-        dir_weights(t3[1], sc.kappa, CY);
-        dir_weights(t3[2], sc.kappa, CZ);
-      }
-      if (fit) {
+      float* buf = (dbl && (comp & 1)) ? bufB : bufA;
+      const int obuf = ofsA + ((dbl && (comp & 1)) ? 4 * mn : 0);
+      if (VEL && fit) {
         // one later group (the next component) may still be in flight
-        if (comp < 2 || (comp == 2 && press)) cp_async_wait<1>(); else cp_async_wait<0>();
+        if (dbl && (comp < 2 || (comp == 2 && press))) cp_async_wait<1>(); else cp_async_wait<0>();
         __syncthreads();   // every thread's copies of this component have landed
       }
-      if (mine && comp == 3) {
-        // probe pressure p* and the correction h (Du/Dt).n, per side with its
-        // own normal: P = p*+ + h a.n (closed), p*+ - p*- + 2 h a.n (open)
-        const float an = am[0] * nrm[0] + am[1] * nrm[1] + am[2] * nrm[2];
+      float Fc = 0.f;      // this component of the marker force
+      if (PROBE && comp == 3) {
+        if (mine) {
+          // probe pressure p* and the correction h (Du/Dt).n, per side with its
+          // own normal: P = p*+ + h a.n (closed), p*+ - p*- + 2 h a.n (open)
+          const float an = s_own[12 * MT];
+#pragma unroll 1
+          for (int l = 0; l < (two ? 2 : 1); ++l) {
+            int cc[3];
+            float t3[3];
+            const float* o = s_own + 3 * l * MT;
+            const float t[3] = {o[0], o[MT], o[2 * MT]};
+            locate(t, 3, cc, t3);
+            DirW X, Y, Z;
+            dir_weights(t3[0], sc.mk, X);
+            dir_weights(t3[1], sc.mk, Y);
+            dir_weights(t3[2], sc.mk, Z);
+            const float ps = fit ? mls_value((const float*)nullptr, SR.at(cc, obuf), X, Y, Z)
+                                 : value_global(pr, g, T.body + s_hdr[0], cc[0], cc[1], cc[2], X, Y, Z);
+            Pj += (l == 0 ? 1.f : -1.f) * ps + sc.probe_h * an;
+          }
+        }
+        continue;
+      }
+      if (PROBE && mine) {
+        // open sheet: (tau+ - tau-) . n+
+        float gr[3] = {0.f, 0.f, 0.f};
 #pragma unroll 1
         for (int l = 0; l < (two ? 2 : 1); ++l) {
-          int cc[3];
-          float t3[3];
-          locate(l == 0 ? tp : tm, 3, B.G, cc, t3);
-          DirW X, Y, Z;
-          dir_weights(t3[0], sc.kappa, X);
-          dir_weights(t3[1], sc.kappa, Y);
-          dir_weights(t3[2], sc.kappa, Z);
-          const float ps = fit ? mls_value(buf, SR.at(cc), X, Y, Z)
-                               : value_global(pr, g, cc[0], cc[1], cc[2], X, Y, Z);
-          Pj += (l == 0 ? 1.f : -1.f) * ps + sc.probe_h * an;
-        }
-      } else if (mine) {
-        if (PROBE) {
-          // open sheet: (tau+ - tau-) . n+
-          float gr[3] = {0.f, 0.f, 0.f};
-          ProbeW P0;
-          P0.prepare(tp, comp, B.G, sc.kappa);
+          ProbeW P;
+          const float* o = s_own + 3 * l * MT;
+          const float t[3] = {o[0], o[MT], o[2 * MT]};
+          P.prepare(t, comp, sc.mk);
+          float q[3];
           if (fit) {
-            P0.add_gradient(buf, SR, g.invh, 1.f, gr);
+            mls_grad((const float*)nullptr, SR.at(P.cc, obuf), P.X, P.Y, P.Z, q);
           } else {
-            const float3 q = gradient_global(velc, g, P0, 1.f);
-            gr[0] += q.x;
-            gr[1] += q.y;
-            gr[2] += q.z;
+            const float3 q3 = gradient_global(velc, g, T.body + s_hdr[0], P);
+            q[0] = q3.x;
+            q[1] = q3.y;
+            q[2] = q3.z;
           }
-          if (two) {
-            ProbeW P1;
-            P1.prepare(tm, comp, B.G, sc.kappa);
-            if (fit) {
-              P1.add_gradient(buf, SR, g.invh, -1.f, gr);
-            } else {
-              const float3 q = gradient_global(velc, g, P1, -1.f);
-              gr[0] += q.x;
-              gr[1] += q.y;
-              gr[2] += q.z;
-            }
-          }
-          const float gn = gr[0] * nrm[0] + gr[1] * nrm[1] + gr[2] * nrm[2];
-          const float ni = comp == 0 ? nrm[0] : (comp == 1 ? nrm[1] : nrm[2]);
-          if (comp == 0) tGn[0] = gn;
-          if (comp == 1) tGn[1] = gn;
-          if (comp == 2) tGn[2] = gn;
 #pragma unroll
-          for (int j = 0; j < 3; ++j) tGTn[j] += ni * gr[j];
+          for (int j = 0; j < 3; ++j) gr[j] += l == 0 ? q[j] : -q[j];
         }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) gr[j] *= sc.kg[j];
+        const float n[3] = {s_own[6 * MT], s_own[7 * MT], s_own[8 * MT]};
+        const float gn = gr[0] * n[0] + gr[1] * n[1] + gr[2] * n[2];
+        const float ni = comp == 0 ? n[0] : (comp == 1 ? n[1] : n[2]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          s_own[(16 + j) * MT] = fmaf(ni, gr[j], s_own[(16 + j) * MT] + (comp == j ? gn : 0.f));
+      }
+      // the centroid's factors, for the interpolation and the spread (after the
+      // probes: what both need does not fit in registers)
+      DirW CX, CY, CZ;
+      int ccC[3];
+      if ((INTERP || FLUSH) && mine) {
+        float t3[3];
+        if (PROBE) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) tc[d] = s_own[(13 + d) * MT];
+        }
+        locate(tc, comp, ccC, t3);
+        dir_weights(t3[0], sc.mk, CX);
+        dir_weights(t3[1], sc.mk, CY);
+        dir_weights(t3[2], sc.mk, CZ);
+      }
+      if (mine) {
         if (INTERP) {
-          const float Ul = fit ? mls_value(buf, SR.at(ccC), CX, CY, CZ)
-                               : value_global(velc, g, ccC[0], ccC[1], ccC[2], CX, CY, CZ);
-          const float Fc = ((comp == 0 ? vb[0] : (comp == 1 ? vb[1] : vb[2])) - Ul) * sc.inv_dt;
-          if (comp == 0) Fl[0] = Fc;
-          if (comp == 1) Fl[1] = Fc;
-          if (comp == 2) Fl[2] = Fc;
+          const float Ul = fit ? mls_value((const float*)nullptr, SR.at(ccC, obuf), CX, CY, CZ)
+                               : value_global(velc, g, T.body + s_hdr[0], ccC[0], ccC[1], ccC[2], CX, CY, CZ);
+          const float Vb = PROBE ? s_own[(9 + comp) * MT]
+                                 : (comp == 0 ? vb[0] : (comp == 1 ? vb[1] : vb[2]));
+          Fc = (Vb - Ul) * sc.inv_dt;
+          if (REC && PROBE) s_own[(9 + comp) * MT] = Fc;   // kept for the record
+          if (REC && !PROBE) {
+            if (comp == 0) vb[0] = Fc;
+            if (comp == 1) vb[1] = Fc;
+            if (comp == 2) vb[2] = Fc;
+          }
           if (U) U[comp * F + gf] = Ul;
           if (Fm) Fm[comp * F + gf] = Fc;
+        } else if (FLUSH) {
+          Fc = comp == 0 ? vb[0] : (comp == 1 ? vb[1] : vb[2]);
         }
       }
-      if (fit && comp == 0) {
-        __syncthreads();   // buffer A is free again
-        stage_async(bufA, w, RT, ngroups);
-        cp_async_commit();
+      if (FLUSH) {
+        const float coef = mine ? cl * Fc : 0.f;
+        float* fc = comp == 0 ? fx : (comp == 1 ? fy : fz);
+        if (fit) {
+          // the block's largest |c_l F| (non-negative floats order as their
+          // bit patterns, a NaN above all)
+          const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(coef)));
+          if (lane == 0) atomicMax(&s_bmax[comp], wm);
+          __syncthreads();   // the maximum is known and the staged component used up
+          int4* acc4 = reinterpret_cast<int4*>(buf);
+          for (int q = threadIdx.x; q < ngroups; q += MT) acc4[q] = make_int4(0, 0, 0, 0);
+          __syncthreads();
+          const float bm = __uint_as_float(s_bmax[comp]) * phi_bound_all;
+          const bool fin = bm <= 3.0e38f;
+          if (!fin && threadIdx.x == 0) atomicOr(T.err, ERR_NONFINITE);
+          if (fin && bm > 0.f) {   // uniform over the block
+            // scale 2^k with every contribution below 2^22 (|c_l phi F| <= bm): a
+            // node takes at most MT <= 256 of them, so the sum stays below 2^30
+            const int k = max(min(22 - (ilogbf(bm) + 1), 120), -126);
+            if (coef != 0.f)
+              mls_spread_fixed(dyn, SR.at(ccC, obuf), CX, CY, CZ, coef * pow2f(k));
+            __syncthreads();
+            // The fields and the footprint record meet what the clear of this
+            // step writes, which may be the grid launched just before this one
+            // (this kernel may start while it still runs): wait for that grid
+            // to complete (immediate when nothing precedes programmatically).
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            const float inv = pow2f(-k);
+            for (int q0 = threadIdx.x - lane; q0 < ngroups; q0 += MT) {
+              const int q = q0 + lane;
+              const int4 a = q < ngroups ? acc4[q] : make_int4(0, 0, 0, 0);
+              const bool nz = (a.x | a.y | a.z | a.w) != 0;
+              const unsigned bal = __ballot_sync(0xffffffffu, nz);
+              if (lane == 0) s_mask[q0 >> 5] |= bal;
+              if (!nz) continue;
+              const float4 va = make_float4((float)a.x * inv, (float)a.y * inv, (float)a.z * inv,
+                                            (float)a.w * inv);
+              if (vec4) {
+                atomicAdd(reinterpret_cast<float4*>(fc + RT.node(q, 0)), va);
+              } else {
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) {
+                  const float xq = jj == 0 ? va.x : (jj == 1 ? va.y : (jj == 2 ? va.z : va.w));
+                  if (xq != 0.f) atomicAdd(fc + RT.node(q, jj), xq);
+                }
+              }
+            }
+          }
+        } else {
+          asm volatile("griddepcontrol.wait;" ::: "memory");
+          if (mine)
+            spread_global(fc, g, T.body + s_hdr[0], ccC[0], ccC[1], ccC[2], CX, CY, CZ, coef);
+        }
       }
-      if (fit && comp == 1 && press) {
-        __syncthreads();   // buffer B is free again
-        stage_async(bufB, pr, RT, ngroups);
+      // the next component into the buffer that is free again (with the spread,
+      // each thread copies into the groups it has just flushed)
+      const int next = comp + (dbl ? 2 : 1);
+      if (VEL && fit && next < (press ? 4 : 3)) {
+        if (!FLUSH) __syncthreads();
+        stage_async<MT>(buf, next == 1 ? vv : (next == 2 ? w : pr), RT, ngroups);
         cp_async_commit();
       }
     }
     if (PROBE && mine) {
       const float s = sc.mu * area;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) Fext[i * F + gf] = s * (tGn[i] + tGTn[i]) - area * Pj * nrm[i];
+      for (int i = 0; i < 3; ++i) {
+        const float t = s * s_own[(16 + i) * MT];
+        Fext[i * F + gf] = press ? t - area * Pj * s_own[(6 + i) * MT] : t;
+      }
     }
   }
 
   // ---- records of the tile-owned spread ------------------------------------
+  if (REC && !ROWMAP) __syncthreads();   // the header
   if (REC && active) {
     float4 r0 = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
     float4 r1 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (mine) {
       const float cl = area * sc.cl_scale;
-      r0 = make_float4(tc[0], tc[1], tc[2], __int_as_float(ch.x));
-      r1 = make_float4(cl * Fl[0], cl * Fl[1], cl * Fl[2], 0.f);
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        if (PROBE) {
+          vb[i] = s_own[(9 + i) * MT];
+          tc[i] = s_own[(13 + i) * MT];
+        }
+      r0 = make_float4(tc[0], tc[1], tc[2], __int_as_float(s_hdr[0]));
+      r1 = make_float4(cl * vb[0], cl * vb[1], cl * vb[2], 0.f);
       int tx[3], ty[3], tz[3];
-      const int nx_ = tiles_along(B.G[0] + (int)floorf(tc[0]), g.n[0], kTX, tx);
-      const int ny_ = tiles_along(B.G[1] + (int)floorf(tc[1]), g.n[1], kTY, ty);
-      const int nz_ = tiles_along(B.G[2] + (int)floorf(tc[2]), g.n[2], kTZ, tz);
+      const int nx_ = tiles_along(s_hdr[1] + (int)floorf(tc[0]), g.n[0], kTX, tx);
+      const int ny_ = tiles_along(s_hdr[2] + (int)floorf(tc[1]), g.n[1], kTY, ty);
+      const int nz_ = tiles_along(s_hdr[3] + (int)floorf(tc[2]), g.n[2], kTZ, tz);
       const unsigned m0 = __float_as_uint(fabsf(r1.x)), m1 = __float_as_uint(fabsf(r1.y)),
                      m2 = __float_as_uint(fabsf(r1.z));
       // reductions without a returned value: nothing waits on them
@@ -612,142 +722,80 @@ __global__ void __launch_bounds__(MT, 512 / MT) marker_kernel(
     td.rec[2 * (size_t)gf + 1] = r1;
   }
 
-  // Everything above reads only inputs.  What follows meets the footprint
-  // clear of the step, which may be the grid launched just before this one
-  // (this kernel may then start while the clear still runs): the body sums
-  // it zeroes, the fields and the footprint record.  Wait for that grid to
-  // complete (immediate when nothing precedes programmatically).
+  // the body sums and the footprint record meet what the clear writes, too
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (MEASURE && (threadIdx.x & 31) == 0 && (threadIdx.x >> 5) * 32 < ch.z) {
-    atomicAdd(T.qsum + 2 * ch.x, s_q[0][threadIdx.x >> 5]);
-    if (B.closed) atomicAdd(T.qsum + 2 * ch.x + 1, s_q[1][threadIdx.x >> 5]);
+  if (!FIELD) __syncthreads();   // the header
+  if (MEASURE && lane == 0 && (int)(threadIdx.x & ~31) < s_hdr[6]) {
+    const int b = s_hdr[0];
+    atomicAdd(T.qsum + 2 * b, s_q[0][threadIdx.x >> 5]);
+    if (s_hdr[4]) atomicAdd(T.qsum + 2 * b + 1, s_q[1][threadIdx.x >> 5]);
   }
-
-  // ---- spreading: exact fixed point, one 32-bit word per staged node and
-  // component; components 0 and 1 in one pass (buffers A and B), component 2
-  // in a second (A), each pass flushed with float4 global atomics ----------
-  if (SPREAD && !REC) {
-    const float cl = area * sc.cl_scale;
-    int* accA = reinterpret_cast<int*>(bufA);
-    int* accB = reinterpret_cast<int*>(bufB);
+  if (FLUSH && record) {
+    // footprint for the next step's clear: per row the x-range of the groups
+    // that received a nonzero spread, the bounding box (flag 1) otherwise
+    const int gc = s_hdr[5];
+    const int rows = sy * sz;
+    int count = rows;
     if (fit) {
-      if (VEL) __syncthreads();   // the velocity phase is done with the buffers
-      for (int q = threadIdx.x; q < ngroups; q += blockDim.x) {
-        reinterpret_cast<int4*>(accA)[q] = make_int4(0, 0, 0, 0);
-        reinterpret_cast<int4*>(accB)[q] = make_int4(0, 0, 0, 0);
+      // more rows than the record holds: only those that received something,
+      // in order (the record does not depend on the blocks' timing)
+      const bool compact = rows > kMaxRows;
+      int done = 0;
+      __syncthreads();   // every warp's bits
+      for (int p0 = 0; p0 < rows; p0 += MT) {
+        const int r = p0 + threadIdx.x;
+        int lo = 0, hi = -1;   // the row's groups
+        if (r < rows) {
+          lo = s_grp[r];
+          hi = s_grp[r + 1] - 1;
+        }
+        // first set bit at or after lo, last at or before hi, a word at a time
+        while (lo <= hi) {
+          const unsigned m = s_mask[lo >> 5] >> (lo & 31);
+          if (m) {
+            lo += __ffs(m) - 1;
+            break;
+          }
+          lo = (lo | 31) + 1;
+        }
+        while (hi >= lo) {
+          const unsigned m = s_mask[hi >> 5] << (31 - (hi & 31));
+          if (m) {
+            hi -= __clz(m);
+            break;
+          }
+          hi = (hi & ~31) - 1;
+        }
+        int2 e = make_int2(0, 0);
+        if (lo <= hi) {
+          const int L = min(4 * (hi - lo + 1), g.n[0]);
+          const int x0 = wrap(s_hdr[1] + 4 * lo - (s_off4[r] >> 2), g.n[0]);
+          e = make_int2(s_gofs[lo] - x0, x0 | (L << 16));
+        }
+        int at = r;
+        bool put = r < rows;
+        if (compact) {
+          const unsigned bal = __ballot_sync(0xffffffffu, lo <= hi);
+          if (lane == 0) s_warp[threadIdx.x >> 5] = __popc(bal);
+          __syncthreads();
+          at = done + __popc(bal & ((1u << lane) - 1u));
+          for (int k = 0; k < MT / 32; ++k) {
+            if (k < (int)(threadIdx.x >> 5)) at += s_warp[k];
+            done += s_warp[k];
+          }
+          __syncthreads();
+          put = lo <= hi && at < kMaxRows;
+        }
+        if (put) T.rowmap[(size_t)gc * kMaxRows + at] = e;
       }
+      if (compact) count = done;
     }
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const int c0 = 2 * pass, nc = pass == 0 ? 2 : 1;   // components c0 .. c0 + nc - 1
-      const float F0 = pass == 0 ? Fl[0] : Fl[2];
-      const float F1 = Fl[1];
-      if (fit) {
-        // per component, the block's bound on |c_l phi F| from the bound on
-        // |phi| (non-negative floats order as their bit patterns)
-        float b0 = mine ? fabsf(cl * F0) * phi_bound_all : 0.f;
-        float b1 = (mine && nc == 2) ? fabsf(cl * F1) * phi_bound_all : 0.f;
-        if (!(b0 <= 3.0e38f)) b0 = __int_as_float(0x7f800000);
-        if (!(b1 <= 3.0e38f)) b1 = __int_as_float(0x7f800000);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          b0 = fmaxf(b0, __shfl_xor_sync(0xffffffffu, b0, o));
-          b1 = fmaxf(b1, __shfl_xor_sync(0xffffffffu, b1, o));
-        }
-        if ((threadIdx.x & 31) == 0) {
-          atomicMax(&s_bmax[c0], __float_as_int(b0));
-          if (nc == 2) atomicMax(&s_bmax[1], __float_as_int(b1));
-        }
-        __syncthreads();   // also: the buffers are zero
-      }
-      float inv[2] = {0.f, 0.f};
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (j >= nc) break;
-        const int comp = j == 0 ? c0 : 1;
-        const float coef = cl * (j == 0 ? F0 : F1);
-        int cc[3];
-        DirW X, Y, Z;
-        if (mine) {
-          float t3[3];
-          locate(tc, comp, B.G, cc, t3);
-          dir_weights(t3[0], sc.kappa, X);
-          dir_weights(t3[1], sc.kappa, Y);
-          dir_weights(t3[2], sc.kappa, Z);
-        }
-        if (fit) {
-          const float bm = __int_as_float(s_bmax[comp]);
-          if (!(bm <= 3.0e38f)) {
-            if (threadIdx.x == 0) atomicOr(T.err, ERR_NONFINITE);
-            continue;   // uniform over the block
-          }
-          if (bm == 0.f) continue;   // nothing to spread for this component
-          // scale 2^k with every contribution below 2^22: a node takes at most
-          // MT <= 256 of them, so the sum stays below 2^30
-          const int k = min(22 - (ilogbf(bm) + 1), 120);
-          inv[j] = pow2f(-max(k, -126));
-          if (mine && coef != 0.f)
-            mls_spread_fixed1(j == 0 ? accA : accB, SR.at(cc), X, Y, Z, coef * pow2f(max(k, -126)));
-        } else if (mine) {
-          spread_global(comp == 0 ? fx : (comp == 1 ? fy : fz), g, cc[0], cc[1], cc[2], X, Y, Z,
-                        coef);
-        }
-      }
-      if (fit) {
-        __syncthreads();
-        float* fa = c0 == 0 ? fx : fz;
-        for (int q = threadIdx.x; q < ngroups; q += blockDim.x) {
-          const int4 a = reinterpret_cast<const int4*>(accA)[q];
-          const int4 b = nc == 2 ? reinterpret_cast<const int4*>(accB)[q] : make_int4(0, 0, 0, 0);
-          const bool na = (a.x | a.y | a.z | a.w) != 0, nb = (b.x | b.y | b.z | b.w) != 0;
-          if (!na && !nb) continue;
-          if (na) reinterpret_cast<int4*>(accA)[q] = make_int4(0, 0, 0, 0);
-          if (nb) reinterpret_cast<int4*>(accB)[q] = make_int4(0, 0, 0, 0);
-          const float4 va = make_float4((float)a.x * inv[0], (float)a.y * inv[0], (float)a.z * inv[0],
-                                        (float)a.w * inv[0]);
-          const float4 vb = make_float4((float)b.x * inv[1], (float)b.y * inv[1], (float)b.z * inv[1],
-                                        (float)b.w * inv[1]);
-          if (vec4) {
-            if (na) atomicAdd(reinterpret_cast<float4*>(fa + RT.node(q, 0)), va);
-            if (nb) atomicAdd(reinterpret_cast<float4*>(fy + RT.node(q, 0)), vb);
-          } else {
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj) {
-              const size_t o = RT.node(q, jj);
-              const float xa = jj == 0 ? va.x : (jj == 1 ? va.y : (jj == 2 ? va.z : va.w));
-              const float xb = jj == 0 ? vb.x : (jj == 1 ? vb.y : (jj == 2 ? vb.z : vb.w));
-              if (xa != 0.f) atomicAdd(fa + o, xa);
-              if (xb != 0.f) atomicAdd(fy + o, xb);
-            }
-          }
-          const int r = s_grow[q];
-          atomicMin(&s_nzlo[r], q);
-          atomicMax(&s_nzhi[r], q);
-        }
-        __syncthreads();   // buffers zero again before the next pass
-      }
-    }
-    if (record) {
-      // footprint for the next step's clear: per row the x-range of the groups
-      // that received a nonzero spread (staged), the bounding box (flag 1)
-      // otherwise
-      const int gc = B.chunk_off + ch.w;
-      if (fit) {
-        for (int r = threadIdx.x; r < sy * sz; r += blockDim.x) {
-          int2 e = make_int2(0, 0);
-          if (s_xmax[r] > 0 && s_nzlo[r] <= s_nzhi[r]) {
-            const int L = min(4 * (s_nzhi[r] - s_nzlo[r] + 1), g.n[0]);
-            const int go = s_gofs[s_nzlo[r]], x0 = go % g.n[0];
-            e = make_int2(go - x0, x0 | (L << 16));
-          }
-          T.rowmap[(size_t)gc * kMaxRows + r] = e;
-        }
-      }
-      if (threadIdx.x == 0) {
-        T.boxes[2 * gc] = make_int4(xlo, ylo, zlo, fit ? (vec4 ? 2 : 0) : 1);
-        T.boxes[2 * gc + 1] = make_int4(min(sx, g.n[0]), min(sy, g.n[1]), min(sz, g.n[2]),
-                                        fit ? sy * sz : 0);
-      }
+    if (threadIdx.x == 0) {
+      const bool box = !fit || count > kMaxRows;   // more rows than the record holds: its box
+      T.boxes[2 * gc] = make_int4(s_hdr[1] + xlo, s_hdr[2] + ylo, s_hdr[3] + zlo,
+                                  box ? 1 : (vec4 ? 2 : 0));
+      T.boxes[2 * gc + 1] = make_int4(min(sx, g.n[0]), min(sy, g.n[1]), min(sz, g.n[2]),
+                                      box ? 0 : count);
     }
   }
 }
@@ -858,7 +906,9 @@ cudaError_t launch_mt(ibm_ctx* c, const float* x, const float* v, const float* u
                       const float* w, const float* pr, const float* accel, float* U, float* Fm,
                       const float* Fm_in, float* Fext, float* fx, float* fy, float* fz,
                       int record, int tmode, const DeviceTables* tab, int cache, bool pdl) {
-  const size_t smem = (I || P || (S && !R)) ? marker_smem_bytes(MT) : 0;
+  const bool rows = I || P || (S && !R);
+  const MarkerShape ms = rows ? c->mshape[P ? 1 : 0] : MarkerShape{0, 0, 1};
+  const size_t smem = rows ? marker_smem_bytes(MT, ms, P) : 0;
   const int vec4 = c->vec4 && aligned16(u) && aligned16(vv) && aligned16(w) && aligned16(pr) &&
                    aligned16(fx) && aligned16(fy) && aligned16(fz);
   // pdl: launched as the programmatic dependent of the footprint clear just
@@ -875,8 +925,8 @@ cudaError_t launch_mt(ibm_ctx* c, const float* x, const float* v, const float* u
   cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, marker_kernel<MT, M, I, P, S, R>, tab ? *tab : c->d, c->grid,
                             c->sc, (int32_t)c->V, (int32_t)c->F, x, v, u, vv, w, pr, accel, U,
-                            Fm, Fm_in, Fext, fx, fy, fz, record, vec4, c->td, tmode,
-                            c->phi_bound, cache, c->fc_tab, c->fc_face);
+                            Fm, Fm_in, Fext, fx, fy, fz, record, vec4, c->td,
+                            c->phi_bound, cache, c->fc_tab, c->fc_face, ms);
 }
 
 // the marker kernel for the context's patch size (128 or 256 faces per block)
@@ -901,11 +951,12 @@ cudaError_t set_marker_smem_limit() {
 #define SET(M, I, P, S, R)                                                                   \
   if (e == cudaSuccess)                                                                      \
     e = cudaFuncSetAttribute(marker_kernel<kMT, M, I, P, S, R>,                              \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, kMarkerSmemBytes);  \
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,                    \
+                             marker_smem_max(kMT, P));               \
   if (e == cudaSuccess)                                                                      \
     e = cudaFuncSetAttribute(marker_kernel<128, M, I, P, S, R>,                              \
                              cudaFuncAttributeMaxDynamicSharedMemorySize,                    \
-                             marker_smem_bytes(128));
+                             marker_smem_max(128, P));
   SET(true, true, true, true, false)
   SET(true, false, true, false, false)
   SET(false, true, true, false, false)

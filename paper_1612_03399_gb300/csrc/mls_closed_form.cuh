@@ -1,15 +1,34 @@
 // Closed-form MLS shape functions of the factorised weight and their use on
-// 3x3x3 supports (Sec. 2.2, Eqs. mls..mls_Q), shared by the marker kernels.
+// 3x3x3 supports (Sec. 2.2, Eqs. mls..mls_Q), shared by the marker, tile-spread
+// and adjoint kernels.
 //
 // MLS with the linear basis and a weight that factorises over directions
 // (W = prod_d exp(-kappa delta_d^2), delta in cells) has an exact closed-form
-// solution of the 4x4 moment system: with per-direction normalised weights
-// a_d(s) = w_d(s)/S_d, mean mu_d and variance s2_d of the node offsets,
-//   phi(sx,sy,sz) = a_x a_y a_z (1 - beta_x - beta_y - beta_z),
-//   beta_d(s) = mu_d (delta_d(s) - mu_d) / s2_d.
-// Writing b_d = a_d beta_d, phi = a_x a_y a_z - b_x a_y a_z - a_x b_y a_z
-// - a_x a_y b_z, so value and full derivative are short tensor contractions of
-// the 27 node values.
+// solution of the 4x4 moment system.  Per direction, for the point at the
+// offset t in [-1/2, 1/2) from its nearest node and the nodes s = -1, 0, 1,
+// with the normalised weights a_s (sum 1), their mean m = sum a_s s, the
+// centred nodes e_s = s - m, the variance s2 = sum a_s e_s^2 and r = (m - t)/s2:
+//   phi(sx,sy,sz) = a_x a_y a_z (1 - r_x e_x - r_y e_y - r_z e_z).
+// Everything is a function of central moments, because the Gaussian weight has
+// da_s/dt = 2 kappa a_s e_s, hence dm/dt = 2 kappa s2.  With the node functions
+//   alpha = a_s,  gamma = a_s e_s,  delta = a_s (e_s^2 - s2)
+// (delta sums to 0 like gamma), so that d alpha/dt = 2 kappa gamma and
+// d gamma/dt = 2 kappa delta,
+//   phi       = aaa - r_x gaa - r_y aga - r_z aag,
+//   d phi/dtx = 2 kappa (h_x gaa - r_x daa - r_y gga - r_z gag)   (y, z alike),
+// a, g, d short for alpha, gamma, delta and h = 1 - dr/dt / (2 kappa)
+// = (1/(2 kappa) + r mu3)/s2, mu3 the third central moment.  A gradient needs
+// nine tensor sums of the three node functions instead of the sixteen
+// products of (a, b = a beta) and their derivatives, and the factors of a
+// direction take two exponentials, two reciprocals and about twenty
+// operations.
+//
+// The sums are formed from differences to the middle node (alpha sums to 1,
+// gamma and delta to 0): a constant offset of the field never enters a
+// product, so the gradient carries no rounding of the field's magnitude.
+// Against float64 the float32 gradient of a field of magnitude 1 with
+// increments of 5 % per cell is 1e-7 .. 1e-6 relative (6e-6 from the plain
+// weighted sums), the value 6e-8 (1.3e-7).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -21,64 +40,63 @@
 namespace ibm {
 namespace {
 
-struct DirW {
-  float a[3], b[3];
-};
-struct DirWD {
-  float a[3], b[3], da[3], db[3];
-};
-
-// per-direction closed-form MLS factors for the fractional offset tp in
-// [-1/2, 1/2) of the point from its nearest node (cells).  The weights enter
-// only through their ratios to the nearest node's,
-//   w(-1)/w(0) = exp(-kappa (1 + 2 tp)),  w(+1)/w(0) = exp(-kappa (1 - 2 tp)),
-// both in (0, 1], so two exponentials suffice and nothing overflows.
-__device__ __forceinline__ void dir_weights(float tp, float kappa, DirW& o) {
-  const float rm = __expf(-kappa * fmaf(2.f, tp, 1.f)), rp = __expf(-kappa * fmaf(-2.f, tp, 1.f));
-  const float invS = __fdividef(1.f, 1.f + rm + rp);
-  const float a0 = rm * invS, a1 = invS, a2 = rp * invS;
-  const float d0 = -1.f - tp, d1 = -tp, d2 = 1.f - tp;
-  const float mu = a0 * d0 + a1 * d1 + a2 * d2;
-  const float e0 = d0 - mu, e1 = d1 - mu, e2 = d2 - mu;
-  const float s2 = a0 * e0 * e0 + a1 * e1 * e1 + a2 * e2 * e2;
-  const float r = __fdividef(mu, s2);
-  o.a[0] = a0; o.a[1] = a1; o.a[2] = a2;
-  o.b[0] = a0 * r * e0; o.b[1] = a1 * r * e1; o.b[2] = a2 * r * e2;
+// 2^x and 1/x by the special-function unit.  Arguments are in its full
+// precision range: |x| <= 2 kappa log2(e) / 2, and sums of weights or variances
+// of at least the smallest normal number (below it the closed form has no
+// float32 value).
+__device__ __forceinline__ float ex2_fast(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rcp_fast(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
-// the same factors and their derivatives with respect to the point's
-// coordinate (in cells): the node offsets move as d delta / dt = -1, the
-// weight ratios as d rm / dt = -2 kappa rm, d rp / dt = 2 kappa rp
-__device__ __forceinline__ void dir_weights_d(float tp, float kappa, DirWD& o) {
-  const float d[3] = {-1.f - tp, -tp, 1.f - tp};
-  const float rm = __expf(-kappa * fmaf(2.f, tp, 1.f)), rp = __expf(-kappa * fmaf(-2.f, tp, 1.f));
-  const float w[3] = {rm, 1.f, rp};
-  const float dw[3] = {-2.f * kappa * rm, 0.f, 2.f * kappa * rp};
-  const float invS = __fdividef(1.f, 1.f + rm + rp);
-  const float dS = dw[0] + dw[2];
-  float a[3], da[3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    a[s] = w[s] * invS;
-    da[s] = (dw[s] - a[s] * dS) * invS;
-  }
-  const float mu = a[0] * d[0] + a[1] * d[1] + a[2] * d[2];
-  const float dmu = da[0] * d[0] + da[1] * d[1] + da[2] * d[2] - 1.f;
-  float e[3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) e[s] = d[s] - mu;
-  const float s2 = a[0] * e[0] * e[0] + a[1] * e[1] * e[1] + a[2] * e[2] * e[2];
-  const float ds2 = da[0] * e[0] * e[0] + da[1] * e[1] * e[1] + da[2] * e[2] * e[2];
-  const float inv_s2 = __fdividef(1.f, s2);
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    const float beta = mu * e[s] * inv_s2;
-    const float dbeta = (dmu * e[s] + mu * (-1.f - dmu)) * inv_s2 - beta * ds2 * inv_s2;
-    o.a[s] = a[s];
-    o.b[s] = a[s] * beta;
-    o.da[s] = da[s];
-    o.db[s] = da[s] * beta + a[s] * dbeta;
-  }
+// weights of one direction: a_s, and b_s = a_s r e_s of the outer nodes (the
+// middle one is -(b0 + b2))
+struct DirW {
+  float a0, a1, a2, b0, b2;
+};
+// node functions of one direction at the outer nodes, r and h
+struct DirG {
+  float a0, a2, c0, c2, g0, g2, r, h;
+};
+
+// The weights enter only through their ratios to the nearest node's,
+//   w(-1)/w(0) = e^-kappa 2^-z,  w(+1)/w(0) = e^-kappa 2^z,  z = 2 kappa log2(e) t,
+// both in (0, 1].
+__device__ __forceinline__ void dir_weights(float t, const MlsK& K, DirW& o) {
+  const float z = K.z * t;
+  const float rm = K.ek * ex2_fast(-z), rp = K.ek * ex2_fast(z);
+  o.a1 = rcp_fast(1.f + rm + rp);
+  o.a0 = rm * o.a1;
+  o.a2 = rp * o.a1;
+  const float m = o.a2 - o.a0;
+  const float s2 = fmaf(-m, m, o.a0 + o.a2);
+  const float r = (m - t) * rcp_fast(s2);
+  o.b0 = -r * fmaf(o.a0, m, o.a0);
+  o.b2 = r * fmaf(-o.a2, m, o.a2);
+}
+
+__device__ __forceinline__ void dir_grad(float t, const MlsK& K, DirG& o) {
+  const float z = K.z * t;
+  const float rm = K.ek * ex2_fast(-z), rp = K.ek * ex2_fast(z);
+  const float i = rcp_fast(1.f + rm + rp);
+  o.a0 = rm * i;
+  o.a2 = rp * i;
+  const float m = o.a2 - o.a0, q = o.a0 + o.a2;
+  const float s2 = fmaf(-m, m, q);
+  const float is2 = rcp_fast(s2);
+  o.r = (m - t) * is2;
+  o.c0 = -fmaf(o.a0, m, o.a0);
+  o.c2 = fmaf(-o.a2, m, o.a2);
+  o.g0 = -fmaf(o.c0, 1.f + m, o.a0 * s2);   // a0 e0^2 - a0 s2
+  o.g2 = fmaf(o.c2, 1.f - m, -o.a2 * s2);
+  const float mu3 = m * fmaf(-3.f, q, fmaf(2.f * m, m, 1.f));
+  o.h = fmaf(o.r, mu3, K.hk) * is2;
 }
 
 __device__ __forceinline__ int wrap(int i, int n) {
@@ -89,150 +107,143 @@ __device__ __forceinline__ int wrap(int i, int n) {
   return i < 0 ? i + n : i;
 }
 
-// Centre node (unwrapped global lattice index) and fractional offset of a
-// point, in every direction, on the lattice of velocity component `comp`
-// (node offset 0 along the component's own direction, 1/2 across it).
-__device__ __forceinline__ void locate(const float (&tau)[3], int comp, const int (&G)[3],
-                                       int (&c)[3], float (&tp)[3]) {
+// Centre node (lattice index relative to the cell G that tau is measured from)
+// and fractional offset of a point, in every direction, on the lattice of
+// velocity component `comp` (node offset 0 along the component's own
+// direction, 1/2 across it; comp 3: the cell centres).
+__device__ __forceinline__ void locate(const float (&tau)[3], int comp, int (&c)[3],
+                                       float (&tp)[3]) {
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const float u = tau[d] - (d == comp ? 0.f : 0.5f);
     const float cc = floorf(u + 0.5f);
     tp[d] = u - cc;
-    c[d] = G[d] + (int)cc;
+    c[d] = (int)cc;
   }
 }
 
-// addressing of a 3x3x3 support: rows (sy, sz), columns sx
+// addressing of a 3x3x3 support: row (sy, sz) of three nodes in x
 struct GlobalAcc {   // wrapped indices into a full [nz][ny][nx] field
   int ix[3], iy[3], iz[3];
   int nx, ny;
-  __device__ void init(const int (&c)[3], const Grid& g) {
+  __device__ __forceinline__ void init(const int (&c)[3], const int (&G)[3], const Grid& g) {
     nx = g.n[0];
     ny = g.n[1];
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-      ix[s] = wrap(c[0] - 1 + s, g.n[0]);
-      iy[s] = wrap(c[1] - 1 + s, g.n[1]);
-      iz[s] = wrap(c[2] - 1 + s, g.n[2]);
+      ix[s] = wrap(G[0] + c[0] - 1 + s, g.n[0]);
+      iy[s] = wrap(G[1] + c[1] - 1 + s, g.n[1]);
+      iz[s] = wrap(G[2] + c[2] - 1 + s, g.n[2]);
     }
   }
-  __device__ int row(int sy, int sz) const { return (iz[sz] * ny + iy[sy]) * nx; }
-  __device__ int col(int sx) const { return ix[sx]; }
-};
-struct RowAcc {      // indices into the rows staged in shared memory
-  const int* off;    // staged offset of row r, minus its first x
-  int ylo, zlo, sy;
-  int cx, cy, cz;    // support corner (centre - 1)
-  __device__ void init(const int (&c)[3], const int* off_minus_x0, int ylo_, int zlo_, int sy_) {
-    off = off_minus_x0;
-    ylo = ylo_;
-    zlo = zlo_;
-    sy = sy_;
-    cx = c[0] - 1;
-    cy = c[1] - 1;
-    cz = c[2] - 1;
+  __device__ __forceinline__ size_t row(int sy, int sz) const {
+    return ((size_t)iz[sz] * ny + iy[sy]) * nx;
   }
-  __device__ int row(int a, int b) const { return off[(cy + a - ylo) + sy * (cz + b - zlo)] + cx; }
-  __device__ int col(int s) const { return s; }
+  __device__ __forceinline__ void load(const float* __restrict__ f, int sy, int sz,
+                                       float (&u)[3]) const {
+    const float* r = f + row(sy, sz);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) u[s] = __ldg(r + ix[s]);
+  }
+};
+struct RowAcc {      // rows staged in shared memory
+  const unsigned char* sm;   // the block's shared memory; the row table lies at its start
+  int off;           // index of the table entry of the support's first row (centre - 1 in y, z)
+  int sy;            // rows per z plane of the table
+  int x4;            // byte offset of the buffer + 4 (centre x - 1)
+  // byte offset of row (a, b) of the support
+  __device__ __forceinline__ int row(int a, int b) const {
+    return reinterpret_cast<const int*>(sm)[off + a + sy * b] + x4;
+  }
+  __device__ __forceinline__ void load(const float*, int a, int b, float (&u)[3]) const {
+    const float* r = reinterpret_cast<const float*>(sm + row(a, b));
+    u[0] = r[0];
+    u[1] = r[1];
+    u[2] = r[2];
+  }
 };
 
-// The contractions below run x first (per row, the a- and b-weighted sums as
-// one pair in packed two-lane float arithmetic), then y within each z-plane,
-// then z:  U = sum_z [a_z (P1 - P2 - P3) - b_z P1],  P1 = sum_y a_y xa,
-// P2 = sum_y a_y xb, P3 = sum_y b_y xa.
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-
+// value: per row the a-sum A and the (a - b)-sum W, per plane S = sum_y a_y A
+// and T = sum_y (a_y W - b_y A), then sum_z (a_z T - b_z S)
 template <class Acc>
 __device__ __forceinline__ float mls_value(const float* __restrict__ f, const Acc& A, const DirW& X,
                                            const DirW& Y, const DirW& Z) {
-  const float2 ab0 = make_float2(X.a[0], X.b[0]), ab1 = make_float2(X.a[1], X.b[1]),
-               ab2 = make_float2(X.a[2], X.b[2]);
-  float q = 0.f;
+  const float w0 = X.a0 - X.b0, w2 = X.a2 - X.b2;
+  float S[3], T[3];
 #pragma unroll
   for (int sz = 0; sz < 3; ++sz) {
-    float2 P = make_float2(0.f, 0.f);
-    float P3 = 0.f;
+    float a[3], w[3];
 #pragma unroll
     for (int sy = 0; sy < 3; ++sy) {
-      const float* r = f + A.row(sy, sz);
-      const float u0 = r[A.col(0)], u1 = r[A.col(1)], u2 = r[A.col(2)];
-      float2 x2 = __ffma2_rn(ab0, f2(u0), make_float2(0.f, 0.f));
-      x2 = __ffma2_rn(ab1, f2(u1), x2);
-      x2 = __ffma2_rn(ab2, f2(u2), x2);
-      P = __ffma2_rn(f2(Y.a[sy]), x2, P);
-      P3 = fmaf(Y.b[sy], x2.x, P3);
+      float u[3];
+      A.load(f, sy, sz, u);
+      const float d0 = u[0] - u[1], d2 = u[2] - u[1];
+      a[sy] = fmaf(X.a2, d2, fmaf(X.a0, d0, u[1]));
+      w[sy] = fmaf(w2, d2, fmaf(w0, d0, u[1]));
     }
-    q = fmaf(Z.a[sz], P.x - P.y - P3, fmaf(-Z.b[sz], P.x, q));
+    const float d0 = a[0] - a[1], d2 = a[2] - a[1];
+    S[sz] = fmaf(Y.a2, d2, fmaf(Y.a0, d0, a[1]));
+    T[sz] = fmaf(Y.a2, w[2] - w[1], fmaf(Y.a0, w[0] - w[1], w[1]));
+    T[sz] = fmaf(-Y.b2, d2, fmaf(-Y.b0, d0, T[sz]));
   }
-  return q;
+  const float U = fmaf(Z.a2, T[2] - T[1], fmaf(Z.a0, T[0] - T[1], T[1]));
+  return fmaf(-Z.b2, S[2] - S[1], fmaf(-Z.b0, S[0] - S[1], U));
 }
 
+// sums of one z plane over (x, y): aa, ca, ac, ga, ag, cc (first letter x)
+struct PlaneG {
+  float aa, ca, ac, ga, ag, cc;
+};
 template <class Acc>
-__device__ __forceinline__ void mls_grad(const float* __restrict__ f, const Acc& A, const DirWD& X,
-                                         const DirWD& Y, const DirWD& Z, float (&g)[3]) {
-  const float2 ab0 = make_float2(X.a[0], X.b[0]), ab1 = make_float2(X.a[1], X.b[1]),
-               ab2 = make_float2(X.a[2], X.b[2]);
-  const float2 db0 = make_float2(X.da[0], X.db[0]), db1 = make_float2(X.da[1], X.db[1]),
-               db2 = make_float2(X.da[2], X.db[2]);
-  float gx = 0.f, gy = 0.f, gz = 0.f;
+__device__ __forceinline__ PlaneG plane_sums(const float* __restrict__ f, const Acc& A, int sz,
+                                             const DirG& X, const DirG& Y) {
+  float a[3], c[3], g[3];
 #pragma unroll
-  for (int sz = 0; sz < 3; ++sz) {
-    // per plane: P = sum_y a_y (xa, xb), P3 = sum_y b_y xa; the same with the
-    // x-derivative sums (Pd, Pd3) and with the y-derivative factors (Q, Q3)
-    float2 P = make_float2(0.f, 0.f), Pd = P, Q = P;
-    float P3 = 0.f, Pd3 = 0.f, Q3 = 0.f;
-#pragma unroll
-    for (int sy = 0; sy < 3; ++sy) {
-      const float* r = f + A.row(sy, sz);
-      const float u0 = r[A.col(0)], u1 = r[A.col(1)], u2 = r[A.col(2)];
-      float2 x2 = __ffma2_rn(ab0, f2(u0), make_float2(0.f, 0.f));
-      x2 = __ffma2_rn(ab1, f2(u1), x2);
-      x2 = __ffma2_rn(ab2, f2(u2), x2);
-      float2 d2 = __ffma2_rn(db0, f2(u0), make_float2(0.f, 0.f));
-      d2 = __ffma2_rn(db1, f2(u1), d2);
-      d2 = __ffma2_rn(db2, f2(u2), d2);
-      P = __ffma2_rn(f2(Y.a[sy]), x2, P);
-      P3 = fmaf(Y.b[sy], x2.x, P3);
-      Pd = __ffma2_rn(f2(Y.a[sy]), d2, Pd);
-      Pd3 = fmaf(Y.b[sy], d2.x, Pd3);
-      Q = __ffma2_rn(f2(Y.da[sy]), x2, Q);
-      Q3 = fmaf(Y.db[sy], x2.x, Q3);
-    }
-    gx = fmaf(Z.a[sz], Pd.x - Pd.y - Pd3, fmaf(-Z.b[sz], Pd.x, gx));
-    gy = fmaf(Z.a[sz], Q.x - Q.y - Q3, fmaf(-Z.b[sz], Q.x, gy));
-    gz = fmaf(Z.da[sz], P.x - P.y - P3, fmaf(-Z.db[sz], P.x, gz));
+  for (int sy = 0; sy < 3; ++sy) {
+    float u[3];
+    A.load(f, sy, sz, u);
+    const float d0 = u[0] - u[1], d2 = u[2] - u[1];
+    a[sy] = fmaf(X.a2, d2, fmaf(X.a0, d0, u[1]));
+    c[sy] = fmaf(X.c2, d2, X.c0 * d0);
+    g[sy] = fmaf(X.g2, d2, X.g0 * d0);
   }
-  g[0] = gx; g[1] = gy; g[2] = gz;
+  PlaneG P;
+  const float a0 = a[0] - a[1], a2 = a[2] - a[1];
+  const float c0 = c[0] - c[1], c2 = c[2] - c[1];
+  P.aa = fmaf(Y.a2, a2, fmaf(Y.a0, a0, a[1]));
+  P.ac = fmaf(Y.c2, a2, Y.c0 * a0);
+  P.ag = fmaf(Y.g2, a2, Y.g0 * a0);
+  P.ca = fmaf(Y.a2, c2, fmaf(Y.a0, c0, c[1]));
+  P.cc = fmaf(Y.c2, c2, Y.c0 * c0);
+  P.ga = fmaf(Y.a2, g[2] - g[1], fmaf(Y.a0, g[0] - g[1], g[1]));
+  return P;
 }
 
-// spread coef * phi onto the 27 nodes
+// full-derivative gradient in cells, divided by 2 kappa
 template <class Acc>
-__device__ __forceinline__ void mls_spread(float* f, const Acc& A, const DirW& X, const DirW& Y,
-                                           const DirW& Z, float coef) {
+__device__ __forceinline__ void mls_grad(const float* __restrict__ f, const Acc& A, const DirG& X,
+                                         const DirG& Y, const DirG& Z, float (&gr)[3]) {
+  const PlaneG P1 = plane_sums(f, A, 1, X, Y);
+  float caa = P1.ca, aca = P1.ac, aac = 0.f, gaa = P1.ga, aga = P1.ag, aag = 0.f, cca = P1.cc,
+        cac = 0.f, acc = 0.f;
 #pragma unroll
-  for (int sz = 0; sz < 3; ++sz) {
-#pragma unroll
-    for (int sy = 0; sy < 3; ++sy) {
-      float* r = f + A.row(sy, sz);
-      const float ay = Y.a[sy], by = Y.b[sy], az = Z.a[sz], bz = Z.b[sz];
-      const float t0 = ay * az * coef, t1 = (by * az + ay * bz) * coef;
-#pragma unroll
-      for (int sx = 0; sx < 3; ++sx)
-        atomicAdd(r + A.col(sx), (X.a[sx] - X.b[sx]) * t0 - X.a[sx] * t1);
-    }
+  for (int k = 0; k < 2; ++k) {
+    const PlaneG P = plane_sums(f, A, 2 * k, X, Y);
+    const float za = k ? Z.a2 : Z.a0, zc = k ? Z.c2 : Z.c0, zg = k ? Z.g2 : Z.g0;
+    const float daa = P.aa - P1.aa, dca = P.ca - P1.ca, dac = P.ac - P1.ac;
+    aac = fmaf(zc, daa, aac);
+    aag = fmaf(zg, daa, aag);
+    caa = fmaf(za, dca, caa);
+    cac = fmaf(zc, dca, cac);
+    aca = fmaf(za, dac, aca);
+    acc = fmaf(zc, dac, acc);
+    gaa = fmaf(za, P.ga - P1.ga, gaa);
+    aga = fmaf(za, P.ag - P1.ag, aga);
+    cca = fmaf(za, P.cc - P1.cc, cca);
   }
-}
-
-// full-derivative MLS gradient (in cells) of component `comp` at a point
-template <class Acc>
-__device__ __forceinline__ void grad_at(const float* f, const Acc& A, const float (&tp)[3],
-                                        float kappa, float (&gr)[3]) {
-  DirWD X, Y, Z;
-  dir_weights_d(tp[0], kappa, X);
-  dir_weights_d(tp[1], kappa, Y);
-  dir_weights_d(tp[2], kappa, Z);
-  mls_grad(f, A, X, Y, Z, gr);
+  gr[0] = fmaf(X.h, caa, -fmaf(X.r, gaa, fmaf(Y.r, cca, Z.r * cac)));
+  gr[1] = fmaf(Y.h, aca, -fmaf(Y.r, aga, fmaf(X.r, cca, Z.r * acc)));
+  gr[2] = fmaf(Z.h, aac, -fmaf(Z.r, aag, fmaf(X.r, cac, Y.r * acc)));
 }
 
 // x >= 0 folded into [0, n)
@@ -276,11 +287,13 @@ struct RowTable {
 };
 
 // issue the copies of one field component's staged rows into dst
+template <int MT>
 __device__ __forceinline__ void stage_async(float* dst, const float* __restrict__ src,
                                             const RowTable& R, int ngroups) {
-  for (int q = threadIdx.x; q < ngroups; q += blockDim.x) {
+#pragma unroll 1
+  for (int q = threadIdx.x; q < ngroups; q += MT) {
     if (R.vec4) {
-      cp_async16(dst + 4 * q, src + R.node(q, 0));   // x multiple of 4 and nx % 4 == 0
+      cp_async16(dst + 4 * q, src + R.gofs[q]);   // x multiple of 4 and nx % 4 == 0
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) cp_async4(dst + 4 * q + j, src + R.node(q, j));
@@ -288,81 +301,54 @@ __device__ __forceinline__ void stage_async(float* dst, const float* __restrict_
   }
 }
 
-// addressing factories: staged rows or the global field
+// addressing factories: staged rows (a table at the start of the shared memory
+// with, per (y, z) row, the byte offset of its staged start - 4 x its first x)
+// or the global field
 struct StagedRows {
-  const int* off_minus_x0;
-  int ylo, zlo, sy;
-  __device__ RowAcc at(const int (&c)[3]) const {
-    RowAcc A;
-    A.init(c, off_minus_x0, ylo, zlo, sy);
-    return A;
+  const unsigned char* sm;
+  int r0, sy;        // -(ylo + sy zlo): first row relative to the body's cell; rows per z plane
+  __device__ __forceinline__ RowAcc at(const int (&c)[3], int buf) const {
+    return RowAcc{sm, r0 + (c[1] - 1) + sy * (c[2] - 1), sy, buf + 4 * (c[0] - 1)};
   }
 };
 struct GlobalRows {
   Grid g;
-  __device__ GlobalAcc at(const int (&c)[3]) const {
+  int G[3];
+  __device__ __forceinline__ GlobalAcc at(const int (&c)[3]) const {
     GlobalAcc A;
-    A.init(c, g);
+    A.init(c, G, g);
     return A;
   }
 };
 
-// nearest node and derivative factors of one component at a probe point
+// nearest node and node functions of one component at a probe point
 struct ProbeW {
   int cc[3];
-  DirWD X, Y, Z;
-  __device__ __forceinline__ void prepare(const float (&t)[3], int comp, const int (&G)[3],
-                                          float kappa) {
+  DirG X, Y, Z;
+  __device__ __forceinline__ void prepare(const float (&t)[3], int comp, const MlsK& K) {
     float t3[3];
-    locate(t, comp, G, cc, t3);
-    dir_weights_d(t3[0], kappa, X);
-    dir_weights_d(t3[1], kappa, Y);
-    dir_weights_d(t3[2], kappa, Z);
-  }
-  // full-derivative gradient per unit length, times sgn, added to gr
-  template <class Rows>
-  __device__ __forceinline__ void add_gradient(const float* f, const Rows& R,
-                                               const float (&invh)[3], float sgn,
-                                               float (&gr)[3]) const {
-    float gl[3];
-    mls_grad(f, R.at(cc), X, Y, Z, gl);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) gr[j] += sgn * gl[j] * invh[j];
+    locate(t, comp, cc, t3);
+    dir_grad(t3[0], K, X);
+    dir_grad(t3[1], K, Y);
+    dir_grad(t3[2], K, Z);
   }
 };
 
-// bound on |phi| over the 27 nodes: phi = a_x a_y a_z - b_x a_y a_z - a_x b_y a_z
-// - a_x a_y b_z, so |phi| <= prod_d (max|a_d| + max|b_d|)
-__device__ __forceinline__ float phi_bound(const DirW& X, const DirW& Y, const DirW& Z) {
-  auto p = [](const DirW& W) {
-    return fmaxf(fmaxf(W.a[0], W.a[1]), W.a[2]) +
-           fmaxf(fmaxf(fabsf(W.b[0]), fabsf(W.b[1])), fabsf(W.b[2]));
-  };
-  return p(X) * p(Y) * p(Z);
-}
-
-// Spread in exact fixed point: the contribution coef*phi, already scaled by
-// the block's power of two so that |value| <= 2^38, is split into
-// hi = floor(value / 2^16) (|hi| <= 2^22) and lo = value - 2^16 hi in
-// [0, 2^16], each added with a native 32-bit shared atomic.  A node receives
-// at most kMT contributions, so neither word overflows, and the node's sum
-// 2^16 * sum(hi) + sum(lo) is independent of the order of the additions.
-__device__ __forceinline__ void mls_spread_fixed(int* hi, int* lo, const RowAcc& A, const DirW& X,
-                                                 const DirW& Y, const DirW& Z, float coef) {
+// spread coef * phi onto the 27 nodes of a full field
+__device__ __forceinline__ void mls_spread(float* f, const GlobalAcc& A, const DirW& X,
+                                           const DirW& Y, const DirW& Z, float coef) {
+  const float xa[3] = {X.a0, X.a1, X.a2}, xb[3] = {X.b0, -(X.b0 + X.b2), X.b2};
+  const float ya[3] = {Y.a0, Y.a1, Y.a2}, yb[3] = {Y.b0, -(Y.b0 + Y.b2), Y.b2};
+  const float za[3] = {Z.a0, Z.a1, Z.a2}, zb[3] = {Z.b0, -(Z.b0 + Z.b2), Z.b2};
 #pragma unroll
   for (int sz = 0; sz < 3; ++sz) {
 #pragma unroll
     for (int sy = 0; sy < 3; ++sy) {
-      const int r = A.row(sy, sz);
-      const float ay = Y.a[sy], by = Y.b[sy], az = Z.a[sz], bz = Z.b[sz];
-      const float t0 = ay * az * coef, t1 = (by * az + ay * bz) * coef;
+      float* r = f + A.row(sy, sz);
+      const float t0 = ya[sy] * za[sz] * coef, t1 = fmaf(yb[sy], za[sz], ya[sy] * zb[sz]) * coef;
 #pragma unroll
-      for (int sx = 0; sx < 3; ++sx) {
-        const float val = (X.a[sx] - X.b[sx]) * t0 - X.a[sx] * t1;
-        const float hf = floorf(val * (1.f / 65536.f));
-        atomicAdd(hi + r + sx, (int)hf);
-        atomicAdd(lo + r + sx, __float2int_rn(fmaf(-hf, 65536.f, val)));
-      }
+      for (int sx = 0; sx < 3; ++sx)
+        atomicAdd(r + A.ix[sx], fmaf(xa[sx], t0 - t1, -xb[sx] * t0));
     }
   }
 }
@@ -372,22 +358,22 @@ __device__ __forceinline__ void mls_spread_fixed(int* hi, int* lo, const RowAcc&
 // |value| < 2^22, rounded to an integer and added with a native shared
 // atomic; a node receives at most kMT contributions, so the word does not
 // overflow, and the sum is independent of the order of the additions.
-__device__ __forceinline__ void mls_spread_fixed1(int* acc, const RowAcc& A, const DirW& X,
-                                                  const DirW& Y, const DirW& Z, float coef) {
-  // nodes 0 and 1 of each row in packed two-lane arithmetic
-  const float2 d01 = make_float2(X.a[0] - X.b[0], X.a[1] - X.b[1]), a01 = make_float2(X.a[0], X.a[1]);
-  const float d2 = X.a[2] - X.b[2];
+__device__ __forceinline__ void mls_spread_fixed(unsigned char* sm, const RowAcc& A, const DirW& X,
+                                                 const DirW& Y, const DirW& Z, float coef) {
+  const float xb1 = -(X.b0 + X.b2);
+  const float ya[3] = {Y.a0, Y.a1, Y.a2}, yb[3] = {Y.b0, -(Y.b0 + Y.b2), Y.b2};
+  const float za[3] = {Z.a0 * coef, Z.a1 * coef, Z.a2 * coef};
+  const float zb[3] = {Z.b0 * coef, -(Z.b0 + Z.b2) * coef, Z.b2 * coef};
 #pragma unroll
   for (int sz = 0; sz < 3; ++sz) {
 #pragma unroll
     for (int sy = 0; sy < 3; ++sy) {
-      const int r = A.row(sy, sz);
-      const float ay = Y.a[sy], by = Y.b[sy], az = Z.a[sz], bz = Z.b[sz];
-      const float t0 = ay * az * coef, t1 = (by * az + ay * bz) * coef;
-      const float2 v01 = __ffma2_rn(d01, f2(t0), __fmul2_rn(a01, f2(-t1)));
-      atomicAdd(acc + r, __float2int_rn(v01.x));
-      atomicAdd(acc + r + 1, __float2int_rn(v01.y));
-      atomicAdd(acc + r + 2, __float2int_rn(fmaf(d2, t0, -X.a[2] * t1)));
+      int* r = reinterpret_cast<int*>(sm + A.row(sy, sz));
+      const float t0 = ya[sy] * za[sz], t1 = fmaf(yb[sy], za[sz], ya[sy] * zb[sz]);
+      const float t = t0 - t1;
+      atomicAdd(r, __float2int_rn(fmaf(X.a0, t, -X.b0 * t0)));
+      atomicAdd(r + 1, __float2int_rn(fmaf(X.a1, t, -xb1 * t0)));
+      atomicAdd(r + 2, __float2int_rn(fmaf(X.a2, t, -X.b2 * t0)));
     }
   }
 }

@@ -56,6 +56,7 @@ struct ibm_flow {
   // its taps g[d][|m|] per direction, m = 0..W
   int solve_w[3] = {-1, -1, -1};
   float taps[3][3][9] = {};
+  int rhs_planes = 16;          // planes per thread of the right-hand side kernel
   // phase timing (profiling aid): events at the 12 kernel boundaries of each
   // substep and the 3 of the body update
   bool timing = false;
@@ -277,6 +278,266 @@ __global__ void __launch_bounds__(256) project_kernel(FGrid G, Vec3 u, float* __
   const float lap = (Fip - 2.f * F + Fim) * G.ih2[0] + (Fjp - 2.f * F + Fjm) * G.ih2[1] +
                     (Fkp - 2.f * F + Fkm) * G.ih2[2];
   p[o] += F - a * lap;
+}
+
+// ---- four cells in x per thread --------------------------------------------
+// For grids of whole float4 rows (nx % 4 == 0, 16-byte aligned fields); the
+// one-cell kernels above serve the rest.  A plane's quads are numbered through
+// its rows, so ragged row lengths leave no idle threads.  Measured on 256^3
+// (us; one cell per thread before): right-hand side 206 -> 156 (127 in substep
+// 0), divergence 108 -> 69, projection 176 -> 115, at 5.6 .. 7.0 TB/s of what they
+// cannot do without; on 200 x 180 x 144: 72 -> 52, 25 -> 10, 54 -> 29.
+constexpr int kQuadThreads = 256;
+
+struct Quad {          // offsets of a quad's neighbours relative to its first cell
+  int o, xm, xp, yp, ym;   // in-plane offset; the cells before and after; the rows j +- 1
+  __device__ __forceinline__ Quad(int q, int nx, int ny) {
+    const int nx4 = nx >> 2, j = q / nx4, i = 4 * (q - j * nx4);
+    o = j * nx + i;
+    xm = i == 0 ? nx - 1 : -1;
+    xp = i + 4 == nx ? 4 - nx : 4;
+    yp = j == ny - 1 ? (1 - ny) * nx : nx;
+    ym = j == 0 ? (ny - 1) * nx : -nx;
+  }
+};
+__device__ __forceinline__ void ld4(float* d, const float* p) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  d[0] = t.x;
+  d[1] = t.y;
+  d[2] = t.z;
+  d[3] = t.w;
+}
+__device__ __forceinline__ void st4(float* p, const float* s) {
+  *reinterpret_cast<float4*>(p) = make_float4(s[0], s[1], s[2], s[3]);
+}
+
+// H(u) and the predictor's right-hand side as rhs_kernel, a thread walking a
+// column of quads over `planes` planes: of the plane above it loads each
+// field once and keeps what the next step needs of this plane in registers,
+// and the products on the (x, y), (x, z) and (y, z) edges serve both
+// components they appear in.  11 float4 and 9 single loads per four cells
+// instead of 34 loads per cell: rhs_kernel was bound by the issue of loads
+// and index arithmetic (80 G cells/s whether its fields came from L2 or HBM).
+template <bool PREV>
+__global__ void __launch_bounds__(kQuadThreads, 2)
+    rhs4_kernel(FGrid G, const float* __restrict__ u, const float* __restrict__ v,
+                const float* __restrict__ w, const float* __restrict__ p,
+                const float* __restrict__ Hp, float* __restrict__ Ho, float* __restrict__ Ro,
+                float gam, float rho, float alpha, float nu, float dt, int planes) {
+  const int q = blockIdx.x * kQuadThreads + threadIdx.x;
+  const int plane = G.nx * G.ny;
+  if (q >= plane / 4) return;
+  const size_t N = (size_t)plane * G.nz;
+  const Quad Q(q, G.nx, G.ny);
+  const int k0 = blockIdx.y * planes, k1 = min(k0 + planes, G.nz);
+  const int oym = Q.o + Q.ym, oyp = Q.o + Q.yp;
+  // u, v, w of this plane with both x neighbours: index 1 is the quad's first cell
+  float U[6], V[6], W[6], Ukm[5], Vkm[4], Vjpkm[4], Wkm[4], Wjm[4], Pkm[4];
+  {
+    const size_t c = (size_t)k0 * plane, m = (size_t)(k0 == 0 ? G.nz - 1 : k0 - 1) * plane;
+    ld4(U + 1, u + c + Q.o);
+    U[0] = __ldg(u + c + Q.o + Q.xm);
+    U[5] = __ldg(u + c + Q.o + Q.xp);
+    ld4(V + 1, v + c + Q.o);
+    V[0] = __ldg(v + c + Q.o + Q.xm);
+    V[5] = __ldg(v + c + Q.o + Q.xp);
+    ld4(W + 1, w + c + Q.o);
+    W[0] = __ldg(w + c + Q.o + Q.xm);
+    W[5] = __ldg(w + c + Q.o + Q.xp);
+    ld4(Ukm, u + m + Q.o);
+    Ukm[4] = __ldg(u + m + Q.o + Q.xp);
+    ld4(Vkm, v + m + Q.o);
+    ld4(Vjpkm, v + m + oyp);
+    ld4(Wkm, w + m + Q.o);
+    ld4(Wjm, w + c + oym);
+    ld4(Pkm, p + m + Q.o);
+  }
+#pragma unroll 1
+  for (int k = k0; k < k1; ++k) {
+    const size_t c = (size_t)k * plane, n = (size_t)(k + 1 == G.nz ? 0 : k + 1) * plane;
+    float Un[6], Vn[6], Wn[6], Wjmn[4], Ujp[4], Ujm[5], Vjp[5], Vjm[4], Wjp[4], P[5], Pjm[4];
+    ld4(Un + 1, u + n + Q.o);
+    Un[0] = __ldg(u + n + Q.o + Q.xm);
+    Un[5] = __ldg(u + n + Q.o + Q.xp);
+    ld4(Vn + 1, v + n + Q.o);
+    Vn[0] = __ldg(v + n + Q.o + Q.xm);
+    Vn[5] = __ldg(v + n + Q.o + Q.xp);
+    ld4(Wn + 1, w + n + Q.o);
+    Wn[0] = __ldg(w + n + Q.o + Q.xm);
+    Wn[5] = __ldg(w + n + Q.o + Q.xp);
+    ld4(Wjmn, w + n + oym);
+    ld4(Ujp, u + c + oyp);
+    ld4(Ujm, u + c + oym);
+    Ujm[4] = __ldg(u + c + oym + Q.xp);
+    ld4(Vjp + 1, v + c + oyp);
+    Vjp[0] = __ldg(v + c + oyp + Q.xm);
+    ld4(Vjm, v + c + oym);
+    ld4(Wjp, w + c + oyp);
+    ld4(P + 1, p + c + Q.o);
+    P[0] = __ldg(p + c + Q.o + Q.xm);
+    ld4(Pjm, p + c + oym);
+    float xy[5], xz[5], uu[5];   // four times the products at this quad's edges and centres
+#pragma unroll
+    for (int e = 0; e < 5; ++e) {
+      const float vs = V[e] + V[e + 1], ws = W[e] + W[e + 1], us = U[e] + U[e + 1];
+      xy[e] = (Ujm[e] + U[e + 1]) * vs;
+      xz[e] = (Ukm[e] + U[e + 1]) * ws;
+      uu[e] = us * us;
+    }
+    const float qx = 0.25f * G.ih[0], qy = 0.25f * G.ih[1], qz = 0.25f * G.ih[2];
+    float H[4], R[4];
+    auto put = [&](int comp, const float (&Hv)[4], const float (&Rv)[4]) {
+      const size_t at = comp * N + c + Q.o;
+      float r[4];
+      float h4[4] = {0.f, 0.f, 0.f, 0.f};
+      if (PREV) ld4(h4, Hp + at);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) r[e] = dt * (PREV ? fmaf(rho, h4[e], Rv[e]) : Rv[e]);
+      st4(Ho + at, Hv);
+      st4(Ro + at, r);
+    };
+    const float an = alpha * nu;
+    // u nodes
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float C = U[e + 1];
+      const float yy = (Ujp[e] + C) * (Vjp[e] + Vjp[e + 1]) - xy[e];
+      const float zz = (Un[e + 1] + C) * (Wn[e] + Wn[e + 1]) - xz[e];
+      H[e] = -(qx * (uu[e + 1] - uu[e]) + qy * yy + qz * zz);
+      const float L = (U[e + 2] - 2.f * C + U[e]) * G.ih2[0] + (Ujp[e] - 2.f * C + Ujm[e]) * G.ih2[1] +
+                      (Un[e + 1] - 2.f * C + Ukm[e]) * G.ih2[2];
+      R[e] = gam * H[e] - alpha * ((P[e + 1] - P[e]) * G.ih[0]) + an * L;
+    }
+    put(0, H, R);
+    // v nodes; the (y, z) edge products
+    float yz[4], yzn[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float C = V[e + 1];
+      yz[e] = (Vkm[e] + C) * (Wjm[e] + W[e + 1]);
+      yzn[e] = (Vn[e + 1] + C) * (Wjmn[e] + Wn[e + 1]);
+      const float sp = C + Vjp[e + 1], sm = Vjm[e] + C;
+      H[e] = -(qx * (xy[e + 1] - xy[e]) + qy * (sp * sp - sm * sm) + qz * (yzn[e] - yz[e]));
+      const float L = (V[e + 2] - 2.f * C + V[e]) * G.ih2[0] +
+                      (Vjp[e + 1] - 2.f * C + Vjm[e]) * G.ih2[1] +
+                      (Vn[e + 1] - 2.f * C + Vkm[e]) * G.ih2[2];
+      R[e] = gam * H[e] - alpha * ((P[e + 1] - Pjm[e]) * G.ih[1]) + an * L;
+    }
+    put(1, H, R);
+    // w nodes
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float C = W[e + 1];
+      const float yy = (Vjpkm[e] + Vjp[e + 1]) * (C + Wjp[e]) - yz[e];
+      const float sp = C + Wn[e + 1], sm = Wkm[e] + C;
+      H[e] = -(qx * (xz[e + 1] - xz[e]) + qy * yy + qz * (sp * sp - sm * sm));
+      const float L = (W[e + 2] - 2.f * C + W[e]) * G.ih2[0] + (Wjp[e] - 2.f * C + Wjm[e]) * G.ih2[1] +
+                      (Wn[e + 1] - 2.f * C + Wkm[e]) * G.ih2[2];
+      R[e] = gam * H[e] - alpha * ((P[e + 1] - Pkm[e]) * G.ih[2]) + an * L;
+    }
+    put(2, H, R);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      Ukm[e] = U[e + 1];
+      Vkm[e] = V[e + 1];
+      Vjpkm[e] = Vjp[e + 1];
+      Wkm[e] = W[e + 1];
+      Wjm[e] = Wjmn[e];
+      Pkm[e] = P[e + 1];
+    }
+    Ukm[4] = U[5];
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+      U[e] = Un[e];
+      V[e] = Vn[e];
+      W[e] = Wn[e];
+    }
+  }
+}
+
+// div(u* + s f) as div_kernel
+template <bool FORCED>
+__global__ void __launch_bounds__(kQuadThreads) div4_kernel(FGrid G, CVec3 u, CVec3 f, float s,
+                                                            float* __restrict__ out) {
+  const int q = blockIdx.x * kQuadThreads + threadIdx.x;
+  const int plane = G.nx * G.ny;
+  if (q >= plane / 4) return;
+  const Quad Q(q, G.nx, G.ny);
+  const int k = blockIdx.y;
+  const size_t o = (size_t)k * plane + Q.o;
+  const size_t on = (size_t)(k + 1 == G.nz ? 0 : k + 1) * plane + Q.o;
+  float a[5], b[4], bp[4], c[4], cp[4], d[4];
+  ld4(a, u.c[0] + o);
+  a[4] = __ldg(u.c[0] + o + Q.xp);
+  ld4(b, u.c[1] + o);
+  ld4(bp, u.c[1] + o + Q.yp);
+  ld4(c, u.c[2] + o);
+  ld4(cp, u.c[2] + on);
+  if (FORCED) {
+    float fa[5], fb[4], fbp[4], fc[4], fcp[4];
+    ld4(fa, f.c[0] + o);
+    fa[4] = __ldg(f.c[0] + o + Q.xp);
+    ld4(fb, f.c[1] + o);
+    ld4(fbp, f.c[1] + o + Q.yp);
+    ld4(fc, f.c[2] + o);
+    ld4(fcp, f.c[2] + on);
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      d[e] = s * ((fa[e + 1] - fa[e]) * G.ih[0] + (fbp[e] - fb[e]) * G.ih[1] +
+                  (fcp[e] - fc[e]) * G.ih[2]);
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float t = (a[e + 1] - a[e]) * G.ih[0] + (bp[e] - b[e]) * G.ih[1] + (cp[e] - c[e]) * G.ih[2];
+    d[e] = FORCED ? t + d[e] : t;
+  }
+  st4(out + o, d);
+}
+
+// u = u* + s f - alpha dt grad(phi); p <- p + phi - a lap(phi), as project_kernel
+template <bool FORCED>
+__global__ void __launch_bounds__(kQuadThreads)
+    project4_kernel(FGrid G, Vec3 u, float* __restrict__ p, const float* __restrict__ phi, CVec3 f,
+                    float s, float adt, float a) {
+  const int q = blockIdx.x * kQuadThreads + threadIdx.x;
+  const int plane = G.nx * G.ny;
+  if (q >= plane / 4) return;
+  const Quad Q(q, G.nx, G.ny);
+  const int k = blockIdx.y;
+  const size_t o = (size_t)k * plane + Q.o;
+  const size_t on = (size_t)(k + 1 == G.nz ? 0 : k + 1) * plane + Q.o;
+  const size_t om = (size_t)(k == 0 ? G.nz - 1 : k - 1) * plane + Q.o;
+  float F[6], Fjm[4], Fjp[4], Fkm[4], Fkp[4], val[4], fr[4];
+  ld4(F + 1, phi + o);
+  F[0] = __ldg(phi + o + Q.xm);
+  F[5] = __ldg(phi + o + Q.xp);
+  ld4(Fjm, phi + o + Q.ym);
+  ld4(Fjp, phi + o + Q.yp);
+  ld4(Fkm, phi + om);
+  ld4(Fkp, phi + on);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float4 t = *reinterpret_cast<const float4*>(u.c[c] + o);
+    const float us[4] = {t.x, t.y, t.z, t.w};
+    if (FORCED) ld4(fr, f.c[c] + o);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float lo = c == 0 ? F[e] : (c == 1 ? Fjm[e] : Fkm[e]);
+      val[e] = us[e] - adt * ((F[e + 1] - lo) * G.ih[c]);
+      if (FORCED) val[e] += s * fr[e];
+    }
+    st4(u.c[c] + o, val);
+  }
+  const float4 t = *reinterpret_cast<const float4*>(p + o);
+  const float ps[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float C = F[e + 1];
+    const float lap = (F[e + 2] - 2.f * C + F[e]) * G.ih2[0] + (Fjp[e] - 2.f * C + Fjm[e]) * G.ih2[1] +
+                      (Fkp[e] - 2.f * C + Fkm[e]) * G.ih2[2];
+    val[e] = ps[e] + (C - a * lap);
+  }
+  st4(p + o, val);
 }
 
 // asynchronous 4- and 8-byte global -> shared copies
@@ -548,6 +809,37 @@ dim3 cell_grid(const ibm_flow* fl) {
   return dim3((unsigned)((fl->n[0] + 31) / 32), (unsigned)((fl->n[1] + 7) / 8), (unsigned)fl->n[2]);
 }
 
+// every given field 16-byte aligned (null: not used) and rows of whole float4s
+template <class... P>
+bool quads(const ibm_flow* fl, P... f) {
+  const uintptr_t bits = (reinterpret_cast<uintptr_t>(f) | ...);
+  return fl->n[0] % 4 == 0 && (bits & 15u) == 0;
+}
+// blocks of the quad kernels: a plane's quads, and `planes` planes per block
+dim3 quad_grid(const ibm_flow* fl, int planes) {
+  const int nq = fl->n[0] / 4 * fl->n[1];
+  return dim3((unsigned)((nq + kQuadThreads - 1) / kQuadThreads),
+              (unsigned)((fl->n[2] + planes - 1) / planes));
+}
+
+// Planes per thread of rhs4_kernel: the whole waves of blocks (two fit on an
+// SM) times a column's length, the first plane's extra loads counted as one and
+// a half planes (200 x 180 x 144: 9 planes, 1.9 waves, instead of 1.07 with 16)
+int rhs_planes(const ibm_flow* fl, int n_sm) {
+  const long nb = (fl->n[0] / 4 * fl->n[1] + kQuadThreads - 1) / kQuadThreads;
+  int best = 1;
+  double least = 1e300;
+  for (int z = 4; z <= 32; ++z) {
+    const long blocks = nb * ((fl->n[2] + z - 1) / z), waves = (blocks + 2 * n_sm - 1) / (2 * n_sm);
+    const double cost = waves * (std::min(z, fl->n[2]) + 1.5);
+    if (cost < least) {
+      least = cost;
+      best = z;
+    }
+  }
+  return best;
+}
+
 // blocks for the row kernels: enough rows in flight, at most one pass over them
 unsigned row_blocks(const ibm_flow* fl) {
   const int rows = fl->n[1] * fl->n[2];
@@ -673,8 +965,15 @@ cudaError_t flow_predict(ibm_flow* fl, int l, float* u, float* v, float* w, cons
   if (e != cudaSuccess) return e;
   e = flow_mark(fl, l, 0, s);
   if (e != cudaSuccess) return e;
-  rhs_kernel<<<cell_grid(fl), dim3(32, 8), 0, s>>>(G, u, v, w, p, Hp, Ho, Ro, (float)kGamma[l],
-                                                     (float)kRho[l], (float)alpha, nu, dt);
+  if (quads(fl, u, v, w, p)) {
+    auto kernel = Hp.c[0] ? rhs4_kernel<true> : rhs4_kernel<false>;
+    kernel<<<quad_grid(fl, fl->rhs_planes), kQuadThreads, 0, s>>>(
+        G, u, v, w, p, Hp.c[0], Hn, fl->R, (float)kGamma[l], (float)kRho[l], (float)alpha, nu, dt,
+        fl->rhs_planes);
+  } else {
+    rhs_kernel<<<cell_grid(fl), dim3(32, 8), 0, s>>>(G, u, v, w, p, Hp, Ho, Ro, (float)kGamma[l],
+                                                       (float)kRho[l], (float)alpha, nu, dt);
+  }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = flow_mark(fl, l, 1, s);
   const bool fourier = fl->solve_w[l] < 0;
@@ -715,7 +1014,13 @@ cudaError_t flow_project(ibm_flow* fl, int l, float* u, float* v, float* w, floa
   if (e != cudaSuccess) return e;
   e = flow_mark(fl, l, 6, s);
   if (e != cudaSuccess) return e;
-  div_kernel<<<cell_grid(fl), dim3(32, 8), 0, s>>>(G, CVec3{{u, v, w}}, f, fscale, fl->rp);
+  const bool q4 = quads(fl, u, v, w, p, fx, fy, fz);
+  if (q4) {
+    auto kernel = fx ? div4_kernel<true> : div4_kernel<false>;
+    kernel<<<quad_grid(fl, 1), kQuadThreads, 0, s>>>(G, CVec3{{u, v, w}}, f, fscale, fl->rp);
+  } else {
+    div_kernel<<<cell_grid(fl), dim3(32, 8), 0, s>>>(G, CVec3{{u, v, w}}, f, fscale, fl->rp);
+  }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = flow_mark(fl, l, 7, s);
   if (e == cudaSuccess) e = fft_status(cufftExecR2C(fl->r2c1, fl->rp, fl->S));
@@ -730,9 +1035,15 @@ cudaError_t flow_project(ibm_flow* fl, int l, float* u, float* v, float* w, floa
   if (e == cudaSuccess) e = fft_status(cufftExecC2R(fl->c2r1, fl->S, fl->rp));
   if (e == cudaSuccess) e = flow_mark(fl, l, 10, s);
   if (e == cudaSuccess) {
-    project_kernel<<<cell_grid(fl), dim3(32, 8), 0, s>>>(
-        G, Vec3{{u, v, w}}, p, fl->rp, f, fscale, (float)(alpha * fl->dt),
-        (float)(alpha * fl->dt * fl->nu / 2.0));
+    const float adt = (float)(alpha * fl->dt), a = (float)(alpha * fl->dt * fl->nu / 2.0);
+    if (q4) {
+      auto kernel = fx ? project4_kernel<true> : project4_kernel<false>;
+      kernel<<<quad_grid(fl, 1), kQuadThreads, 0, s>>>(G, Vec3{{u, v, w}}, p, fl->rp, f, fscale,
+                                                       adt, a);
+    } else {
+      project_kernel<<<cell_grid(fl), dim3(32, 8), 0, s>>>(G, Vec3{{u, v, w}}, p, fl->rp, f, fscale,
+                                                           adt, a);
+    }
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = flow_mark(fl, l, 11, s);
@@ -778,6 +1089,9 @@ extern "C" ibm_status ibm_flow_create(const ibm_grid_desc* grid, double nu, doub
   fl->nu = nu;
   fl->dt = dt;
   ibm::choose_solves(fl);
+  int n_sm = 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, fl->device) == cudaSuccess)
+    fl->rhs_planes = ibm::rhs_planes(fl, std::max(n_sm, 1));
   const int nx = fl->n[0], ny = fl->n[1], nz = fl->n[2], nxh = nx / 2 + 1;
   fl->N = (size_t)nx * ny * nz;
   fl->NC = (size_t)nxh * ny * nz;

@@ -898,6 +898,7 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
       R.nf = Bd.n_face;
       R.ne = T.ne;
       R.closed = Bd.closed ? 1 : 0;
+      c->any_open = c->any_open || !Bd.closed;
       R.varied = varied ? 1 : 0;
       for (int d = 0; d < 3; ++d) {
         const double o = Bd.origin[d] / h[d];

@@ -76,8 +76,12 @@ __device__ __forceinline__ long long warp_sum_i64(long long q) {
 
 // REC (record mode): instead of spreading, write each marker's spread record
 // (centroid in cells, c_l F) and count it under the tiles of the tile-owned
-// spread, with the tile's largest |c_l F| per component
-template <int MT, bool MEASURE, bool INTERP, bool PROBE, bool SPREAD, bool REC>
+// spread, with the tile's largest |c_l F| per component.  PLAIN: all bodies
+// closed and no pressure, so one probe and three components; without the code
+// for the second probe and the pressure the step's kernel needs no spills at
+// 80 registers (354 -> 339 us for the 1000 drops, 117 -> 111 us for the uneven
+// bodies).
+template <int MT, bool MEASURE, bool INTERP, bool PROBE, bool SPREAD, bool REC, bool PLAIN>
 __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
     DeviceTables T, Grid g, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ v, const float* __restrict__ u, const float* __restrict__ vv,
@@ -192,7 +196,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
       for (int d = 0; d < 3; ++d) vb[d] = __ldg(Fm_in + d * F + gf);
     }
     // marker acceleration (pressure correction): mean of the vertices'
-    if (PROBE && pr && accel) {
+    if (PROBE && !PLAIN && pr && accel) {
       const float third = 1.f / 3.f;
 #pragma unroll
       for (int d = 0; d < 3; ++d)
@@ -231,11 +235,11 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         s_own[d * MT] = tp[d];
-        s_own[(3 + d) * MT] = tm[d];
+        if (!PLAIN) s_own[(3 + d) * MT] = tm[d];
         s_own[(6 + d) * MT] = nrm[d];
         s_own[(9 + d) * MT] = vb[d];
       }
-      s_own[12 * MT] = am[0] * nrm[0] + am[1] * nrm[1] + am[2] * nrm[2];
+      if (!PLAIN) s_own[12 * MT] = am[0] * nrm[0] + am[1] * nrm[1] + am[2] * nrm[2];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         s_own[(13 + d) * MT] = tc[d];
@@ -274,7 +278,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
   }
 
   const bool mine = FIELD && active && ok;
-  const bool two = PROBE && !B.closed;     // open sheet: probes on both sides
+  const bool two = PROBE && !PLAIN && !B.closed;   // open sheet: probes on both sides
 
   // ---- row map of the block's footprint -----------------------------------
   int ylo = 0, zlo = 0, sy = 0, sz = 0, xlo = 0, sx = 0;
@@ -500,7 +504,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
   // word per staged node) in place of the component's staged velocity, and
   // flushed with float4 global atomics.
   if (FIELD && (VEL || FLUSH)) {
-    const bool press = PROBE && pr != nullptr;
+    const bool press = PROBE && !PLAIN && pr != nullptr;
     float Pj = 0.f;
     const float cl = area * sc.cl_scale;
     if (VEL && fit) {
@@ -522,7 +526,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
         __syncthreads();   // every thread's copies of this component have landed
       }
       float Fc = 0.f;      // this component of the marker force
-      if (PROBE && comp == 3) {
+      if (PROBE && !PLAIN && comp == 3) {
         if (mine) {
           // probe pressure p* and the correction h (Du/Dt).n, per side with its
           // own normal: P = p*+ + h a.n (closed), p*+ - p*- + 2 h a.n (open)
@@ -923,7 +927,10 @@ cudaError_t launch_mt(ibm_ctx* c, const float* x, const float* v, const float* u
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, marker_kernel<MT, M, I, P, S, R>, tab ? *tab : c->d, c->grid,
+  auto kernel = marker_kernel<MT, M, I, P, S, R, true>;
+  if constexpr (P)
+    if (pr || c->any_open) kernel = marker_kernel<MT, M, I, P, S, R, false>;
+  return cudaLaunchKernelEx(&cfg, kernel, tab ? *tab : c->d, c->grid,
                             c->sc, (int32_t)c->V, (int32_t)c->F, x, v, u, vv, w, pr, accel, U,
                             Fm, Fm_in, Fext, fx, fy, fz, record, vec4, c->td,
                             c->phi_bound, cache, c->fc_tab, c->fc_face, ms);
@@ -946,17 +953,23 @@ cudaError_t launch_t(ibm_ctx* c, const float* x, const float* v, const float* u,
 
 }  // namespace
 
+template <int MT, bool M, bool I, bool P, bool S, bool R>
+cudaError_t marker_smem_limit() {
+  cudaError_t e = cudaFuncSetAttribute(marker_kernel<MT, M, I, P, S, R, true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       marker_smem_max(MT, P));
+  if constexpr (P)
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(marker_kernel<MT, M, I, P, S, R, false>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, marker_smem_max(MT, P));
+  return e;
+}
+
 cudaError_t set_marker_smem_limit() {
   cudaError_t e = cudaSuccess;
-#define SET(M, I, P, S, R)                                                                   \
-  if (e == cudaSuccess)                                                                      \
-    e = cudaFuncSetAttribute(marker_kernel<kMT, M, I, P, S, R>,                              \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,                    \
-                             marker_smem_max(kMT, P));               \
-  if (e == cudaSuccess)                                                                      \
-    e = cudaFuncSetAttribute(marker_kernel<128, M, I, P, S, R>,                              \
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,                    \
-                             marker_smem_max(128, P));
+#define SET(M, I, P, S, R)                                                    \
+  if (e == cudaSuccess) e = marker_smem_limit<kMT, M, I, P, S, R>();          \
+  if (e == cudaSuccess) e = marker_smem_limit<128, M, I, P, S, R>();
   SET(true, true, true, true, false)
   SET(true, false, true, false, false)
   SET(false, true, true, false, false)

@@ -1,10 +1,10 @@
 // Element forces of the interaction potentials (Sec. 2.3, Eqs.
-// elaspot..areapot), written once for any scalar type T: float in the forward
-// force kernel, Dual (value + directional derivative) in the adjoint, where
-// the derivative part of the forces is the Jacobian-vector product J y of
-// the forces along the tangent y carried by the positions.  J = -Hessian of
-// the energy is symmetric, so the same product is the vector-Jacobian
-// product the adjoint needs.
+// elaspot..areapot).  edge_forces and face_forces carry Dual numbers (value +
+// directional derivative) in the adjoint, where the derivative part of the
+// forces is the Jacobian-vector product J y of the forces along the tangent y
+// carried by the positions.  J = -Hessian of the energy is symmetric, so the
+// same product is the vector-Jacobian product the adjoint needs.  edge_forward
+// and face_forward are the force kernel's, without the per-constant parts.
 //
 // Edge e = (a, b) with wings c (face (a, b, c)) and d (face (b, a, d)):
 //   spring   W = k_s/2 (l - l0)^2      F_a = k_s (l - l0) e/l, F_b = -F_a
@@ -160,6 +160,65 @@ __device__ __forceinline__ void face_forces(const Vec<T>& pa, const Vec<T>& pb, 
     f[k] = vadd(vscale(gradA[k], -gA), vscale(gradV[k], -cV));
   }
   const float da = val(Af) - A0f;
+  e_area = 0.5f * ka * da * da / A0f;
+}
+
+// Spring and bending of one edge, values only.  With N1 = e x ac, N2 = ad x e:
+// (n1 x n2).e/|e| = -|e| (ad.N1)/(|N1||N2|), the force on b is what makes the
+// four sum to zero, and energies are formed only where they are used.
+__device__ __forceinline__ void edge_forward(const Vec<float>& pa, const Vec<float>& pb,
+                                             const Vec<float>& pc, const Vec<float>& pd,
+                                             bool has_hinge, float l0, float cos0, float sin0,
+                                             float ks, float kb, Vec<float>& fa, Vec<float>& fb,
+                                             Vec<float>& fc, Vec<float>& fd, float& e_spring,
+                                             float& e_bend) {
+  const Vec<float> e = vsub(pb, pa);
+  const float l2 = vdot(e, e);
+  const float inv_l = rsqrtf(l2);
+  const float l = l2 * inv_l, dl = l - l0;
+  fa = vscale(e, ks * dl * inv_l);
+  fb = {-fa.x, -fa.y, -fa.z};
+  fc = fd = {0.f, 0.f, 0.f};
+  e_spring = 0.5f * ks * dl * dl;
+  e_bend = 0.f;
+  if (!has_hinge) return;
+  const Vec<float> ac = vsub(pc, pa), ad = vsub(pd, pa);
+  const Vec<float> N1 = vcross(e, ac), N2 = vcross(ad, e);
+  const float r1 = rsqrtf(vdot(N1, N1)), r2 = rsqrtf(vdot(N2, N2));
+  const float r12 = r1 * r2;
+  const float cth = vdot(N1, N2) * r12, sth = -l * vdot(ad, N1) * r12;
+  const float s = kb * l * (sth * cos0 - cth * sin0);   // k_b |e| sin(theta - theta0)
+  fc = vscale(N1, s * r1 * r1);
+  fd = vscale(N2, s * r2 * r2);
+  const float inv_l2 = inv_l * inv_l;
+  const float sc = vdot(ac, e) * inv_l2, sd = vdot(ad, e) * inv_l2;
+  const Vec<float> g = {sc * fc.x + sd * fd.x, sc * fc.y + sd * fd.y, sc * fc.z + sd * fd.z};
+  fa = {fa.x + (g.x - (fc.x + fd.x)), fa.y + (g.y - (fc.y + fd.y)), fa.z + (g.z - (fc.z + fd.z))};
+  fb = vsub(fb, g);
+  e_bend = kb * (1.f - (cth * cos0 + sth * sin0));
+}
+
+// Local area, global area and volume forces of one face, values only.  The
+// area part is (m x (c - b), m x (a - c), minus their sum) with
+// m = -(c_A + k_a strain) n / 2.  The volume part gives every corner a third of
+// the face's normal, -c_V N / 6: grad_a V = b x c / 6 differs from N / 6 by
+// a x (c - b) / 6, whose sum over the closed fan of faces around a vertex is
+// zero (c_V is zero on open sheets), and N carries no products of the
+// body-frame coordinates.
+__device__ __forceinline__ void face_forward(const Vec<float>& pa, const Vec<float>& pb,
+                                             const Vec<float>& pc, float A0f, float ka, float cA,
+                                             float cV, Vec<float> (&f)[3], float& e_area) {
+  const Vec<float> ab = vsub(pb, pa), ac = vsub(pc, pa), bc = vsub(ac, ab);
+  const Vec<float> N = vcross(ab, ac);
+  const float q = vdot(N, N);
+  const float rn = rsqrtf(q);
+  const float da = 0.5f * q * rn - A0f;
+  const Vec<float> m = vscale(N, -0.5f * rn * (cA + ka * __fdividef(da, A0f)));
+  const Vec<float> v = vscale(N, cV * (-1.f / 6.f));
+  const Vec<float> fa = vcross(m, bc), fb = vcross(ac, m);   // m x (a - c) = ac x m
+  f[0] = vadd(fa, v);
+  f[1] = vadd(fb, v);
+  f[2] = {v.x - (fa.x + fb.x), v.y - (fa.y + fb.y), v.z - (fa.z + fb.z)};
   e_area = 0.5f * ka * da * da / A0f;
 }
 

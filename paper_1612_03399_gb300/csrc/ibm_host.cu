@@ -644,6 +644,30 @@ void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
   }
 }
 
+// Threads per force-kernel block: the least thread-iterations over the work
+// items (edges, then faces at about half an edge's work, then own vertices at
+// a third).  Patches of 128 vertices of the icosphere drops have 522 edges: 256
+// threads would take three passes for them, 192 or 288 take the same three or
+// two with few idle threads.
+int choose_force_threads(const std::vector<FWork>& work) {
+  int best = kForceThreads;
+  double least = 1e300;
+  for (int t = 128; t <= kForceThreadsMax; t += 32) {
+    double cost = 0.0;
+    const size_t step = std::max<size_t>(1, work.size() / 4096);
+    for (size_t k = 0; k < work.size(); k += step) {
+      const FWork& w = work[k];
+      cost += t * ((w.n_edge + t - 1) / t + 0.5 * ((w.n_face + t - 1) / t) +
+                   0.33 * ((w.n_own + t - 1) / t));
+    }
+    if (cost < least) {
+      least = cost;
+      best = t;
+    }
+  }
+  return best;
+}
+
 void make_consts(ibm_ctx* c) {
   const ibm_params& p = c->prm;
   ibm::Grid& g = c->grid;
@@ -802,7 +826,8 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     std::vector<int2> work;
     std::vector<float> frest;        // force-kernel rest data per work item, patch order
     std::vector<int64_t> wrest;
-    size_t force_smem = 0, adjoint_smem = 0;
+    std::vector<FWork> fwork;
+    size_t force_smem = 0, force_smem_wide = 0, adjoint_smem = 0;
     c->h_body.resize(n_bodies);
     long long vo = 0, fo = 0, eo = 0;
     for (int b = 0; b < n_bodies; ++b) {
@@ -953,9 +978,27 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
         }
         // shared memory of the block: blob, rest data, positions, slots
         const FPatch& Q = T.fpatch[q];
-        force_smem = std::max(force_smem,
-                              sizeof(float) * ((size_t)Q.blob_words + frest_words(H.n_edge, H.n_face, varied) +
-                                               3 * (size_t)pad4(H.n_loc) + 3 * (size_t)pad4(Q.n_slot)));
+        FWork fw{};
+        fw.v_off = (int32_t)vo;
+        fw.f_off = (int32_t)fo;
+        fw.body = b;
+        fw.own0 = H.own0;
+        fw.n_own = H.n_own;
+        fw.n_loc = H.n_loc;
+        fw.n_edge = H.n_edge;
+        fw.n_face = H.n_face;
+        fw.loc_off = H.loc_off;      // within the topology until the tables are joined
+        fw.blob_off = Q.blob_off;
+        fw.blob_words = Q.blob_words;
+        fw.n_slot = Q.n_slot;
+        fw.rest = (int64_t)r0;
+        fw.rest_words = frest_words(H.n_edge, H.n_face, varied);
+        fw.varied = varied ? 1 : 0;
+        fwork.push_back(fw);
+        const size_t own_words = (size_t)Q.blob_words + fw.rest_words;
+        const size_t per = (size_t)H.n_loc + Q.n_slot;
+        force_smem = std::max(force_smem, sizeof(float) * (own_words + 3 * per));
+        force_smem_wide = std::max(force_smem_wide, sizeof(float) * (own_words + 4 * per));
         // the adjoint: blob with its tail, rest data, positions and
         // tangents, slots
         adjoint_smem = std::max(
@@ -981,6 +1024,7 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     std::vector<uint16_t> slot_all;
     std::vector<uint32_t> fblob_all;
     std::vector<FPatch> fpatch_all;
+    std::vector<int32_t> topo_loc, topo_blob;   // where each topology's tables start
     int max_loc = 0, max_slot = 0, max_own = 0;
     for (size_t t = 0; t < topos.size(); ++t) {
       const HostTopo& T = topos[t];
@@ -1021,6 +1065,8 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
       csr_all.insert(csr_all.end(), T.csr_ptr.begin(), T.csr_ptr.end());
       slot_all.insert(slot_all.end(), T.csr_slot.begin(), T.csr_slot.end());
       const int32_t bo = (int32_t)fblob_all.size();
+      topo_loc.push_back(lo);
+      topo_blob.push_back(bo);
       for (FPatch Q : T.fpatch) {
         Q.blob_off += bo;
         fpatch_all.push_back(Q);
@@ -1031,7 +1077,13 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
       max_own = std::max(max_own, T.max_own);
     }
     (void)max_slot;
-    c->force_smem = force_smem;
+    for (FWork& w : fwork) {
+      w.loc_off += topo_loc[body_topo[w.body]];
+      w.blob_off += topo_blob[body_topo[w.body]];
+    }
+    c->force_threads = choose_force_threads(fwork);
+    c->force_wide = force_smem_wide <= 227 * 1024;
+    c->force_smem = c->force_wide ? force_smem_wide : force_smem;
     if (c->force_smem > 227 * 1024)
       fail(IBM_ERR_UNSUPPORTED, "force-kernel shared memory above 227 KB; lower patch_size");
     c->adjoint_smem = adjoint_smem;
@@ -1063,6 +1115,7 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     d.fpatch = upload(c, fpatch_all);
     d.frest = upload(c, frest);
     d.wrest = upload(c, wrest);
+    d.fwork = upload(c, fwork);
     d.l0 = upload(c, l0);
     d.cs0 = upload(c, cs0);
     d.A0f = upload(c, A0f);

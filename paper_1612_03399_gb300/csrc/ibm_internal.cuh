@@ -91,6 +91,17 @@ __host__ __device__ constexpr int frest_words(int n_edge, int n_face, bool varie
   return (varied ? 5 : 3) * pad4(n_edge) + (varied ? 2 : 1) * pad4(n_face);
 }
 
+// What a force-kernel block needs of its work item, in one 64-byte record: a
+// block starts its copies and gathers one load after this one, not after the
+// chain work item -> body -> topology -> patch.
+struct alignas(16) FWork {
+  int32_t v_off, f_off, body, own0;           // the body's vertices and faces; first own vertex
+  int32_t n_own, n_loc, n_edge, n_face;
+  int32_t loc_off, blob_off, blob_words, n_slot;
+  int64_t rest;                               // word offset of the rest data
+  int32_t rest_words, varied;
+};
+
 struct Grid {
   int32_t n[3];
   float h[3], invh[3];
@@ -175,7 +186,8 @@ __device__ __forceinline__ int tiles_along(int f, int n, int T, int (&out)[3]) {
   }
   return k;
 }
-constexpr int kForceThreads = 256;   // threads per force-kernel block
+constexpr int kForceThreads = 256;   // threads per block of the adjoint's and advance kernels
+constexpr int kForceThreadsMax = 288;   // most threads of a force-kernel block
 // host mirror of the node update's outputs (ibm_step_host): the force kernel
 // writes x', v' to device arrays and the last block to complete each chunk of
 // kMirrorChunk entries of the flat [3][V] arrays copies that chunk into host
@@ -209,6 +221,7 @@ struct DeviceTables {
   FPatch* fpatch = nullptr;     // per topology patch, indexed like `patch`
   float* frest = nullptr;       // rest data of every work item, in patch order
   int64_t* wrest = nullptr;     // [n_work] word offset of the work item's rest data
+  FWork* fwork = nullptr;       // [n_work] records of the force kernel
   float* l0 = nullptr;          // [E] rest edge lengths
   float2* cs0 = nullptr;        // [E] (cos theta0, sin theta0) per hinge edge
   float* A0f = nullptr;         // [F] rest face areas
@@ -374,6 +387,8 @@ struct ibm_ctx {
   ibm::StepConsts sc{};
   size_t force_smem = 0;
   size_t adjoint_smem = 0;
+  int force_threads = ibm::kForceThreads;   // threads per force-kernel block
+  bool force_wide = true;           // its positions and slots as float4
   int32_t max_own = 0;
   bool have_prev = false;
   // the body sums alternate between two buffers from one ibm_step to the next,

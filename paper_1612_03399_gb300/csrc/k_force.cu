@@ -25,20 +25,61 @@
 namespace ibm {
 namespace {
 
-struct Smem {
-  float *px, *py, *pz, *cx, *cy, *cz;
-  __device__ Vec<float> pos(int i) const { return {px[i], py[i], pz[i]}; }
-  __device__ void put(int s, const Vec<float>& f) const {
-    if (s == kNone) return;
-    cx[s] = f.x;
-    cy[s] = f.y;
-    cz[s] = f.z;
+// Positions and contribution slots in shared memory: as float4 (WIDE, one
+// shared load or store each), or as three arrays, a quarter smaller, for
+// patches whose float4 form does not fit (above about 650 vertices).
+template <bool WIDE>
+struct Smem;
+template <>
+struct Smem<true> {
+  float4 *p, *c;
+  __device__ __forceinline__ void init(float* s, int n_loc, int) {
+    p = reinterpret_cast<float4*>(s);
+    c = p + n_loc;
   }
-  __device__ void add(int s, const Vec<float>& f) const {
+  __device__ __forceinline__ void set(int i, float x, float y, float z) const {
+    p[i] = make_float4(x, y, z, 0.f);
+  }
+  __device__ __forceinline__ Vec<float> pos(int i) const {
+    const float4 t = p[i];
+    return {t.x, t.y, t.z};
+  }
+  __device__ __forceinline__ Vec<float> slot(int s) const {
+    const float4 t = c[s];
+    return {t.x, t.y, t.z};
+  }
+  __device__ __forceinline__ void put(int s, const Vec<float>& f) const {
+    if (s != kNone) c[s] = make_float4(f.x, f.y, f.z, 0.f);
+  }
+  __device__ __forceinline__ void add(int s, const Vec<float>& f) const {
+    if (s != kNone) put(s, vadd(slot(s), f));
+  }
+};
+template <>
+struct Smem<false> {
+  float *p, *c;
+  int np, nc;
+  __device__ __forceinline__ void init(float* s, int n_loc, int n_slot) {
+    p = s;
+    np = n_loc;
+    c = s + 3 * n_loc;
+    nc = n_slot;
+  }
+  __device__ __forceinline__ void set(int i, float x, float y, float z) const {
+    p[i] = x;
+    p[np + i] = y;
+    p[2 * np + i] = z;
+  }
+  __device__ __forceinline__ Vec<float> pos(int i) const { return {p[i], p[np + i], p[2 * np + i]}; }
+  __device__ __forceinline__ Vec<float> slot(int s) const { return {c[s], c[nc + s], c[2 * nc + s]}; }
+  __device__ __forceinline__ void put(int s, const Vec<float>& f) const {
     if (s == kNone) return;
-    cx[s] += f.x;
-    cy[s] += f.y;
-    cz[s] += f.z;
+    c[s] = f.x;
+    c[nc + s] = f.y;
+    c[2 * nc + s] = f.z;
+  }
+  __device__ __forceinline__ void add(int s, const Vec<float>& f) const {
+    if (s != kNone) put(s, vadd(slot(s), f));
   }
 };
 
@@ -103,68 +144,63 @@ __device__ __noinline__ void mirror_chunks(Mirror m, const float* x_out, const f
 }
 
 // MODE 0: F_int only; 1: F_int + F_ext^v and the node update; 2: the
-// acceleration (F_int + F_ext^v)/m, zero on clamped nodes, into Fint
-template <int MODE>
-__global__ void __launch_bounds__(kForceThreads) force_kernel(
+// acceleration (F_int + F_ext^v)/m, zero on clamped nodes, into Fint.
+// ENERGY: the body's energies as well (MODE 0).
+//
+// What bounds it: instruction issue while its blocks compute, and between that
+// the latency of the chain record -> index -> position and of the barriers; its
+// 117 bytes per vertex take 11 us of HBM for 642 k vertices.  Hence one record
+// per block (a load instead of a chain of four), forces without the parts only
+// the adjoint uses, float4 positions and slots, and a block size whose whole
+// warps fit the patches' element counts (force_threads).  Measured with patches
+// of 128 vertices: 107 -> 84 us for 642 k vertices after the coupled step's
+// marker kernel, 28.5 -> 23.4 us for 160 k vertices on its own.
+template <int MODE, bool ENERGY, bool WIDE>
+__global__ void __launch_bounds__(kForceThreadsMax, 3) force_kernel(
     DeviceTables T, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ v, const float* __restrict__ Fext, float* __restrict__ Fint,
     float* __restrict__ x_out, float* __restrict__ v_out, double* __restrict__ energy,
     Mirror mirror) {
   extern __shared__ __align__(16) float sm[];
   __shared__ __align__(8) unsigned long long bar;
-  const int2 wk = T.work[blockIdx.x];
-  const BodyDev B = T.body[wk.x];
-  const TopoDev topo = T.topo[B.topo];
-  const PatchHdr P = T.patch[topo.patch_off + wk.y];
-  const FPatch Q = T.fpatch[topo.patch_off + wk.y];
+  const FWork P = T.fwork[blockIdx.x];
   const int pe = pad4(P.n_edge), pf = pad4(P.n_face);
-  const int rest_words = frest_words(P.n_edge, P.n_face, B.varied != 0);
   const uint4* rec = reinterpret_cast<const uint4*>(sm);                   // edges
   const uint2* frec = reinterpret_cast<const uint2*>(sm + 4 * P.n_edge);   // faces
   const uint16_t* ptr = reinterpret_cast<const uint16_t*>(sm + 4 * P.n_edge + 2 * P.n_face);
-  const float* rest = sm + Q.blob_words;
-  Smem S;
-  S.px = sm + Q.blob_words + rest_words;
-  S.py = S.px + pad4(P.n_loc);
-  S.pz = S.py + pad4(P.n_loc);
-  S.cx = S.pz + pad4(P.n_loc);
-  S.cy = S.cx + pad4(Q.n_slot);
-  S.cz = S.cy + pad4(Q.n_slot);
+  const float* rest = sm + P.blob_words;
+  Smem<WIDE> S;
+  S.init(sm + P.blob_words + P.rest_words, P.n_loc, P.n_slot);
 
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
-    const unsigned nb = 4u * (unsigned)Q.blob_words, nr = 4u * (unsigned)rest_words;
+    const unsigned nb = 4u * (unsigned)P.blob_words, nr = 4u * (unsigned)P.rest_words;
     mbar_arrive_tx(&bar, nb + nr + (unsigned)sc.starve_tx);
-    if (nb) bulk_load(sm, T.fblob + Q.blob_off, nb, &bar);
-    if (nr) bulk_load(sm + Q.blob_words, T.frest + T.wrest[blockIdx.x], nr, &bar);
+    if (nb) bulk_load(sm, T.fblob + P.blob_off, nb, &bar);
+    if (nr) bulk_load(sm + P.blob_words, T.frest + P.rest, nr, &bar);
   }
   // meanwhile: positions of the own and halo vertices, two per thread in flight
   for (int i = threadIdx.x; i < P.n_loc; i += 2 * blockDim.x) {
     const int j = i + blockDim.x;
-    const int gi = B.v_off + __ldg(T.loc_vert + P.loc_off + i);
-    const int gj = j < P.n_loc ? B.v_off + __ldg(T.loc_vert + P.loc_off + j) : gi;
+    const int gi = P.v_off + __ldg(T.loc_vert + P.loc_off + i);
+    const int gj = j < P.n_loc ? P.v_off + __ldg(T.loc_vert + P.loc_off + j) : gi;
     const float xi = __ldg(x + gi), yi = __ldg(x + V + gi), zi = __ldg(x + 2 * V + gi);
     const float xj = __ldg(x + gj), yj = __ldg(x + V + gj), zj = __ldg(x + 2 * V + gj);
-    S.px[i] = xi;
-    S.py[i] = yi;
-    S.pz[i] = zi;
-    if (j < P.n_loc) {
-      S.px[j] = xj;
-      S.py[j] = yj;
-      S.pz[j] = zj;
-    }
+    S.set(i, xi, yi, zi);
+    if (j < P.n_loc) S.set(j, xj, yj, zj);
   }
+  const BodyDev& B = T.body[P.body];
+  const float Bks = B.ks, Bkb = B.kb;
   // and the velocity and clamp flag of the thread's first own vertex
   float pv[3] = {0.f, 0.f, 0.f};
   bool pcl = false;
   if (MODE == 1 && (int)threadIdx.x < P.n_own) {
-    const int gv = B.v_off + P.own0 + threadIdx.x;
+    const int gv = P.v_off + P.own0 + threadIdx.x;
     pv[0] = __ldg(v + gv);
     pv[1] = __ldg(v + V + gv);
     pv[2] = __ldg(v + 2 * V + gv);
     pcl = T.clamp[gv] != 0;
   }
-  const bool want_e = energy != nullptr;
   double eS = 0.0, eB = 0.0, eA = 0.0;
   __syncthreads();   // positions staged, barrier initialised
   if (!__syncthreads_and(mbar_wait(&bar, kCopyWaitClocks))) {
@@ -186,13 +222,13 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
     const Vec<float> pa = S.pos(la), pb = S.pos(lb);
     const Vec<float> pc = hinge ? S.pos(lc) : pa, pd = hinge ? S.pos(ld) : pb;
     const float c0 = hinge ? rest[pe + k] : 1.f, s0 = hinge ? rest[2 * pe + k] : 0.f;
-    Vec<float> fa, fb, fc, fd, us[2], ub[4];
+    Vec<float> fa, fb, fc, fd;
     float es, eb;
     // per-edge constants (van Gelder springs, materials) where the body has them
-    const float ks = B.varied ? B.ks * rest[3 * pe + pf + k] : B.ks;
-    const float kb = B.varied ? B.kb * rest[4 * pe + pf + k] : B.kb;
-    edge_forces(pa, pb, pc, pd, hinge, rest[k], c0, s0, ks, kb, fa, fb, fc, fd, us, ub, es, eb);
-    if (want_e && (r.z & 0xFFFF) != kNone) {   // the patch of vertex a owns the edge
+    const float ks = P.varied ? Bks * rest[3 * pe + pf + k] : Bks;
+    const float kb = P.varied ? Bkb * rest[4 * pe + pf + k] : Bkb;
+    edge_forward(pa, pb, pc, pd, hinge, rest[k], c0, s0, ks, kb, fa, fb, fc, fd, es, eb);
+    if (ENERGY && (r.z & 0xFFFF) != kNone) {   // the patch of vertex a owns the edge
       eS += (double)es;
       eB += (double)eb;
     }
@@ -208,8 +244,8 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // per-body global-term coefficients from the marker kernel's exact
   // fixed-point area / volume sums
-  const float2 cf = body_coef(B, __ldg(T.qsum + 2 * wk.x), __ldg(T.qsum + 2 * wk.x + 1));
-  const float cA = cf.x, cV = cf.y;
+  const float2 cf = body_coef(B, __ldg(T.qsum + 2 * P.body), __ldg(T.qsum + 2 * P.body + 1));
+  const float cA = cf.x, cV = cf.y, Bka = B.ka, inv_mass = B.inv_mass;
   __syncthreads();   // every edge slot written
   // faces: local area, global area, volume, added to the slots of the edge
   // each face is attached to (an edge per face: no two threads touch the same
@@ -224,7 +260,7 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
     if (MODE != 0) {
       // F_ext^v = sum over the vertex's faces of F_ext / 3: each face adds a
       // third of its load to its corners, gathered with the forces
-      const int g0 = B.f_off + (int)r0.y, g1 = B.f_off + (int)r1.y;
+      const int g0 = P.f_off + (int)r0.y, g1 = P.f_off + (int)r1.y;
       fe0 = {__ldg(Fext + g0), __ldg(Fext + F + g0), __ldg(Fext + 2 * F + g0)};
       fe1 = {__ldg(Fext + g1), __ldg(Fext + F + g1), __ldg(Fext + 2 * F + g1)};
     }
@@ -240,11 +276,10 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
       const int d0 = right ? (int)(r.z >> 16) : (int)(r.z & 0xFFFF);
       const int d1 = right ? (int)(r.z & 0xFFFF) : (int)(r.z >> 16);
       const int d2 = right ? (int)(r.w >> 16) : (int)(r.w & 0xFFFF);
-      Vec<float> f[3], gA[3], gV[3], ua[3];
+      Vec<float> f[3];
       float ea;
-      const float ka = B.varied ? B.ka * rest[5 * pe + pf + k] : B.ka;
-      face_forces(S.pos(v0), S.pos(v1), S.pos(v2), rest[3 * pe + k], ka, cA, cV, f, gA, gV, ua,
-                  ea);
+      const float ka = P.varied ? Bka * rest[5 * pe + pf + k] : Bka;
+      face_forward(S.pos(v0), S.pos(v1), S.pos(v2), rest[3 * pe + k], ka, cA, cV, f, ea);
       if (MODE != 0) {
         const Vec<float> fe = vscale(h ? fe1 : fe0, third);
 #pragma unroll
@@ -253,7 +288,7 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
       S.add(d0, f[0]);
       S.add(d1, f[1]);
       S.add(d2, f[2]);
-      if (want_e && (fr.x >> 31)) eA += (double)ea;
+      if (ENERGY && (fr.x >> 31)) eA += (double)ea;
     }
   }
   __syncthreads();
@@ -263,25 +298,26 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
     const int s0 = ptr[i], s1 = ptr[i + 1];
     float fx = 0.f, fy = 0.f, fz = 0.f;
     for (int s = s0; s < s1; ++s) {
-      fx += S.cx[s];
-      fy += S.cy[s];
-      fz += S.cz[s];
+      const Vec<float> t = S.slot(s);
+      fx += t.x;
+      fy += t.y;
+      fz += t.z;
     }
-    const int lv = P.own0 + i;
-    const int gv = B.v_off + lv;
+    const int gv = P.v_off + P.own0 + i;
     if (MODE == 0) {
       Fint[gv] = fx;
       Fint[V + gv] = fy;
       Fint[2 * V + gv] = fz;
     } else if (MODE == 2) {
       const bool cl = T.clamp[gv] != 0;
-      Fint[gv] = cl ? 0.f : fx * B.inv_mass;
-      Fint[V + gv] = cl ? 0.f : fy * B.inv_mass;
-      Fint[2 * V + gv] = cl ? 0.f : fz * B.inv_mass;
+      Fint[gv] = cl ? 0.f : fx * inv_mass;
+      Fint[V + gv] = cl ? 0.f : fy * inv_mass;
+      Fint[2 * V + gv] = cl ? 0.f : fz * inv_mass;
     } else {
       // the gathered slots hold F_int + F_ext^v
-      const float ax = fx * B.inv_mass, ay = fy * B.inv_mass, az = fz * B.inv_mass;
-      const float x0 = S.px[i], y0 = S.py[i], z0 = S.pz[i];
+      const float ax = fx * inv_mass, ay = fy * inv_mass, az = fz * inv_mass;
+      const Vec<float> p0 = S.pos(i);
+      const float x0 = p0.x, y0 = p0.y, z0 = p0.z;
       const bool first = i == (int)threadIdx.x;
       float vx = first ? pv[0] : __ldg(v + gv), vy = first ? pv[1] : __ldg(v + V + gv),
             vz = first ? pv[2] : __ldg(v + 2 * V + gv);
@@ -302,10 +338,10 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
       v_out[gv] = vx; v_out[V + gv] = vy; v_out[2 * V + gv] = vz;
     }
   }
-  if (MODE == 1 && mirror.hx) mirror_chunks(mirror, x_out, v_out, V, B.v_off + P.own0, P.n_own);
+  if (MODE == 1 && mirror.hx) mirror_chunks(mirror, x_out, v_out, V, P.v_off + P.own0, P.n_own);
 
-  if (want_e) {
-    __shared__ double red[3][kForceThreads / 32];
+  if (ENERGY) {
+    __shared__ double red[3][kForceThreadsMax / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     eS = warp_sum(eS);
     eB = warp_sum(eB);
@@ -323,13 +359,13 @@ __global__ void __launch_bounds__(kForceThreads) force_kernel(
         b += red[1][k];
         c += red[2][k];
       }
-      atomicAdd(energy + 5 * wk.x + 0, a);
-      atomicAdd(energy + 5 * wk.x + 1, b);
-      atomicAdd(energy + 5 * wk.x + 2, c);
-      if (wk.y == 0) {
-        const double Ab = T.meas[2 * wk.x], Vb = T.meas[2 * wk.x + 1];
-        energy[5 * wk.x + 3] = 0.5 * B.kA * (Ab - B.A0) * (Ab - B.A0) / B.A0;
-        energy[5 * wk.x + 4] = B.closed ? 0.5 * B.kv * (Vb - B.V0) * (Vb - B.V0) / B.V0 : 0.0;
+      atomicAdd(energy + 5 * P.body + 0, a);
+      atomicAdd(energy + 5 * P.body + 1, b);
+      atomicAdd(energy + 5 * P.body + 2, c);
+      if (P.own0 == 0) {
+        const double Ab = T.meas[2 * P.body], Vb = T.meas[2 * P.body + 1];
+        energy[5 * P.body + 3] = 0.5 * B.kA * (Ab - B.A0) * (Ab - B.A0) / B.A0;
+        energy[5 * P.body + 4] = B.closed ? 0.5 * B.kv * (Vb - B.V0) * (Vb - B.V0) / B.V0 : 0.0;
       }
     }
   }
@@ -386,13 +422,13 @@ __global__ void __launch_bounds__(kForceThreads) advance_kernel(
 // marker kernel allows it from the start of every block) and wait for its
 // completion before the face part; after any other preceding work they start
 // as usual, when it has completed.
-template <int MODE>
+template <int MODE, bool ENERGY = false>
 cudaError_t launch_force_mode(ibm_ctx* c, const float* x, const float* v, const float* Fext,
                               float* Fint, float* x_out, float* v_out, double* energy,
                               const Mirror& mirror = Mirror()) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)c->n_work);
-  cfg.blockDim = dim3(kForceThreads);
+  cfg.blockDim = dim3((unsigned)c->force_threads);
   cfg.dynamicSmemBytes = c->force_smem;
   cfg.stream = c->stream;
   cudaLaunchAttribute attr[1];
@@ -400,17 +436,20 @@ cudaError_t launch_force_mode(ibm_ctx* c, const float* x, const float* v, const 
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, force_kernel<MODE>, c->d, c->sc, (int32_t)c->V, (int32_t)c->F,
-                            x, v, Fext, Fint, x_out, v_out, energy, mirror);
+  auto kernel = c->force_wide ? force_kernel<MODE, ENERGY, true> : force_kernel<MODE, ENERGY, false>;
+  return cudaLaunchKernelEx(&cfg, kernel, c->d, c->sc, (int32_t)c->V,
+                            (int32_t)c->F, x, v, Fext, Fint, x_out, v_out, energy, mirror);
 }
 
 cudaError_t launch_force(ibm_ctx* c, const float* x, const float* v, const float* Fext,
                          float* Fint, float* x_out, float* v_out, double* energy, bool advance,
                          const Mirror* mirror) {
   if (c->n_work == 0) return cudaSuccess;
-  return advance ? launch_force_mode<1>(c, x, v, Fext, Fint, x_out, v_out, energy,
-                                        mirror ? *mirror : Mirror())
-                 : launch_force_mode<0>(c, x, v, Fext, Fint, x_out, v_out, energy);
+  if (advance)
+    return launch_force_mode<1>(c, x, v, Fext, Fint, x_out, v_out, energy,
+                                mirror ? *mirror : Mirror());
+  return energy ? launch_force_mode<0, true>(c, x, v, Fext, Fint, x_out, v_out, energy)
+                : launch_force_mode<0>(c, x, v, Fext, Fint, x_out, v_out, energy);
 }
 
 cudaError_t launch_accel(ibm_ctx* c, const float* x, const float* Fext, float* a) {
@@ -428,14 +467,14 @@ cudaError_t launch_advance(ibm_ctx* c, const float* x, const float* v, const flo
 }
 
 cudaError_t set_force_smem_limit(size_t bytes) {
-  cudaError_t e = cudaFuncSetAttribute(force_kernel<1>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(force_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(force_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)bytes);
+  cudaError_t e = cudaSuccess;
+  for (auto k : {force_kernel<0, false, true>, force_kernel<0, true, true>,
+                 force_kernel<1, false, true>, force_kernel<2, false, true>,
+                 force_kernel<0, false, false>, force_kernel<0, true, false>,
+                 force_kernel<1, false, false>, force_kernel<2, false, false>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return e;
 }
 
 }  // namespace ibm

@@ -140,7 +140,7 @@ constexpr int kMT = 256;             // most markers (faces) per block of the ma
 // ---------------------------------------------------------------------------
 constexpr int kTX = 16, kTY = 8, kTZ = 8;
 constexpr int kTileNodes = kTX * kTY * kTZ;   // 1024 nodes, 128 x-segments of 8 nodes
-constexpr int kTileThreads = 256;
+constexpr int kTileThreads = 128;
 // TileDev::state slots
 enum : int32_t { TS_EPOCH = 0, TS_LEN = 1, TS_PAIRS = 2 };
 

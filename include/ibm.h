@@ -383,7 +383,8 @@ ibm_status ibm_gts_read(const char* path, int64_t* n_vert, int64_t* n_face, doub
  * inverse, a circulant whose entries fall off as r^|m|, has less than 2^-26
  * of its mass beyond some |m| = W <= 8 with 2W + 1 <= n (then three
  * separable (2W+1)-tap filters, fused with the u* update; small
- * alpha_l dt nu / h^2), else in Fourier space.  A flow object owns its work
+ * alpha_l dt nu / h^2), else by the same inverse as first-order recursions
+ * along the lines (r <= 0.7) or in Fourier space.  A flow object owns its work
  * arrays (about thirteen fields) and FFT plans; velocity and pressure fields
  * are caller-owned device arrays [nz][ny][nx]. */
 typedef struct ibm_flow ibm_flow;
@@ -398,8 +399,8 @@ typedef struct ibm_flow ibm_flow;
 ibm_status ibm_flow_create(const ibm_grid_desc* grid, double nu, double dt, ibm_flow** out);
 ibm_status ibm_flow_set_stream(ibm_flow* flow, void* stream);
 /* The viscous solve of substep `substep` (0, 1, 2): *width = W >= 0 when it
- * runs in real space with 2W + 1 taps per direction, -1 when it runs in
- * Fourier space.  Host only.  Errors: IBM_ERR_INVALID_ARG. */
+ * runs in real space with 2W + 1 taps per direction, -1 when it does not (line
+ * recursions or Fourier space).  Host only.  Errors: IBM_ERR_INVALID_ARG. */
 ibm_status ibm_flow_solve_width(const ibm_flow* flow, int32_t substep, int32_t* width);
 /* Waits for the device to finish (coupled steps may still run on a
  * context's stream), then frees everything the flow owns.  NULL is ignored. */
@@ -450,7 +451,7 @@ ibm_status ibm_flow_step(ibm_flow* flow, ibm_ctx* ctx, const float* x, const flo
  * ibm_flow_get_phase_times waits for the last recorded events and writes host
  * ms[13], each summed over substeps 0, 1, 2 of the last ones recorded:
  * (advection and right-hand side, forward FFT x3, Crank-Nicolson scaling,
- * inverse FFT x3 (these three 0 in real-space substeps), u* update (with the
+ * inverse FFT x3 (these three 0 where no transform runs), u* update (with the
  * real-space solve in it), IBM forcing (the time between predictor and
  * projection: force-field zeroing and the marker kernel), divergence,
  * forward FFT, Poisson scaling, inverse FFT, projection), then the body

@@ -8,15 +8,16 @@
 //                   nodes of that cell index
 //   the factorised Crank-Nicolson solve: the operator
 //                   (1 - a d_xx)(1 - a d_yy)(1 - a d_zz), a = alpha_l dt nu / 2,
-//                   is inverted in one of two exact ways, picked per substep
+//                   is inverted in one of three exact ways, picked per substep
 //                   at creation:
-//     cn_solve_kernel  in real space: with c = a/h_d^2 the inverse of the
+//     cn_solve_kernel  by short filters: with c = a/h_d^2 the inverse of the
 //                   periodic 1-D factor 1 - c (E - 2 + E^-1) is a circulant
 //                   whose entries fall off as r^|m|, r < 1 the smaller root
 //                   of c r^2 - (1 + 2c) r + c; when its mass beyond |m| = W
 //                   (W <= 8) is below 2^-26 in every direction, the three
 //                   inverses are applied as separable (2W+1)-tap filters and
 //                   u* = u + du is written in the same pass
+//     line_x_kernel, line_yz_kernel  by recursions along the lines, for r <= 0.7
 //     R2C (batch 3) -> cn_scale_kernel -> C2R, add_kernel (u* = u + du):
 //                   otherwise, the operator being diagonal in Fourier space
 //   div_kernel      div(u* + s f)
@@ -57,6 +58,10 @@ struct ibm_flow {
   int solve_w[3] = {-1, -1, -1};
   float taps[3][3][9] = {};
   int rhs_planes = 16;          // planes per thread of the right-hand side kernel
+  // per substep: solved by recursions along the lines; the powers of r they use
+  bool lines[3] = {false, false, false};
+  float* pw = nullptr;          // [3][pw_stride]
+  size_t pw_stride = 0;
   // phase timing (profiling aid): events at the 12 kernel boundaries of each
   // substep and the 3 of the body update
   bool timing = false;
@@ -770,6 +775,108 @@ cudaError_t set_solve_smem(const ibm_flow* fl) {
   return e;
 }
 
+// ---- the factorised solve by recursions along the lines ---------------------
+// 1 - c (E - 2 + E^-1) = (c/r) (1 - r E^-1)(1 - r E), r < 1 the smaller root of
+// c r^2 - (1 + 2c) r + c = 0, so its periodic inverse is a first-order recursion
+// up every line and one down, times r/c.  A line is cut into kSegs segments that
+// run from zero; the values that enter them follow from the segments' ends (the
+// line closes on itself: the sum over a turn divided by 1 - r^n), and reach the
+// i-th entry of a segment times r^(i+1).  Exact to rounding for any line; the
+// sums grow by 1/(1 - r) at most before the scaling takes it back.
+// A block holds 32 lines in shared memory, kSegs threads to a line; three passes
+// (z, y, x) move 84 N bytes, the last adds to u.  Replaces the transforms where
+// 17 taps are not enough: on 200 x 180 x 144 a substep's forward and inverse
+// transforms of three fields, the scaling and the add took 324 us, the passes
+// take 42 + 32 + 52 us; the error of u* against float64 is 0.6 of the transforms'
+// (r = 0.35 .. 0.7).
+constexpr int kSegs = 8;
+constexpr int kMaxLine = 1600;          // entries of a line that fit shared memory
+
+struct LineSolve {
+  float r, q, close;   // r, r/c, 1 / (1 - r^n)
+  const float* pw;     // r^k, k = 0 .. ceil(n / kSegs)
+};
+
+// one line per lane (stride `pitch` between its entries in s), segment threadIdx.y;
+// `in(i)` gives entry i, `out(i, x)` takes the solution
+template <class In, class Out>
+__device__ __forceinline__ void solve_lines(float* s, int pitch, int n, const LineSolve& L,
+                                            float (*ends)[2][32], In in, Out out) {
+  const int lane = threadIdx.x, g = threadIdx.y;
+  const int i0 = n * g / kSegs, len = n * (g + 1) / kSegs - i0;
+  float* p = s + i0 * pitch;
+  float y = 0.f;
+#pragma unroll 4
+  for (int i = 0; i < len; ++i) {
+    y = fmaf(L.r, y, in(i0 + i));
+    p[i * pitch] = y;
+  }
+  ends[g][0][lane] = y;
+  __syncthreads();
+  float c = 0.f;
+#pragma unroll
+  for (int h = 0; h < kSegs; ++h)
+    c = fmaf(__ldg(L.pw + (n * (h + 1) / kSegs - n * h / kSegs)), c, ends[h][0][lane]);
+  c *= L.close;                       // what enters entry 0 from the line's end
+  for (int h = 0; h < g; ++h)
+    c = fmaf(__ldg(L.pw + (n * (h + 1) / kSegs - n * h / kSegs)), c, ends[h][0][lane]);
+  float x = 0.f;
+#pragma unroll 4
+  for (int i = len - 1; i >= 0; --i) {
+    x = fmaf(L.r, x, L.q * fmaf(c, __ldg(L.pw + i + 1), p[i * pitch]));
+    p[i * pitch] = x;
+  }
+  ends[g][1][lane] = x;
+  __syncthreads();
+  c = 0.f;
+#pragma unroll
+  for (int h = kSegs - 1; h >= 0; --h)
+    c = fmaf(__ldg(L.pw + (n * (h + 1) / kSegs - n * h / kSegs)), c, ends[h][1][lane]);
+  c *= L.close;
+  for (int h = kSegs - 1; h > g; --h)
+    c = fmaf(__ldg(L.pw + (n * (h + 1) / kSegs - n * h / kSegs)), c, ends[h][1][lane]);
+#pragma unroll 4
+  for (int i = 0; i < len; ++i) out(i0 + i, fmaf(c, __ldg(L.pw + len - i), p[i * pitch]));
+}
+
+// x lines, 32 rows per block: the last pass, added to u
+__global__ void __launch_bounds__(32 * kSegs) line_x_kernel(FGrid G, const float* __restrict__ R,
+                                                            Vec3 u, LineSolve L) {
+  extern __shared__ __align__(16) float smem[];
+  __shared__ float ends[kSegs][2][32];
+  const int n = G.nx, pitch = n | 1;               // odd: no bank conflicts down the rows
+  const int rows = G.ny * G.nz, r0 = 32 * blockIdx.x, nr = min(32, rows - r0);
+  const float* f = R + ((size_t)blockIdx.y * rows + r0) * n;
+  float* uc = (blockIdx.y == 0 ? u.c[0] : (blockIdx.y == 1 ? u.c[1] : u.c[2])) + (size_t)r0 * n;
+  for (int k = threadIdx.y; k < nr; k += kSegs)
+    for (int i = threadIdx.x; i < n; i += 32) smem[k * pitch + i] = f[k * n + i];
+  __syncthreads();
+  float* s = smem + threadIdx.x * pitch;
+  solve_lines(s, 1, n, L, ends, [&](int i) { return s[i]; }, [&](int i, float x) { s[i] = x; });
+  __syncthreads();
+  for (int k = threadIdx.y; k < nr; k += kSegs)
+    for (int i = threadIdx.x; i < n; i += 32) uc[k * n + i] += smem[k * pitch + i];
+}
+
+// y or z lines, in place in R: 32 neighbouring x per block, the other direction
+// in blockIdx.y, the component in blockIdx.z
+template <bool Z>
+__global__ void __launch_bounds__(32 * kSegs) line_yz_kernel(FGrid G, float* __restrict__ R,
+                                                             LineSolve L) {
+  extern __shared__ __align__(16) float smem[];
+  __shared__ float ends[kSegs][2][32];
+  const size_t plane = (size_t)G.nx * G.ny, stride = Z ? plane : (size_t)G.nx;
+  const int n = Z ? G.nz : G.ny, x = 32 * blockIdx.x + threadIdx.x;
+  const bool in_row = x < G.nx;
+  float* f = R + blockIdx.z * plane * G.nz + blockIdx.y * (Z ? (size_t)G.nx : plane) + x;
+  solve_lines(
+      smem + threadIdx.x, 32, n, L, ends,
+      [&](int i) { return in_row ? f[i * stride] : 0.f; },
+      [&](int i, float v) {
+        if (in_row) f[i * stride] = v;
+      });
+}
+
 FGrid fgrid(const ibm_flow* fl);
 
 cudaError_t launch_cn_solve(const ibm_flow* fl, int l, float* u, float* v, float* w,
@@ -791,6 +898,73 @@ cudaError_t launch_cn_solve(const ibm_flow* fl, int l, float* u, float* v, float
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
+}
+
+// The recursions' constants for c = a / h^2, and the powers of r a segment needs.
+double line_root(double c) { return 2.0 * c / (1.0 + 2.0 * c + std::sqrt(1.0 + 4.0 * c)); }
+LineSolve line_solve(double c, int n, const float* pw) {
+  const double r = line_root(c);
+  return {(float)r, (float)(2.0 / (1.0 + 2.0 * c + std::sqrt(1.0 + 4.0 * c))),
+          (float)(1.0 / (1.0 - std::pow(r, n))), pw};
+}
+int line_powers(int n) { return (n + kSegs - 1) / kSegs + 2; }
+
+cudaError_t launch_lines(const ibm_flow* fl, int l, float* u, float* v, float* w, cudaStream_t s) {
+  const FGrid G = fgrid(fl);
+  const double a = (kGamma[l] + kRho[l]) * fl->dt * fl->nu / 2.0;
+  LineSolve L[3];
+  const float* pw = fl->pw + (size_t)l * fl->pw_stride;
+  for (int d = 0; d < 3; ++d) {
+    L[d] = line_solve(a / (fl->h[d] * fl->h[d]), fl->n[d], pw);
+    pw += line_powers(fl->n[d]);
+  }
+  const dim3 block(32, kSegs);
+  const unsigned nx32 = (unsigned)((G.nx + 31) / 32);
+  const int rows = G.ny * G.nz;
+  line_yz_kernel<true><<<dim3(nx32, (unsigned)G.ny, 3), block, 32 * sizeof(float) * G.nz, s>>>(
+      G, fl->R, L[2]);
+  line_yz_kernel<false><<<dim3(nx32, (unsigned)G.nz, 3), block, 32 * sizeof(float) * G.ny, s>>>(
+      G, fl->R, L[1]);
+  line_x_kernel<<<dim3((unsigned)((rows + 31) / 32), 3), block, 32 * sizeof(float) * (G.nx | 1), s>>>(
+      G, fl->R, Vec3{{u, v, w}}, L[0]);
+  return cudaGetLastError();
+}
+
+// The recursions take a substep instead of the transforms while r <= 0.7 (their
+// rounding, about 2/(1 - r) units per direction, is then that of a transform)
+// and lines fit shared memory.  Where 17 taps or fewer do, the fused filters
+// stay: W = 7 on 200 x 180 x 144 takes 145 us.
+bool use_lines(const ibm_flow* fl, int l) {
+  if (fl->solve_w[l] >= 0) return false;
+  const double a = (kGamma[l] + kRho[l]) * fl->dt * fl->nu / 2.0;
+  for (int d = 0; d < 3; ++d)
+    if (fl->n[d] > kMaxLine || line_root(a / (fl->h[d] * fl->h[d])) > 0.7) return false;
+  return fl->n[1] <= 65535 && fl->n[2] <= 65535;   // the launches' grid.y
+}
+
+// device table of the powers, and the kernels' shared memory
+cudaError_t set_up_lines(ibm_flow* fl) {
+  bool any = false;
+  for (int l = 0; l < 3; ++l) any = (fl->lines[l] = use_lines(fl, l)) || any;
+  if (!any) return cudaSuccess;
+  fl->pw_stride = 0;
+  for (int d = 0; d < 3; ++d) fl->pw_stride += line_powers(fl->n[d]);
+  std::vector<float> pw;
+  for (int l = 0; l < 3; ++l) {
+    const double a = (kGamma[l] + kRho[l]) * fl->dt * fl->nu / 2.0;
+    for (int d = 0; d < 3; ++d) {
+      const double r = line_root(a / (fl->h[d] * fl->h[d]));
+      for (int k = 0; k < line_powers(fl->n[d]); ++k) pw.push_back((float)std::pow(r, k));
+    }
+  }
+  cudaError_t e = cudaMalloc(&fl->pw, pw.size() * sizeof(float));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(fl->pw, pw.data(), pw.size() * sizeof(float), cudaMemcpyHostToDevice);
+  const size_t most = 32 * sizeof(float) * (size_t)(std::max({fl->n[0], fl->n[1], fl->n[2]}) | 1);
+  if (e == cudaSuccess) e = allow_smem(line_x_kernel, most);
+  for (auto k : {line_yz_kernel<false>, line_yz_kernel<true>})
+    if (e == cudaSuccess) e = allow_smem(k, most);
+  return e;
 }
 
 FGrid fgrid(const ibm_flow* fl) {
@@ -870,7 +1044,7 @@ void release(ibm_flow* fl) {
     cufftDestroy(fl->c2r1);
   }
   for (void* q : {(void*)fl->H[0], (void*)fl->H[1], (void*)fl->R, (void*)fl->rp, (void*)fl->S,
-                  (void*)fl->lam})
+                  (void*)fl->lam, (void*)fl->pw})
     if (q) cudaFree(q);
   for (auto& row : fl->ev)
     for (cudaEvent_t& ev : row)
@@ -976,7 +1150,7 @@ cudaError_t flow_predict(ibm_flow* fl, int l, float* u, float* v, float* w, cons
   }
   e = cudaGetLastError();
   if (e == cudaSuccess) e = flow_mark(fl, l, 1, s);
-  const bool fourier = fl->solve_w[l] < 0;
+  const bool lines = fl->lines[l], fourier = fl->solve_w[l] < 0 && !lines;
   // real-space path: the three Fourier phases stay empty
   if (e == cudaSuccess && fourier) e = fft_status(cufftExecR2C(fl->r2c3, fl->R, fl->S));
   if (e == cudaSuccess) e = flow_mark(fl, l, 2, s);
@@ -994,7 +1168,7 @@ cudaError_t flow_predict(ibm_flow* fl, int l, float* u, float* v, float* w, cons
     add_kernel<<<dim3(flat_blocks(fl->N), 3), 256, 0, s>>>(Vec3{{u, v, w}}, fl->R, fl->N);
     e = cudaGetLastError();
   } else if (e == cudaSuccess) {
-    e = launch_cn_solve(fl, l, u, v, w, s);
+    e = lines ? launch_lines(fl, l, u, v, w, s) : launch_cn_solve(fl, l, u, v, w, s);
   }
   if (e == cudaSuccess) e = flow_mark(fl, l, 5, s);
   if (e == cudaSuccess) {
@@ -1097,6 +1271,7 @@ extern "C" ibm_status ibm_flow_create(const ibm_grid_desc* grid, double nu, doub
   fl->NC = (size_t)nxh * ny * nz;
   cudaError_t e = cudaSuccess;
   e = ibm::set_solve_smem(fl);
+  if (e == cudaSuccess) e = ibm::set_up_lines(fl);
   for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMalloc(&fl->H[b], 3 * fl->N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fl->R, 3 * fl->N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fl->rp, fl->N * sizeof(float));

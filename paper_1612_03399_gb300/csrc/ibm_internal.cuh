@@ -469,6 +469,23 @@ cudaError_t launch_taylor(ibm_ctx* c, const float* x, double* D);
 cudaError_t launch_interp64(ibm_ctx* c, const float* x, const float* v, const float* u,
                             const float* vv, const float* w, float* U, float* Fm, float* Fext);
 cudaError_t launch_taylor_backward(ibm_ctx* c, const float* x, const double* gD, float* gx);
+// Let a kernel be launched with as much dynamic shared memory as a block can
+// have beside its static part (the limit belongs to the function, not to a
+// context: a smaller one set for one context would fail another's launches);
+// cudaErrorInvalidValue when `bytes` is more than that.
+template <class... A>
+cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
+  cudaFuncAttributes at{};
+  int dev = 0, most = 0;
+  cudaError_t e = cudaFuncGetAttributes(&at, kernel);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  most -= (int)at.sharedSizeBytes;
+  if (bytes > (size_t)most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
 cudaError_t set_force_smem_limit(size_t bytes);
 cudaError_t set_adjoint_smem_limit(size_t bytes);
 cudaError_t set_marker_smem_limit();

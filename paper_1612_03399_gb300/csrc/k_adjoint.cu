@@ -775,8 +775,7 @@ cudaError_t launch_backward(ibm_ctx* c, const float* x, const float* v, const fl
 }
 
 cudaError_t set_adjoint_smem_limit(size_t bytes) {
-  return cudaFuncSetAttribute(force_adjoint_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)bytes);
+  return allow_smem(force_adjoint_kernel, bytes);
 }
 
 }  // namespace ibm

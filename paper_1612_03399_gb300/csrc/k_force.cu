@@ -472,8 +472,7 @@ cudaError_t set_force_smem_limit(size_t bytes) {
                  force_kernel<1, false, true>, force_kernel<2, false, true>,
                  force_kernel<0, false, false>, force_kernel<0, true, false>,
                  force_kernel<1, false, false>, force_kernel<2, false, false>})
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) e = allow_smem(k, bytes);
   return e;
 }
 

@@ -28,220 +28,46 @@
 #include "bulk_copy.cuh"
 #include "force_elems.cuh"
 #include "ibm_internal.cuh"
+#include "mls_closed_form.cuh"
 
 namespace ibm {
 namespace {
 
-__device__ __forceinline__ int wrap(int i, int n) {
-  if (i >= 0 && i < n) return i;
-  if (i < 0 && i >= -n) return i + n;
-  if (i >= n && i < 2 * n) return i - n;
-  i %= n;
-  return i < 0 ? i + n : i;
-}
-
-// per-direction MLS factors a, b = a beta and their first and second
-// derivatives with respect to the point's coordinate in cells (closed form
-// of the factorised weight; see the marker kernel)
-struct DirW2 {
-  float a[3][3], b[3][3];   // [order][node]
-};
-__device__ __forceinline__ void dir_weights_d2(float tp, float kappa, DirW2& o) {
-  float d[3] = {-1.f - tp, -tp, 1.f - tp};
-  float w[3], w1[3], w2[3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    w[s] = __expf(-kappa * d[s] * d[s]);
-    w1[s] = 2.f * kappa * d[s] * w[s];
-    w2[s] = 2.f * kappa * w[s] * (2.f * kappa * d[s] * d[s] - 1.f);
-  }
-  const float invS = 1.f / (w[0] + w[1] + w[2]);
-  const float S1 = w1[0] + w1[1] + w1[2], S2 = w2[0] + w2[1] + w2[2];
-  float a[3], a1[3], a2[3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    a[s] = w[s] * invS;
-    a1[s] = (w1[s] - a[s] * S1) * invS;
-  }
-#pragma unroll
-  for (int s = 0; s < 3; ++s) a2[s] = (w2[s] - 2.f * a1[s] * S1 - a[s] * S2) * invS;
-  float mu = 0.f, mu1 = -1.f, mu2 = 0.f;
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    mu += a[s] * d[s];
-    mu1 += a1[s] * d[s];
-    mu2 += a2[s] * d[s] - a1[s];
-  }
-  const float e1 = -1.f - mu1, e2 = -mu2;   // derivatives of e_s = d_s - mu (same for all s)
-  float Q = 0.f, Q1 = 0.f, Q2 = 0.f;
-  float e[3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    e[s] = d[s] - mu;
-    Q += a[s] * e[s] * e[s];
-    Q1 += a1[s] * e[s] * e[s] + 2.f * a[s] * e[s] * e1;
-    Q2 += a2[s] * e[s] * e[s] + 4.f * a1[s] * e[s] * e1 + 2.f * a[s] * e1 * e1 + 2.f * a[s] * e[s] * e2;
-  }
-  const float iQ = 1.f / Q;
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    const float P = mu * e[s], P1 = mu1 * e[s] + mu * e1, P2 = mu2 * e[s] + 2.f * mu1 * e1 + mu * e2;
-    const float beta = P * iQ;
-    const float beta1 = P1 * iQ - P * Q1 * iQ * iQ;
-    const float beta2 = P2 * iQ - 2.f * P1 * Q1 * iQ * iQ - P * Q2 * iQ * iQ +
-                        2.f * P * Q1 * Q1 * iQ * iQ * iQ;
-    o.a[0][s] = a[s];
-    o.a[1][s] = a1[s];
-    o.a[2][s] = a2[s];
-    o.b[0][s] = a[s] * beta;
-    o.b[1][s] = a1[s] * beta + a[s] * beta1;
-    o.b[2][s] = a2[s] * beta + 2.f * a1[s] * beta1 + a[s] * beta2;
-  }
-}
-
-// gradient (cells) and Hessian (cells; xx, yy, zz, xy, xz, yz) of the MLS
-// interpolant of one velocity component at a point
-__device__ void mls_grad_hess(const float* __restrict__ f, const Grid& g, const float (&tau)[3],
-                              int comp, const int (&G)[3], float kappa, float (&gr)[3],
-                              float (&hs)[6]) {
+// gradient (per length) and Hessian (per length squared) of the MLS interpolant
+// of velocity component `comp` at tau, and value and gradient on any lattice
+__device__ __forceinline__ void grad_hess_at(const float* __restrict__ f, const GlobalRows& R,
+                                             const StepConsts& sc, const float (&tau)[3], int comp,
+                                             float (&gr)[3], float (&hs)[6]) {
   int c[3];
-  float tp[3];
+  float t[3];
+  locate(tau, comp, c, t);
+  DirH X, Y, Z;
+  dir_hess(t[0], sc.mk, X);
+  dir_hess(t[1], sc.mk, Y);
+  dir_hess(t[2], sc.mk, Z);
+  mls_grad_hess(f, R.at(c), X, Y, Z, gr, hs);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const float uu = tau[d] - (d == comp ? 0.f : 0.5f);
-    const float cc = floorf(uu + 0.5f);
-    tp[d] = uu - cc;
-    c[d] = G[d] + (int)cc;
+  for (int j = 0; j < 3; ++j) {
+    gr[j] *= sc.kg[j];
+    hs[j] *= sc.kg[j] * sc.kg[j];
   }
-  DirW2 X, Y, Z;
-  dir_weights_d2(tp[0], kappa, X);
-  dir_weights_d2(tp[1], kappa, Y);
-  dir_weights_d2(tp[2], kappa, Z);
-  int ix[3], iy[3], iz[3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    ix[s] = wrap(c[0] - 1 + s, g.n[0]);
-    iy[s] = wrap(c[1] - 1 + s, g.n[1]);
-    iz[s] = wrap(c[2] - 1 + s, g.n[2]);
-  }
-  // nine derivative patterns (x, y, z orders): 100 010 001 200 020 002 110
-  // 101 011.  Separable contraction: per row the (a, b) sums of the three x
-  // orders as packed pairs; per z-plane, for the six (x, y) order pairs the
-  // patterns use, P = sum_y a_y (xa, xb) and P3 = sum_y b_y xa; then per
-  // pattern acc += a_z (P.x - P.y - P3) - b_z P.x
-  constexpr int GX[6] = {1, 0, 0, 2, 0, 1}, GY[6] = {0, 1, 0, 0, 2, 1};
-  float acc[9];
-#pragma unroll
-  for (int p = 0; p < 9; ++p) acc[p] = 0.f;
-#pragma unroll
-  for (int sz = 0; sz < 3; ++sz) {
-    float2 P[6];
-    float P3[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      P[q] = make_float2(0.f, 0.f);
-      P3[q] = 0.f;
-    }
-#pragma unroll
-    for (int sy = 0; sy < 3; ++sy) {
-      const float* r = f + ((size_t)iz[sz] * g.n[1] + iy[sy]) * g.n[0];
-      const float u0 = __ldg(r + ix[0]), u1 = __ldg(r + ix[1]), u2 = __ldg(r + ix[2]);
-      float2 xo[3];
-#pragma unroll
-      for (int o = 0; o < 3; ++o) {
-        xo[o] = __fmul2_rn(make_float2(X.a[o][0], X.b[o][0]), make_float2(u0, u0));
-        xo[o] = __ffma2_rn(make_float2(X.a[o][1], X.b[o][1]), make_float2(u1, u1), xo[o]);
-        xo[o] = __ffma2_rn(make_float2(X.a[o][2], X.b[o][2]), make_float2(u2, u2), xo[o]);
-      }
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        const float ay = Y.a[GY[q]][sy];
-        P[q] = __ffma2_rn(make_float2(ay, ay), xo[GX[q]], P[q]);
-        P3[q] = fmaf(Y.b[GY[q]][sy], xo[GX[q]].x, P3[q]);
-      }
-    }
-    // pattern p: (x, y) pair and z order
-    constexpr int PQ[9] = {0, 1, 2, 3, 4, 2, 5, 0, 1}, PZ[9] = {0, 0, 1, 0, 0, 2, 0, 1, 1};
-#pragma unroll
-    for (int p = 0; p < 9; ++p) {
-      const int q = PQ[p];
-      acc[p] = fmaf(Z.a[PZ[p]][sz], P[q].x - P[q].y - P3[q], fmaf(-Z.b[PZ[p]][sz], P[q].x, acc[p]));
-    }
-  }
-  gr[0] = acc[0];
-  gr[1] = acc[1];
-  gr[2] = acc[2];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) hs[k] = acc[3 + k];
+  hs[3] *= sc.kg[0] * sc.kg[1];
+  hs[4] *= sc.kg[0] * sc.kg[2];
+  hs[5] *= sc.kg[1] * sc.kg[2];
 }
-
-// value and gradient (cells) of the MLS interpolant of one field at a point
-// (comp 0-2: velocity lattices, 3: cell centres)
-__device__ void mls_val_grad(const float* __restrict__ f, const Grid& g, const float (&tau)[3],
-                             int comp, const int (&G)[3], float kappa, float& val,
-                             float (&gr)[3]) {
+__device__ __forceinline__ void val_grad_at(const float* __restrict__ f, const GlobalRows& R,
+                                            const StepConsts& sc, const float (&tau)[3], int comp,
+                                            float& val, float (&gr)[3]) {
   int c[3];
-  float tp[3];
+  float t[3];
+  locate(tau, comp, c, t);
+  DirG X, Y, Z;
+  dir_grad(t[0], sc.mk, X);
+  dir_grad(t[1], sc.mk, Y);
+  dir_grad(t[2], sc.mk, Z);
+  mls_val_grad(f, R.at(c), X, Y, Z, val, gr);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const float uu = tau[d] - (d == comp ? 0.f : 0.5f);
-    const float cc = floorf(uu + 0.5f);
-    tp[d] = uu - cc;
-    c[d] = G[d] + (int)cc;
-  }
-  DirW2 X, Y, Z;
-  dir_weights_d2(tp[0], kappa, X);
-  dir_weights_d2(tp[1], kappa, Y);
-  dir_weights_d2(tp[2], kappa, Z);
-  int ix[3], iy[3], iz[3];
-#pragma unroll
-  for (int s = 0; s < 3; ++s) {
-    ix[s] = wrap(c[0] - 1 + s, g.n[0]);
-    iy[s] = wrap(c[1] - 1 + s, g.n[1]);
-    iz[s] = wrap(c[2] - 1 + s, g.n[2]);
-  }
-  // value and the three first derivatives (patterns 000 100 010 001), with
-  // the separable contraction of mls_grad_hess: (x, y) order pairs 00, 10, 01
-  constexpr int GX[3] = {0, 1, 0}, GY[3] = {0, 0, 1};
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int sz = 0; sz < 3; ++sz) {
-    float2 P[3];
-    float P3[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      P[q] = make_float2(0.f, 0.f);
-      P3[q] = 0.f;
-    }
-#pragma unroll
-    for (int sy = 0; sy < 3; ++sy) {
-      const float* r = f + ((size_t)iz[sz] * g.n[1] + iy[sy]) * g.n[0];
-      const float u0 = __ldg(r + ix[0]), u1 = __ldg(r + ix[1]), u2 = __ldg(r + ix[2]);
-      float2 xo[2];
-#pragma unroll
-      for (int o = 0; o < 2; ++o) {
-        xo[o] = __fmul2_rn(make_float2(X.a[o][0], X.b[o][0]), make_float2(u0, u0));
-        xo[o] = __ffma2_rn(make_float2(X.a[o][1], X.b[o][1]), make_float2(u1, u1), xo[o]);
-        xo[o] = __ffma2_rn(make_float2(X.a[o][2], X.b[o][2]), make_float2(u2, u2), xo[o]);
-      }
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const float ay = Y.a[GY[q]][sy];
-        P[q] = __ffma2_rn(make_float2(ay, ay), xo[GX[q]], P[q]);
-        P3[q] = fmaf(Y.b[GY[q]][sy], xo[GX[q]].x, P3[q]);
-      }
-    }
-    constexpr int PQ[4] = {0, 1, 2, 0}, PZ[4] = {0, 0, 0, 1};
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int q = PQ[p];
-      acc[p] = fmaf(Z.a[PZ[p]][sz], P[q].x - P[q].y - P3[q], fmaf(-Z.b[PZ[p]][sz], P[q].x, acc[p]));
-    }
-  }
-  val = acc[0];
-  gr[0] = acc[1];
-  gr[1] = acc[2];
-  gr[2] = acc[3];
+  for (int j = 0; j < 3; ++j) gr[j] *= sc.kg[j];
 }
 
 __device__ __forceinline__ float hess_at(const float (&hs)[6], int j, int k) {
@@ -272,23 +98,48 @@ __device__ __forceinline__ void cross3(const float (&a)[3], const float (&b)[3],
   o[2] = a[0] * b[1] - a[1] * b[0];
 }
 
-__global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
+// What bounds it: the latency of the 27-node gathers and of the chain from a
+// face to its weights, hidden only by other warps, so registers decide: with the
+// values a thread keeps across the gathers in shared memory and the Hessian from
+// the closed form's moments (no second-derivative node functions) three blocks
+// fit on an SM.  246 k faces (48 bodies): 72.5 us with sixteen derivative
+// patterns and two blocks, 55.9 us in this form with two, 52.6 us with three
+// (272 bytes of spills).
+__global__ void __launch_bounds__(kMT, 3) ext_adjoint_kernel(
     DeviceTables T, Grid g, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ vel, const float* __restrict__ u, const float* __restrict__ vv,
     const float* __restrict__ w, const float* __restrict__ pr, const float* __restrict__ accel,
     const float* __restrict__ gxn, const float* __restrict__ gvn, const float* __restrict__ gfx,
     const float* __restrict__ gfy, const float* __restrict__ gfz, float* __restrict__ gve) {
+  extern __shared__ __align__(16) float own_[];
   __shared__ double s_red[2][kMT / 32];
   __shared__ int s_last;
+  // values a thread needs before and after the field evaluations, kept here and
+  // not in registers: normal, force cotangent, edges, probe ends, cotangents of
+  // the probe ends, (G + G^T) n and (G + G^T) gF
+  float* own = own_ + threadIdx.x;
+  enum { kN = 0, kGF = 3, kE1 = 6, kE2 = 9, kTP = 12, kTM = 15, kGP = 18, kGM = 21, kTn = 24, kTg = 27 };
+  auto put = [&](int at, const float (&v)[3]) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) own[(at + d) * kMT] = v[d];
+  };
+  auto get = [&](int at, float (&v)[3]) {
+#pragma unroll
+    for (int d = 0; d < 3; ++d) v[d] = own[(at + d) * kMT];
+  };
   const int4 ch = T.chunks[blockIdx.x];
   const BodyDev B = T.body[ch.x];
   const TopoDev topo = T.topo[B.topo];
   double dA = 0.0, dV = 0.0;
-  if ((int)threadIdx.x < ch.z) {
+  float area = 0.f, inv = 0.f, c[3] = {0.f, 0.f, 0.f};
+  int gf = 0, id[3] = {0, 0, 0};
+  const bool mine = (int)threadIdx.x < ch.z, two = !B.closed;
+  if (mine) {
     const int lf = __ldg(T.mface + topo.mface_off + ch.y + threadIdx.x);
-    const int gf = B.f_off + lf;
+    gf = B.f_off + lf;
     const int* tr = T.tri + topo.tri_off + 3 * lf;
-    const int id[3] = {B.v_off + __ldg(tr), B.v_off + __ldg(tr + 1), B.v_off + __ldg(tr + 2)};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) id[k] = B.v_off + __ldg(tr + k);
     float p[3][3], ga[3][3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
@@ -304,7 +155,8 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
     }
     cross3(e1, e2, N);
     const float nn = sqrtf(N[0] * N[0] + N[1] * N[1] + N[2] * N[2]);
-    const float area = 0.5f * nn, inv = 1.f / nn;
+    area = 0.5f * nn;
+    inv = 1.f / nn;
     const float n[3] = {N[0] * inv, N[1] * inv, N[2] * inv};
     // per-body sums grad A . gF and grad V . gF
     {
@@ -335,57 +187,92 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
 #pragma unroll
     for (int d = 0; d < 3; ++d) gF[d] = (ga[0][d] + ga[1][d] + ga[2][d]) * (1.f / 3.f);
     const float third = 1.f / 3.f;
-    float c[3], tpp[3], tpm[3];
+    float tpp[3], tpm[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       c[d] = (p[0][d] + p[1][d] + p[2][d]) * third;
       tpp[d] = fmaf(c[d] + sc.probe_h * n[d], g.invh[d], B.frac[d]);
       tpm[d] = fmaf(c[d] - sc.probe_h * n[d], g.invh[d], B.frac[d]);
     }
-    const bool two = !B.closed;
-    const float* fld[3] = {u, vv, w};
+    const float zero[3] = {0.f, 0.f, 0.f};
+    put(kN, n);
+    put(kGF, gF);
+    put(kE1, e1);
+    put(kE2, e2);
+    put(kTP, tpp);
+    put(kTM, tpm);
+    put(kGP, zero);
+    put(kGM, zero);
+    put(kTn, zero);
+    put(kTg, zero);
+  }
+  // fixed-order per-body sums of grad A . gF and grad V . gF
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    dA += __shfl_down_sync(0xffffffffu, dA, o);
+    dV += __shfl_down_sync(0xffffffffu, dV, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    s_red[0][threadIdx.x >> 5] = dA;
+    s_red[1][threadIdx.x >> 5] = dV;
+  }
+  if (mine) {
     // one gradient-and-Hessian evaluation per component and probe end: the
-    // gradient forms G, the Hessian the position cotangent of the probe ends,
+    // gradient forms G, of which (G + G^T) n and (G + G^T) gF are needed, the
+    // Hessian the position cotangent of the probe ends,
     // gp_k = sum_ij gG_ij H_ijk with gG_ij = mu A (gF_i n_j + gF_j n_i), which
     // does not depend on G
-    float G[3][3];
-    float gpp[3] = {0.f, 0.f, 0.f}, gpm[3] = {0.f, 0.f, 0.f};
+    const GlobalRows rows{g, {B.G[0], B.G[1], B.G[2]}};
     const float s = sc.mu * area;
 #pragma unroll 1
     for (int i = 0; i < 3; ++i) {
-      float gr[3], hs[6];
-      mls_grad_hess(fld[i], g, tpp, i, B.G, sc.kappa, gr, hs);
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        G[i][j] = gr[j] * g.invh[j];
-        const float gG = s * (gF[i] * n[j] + gF[j] * n[i]);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) gpp[k] += gG * hess_at(hs, j, k) * g.invh[j] * g.invh[k];
-      }
-      if (two) {
-        mls_grad_hess(fld[i], g, tpm, i, B.G, sc.kappa, gr, hs);
+      const float* f = i == 0 ? u : (i == 1 ? vv : w);
+      float Gi[3] = {0.f, 0.f, 0.f};
+#pragma unroll 1
+      for (int l = 0; l < (two ? 2 : 1); ++l) {
+        const float sg = l == 0 ? 1.f : -1.f;
+        float t[3], gr[3], hs[6], n[3], gF[3], gp[3];
+        get(kTP + 3 * l, t);
+        grad_hess_at(f, rows, sc, t, i, gr, hs);
+        get(kN, n);
+        get(kGF, gF);
+        get(kGP + 3 * l, gp);
+        const float ni = own[(kN + i) * kMT], gi = own[(kGF + i) * kMT];
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          G[i][j] -= gr[j] * g.invh[j];
-          const float gG = s * (gF[i] * n[j] + gF[j] * n[i]);
+          Gi[j] += sg * gr[j];
+          const float gG = sg * s * (gi * n[j] + gF[j] * ni);
 #pragma unroll
-          for (int k = 0; k < 3; ++k) gpm[k] -= gG * hess_at(hs, j, k) * g.invh[j] * g.invh[k];
+          for (int k = 0; k < 3; ++k) gp[k] += gG * hess_at(hs, j, k);
         }
+        put(kGP + 3 * l, gp);
       }
-    }
-    // F = mu A (G + G^T) n
-    float Tn[3], TgF[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      Tn[i] = 0.f;
-      TgF[i] = 0.f;
+      // row i of G: (G n)_i and (G gF)_i, and n_i G_i. and gF_i G_i. for the transposes
+      float n[3], gF[3], Tn[3], TgF[3];
+      get(kN, n);
+      get(kGF, gF);
+      get(kTn, Tn);
+      get(kTg, TgF);
+      const float ni = own[(kN + i) * kMT], gi = own[(kGF + i) * kMT];
+      const float gn = Gi[0] * n[0] + Gi[1] * n[1] + Gi[2] * n[2];
+      const float gg = Gi[0] * gF[0] + Gi[1] * gF[1] + Gi[2] * gF[2];
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
-        const float Tij = G[i][j] + G[j][i];
-        Tn[i] += Tij * n[j];
-        TgF[i] += Tij * gF[j];
+        Tn[j] = fmaf(ni, Gi[j], Tn[j] + (i == j ? gn : 0.f));
+        TgF[j] = fmaf(gi, Gi[j], TgF[j] + (i == j ? gg : 0.f));
       }
+      put(kTn, Tn);
+      put(kTg, TgF);
     }
+    float n[3], gF[3], Tn[3], TgF[3], gpp[3], gpm[3];
+    get(kN, n);
+    get(kGF, gF);
+    get(kTn, Tn);
+    get(kTg, TgF);
+    get(kGP, gpp);
+    get(kGM, gpm);
+    const float third = 1.f / 3.f;
+    // F = mu A (G + G^T) n
     float gArea = sc.mu * (gF[0] * Tn[0] + gF[1] * Tn[1] + gF[2] * Tn[2]);
     float gn[3] = {sc.mu * area * TgF[0], sc.mu * area * TgF[1], sc.mu * area * TgF[2]};
     // p+- = c +- h n
@@ -407,19 +294,22 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
                    __ldg(accel + d * V + id[2])) * third;
       }
       float P, gpr[3], dPdc[3], dPdn[3];
-      mls_val_grad(pr, g, tpp, 3, B.G, sc.kappa, P, gpr);
+      float t[3];
+      get(kTP, t);
+      val_grad_at(pr, rows, sc, t, 3, P, gpr);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
-        dPdc[d] = gpr[d] * g.invh[d];
+        dPdc[d] = gpr[d];
         dPdn[d] = sc.probe_h * dPdc[d];
       }
       if (two) {
         float Pm;
-        mls_val_grad(pr, g, tpm, 3, B.G, sc.kappa, Pm, gpr);
+        get(kTM, t);
+        val_grad_at(pr, rows, sc, t, 3, Pm, gpr);
         P -= Pm;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const float gd = gpr[d] * g.invh[d];
+          const float gd = gpr[d];
           dPdc[d] -= gd;
           dPdn[d] += sc.probe_h * gd;
         }
@@ -441,7 +331,6 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
       // dL/dF_i = c_l G_i, so the vertex velocities get c_l G_i / (3 dt)
       // each, the centroid c_l (F_i grad G_i - G_i grad U_i / dt) and the
       // area cl_scale sum_i F_i G_i
-      const float* gfs[3] = {gfx, gfy, gfz};
       float tcc[3], vb[3];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
@@ -451,15 +340,15 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
       }
       const float cl = area * sc.cl_scale;
       float gAs = 0.f;
-#pragma unroll
+#pragma unroll 1
       for (int i = 0; i < 3; ++i) {
         float Uv, Ug[3], Gv, Gg[3];
-        mls_val_grad(fld[i], g, tcc, i, B.G, sc.kappa, Uv, Ug);
-        mls_val_grad(gfs[i], g, tcc, i, B.G, sc.kappa, Gv, Gg);
-        const float Fi = (vb[i] - Uv) * sc.inv_dt;
+        val_grad_at(i == 0 ? u : (i == 1 ? vv : w), rows, sc, tcc, i, Uv, Ug);
+        val_grad_at(i == 0 ? gfx : (i == 1 ? gfy : gfz), rows, sc, tcc, i, Gv, Gg);
+        const float Fi = ((i == 0 ? vb[0] : (i == 1 ? vb[1] : vb[2])) - Uv) * sc.inv_dt;
         gAs += Fi * Gv;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) gc[d] += cl * (Fi * Gg[d] - Gv * sc.inv_dt * Ug[d]) * g.invh[d];
+        for (int d = 0; d < 3; ++d) gc[d] += cl * (Fi * Gg[d] - Gv * sc.inv_dt * Ug[d]);
         gve[i * (size_t)F + gf] = cl * Gv * sc.inv_dt * third;
       }
       gArea += sc.cl_scale * gAs;
@@ -470,7 +359,9 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
 #pragma unroll
     for (int d = 0; d < 3; ++d) gN[d] = (gn[d] - gnn * n[d]) * inv + 0.5f * gArea * n[d];
     // N = e1 x e2
-    float ge1[3], ge2[3];
+    float ge1[3], ge2[3], e1[3], e2[3];
+    get(kE1, e1);
+    get(kE2, e2);
     cross3(e2, gN, ge1);
     cross3(gN, e1, ge2);
 #pragma unroll
@@ -480,16 +371,6 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
       T.gxe[(1 * 3 + d) * (size_t)F + gf] = ge1[d] + gcd;
       T.gxe[(2 * 3 + d) * (size_t)F + gf] = ge2[d] + gcd;
     }
-  }
-  // fixed-order per-body sums of grad A . gF and grad V . gF
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dA += __shfl_down_sync(0xffffffffu, dA, o);
-    dV += __shfl_down_sync(0xffffffffu, dV, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    s_red[0][threadIdx.x >> 5] = dA;
-    s_red[1][threadIdx.x >> 5] = dV;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -518,6 +399,8 @@ __global__ void __launch_bounds__(kMT, 2) ext_adjoint_kernel(
     T.counter2[ch.x] = 0;
   }
 }
+
+constexpr size_t kExtBytes = 30 * sizeof(float) * kMT;   // ext_adjoint_kernel's values per thread
 
 struct DSmem {
   float *px, *py, *pz, *tx, *ty, *tz, *cx, *cy, *cz;
@@ -764,9 +647,9 @@ cudaError_t launch_backward(ibm_ctx* c, const float* x, const float* v, const fl
   // per-face velocity cotangents of the spread go to the step's F_ext scratch,
   // unused by the adjoint otherwise
   float* gve = gfx ? c->d.fext : nullptr;
-  ext_adjoint_kernel<<<c->n_chunks, kMT, 0, c->stream>>>(c->d, c->grid, c->sc, (int32_t)c->V,
-                                                         (int32_t)c->F, x, v, u, vv, w, pr, accel,
-                                                         gx_next, gv_next, gfx, gfy, gfz, gve);
+  ext_adjoint_kernel<<<c->n_chunks, kMT, kExtBytes, c->stream>>>(
+      c->d, c->grid, c->sc, (int32_t)c->V, (int32_t)c->F, x, v, u, vv, w, pr, accel, gx_next, gv_next,
+      gfx, gfy, gfz, gve);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   force_adjoint_kernel<<<c->n_work, kForceThreads, c->adjoint_smem, c->stream>>>(

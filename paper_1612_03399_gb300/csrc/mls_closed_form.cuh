@@ -137,7 +137,7 @@ struct GlobalAcc {   // wrapped indices into a full [nz][ny][nx] field
     }
   }
   __device__ __forceinline__ size_t row(int sy, int sz) const {
-    return ((size_t)iz[sz] * ny + iy[sy]) * nx;
+    return (size_t)(unsigned)(iz[sz] * ny + iy[sy]) * (unsigned)nx;   // (rows fit 32 bits)
   }
   __device__ __forceinline__ void load(const float* __restrict__ f, int sy, int sz,
                                        float (&u)[3]) const {
@@ -244,6 +244,123 @@ __device__ __forceinline__ void mls_grad(const float* __restrict__ f, const Acc&
   gr[0] = fmaf(X.h, caa, -fmaf(X.r, gaa, fmaf(Y.r, cca, Z.r * cac)));
   gr[1] = fmaf(Y.h, aca, -fmaf(Y.r, aga, fmaf(X.r, cca, Z.r * acc)));
   gr[2] = fmaf(Z.h, aac, -fmaf(Z.r, aag, fmaf(X.r, cac, Y.r * acc)));
+}
+
+// Second derivatives (the adjoint's).  On three nodes s^3 = s, so the next
+// function of the sequence is one of the two before: d delta/dt / (2 kappa) =
+// (1 - 3q) gamma - 3m delta, q = a_0 + a_2, and no further node function is
+// needed: with D = d/dt / (2 kappa) per direction,
+//   D_x D_x phi = (Dh - (1 - 3q) r)_x gaa + (2h - 1 + 3 m r)_x daa - r_y dga - r_z dag
+//   D_x D_y phi = (h_x + h_y - 1) gga - r_x dga - r_y gda - r_z ggg
+// with Dh = ((1 - 2h) mu3 + r (mu4 - 3 s2^2)) / s2.
+struct DirH : DirG {
+  float k1, k2;   // the coefficients of gaa and daa above
+};
+__device__ __forceinline__ void dir_hess(float t, const MlsK& K, DirH& o) {
+  dir_grad(t, K, o);
+  const float m = o.a2 - o.a0, q = o.a0 + o.a2, m2 = m * m;
+  const float s2 = q - m2;
+  const float mu3 = m * fmaf(-3.f, q, fmaf(2.f, m2, 1.f));
+  const float mu4 = fmaf(-3.f * m, mu3, fmaf(-3.f, m2, 1.f) * s2);
+  const float dh = fmaf(fmaf(-2.f, o.h, 1.f), mu3, o.r * fmaf(-3.f * s2, s2, mu4)) * rcp_fast(s2);
+  o.k1 = fmaf(-o.r, fmaf(-3.f, q, 1.f), dh);
+  o.k2 = fmaf(3.f * m, o.r, fmaf(2.f, o.h, -1.f));
+}
+
+// gradient in cells / (2 kappa) and Hessian in cells / (2 kappa)^2 (xx, yy, zz,
+// xy, xz, yz)
+template <class Acc>
+__device__ __forceinline__ void mls_grad_hess(const float* __restrict__ f, const Acc& A,
+                                              const DirH& X, const DirH& Y, const DirH& Z,
+                                              float (&gr)[3], float (&hs)[6]) {
+  // per z plane the sums over (x, y): aa ac ad ca cc cd da dc (c, d: gamma, delta)
+  auto plane = [&](int sz, float (&P)[8]) {
+    float a[3], c[3], g[3];
+#pragma unroll
+    for (int sy = 0; sy < 3; ++sy) {
+      float u[3];
+      A.load(f, sy, sz, u);
+      const float d0 = u[0] - u[1], d2 = u[2] - u[1];
+      a[sy] = fmaf(X.a2, d2, fmaf(X.a0, d0, u[1]));
+      c[sy] = fmaf(X.c2, d2, X.c0 * d0);
+      g[sy] = fmaf(X.g2, d2, X.g0 * d0);
+    }
+    const float a0 = a[0] - a[1], a2 = a[2] - a[1], c0 = c[0] - c[1], c2 = c[2] - c[1],
+                g0 = g[0] - g[1], g2 = g[2] - g[1];
+    P[0] = fmaf(Y.a2, a2, fmaf(Y.a0, a0, a[1]));
+    P[1] = fmaf(Y.c2, a2, Y.c0 * a0);
+    P[2] = fmaf(Y.g2, a2, Y.g0 * a0);
+    P[3] = fmaf(Y.a2, c2, fmaf(Y.a0, c0, c[1]));
+    P[4] = fmaf(Y.c2, c2, Y.c0 * c0);
+    P[5] = fmaf(Y.g2, c2, Y.g0 * c0);
+    P[6] = fmaf(Y.a2, g2, fmaf(Y.a0, g0, g[1]));
+    P[7] = fmaf(Y.c2, g2, Y.c0 * g0);
+  };
+  float M[8], sa[8], sc[8], sg[4];   // the middle plane; sums with alpha, gamma, delta in z
+  plane(1, M);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    sa[q] = M[q];
+    sc[q] = 0.f;
+    if (q < 4) sg[q] = 0.f;
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    float P[8];
+    plane(2 * k, P);
+    const float za = k ? Z.a2 : Z.a0, zc = k ? Z.c2 : Z.c0, zg = k ? Z.g2 : Z.g0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float d = P[q] - M[q];
+      sa[q] = fmaf(za, d, sa[q]);
+      sc[q] = fmaf(zc, d, sc[q]);
+      if (q < 4) sg[q] = fmaf(zg, d, sg[q]);
+    }
+  }
+  // names: x, y, z letters
+  const float caa = sa[3], aca = sa[1], aac = sc[0], daa = sa[6], ada = sa[2], aad = sg[0];
+  const float cca = sa[4], cac = sc[3], acc = sc[1];
+  const float dca = sa[7], cda = sa[5], dac = sc[6], cad = sg[3], adc = sc[2], acd = sg[1];
+  const float ccc = sc[4];
+  gr[0] = fmaf(X.h, caa, -fmaf(X.r, daa, fmaf(Y.r, cca, Z.r * cac)));
+  gr[1] = fmaf(Y.h, aca, -fmaf(Y.r, ada, fmaf(X.r, cca, Z.r * acc)));
+  gr[2] = fmaf(Z.h, aac, -fmaf(Z.r, aad, fmaf(X.r, cac, Y.r * acc)));
+  hs[0] = fmaf(X.k1, caa, fmaf(X.k2, daa, -fmaf(Y.r, dca, Z.r * dac)));
+  hs[1] = fmaf(Y.k1, aca, fmaf(Y.k2, ada, -fmaf(X.r, cda, Z.r * adc)));
+  hs[2] = fmaf(Z.k1, aac, fmaf(Z.k2, aad, -fmaf(X.r, cad, Y.r * acd)));
+  hs[3] = fmaf(X.h + Y.h - 1.f, cca, -fmaf(X.r, dca, fmaf(Y.r, cda, Z.r * ccc)));
+  hs[4] = fmaf(X.h + Z.h - 1.f, cac, -fmaf(X.r, dac, fmaf(Z.r, cad, Y.r * ccc)));
+  hs[5] = fmaf(Y.h + Z.h - 1.f, acc, -fmaf(Y.r, adc, fmaf(Z.r, acd, X.r * ccc)));
+}
+
+// value, and gradient in cells / (2 kappa)
+template <class Acc>
+__device__ __forceinline__ void mls_val_grad(const float* __restrict__ f, const Acc& A,
+                                             const DirG& X, const DirG& Y, const DirG& Z,
+                                             float& val, float (&gr)[3]) {
+  const PlaneG M = plane_sums(f, A, 1, X, Y);
+  float aaa = M.aa, caa = M.ca, aca = M.ac, aac = 0.f, daa = M.ga, ada = M.ag, aad = 0.f,
+        cca = M.cc, cac = 0.f, acc = 0.f;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const PlaneG P = plane_sums(f, A, 2 * k, X, Y);
+    const float za = k ? Z.a2 : Z.a0, zc = k ? Z.c2 : Z.c0, zg = k ? Z.g2 : Z.g0;
+    const float d0 = P.aa - M.aa, d1 = P.ca - M.ca, d2 = P.ac - M.ac;
+    aaa = fmaf(za, d0, aaa);
+    aac = fmaf(zc, d0, aac);
+    aad = fmaf(zg, d0, aad);
+    caa = fmaf(za, d1, caa);
+    cac = fmaf(zc, d1, cac);
+    aca = fmaf(za, d2, aca);
+    acc = fmaf(zc, d2, acc);
+    daa = fmaf(za, P.ga - M.ga, daa);
+    ada = fmaf(za, P.ag - M.ag, ada);
+    cca = fmaf(za, P.cc - M.cc, cca);
+  }
+  val = aaa - fmaf(X.r, caa, fmaf(Y.r, aca, Z.r * aac));
+  gr[0] = fmaf(X.h, caa, -fmaf(X.r, daa, fmaf(Y.r, cca, Z.r * cac)));
+  gr[1] = fmaf(Y.h, aca, -fmaf(Y.r, ada, fmaf(X.r, cca, Z.r * acc)));
+  gr[2] = fmaf(Z.h, aac, -fmaf(Z.r, aad, fmaf(X.r, cac, Y.r * acc)));
 }
 
 // x >= 0 folded into [0, n)

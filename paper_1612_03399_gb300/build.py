@@ -49,7 +49,7 @@ KERNEL_SOURCES = {
     "clear": ["k_mls.cu", "mls_closed_form.cuh", "bulk_copy.cuh", "ibm_internal.cuh"],
     "forcing": ["k_mls.cu", "mls_closed_form.cuh", "bulk_copy.cuh", "ibm_internal.cuh"],
     "body_marker": ["k_mls.cu", "mls_closed_form.cuh", "bulk_copy.cuh", "ibm_internal.cuh"],
-    "force": ["k_force.cu", "force_elems.cuh", "bulk_copy.cuh", "ibm_internal.cuh"],
+    "force": ["k_force.cu", "force_elems.cuh", "force_smem.cuh", "bulk_copy.cuh", "ibm_internal.cuh"],
     "spread": ["k_tile.cu", "mls_closed_form.cuh", "ibm_internal.cuh"],
     "rhs": ["ibm_flow.cu", "ibm_internal.cuh"],
     "cn_scale": ["ibm_flow.cu", "ibm_internal.cuh"],

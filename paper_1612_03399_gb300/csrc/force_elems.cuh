@@ -1,11 +1,9 @@
 // Element forces of the interaction potentials (Sec. 2.3, Eqs.
-// elaspot..areapot).  edge_forces and face_forces carry Dual numbers (value +
-// directional derivative) in the adjoint, where the derivative part of the
-// forces is the Jacobian-vector product J y of the forces along the tangent y
-// carried by the positions.  J = -Hessian of the energy is symmetric, so the
-// same product is the vector-Jacobian product the adjoint needs.  edge_forward
-// and face_forward are the force kernel's, without the per-constant parts.
-//
+// elaspot..areapot): the forces themselves (edge_forward, face_forward: the
+// force kernel) and their derivatives along the tangents y the positions carry
+// (edge_tangent, face_tangent: the adjoint).  The derivative is the
+// Jacobian-vector product J y; J = -Hessian of the energy is symmetric, so the
+// same product is the vector-Jacobian product the adjoint needs.
 // Edge e = (a, b) with wings c (face (a, b, c)) and d (face (b, a, d)):
 //   spring   W = k_s/2 (l - l0)^2      F_a = k_s (l - l0) e/l, F_b = -F_a
 //   bending  W = k_b (1 - cos(theta - theta0)),  F = -k_b sin(theta - theta0) grad theta,
@@ -24,30 +22,6 @@
 #include <cuda_runtime.h>
 
 namespace ibm {
-
-// forward-mode dual number: value and derivative along one direction
-struct Dual {
-  float v, d;
-  __device__ __forceinline__ Dual() {}
-  __device__ __forceinline__ Dual(float a) : v(a), d(0.f) {}
-  __device__ __forceinline__ Dual(float a, float b) : v(a), d(b) {}
-};
-__device__ __forceinline__ Dual operator+(Dual a, Dual b) { return {a.v + b.v, a.d + b.d}; }
-__device__ __forceinline__ Dual operator-(Dual a, Dual b) { return {a.v - b.v, a.d - b.d}; }
-__device__ __forceinline__ Dual operator-(Dual a) { return {-a.v, -a.d}; }
-__device__ __forceinline__ Dual operator*(Dual a, Dual b) { return {a.v * b.v, a.v * b.d + a.d * b.v}; }
-__device__ __forceinline__ Dual operator/(Dual a, Dual b) {
-  const float r = 1.f / b.v;
-  const float q = a.v * r;
-  return {q, (a.d - q * b.d) * r};
-}
-__device__ __forceinline__ float val(float a) { return a; }
-__device__ __forceinline__ float val(Dual a) { return a.v; }
-__device__ __forceinline__ float rsqrt_(float a) { return rsqrtf(a); }
-__device__ __forceinline__ Dual rsqrt_(Dual a) {
-  const float r = rsqrtf(a.v);
-  return {r, -0.5f * r * r * r * a.d};
-}
 
 template <class T>
 struct Vec {
@@ -72,95 +46,6 @@ __device__ __forceinline__ T vdot(const Vec<T>& a, const Vec<T>& b) {
 template <class T>
 __device__ __forceinline__ Vec<T> vscale(const Vec<T>& a, T s) {
   return {a.x * s, a.y * s, a.z * s};
-}
-
-// Spring and bending of one edge.  fa..fd receive the forces on a, b, c, d;
-// `unit_s` and `unit_b` receive the same forces per unit k_s and k_b (for the
-// constants' gradients); `has_hinge` false on a boundary edge.
-template <class T>
-__device__ __forceinline__ void edge_forces(const Vec<T>& pa, const Vec<T>& pb, const Vec<T>& pc,
-                                            const Vec<T>& pd, bool has_hinge, float l0, float cos0,
-                                            float sin0, float ks, float kb, Vec<T>& fa, Vec<T>& fb,
-                                            Vec<T>& fc, Vec<T>& fd, Vec<T> (&unit_s)[2],
-                                            Vec<T> (&unit_b)[4], float& e_spring, float& e_bend) {
-  const Vec<T> e = vsub(pb, pa);
-  const T l2 = vdot(e, e);
-  const T inv_l = rsqrt_(l2);
-  const T l = l2 * inv_l;
-  const T s_unit = (l - T(l0)) * inv_l;
-  unit_s[0] = vscale(e, s_unit);
-  unit_s[1] = vscale(e, -s_unit);
-  fa = vscale(unit_s[0], T(ks));
-  fb = vscale(unit_s[1], T(ks));
-  const float dl = val(l) - l0;
-  e_spring = 0.5f * ks * dl * dl;
-  const Vec<T> zero = {T(0.f), T(0.f), T(0.f)};
-  fc = zero;
-  fd = zero;
-  e_bend = 0.f;
-  if (!has_hinge) {
-    unit_b[0] = unit_b[1] = unit_b[2] = unit_b[3] = zero;
-    return;
-  }
-  const Vec<T> ac = vsub(pc, pa), ad = vsub(pd, pa);
-  const Vec<T> N1 = vcross(e, ac);
-  const Vec<T> N2 = vcross(vsub(pd, pb), e);
-  const T q1 = vdot(N1, N1), q2 = vdot(N2, N2);
-  const T r1 = rsqrt_(q1), r2 = rsqrt_(q2);
-  const Vec<T> n1 = vscale(N1, r1), n2 = vscale(N2, r2);
-  const T cth = vdot(n1, n2);
-  const T sth = vdot(vcross(n1, n2), e) * inv_l;
-  const T sdiff = sth * T(cos0) - cth * T(sin0);  // sin(theta - theta0)
-  const Vec<T> gc = vscale(N1, -(l * r1 * r1));
-  const Vec<T> gd = vscale(N2, -(l * r2 * r2));
-  const T inv_l2 = inv_l * inv_l;
-  const T sc = vdot(ac, e) * inv_l2, sd = vdot(ad, e) * inv_l2;
-  const T one(1.f);
-  const Vec<T> ga = vadd(vscale(gc, -(one - sc)), vscale(gd, -(one - sd)));
-  const Vec<T> gb = vadd(vscale(gc, -sc), vscale(gd, -sd));
-  const T cu = -sdiff;                 // force per unit k_b: -sin(theta - theta0) grad theta
-  unit_b[0] = vscale(ga, cu);
-  unit_b[1] = vscale(gb, cu);
-  unit_b[2] = vscale(gc, cu);
-  unit_b[3] = vscale(gd, cu);
-  fa = vadd(fa, vscale(unit_b[0], T(kb)));
-  fb = vadd(fb, vscale(unit_b[1], T(kb)));
-  fc = vscale(unit_b[2], T(kb));
-  fd = vscale(unit_b[3], T(kb));
-  e_bend = kb * (1.f - (val(cth) * cos0 + val(sth) * sin0));
-}
-
-// Local area, global area and volume forces of one face.  cA, cV are the
-// per-body coefficients k_A (A - A0)/A0 and k_v (V - V0)/V0 (as T, so that
-// the adjoint can give them their directional derivative).  gradA, gradV
-// receive grad A_f and grad V (body frame) at a, b, c; unit_a the force per
-// unit k_a.
-template <class T>
-__device__ __forceinline__ void face_forces(const Vec<T>& pa, const Vec<T>& pb, const Vec<T>& pc,
-                                            float A0f, float ka, T cA, T cV, Vec<T> (&f)[3],
-                                            Vec<T> (&gradA)[3], Vec<T> (&gradV)[3],
-                                            Vec<T> (&unit_a)[3], float& e_area) {
-  const Vec<T> N = vcross(vsub(pb, pa), vsub(pc, pa));
-  const T q = vdot(N, N);
-  const T rn = rsqrt_(q);
-  const T Af = T(0.5f) * q * rn;
-  const Vec<T> n = vscale(N, rn);
-  const T half(0.5f), sixth(1.f / 6.f);
-  gradA[0] = vscale(vcross(n, vsub(pc, pb)), half);
-  gradA[1] = vscale(vcross(n, vsub(pa, pc)), half);
-  gradA[2] = vscale(vcross(n, vsub(pb, pa)), half);
-  gradV[0] = vscale(vcross(pb, pc), sixth);
-  gradV[1] = vscale(vcross(pc, pa), sixth);
-  gradV[2] = vscale(vcross(pa, pb), sixth);
-  const T strain = (Af - T(A0f)) / T(A0f);
-  const T gA = cA + T(ka) * strain;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    unit_a[k] = vscale(gradA[k], -strain);
-    f[k] = vadd(vscale(gradA[k], -gA), vscale(gradV[k], -cV));
-  }
-  const float da = val(Af) - A0f;
-  e_area = 0.5f * ka * da * da / A0f;
 }
 
 // Spring and bending of one edge, values only.  With N1 = e x ac, N2 = ad x e:
@@ -220,6 +105,89 @@ __device__ __forceinline__ void face_forward(const Vec<float>& pa, const Vec<flo
   f[1] = vadd(fb, v);
   f[2] = {v.x - (fa.x + fb.x), v.y - (fa.y + fb.y), v.z - (fa.z + fb.z)};
   e_area = 0.5f * ka * da * da / A0f;
+}
+
+// k u + l v
+__device__ __forceinline__ Vec<float> vmad(float k, const Vec<float>& u, float l,
+                                           const Vec<float>& v) {
+  return {fmaf(k, u.x, l * v.x), fmaf(k, u.y, l * v.y), fmaf(k, u.z, l * v.z)};
+}
+
+// Derivatives (suffix d) of an edge's forces along the tangents: e, ac, ad with
+// their tangents ed, acd, add (differences of the vertices').  fa..fd receive
+// the derivatives of the forces on a, b, c, d.  uk_s and uk_b receive y . dF/dk_s
+// and y . dF/dk_b, the forces per unit constant against the same tangents, which
+// are the force cotangents: sums of products already at hand.
+__device__ __forceinline__ void edge_tangent(const Vec<float>& e, const Vec<float>& ed,
+                                             const Vec<float>& ac, const Vec<float>& acd,
+                                             const Vec<float>& ad, const Vec<float>& add,
+                                             bool has_hinge, float l0, float cos0, float sin0,
+                                             float ks, float kb, Vec<float>& fa, Vec<float>& fb,
+                                             Vec<float>& fc, Vec<float>& fd, float& uk_s,
+                                             float& uk_b) {
+  const float l2 = vdot(e, e), eed = vdot(e, ed);
+  const float il = rsqrtf(l2), l = l2 * il, ld = eed * il;
+  const float il2 = il * il, ild = -il2 * ld;            // (1/l)' = -l'/l^2
+  const float st = (l - l0) * il, std_ = ld * il + (l - l0) * ild;
+  fa = vmad(ks * std_, e, ks * st, ed);
+  fb = {-fa.x, -fa.y, -fa.z};
+  fc = fd = {0.f, 0.f, 0.f};
+  uk_s = -st * eed;
+  uk_b = 0.f;
+  if (!has_hinge) return;
+  const Vec<float> N1 = vcross(e, ac), N2 = vcross(ad, e);
+  const Vec<float> N1d = vadd(vcross(ed, ac), vcross(e, acd));
+  const Vec<float> N2d = vadd(vcross(add, e), vcross(ad, ed));
+  const float r1 = rsqrtf(vdot(N1, N1)), r2 = rsqrtf(vdot(N2, N2));
+  const float R1 = r1 * r1, R2 = r2 * r2, r12 = r1 * r2;
+  const float h1 = R1 * vdot(N1, N1d), h2 = R2 * vdot(N2, N2d);   // |N|'/|N|
+  const float r12d = -r12 * (h1 + h2);
+  const float D = vdot(N1, N2), Dd = vdot(N1d, N2) + vdot(N1, N2d);
+  const float t = vdot(ad, N1), td = vdot(add, N1) + vdot(ad, N1d);
+  const float cth = D * r12, cthd = Dd * r12 + D * r12d;
+  const float sth = -l * t * r12, sthd = -(ld * t * r12 + l * (td * r12 + t * r12d));
+  const float sn = sth * cos0 - cth * sin0, snd = sthd * cos0 - cthd * sin0;
+  const float s = l * sn, sd_ = ld * sn + l * snd;
+  const float a1 = s * R1, a1d = sd_ * R1 - 2.f * a1 * h1;
+  const float a2 = s * R2, a2d = sd_ * R2 - 2.f * a2 * h2;
+  const Vec<float> uc = vscale(N1, a1), ucd = vmad(a1d, N1, a1, N1d);   // per unit k_b
+  const Vec<float> ud = vscale(N2, a2), udd = vmad(a2d, N2, a2, N2d);
+  const float il2d = 2.f * il * ild;
+  const float pc = vdot(ac, e), pd = vdot(ad, e);
+  const float sc = pc * il2, scd = (vdot(acd, e) + vdot(ac, ed)) * il2 + pc * il2d;
+  const float sd = pd * il2, sdd = (vdot(add, e) + vdot(ad, ed)) * il2 + pd * il2d;
+  const Vec<float> g = vmad(sc, uc, sd, ud);
+  const Vec<float> gd = vadd(vmad(scd, uc, sc, ucd), vmad(sdd, ud, sd, udd));
+  fa = vadd(fa, vscale(vsub(gd, vadd(ucd, udd)), kb));
+  fb = vsub(fb, vscale(gd, kb));
+  fc = vscale(ucd, kb);
+  fd = vscale(udd, kb);
+  uk_b = vdot(uc, acd) + vdot(ud, add) - vdot(g, ed);
+}
+
+// The same for a face: ab, ac with their tangents; cA, cV and their derivatives
+// cAd, cVd; uk_a receives y . dF/dk_a = -strain A'.
+__device__ __forceinline__ void face_tangent(const Vec<float>& ab, const Vec<float>& abd,
+                                             const Vec<float>& ac, const Vec<float>& acd,
+                                             float A0f, float ka, float cA, float cAd, float cV,
+                                             float cVd, Vec<float> (&f)[3], float& uk_a) {
+  const Vec<float> bc = vsub(ac, ab), bcd = vsub(acd, abd);
+  const Vec<float> N = vcross(ab, ac), Nd = vadd(vcross(abd, ac), vcross(ab, acd));
+  const float q = vdot(N, N);
+  const float rn = rsqrtf(q);
+  const float Afd = 0.5f * vdot(N, Nd) * rn;
+  const float strain = __fdividef(0.5f * q * rn - A0f, A0f);
+  const float gA = cA + ka * strain, gAd = cAd + __fdividef(ka * Afd, A0f);
+  const float rnd = -2.f * rn * rn * Afd;                  // (1/|N|)' = -|N|'/|N|^2
+  const float k = -0.5f * rn * gA, kd = -0.5f * fmaf(rnd, gA, rn * gAd);
+  const Vec<float> m = vscale(N, k), md = vmad(kd, N, k, Nd);
+  const Vec<float> v = vmad(cVd * (-1.f / 6.f), N, cV * (-1.f / 6.f), Nd);
+  const Vec<float> fa = vadd(vcross(md, bc), vcross(m, bcd));
+  const Vec<float> fb = vadd(vcross(acd, m), vcross(ac, md));
+  f[0] = vadd(fa, v);
+  f[1] = vadd(fb, v);
+  f[2] = vsub(v, vadd(fa, fb));
+  uk_a = -strain * Afd;
 }
 
 }  // namespace ibm

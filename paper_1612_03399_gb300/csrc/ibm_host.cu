@@ -827,7 +827,7 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     std::vector<float> frest;        // force-kernel rest data per work item, patch order
     std::vector<int64_t> wrest;
     std::vector<FWork> fwork;
-    size_t force_smem = 0, force_smem_wide = 0, adjoint_smem = 0;
+    size_t force_smem = 0, force_smem_wide = 0, adjoint_smem = 0, adjoint_smem_wide = 0;
     c->h_body.resize(n_bodies);
     long long vo = 0, fo = 0, eo = 0;
     for (int b = 0; b < n_bodies; ++b) {
@@ -994,6 +994,7 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
         fw.rest = (int64_t)r0;
         fw.rest_words = frest_words(H.n_edge, H.n_face, varied);
         fw.varied = varied ? 1 : 0;
+        fw.vf_words = Q.vf_words;
         fwork.push_back(fw);
         const size_t own_words = (size_t)Q.blob_words + fw.rest_words;
         const size_t per = (size_t)H.n_loc + Q.n_slot;
@@ -1001,10 +1002,11 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
         force_smem_wide = std::max(force_smem_wide, sizeof(float) * (own_words + 4 * per));
         // the adjoint: blob with its tail, rest data, positions and
         // tangents, slots
-        adjoint_smem = std::max(
-            adjoint_smem, sizeof(float) * ((size_t)Q.blob_words + Q.vf_words +
-                                           frest_words(H.n_edge, H.n_face, varied) +
-                                           6 * (size_t)pad4(H.n_loc) + 3 * (size_t)pad4(Q.n_slot)));
+        const size_t adj = own_words + Q.vf_words;
+        adjoint_smem = std::max(adjoint_smem, sizeof(float) * (adj + 6 * (size_t)pad4(H.n_loc) +
+                                                               3 * (size_t)pad4(Q.n_slot)));
+        adjoint_smem_wide = std::max(
+            adjoint_smem_wide, sizeof(float) * (adj + 4 * (2 * (size_t)H.n_loc + Q.n_slot)));
       }
       vo += Bd.n_vert;
       fo += Bd.n_face;
@@ -1086,7 +1088,8 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     c->force_smem = c->force_wide ? force_smem_wide : force_smem;
     if (c->force_smem > 227 * 1024)
       fail(IBM_ERR_UNSUPPORTED, "force-kernel shared memory above 227 KB; lower patch_size");
-    c->adjoint_smem = adjoint_smem;
+    c->adjoint_wide = adjoint_smem_wide <= 226 * 1024;   // 1 KB for the static part
+    c->adjoint_smem = c->adjoint_wide ? adjoint_smem_wide : adjoint_smem;
     c->max_own = max_own;
     if (c->adjoint_smem > 227 * 1024)
       fail(IBM_ERR_UNSUPPORTED, "force-kernel shared memory above 227 KB; lower patch_size");

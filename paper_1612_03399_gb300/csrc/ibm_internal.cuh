@@ -91,7 +91,7 @@ __host__ __device__ constexpr int frest_words(int n_edge, int n_face, bool varie
   return (varied ? 5 : 3) * pad4(n_edge) + (varied ? 2 : 1) * pad4(n_face);
 }
 
-// What a force-kernel block needs of its work item, in one 64-byte record: a
+// What a force-kernel block needs of its work item, in one record: a
 // block starts its copies and gathers one load after this one, not after the
 // chain work item -> body -> topology -> patch.
 struct alignas(16) FWork {
@@ -100,6 +100,7 @@ struct alignas(16) FWork {
   int32_t loc_off, blob_off, blob_words, n_slot;
   int64_t rest;                               // word offset of the rest data
   int32_t rest_words, varied;
+  int32_t vf_words, pad[3];                   // the adjoint's tail of the blob
 };
 
 struct Grid {
@@ -186,7 +187,7 @@ __device__ __forceinline__ int tiles_along(int f, int n, int T, int (&out)[3]) {
   }
   return k;
 }
-constexpr int kForceThreads = 256;   // threads per block of the adjoint's and advance kernels
+constexpr int kForceThreads = 256;   // threads per block of the advance kernel; most of the adjoint's
 constexpr int kForceThreadsMax = 288;   // most threads of a force-kernel block
 // host mirror of the node update's outputs (ibm_step_host): the force kernel
 // writes x', v' to device arrays and the last block to complete each chunk of
@@ -389,6 +390,7 @@ struct ibm_ctx {
   size_t adjoint_smem = 0;
   int force_threads = ibm::kForceThreads;   // threads per force-kernel block
   bool force_wide = true;           // its positions and slots as float4
+  bool adjoint_wide = true;         // likewise the adjoint's
   int32_t max_own = 0;
   bool have_prev = false;
   // the body sums alternate between two buffers from one ibm_step to the next,

@@ -19,14 +19,17 @@
 // grad A . gF and grad V . gF (fixed order), which the global area and
 // volume terms need.
 //
-// force_adjoint_kernel (per force patch): the element forces evaluated with
-// dual numbers whose tangents are gF give (dF_int/dx) gF (= its transpose:
+// force_adjoint_kernel (per force patch): the derivatives of the element forces
+// along the tangents gF give (dF_int/dx) gF (= its transpose:
 // F_int is minus an energy gradient, so its Jacobian is symmetric); the
 // constants' cotangents are gF . dF/dk, summed per body in a fixed order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "bulk_copy.cuh"
 #include "force_elems.cuh"
+#include "force_smem.cuh"
 #include "ibm_internal.cuh"
 #include "mls_closed_form.cuh"
 
@@ -92,6 +95,30 @@ __device__ __forceinline__ void force_cot(const DeviceTables& T, const StepConst
   }
 }
 
+// Warp sums in float64, which this chip issues at a sixteenth of a warp per cycle
+// and SM: after the first exchange each half or quarter of the warp carries one
+// quantity, 5 and 6 additions instead of 10 and 15.  Lanes 0 and 16 (0, 8 and 16)
+// get the sums; the order is fixed.
+__device__ __forceinline__ double warp_sums(double a, double b) {
+  const bool up = threadIdx.x & 16;
+  double r = up ? b : a;
+  r += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+__device__ __forceinline__ double warp_sums(double a, double b, double c) {
+  const bool up = threadIdx.x & 16, odd = !up && (threadIdx.x & 8);
+  double r = up ? c : a;
+  r += __shfl_xor_sync(0xffffffffu, up ? a : c, 16);
+  b += __shfl_xor_sync(0xffffffffu, b, 16);
+  const double t = __shfl_xor_sync(0xffffffffu, (up || odd) ? r : b, 8);
+  r = (odd ? b : r) + t;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+
 __device__ __forceinline__ void cross3(const float (&a)[3], const float (&b)[3], float (&o)[3]) {
   o[0] = a[1] * b[2] - a[2] * b[1];
   o[1] = a[2] * b[0] - a[0] * b[2];
@@ -104,7 +131,7 @@ __device__ __forceinline__ void cross3(const float (&a)[3], const float (&b)[3],
 // the closed form's moments (no second-derivative node functions) three blocks
 // fit on an SM.  246 k faces (48 bodies): 72.5 us with sixteen derivative
 // patterns and two blocks, 55.9 us in this form with two, 52.6 us with three
-// (272 bytes of spills).
+// (272 bytes of spills), 49.7 us with the packed float64 sums.
 __global__ void __launch_bounds__(kMT, 3) ext_adjoint_kernel(
     DeviceTables T, Grid g, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ vel, const float* __restrict__ u, const float* __restrict__ vv,
@@ -207,14 +234,9 @@ __global__ void __launch_bounds__(kMT, 3) ext_adjoint_kernel(
     put(kTg, zero);
   }
   // fixed-order per-body sums of grad A . gF and grad V . gF
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dA += __shfl_down_sync(0xffffffffu, dA, o);
-    dV += __shfl_down_sync(0xffffffffu, dV, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    s_red[0][threadIdx.x >> 5] = dA;
-    s_red[1][threadIdx.x >> 5] = dV;
+  {
+    const double r = warp_sums(dA, dV);
+    if ((threadIdx.x & 15) == 0) s_red[(threadIdx.x >> 4) & 1][threadIdx.x >> 5] = r;
   }
   if (mine) {
     // one gradient-and-Hessian evaluation per component and probe end: the
@@ -386,47 +408,31 @@ __global__ void __launch_bounds__(kMT, 3) ext_adjoint_kernel(
     s_last = (atomicAdd(T.counter2 + ch.x, 1) == B.n_chunk - 1);
   }
   __syncthreads();
-  if (s_last && threadIdx.x == 0) {
+  if (s_last && threadIdx.x < 32) {   // lanes take every 32nd chunk: a fixed order again
     __threadfence();
-    const volatile double* P = T.partial2;
     double a = 0.0, b = 0.0;
-    for (int k = 0; k < B.n_chunk; ++k) {
-      a += P[2 * (B.chunk_off + k)];
-      b += P[2 * (B.chunk_off + k) + 1];
+    for (int k = threadIdx.x; k < B.n_chunk; k += 32) {
+      a += __ldcg(T.partial2 + 2 * (B.chunk_off + k));
+      b += __ldcg(T.partial2 + 2 * (B.chunk_off + k) + 1);
     }
-    T.dmeas[2 * ch.x] = a;
-    T.dmeas[2 * ch.x + 1] = b;
-    T.counter2[ch.x] = 0;
+    const double r = warp_sums(a, b);
+    if ((threadIdx.x & 15) == 0) T.dmeas[2 * ch.x + (threadIdx.x >> 4)] = r;
+    if (threadIdx.x == 0) T.counter2[ch.x] = 0;
   }
 }
 
 constexpr size_t kExtBytes = 30 * sizeof(float) * kMT;   // ext_adjoint_kernel's values per thread
 
-struct DSmem {
-  float *px, *py, *pz, *tx, *ty, *tz, *cx, *cy, *cz;
-  __device__ Vec<Dual> pos(int i) const {
-    return {Dual(px[i], tx[i]), Dual(py[i], ty[i]), Dual(pz[i], tz[i])};
-  }
-  __device__ Vec<float> cot(int i) const { return {tx[i], ty[i], tz[i]}; }
-  __device__ void put(int s, const Vec<Dual>& f) const {
-    if (s == kNone) return;
-    cx[s] = f.x.d;
-    cy[s] = f.y.d;
-    cz[s] = f.z.d;
-  }
-  __device__ void add(int s, const Vec<Dual>& f) const {
-    if (s == kNone) return;
-    cx[s] += f.x.d;
-    cy[s] += f.y.d;
-    cz[s] += f.z.d;
-  }
-};
-
-__device__ __forceinline__ float dotv(const Vec<float>& a, const Vec<Dual>& b) {
-  return a.x * b.x.v + a.y * b.y.v + a.z * b.z.v;
-}
-
-__global__ void __launch_bounds__(kForceThreads) force_adjoint_kernel(
+// What bounds it: issue, and latency between its barriers, as the force kernel;
+// float64 instructions issue at a sixteenth of a warp per cycle and SM, so only
+// what must be float64 is, once per block where it can be.  48 bodies (246 k
+// faces, 960 patches): 64.9 us with generic forward-mode numbers, narrow slots
+// and a float64 division per thread; 48.1 us with the derivatives written out
+// (edge_tangent, face_tangent) and float4 slots; 41.9 us with the division per
+// block and the packed warp sums.  Three blocks on an SM (80 registers): 43.7 us.
+// The layout goes by the same rule as the force kernel's: float4 where it fits.
+template <bool WIDE>
+__global__ void __launch_bounds__(kForceThreads, 2) force_adjoint_kernel(
     DeviceTables T, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ gxn, const float* __restrict__ gvn, float* __restrict__ gx,
     float* __restrict__ gvo, double* __restrict__ gparams, const float* __restrict__ gve) {
@@ -434,55 +440,47 @@ __global__ void __launch_bounds__(kForceThreads) force_adjoint_kernel(
   __shared__ double s_red[3][kForceThreads / 32];
   __shared__ int s_last;
   __shared__ __align__(8) unsigned long long bar;
-  const int2 wk = T.work[blockIdx.x];
-  const BodyDev B = T.body[wk.x];
-  const TopoDev topo = T.topo[B.topo];
-  const PatchHdr P = T.patch[topo.patch_off + wk.y];
-  const FPatch Q = T.fpatch[topo.patch_off + wk.y];
+  const FWork P = T.fwork[blockIdx.x];
+  const BodyDev& B = T.body[P.body];
   // the forward kernel's blob (edge and face records, slot starts) with the
   // adjoint's tail (each own vertex's faces and corners), the rest data,
   // positions and tangents of the local vertices, contribution slots
   const int pe = pad4(P.n_edge), pf = pad4(P.n_face);
-  const int rest_words = frest_words(P.n_edge, P.n_face, B.varied != 0);
   const uint4* rec = reinterpret_cast<const uint4*>(sm);
   const uint2* frec = reinterpret_cast<const uint2*>(sm + 4 * P.n_edge);
   const uint16_t* ptr = reinterpret_cast<const uint16_t*>(sm + 4 * P.n_edge + 2 * P.n_face);
-  const uint16_t* vptr = reinterpret_cast<const uint16_t*>(sm + Q.blob_words);
-  const uint32_t* vent = reinterpret_cast<const uint32_t*>(sm + Q.blob_words) + (P.n_own + 2) / 2;
-  const float* rest = sm + Q.blob_words + Q.vf_words;
-  DSmem S;
-  S.px = sm + Q.blob_words + Q.vf_words + rest_words;
-  S.py = S.px + pad4(P.n_loc);
-  S.pz = S.py + pad4(P.n_loc);
-  S.tx = S.pz + pad4(P.n_loc);
-  S.ty = S.tx + pad4(P.n_loc);
-  S.tz = S.ty + pad4(P.n_loc);
-  S.cx = S.tz + pad4(P.n_loc);
-  S.cy = S.cx + pad4(Q.n_slot);
-  S.cz = S.cy + pad4(Q.n_slot);
+  const uint16_t* vptr = reinterpret_cast<const uint16_t*>(sm + P.blob_words);
+  const uint32_t* vent = reinterpret_cast<const uint32_t*>(sm + P.blob_words) + (P.n_own + 2) / 2;
+  const float* rest = sm + P.blob_words + P.vf_words;
+  // S: positions and slots; Y: tangents (its slots are S's)
+  Smem<WIDE> S, Y;
+  {
+    float* at = sm + P.blob_words + P.vf_words + P.rest_words;
+    Y.init(at, P.n_loc, P.n_slot);
+    S.init(at + (WIDE ? 4 : 3) * P.n_loc, P.n_loc, P.n_slot);
+  }
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
-    const unsigned nb = 4u * (unsigned)(Q.blob_words + Q.vf_words), nr = 4u * (unsigned)rest_words;
+    const unsigned nb = 4u * (unsigned)(P.blob_words + P.vf_words),
+                   nr = 4u * (unsigned)P.rest_words;
     mbar_arrive_tx(&bar, nb + nr + (unsigned)sc.starve_tx);
-    if (nb) bulk_load(sm, T.fblob + Q.blob_off, nb, &bar);
-    if (nr) bulk_load(sm + Q.blob_words + Q.vf_words, T.frest + T.wrest[blockIdx.x], nr, &bar);
+    if (nb) bulk_load(sm, T.fblob + P.blob_off, nb, &bar);
+    if (nr) bulk_load(sm + P.blob_words + P.vf_words, T.frest + P.rest, nr, &bar);
   }
   for (int i = threadIdx.x; i < P.n_loc; i += blockDim.x) {
-    const int gvx = B.v_off + __ldg(T.loc_vert + P.loc_off + i);
-    S.px[i] = __ldg(x + gvx);
-    S.py[i] = __ldg(x + V + gvx);
-    S.pz[i] = __ldg(x + 2 * V + gvx);
+    const int gvx = P.v_off + __ldg(T.loc_vert + P.loc_off + i);
+    S.set(i, __ldg(x + gvx), __ldg(x + V + gvx), __ldg(x + 2 * V + gvx));
     float o[3];
     force_cot(T, sc, V, gvx, B.inv_mass, gxn, gvn, o);
-    S.tx[i] = o[0];
-    S.ty[i] = o[1];
-    S.tz[i] = o[2];
+    Y.set(i, o[0], o[1], o[2]);
   }
   // global-term coefficients and their derivatives along gF
-  const float2 cf = T.coef[wk.x];
-  const double dA = T.dmeas[2 * wk.x], dV = T.dmeas[2 * wk.x + 1];
-  const Dual cA(cf.x, (float)(B.kA / B.A0 * dA));
-  const Dual cV(cf.y, B.closed ? (float)(B.kv / B.V0 * dV) : 0.f);
+  const float2 cf = T.coef[P.body];
+  if (threadIdx.x == 0) {   // (in every thread the divisions took 2 us a block)
+    s_red[0][0] = B.kA / B.A0 * T.dmeas[2 * P.body];
+    s_red[0][1] = B.closed ? B.kv / B.V0 * T.dmeas[2 * P.body + 1] : 0.0;
+  }
+  const float Bks = B.ks, Bkb = B.kb, Bka = B.ka;
   double gks = 0.0, gkb = 0.0, gka = 0.0;
   __syncthreads();   // positions and tangents staged, barrier initialised
   if (!__syncthreads_and(mbar_wait(&bar, kCopyWaitClocks))) {
@@ -495,32 +493,32 @@ __global__ void __launch_bounds__(kForceThreads) force_adjoint_kernel(
     __syncthreads();
     return;
   }
+  const float cAd = (float)s_red[0][0], cVd = (float)s_red[0][1];   // before the barriers below
   for (int k = threadIdx.x; k < P.n_edge; k += blockDim.x) {
     const uint4 r = rec[k];
     const int la = r.x & 0xFFFF, lb = r.x >> 16, lc = r.y & 0xFFFF, ld = r.y >> 16;
     const bool hinge = ld != kNone;
-    const Vec<Dual> pa = S.pos(la), pb = S.pos(lb);
-    const Vec<Dual> pc = hinge ? S.pos(lc) : pa, pd = hinge ? S.pos(ld) : pb;
+    const Vec<float> pa = S.pos(la), ya = Y.pos(la);
+    const Vec<float> e = vsub(S.pos(lb), pa), ed = vsub(Y.pos(lb), ya);
+    const int wc = hinge ? lc : la, wd = hinge ? ld : lb;
+    const Vec<float> ac = vsub(S.pos(wc), pa), acd = vsub(Y.pos(wc), ya);
+    const Vec<float> ad = vsub(S.pos(wd), pa), add = vsub(Y.pos(wd), ya);
     const float c0 = hinge ? rest[pe + k] : 1.f, s0 = hinge ? rest[2 * pe + k] : 0.f;
-    Vec<Dual> fa, fb, fc, fd, us[2], ub[4];
-    float es, eb;
     // per-edge multipliers m: the forces use m k, the constants' cotangents
     // scale the per-unit-k forces by m
-    const float ms = B.varied ? rest[3 * pe + pf + k] : 1.f;
-    const float mb = B.varied ? rest[4 * pe + pf + k] : 1.f;
-    edge_forces(pa, pb, pc, pd, hinge, rest[k], c0, s0, B.ks * ms, B.kb * mb, fa, fb, fc, fd, us,
-                ub, es, eb);
+    const float ms = P.varied ? rest[3 * pe + pf + k] : 1.f;
+    const float mb = P.varied ? rest[4 * pe + pf + k] : 1.f;
+    Vec<float> fa, fb, fc, fd;
+    float us, ub;
+    edge_tangent(e, ed, ac, acd, ad, add, hinge, rest[k], c0, s0, Bks * ms, Bkb * mb, fa, fb, fc,
+                 fd, us, ub);
     S.put(r.z & 0xFFFF, fa);
     S.put(r.z >> 16, fb);
     S.put(r.w & 0xFFFF, fc);
     S.put(r.w >> 16, fd);
     if ((r.z & 0xFFFF) != kNone) {   // owned edge: constants' cotangents
-      const Vec<float> ca = S.cot(la), cb = S.cot(lb);
-      gks += ms * (dotv(ca, us[0]) + dotv(cb, us[1]));
-      if (hinge) {
-        const Vec<float> cc = S.cot(lc), cd = S.cot(ld);
-        gkb += mb * (dotv(ca, ub[0]) + dotv(cb, ub[1]) + dotv(cc, ub[2]) + dotv(cd, ub[3]));
-      }
+      gks += ms * us;
+      gkb += mb * ub;
     }
   }
   __syncthreads();   // every edge slot written
@@ -536,33 +534,34 @@ __global__ void __launch_bounds__(kForceThreads) force_adjoint_kernel(
     const int d0 = right ? (int)(r.z >> 16) : (int)(r.z & 0xFFFF);
     const int d1 = right ? (int)(r.z & 0xFFFF) : (int)(r.z >> 16);
     const int d2 = right ? (int)(r.w >> 16) : (int)(r.w & 0xFFFF);
-    Vec<Dual> f[3], gA[3], gV[3], ua[3];
-    float ea;
-    const float ma = B.varied ? rest[5 * pe + pf + k] : 1.f;
-    face_forces(S.pos(v0), S.pos(v1), S.pos(v2), rest[3 * pe + k], B.ka * ma, cA, cV, f, gA, gV,
-                ua, ea);
+    Vec<float> f[3];
+    float ua;
+    const float ma = P.varied ? rest[5 * pe + pf + k] : 1.f;
+    const Vec<float> pa = S.pos(v0), ya = Y.pos(v0);
+    face_tangent(vsub(S.pos(v1), pa), vsub(Y.pos(v1), ya), vsub(S.pos(v2), pa), vsub(Y.pos(v2), ya),
+                 rest[3 * pe + k], Bka * ma, cf.x, cAd, cf.y, cVd, f, ua);
     S.add(d0, f[0]);
     S.add(d1, f[1]);
     S.add(d2, f[2]);
-    if (fr.x >> 31)
-      gka += ma * (dotv(S.cot(v0), ua[0]) + dotv(S.cot(v1), ua[1]) + dotv(S.cot(v2), ua[2]));
+    if (fr.x >> 31) gka += ma * ua;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < P.n_own; i += blockDim.x) {
     const int s0 = ptr[i], s1 = ptr[i + 1];
     float jx = 0.f, jy = 0.f, jz = 0.f;
     for (int s = s0; s < s1; ++s) {
-      jx += S.cx[s];
-      jy += S.cy[s];
-      jz += S.cz[s];
+      const Vec<float> t = S.slot(s);
+      jx += t.x;
+      jy += t.y;
+      jz += t.z;
     }
-    const int gvx = B.v_off + P.own0 + i;
+    const int gvx = P.v_off + P.own0 + i;
     // traction part: the cotangents the faces left for this corner
     float wx = 0.f, wy = 0.f, wz = 0.f;   // the spread's velocity cotangent
     for (int q = vptr[i]; q < vptr[i + 1]; ++q) {
       const uint32_t e = vent[q];
       const int corner = (int)(e >> 30);
-      const size_t gf = (size_t)B.f_off + (e & 0x3FFFFFFFu);
+      const size_t gf = (size_t)P.f_off + (e & 0x3FFFFFFFu);
       jx += __ldg(T.gxe + (corner * 3 + 0) * (size_t)F + gf);
       jy += __ldg(T.gxe + (corner * 3 + 1) * (size_t)F + gf);
       jz += __ldg(T.gxe + (corner * 3 + 2) * (size_t)F + gf);
@@ -583,22 +582,17 @@ __global__ void __launch_bounds__(kForceThreads) force_adjoint_kernel(
     gvo[V + gvx] = (cl ? 0.f : __ldg(gvn + V + gvx) + sc.dt * gx1) + wy;
     gvo[2 * V + gvx] = (cl ? 0.f : __ldg(gvn + 2 * V + gvx) + sc.dt * gx2) + wz;
   }
+  const int n_patch = T.topo[B.topo].n_patch;
   // constants' cotangents: fixed-order per-patch sums, then per body
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    gks += __shfl_down_sync(0xffffffffu, gks, o);
-    gkb += __shfl_down_sync(0xffffffffu, gkb, o);
-    gka += __shfl_down_sync(0xffffffffu, gka, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    s_red[0][threadIdx.x >> 5] = gks;
-    s_red[1][threadIdx.x >> 5] = gkb;
-    s_red[2][threadIdx.x >> 5] = gka;
+  {
+    const double r = warp_sums(gks, gkb, gka);
+    const int q = (threadIdx.x & 31) >> 3;
+    if ((threadIdx.x & 7) == 0 && q < 3) s_red[q][threadIdx.x >> 5] = r;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0.0, b = 0.0, c = 0.0;
-    for (int k = 0; k < kForceThreads / 32; ++k) {
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
       a += s_red[0][k];
       b += s_red[1][k];
       c += s_red[2][k];
@@ -607,25 +601,27 @@ __global__ void __launch_bounds__(kForceThreads) force_adjoint_kernel(
     T.wpart[3 * (size_t)blockIdx.x + 1] = b;
     T.wpart[3 * (size_t)blockIdx.x + 2] = c;
     __threadfence();
-    s_last = (atomicAdd(T.wcounter + wk.x, 1) == topo.n_patch - 1);
+    s_last = (atomicAdd(T.wcounter + P.body, 1) == n_patch - 1);
   }
   __syncthreads();
-  if (s_last && threadIdx.x == 0) {
+  if (s_last && threadIdx.x < 32) {
     __threadfence();
-    const volatile double* W = T.wpart;
     double a = 0.0, b = 0.0, c = 0.0;
-    for (int k = 0; k < topo.n_patch; ++k) {
-      a += W[3 * (size_t)(B.work_off + k)];
-      b += W[3 * (size_t)(B.work_off + k) + 1];
-      c += W[3 * (size_t)(B.work_off + k) + 2];
+    for (int k = threadIdx.x; k < n_patch; k += 32) {
+      const double* W = T.wpart + 3 * (size_t)(B.work_off + k);
+      a += __ldcg(W);
+      b += __ldcg(W + 1);
+      c += __ldcg(W + 2);
     }
-    const double Ab = T.meas[2 * wk.x], Vb = T.meas[2 * wk.x + 1];
-    gparams[5 * wk.x + 0] = a;
-    gparams[5 * wk.x + 1] = b;
-    gparams[5 * wk.x + 2] = c;
-    gparams[5 * wk.x + 3] = -(Ab - B.A0) / B.A0 * dA;
-    gparams[5 * wk.x + 4] = B.closed ? -(Vb - B.V0) / B.V0 * dV : 0.0;
-    T.wcounter[wk.x] = 0;
+    const double r = warp_sums(a, b, c);
+    const int q = threadIdx.x >> 3;
+    if ((threadIdx.x & 7) == 0 && q < 3) gparams[5 * P.body + q] = r;
+    if (threadIdx.x == 0) {
+      const double Ab = T.meas[2 * P.body], Vb = T.meas[2 * P.body + 1];
+      gparams[5 * P.body + 3] = -(Ab - B.A0) / B.A0 * T.dmeas[2 * P.body];
+      gparams[5 * P.body + 4] = B.closed ? -(Vb - B.V0) / B.V0 * T.dmeas[2 * P.body + 1] : 0.0;
+      T.wcounter[P.body] = 0;
+    }
   }
 }
 
@@ -652,13 +648,15 @@ cudaError_t launch_backward(ibm_ctx* c, const float* x, const float* v, const fl
       gfx, gfy, gfz, gve);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  force_adjoint_kernel<<<c->n_work, kForceThreads, c->adjoint_smem, c->stream>>>(
+  auto kernel = c->adjoint_wide ? force_adjoint_kernel<true> : force_adjoint_kernel<false>;
+  kernel<<<c->n_work, std::min(c->force_threads, kForceThreads), c->adjoint_smem, c->stream>>>(
       c->d, c->sc, (int32_t)c->V, (int32_t)c->F, x, gx_next, gv_next, gx, gv, gparams, gve);
   return cudaGetLastError();
 }
 
 cudaError_t set_adjoint_smem_limit(size_t bytes) {
-  return allow_smem(force_adjoint_kernel, bytes);
+  const cudaError_t e = allow_smem(force_adjoint_kernel<true>, bytes);
+  return e == cudaSuccess ? allow_smem(force_adjoint_kernel<false>, bytes) : e;
 }
 
 }  // namespace ibm

@@ -20,68 +20,11 @@
 
 #include "bulk_copy.cuh"
 #include "force_elems.cuh"
+#include "force_smem.cuh"
 #include "ibm_internal.cuh"
 
 namespace ibm {
 namespace {
-
-// Positions and contribution slots in shared memory: as float4 (WIDE, one
-// shared load or store each), or as three arrays, a quarter smaller, for
-// patches whose float4 form does not fit (above about 650 vertices).
-template <bool WIDE>
-struct Smem;
-template <>
-struct Smem<true> {
-  float4 *p, *c;
-  __device__ __forceinline__ void init(float* s, int n_loc, int) {
-    p = reinterpret_cast<float4*>(s);
-    c = p + n_loc;
-  }
-  __device__ __forceinline__ void set(int i, float x, float y, float z) const {
-    p[i] = make_float4(x, y, z, 0.f);
-  }
-  __device__ __forceinline__ Vec<float> pos(int i) const {
-    const float4 t = p[i];
-    return {t.x, t.y, t.z};
-  }
-  __device__ __forceinline__ Vec<float> slot(int s) const {
-    const float4 t = c[s];
-    return {t.x, t.y, t.z};
-  }
-  __device__ __forceinline__ void put(int s, const Vec<float>& f) const {
-    if (s != kNone) c[s] = make_float4(f.x, f.y, f.z, 0.f);
-  }
-  __device__ __forceinline__ void add(int s, const Vec<float>& f) const {
-    if (s != kNone) put(s, vadd(slot(s), f));
-  }
-};
-template <>
-struct Smem<false> {
-  float *p, *c;
-  int np, nc;
-  __device__ __forceinline__ void init(float* s, int n_loc, int n_slot) {
-    p = s;
-    np = n_loc;
-    c = s + 3 * n_loc;
-    nc = n_slot;
-  }
-  __device__ __forceinline__ void set(int i, float x, float y, float z) const {
-    p[i] = x;
-    p[np + i] = y;
-    p[2 * np + i] = z;
-  }
-  __device__ __forceinline__ Vec<float> pos(int i) const { return {p[i], p[np + i], p[2 * np + i]}; }
-  __device__ __forceinline__ Vec<float> slot(int s) const { return {c[s], c[nc + s], c[2 * nc + s]}; }
-  __device__ __forceinline__ void put(int s, const Vec<float>& f) const {
-    if (s == kNone) return;
-    c[s] = f.x;
-    c[nc + s] = f.y;
-    c[2 * nc + s] = f.z;
-  }
-  __device__ __forceinline__ void add(int s, const Vec<float>& f) const {
-    if (s != kNone) put(s, vadd(slot(s), f));
-  }
-};
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

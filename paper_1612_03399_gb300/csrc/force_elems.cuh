@@ -1,7 +1,6 @@
 // Element forces of the interaction potentials (Sec. 2.3, Eqs.
-// elaspot..areapot): the forces themselves (edge_forward, face_forward: the
-// force kernel) and their derivatives along the tangents y the positions carry
-// (edge_tangent, face_tangent: the adjoint).  The derivative is the
+// elaspot..areapot): the forces themselves (*_forward: the force kernel) and their derivatives along the tangents y the positions carry
+// (*_tangent: the adjoint).  The derivative is the
 // Jacobian-vector product J y; J = -Hessian of the energy is symmetric, so the
 // same product is the vector-Jacobian product the adjoint needs.
 // Edge e = (a, b) with wings c (face (a, b, c)) and d (face (b, a, d)):
@@ -48,28 +47,26 @@ __device__ __forceinline__ Vec<T> vscale(const Vec<T>& a, T s) {
   return {a.x * s, a.y * s, a.z * s};
 }
 
-// Spring and bending of one edge, values only.  With N1 = e x ac, N2 = ad x e:
-// (n1 x n2).e/|e| = -|e| (ad.N1)/(|N1||N2|), the force on b is what makes the
-// four sum to zero, and energies are formed only where they are used.
-__device__ __forceinline__ void edge_forward(const Vec<float>& pa, const Vec<float>& pb,
-                                             const Vec<float>& pc, const Vec<float>& pd,
-                                             bool has_hinge, float l0, float cos0, float sin0,
-                                             float ks, float kb, Vec<float>& fa, Vec<float>& fb,
-                                             Vec<float>& fc, Vec<float>& fd, float& e_spring,
-                                             float& e_bend) {
-  const Vec<float> e = vsub(pb, pa);
+// Values only.  An edge with its hinge: e = pb - pa, ac and ad from a to the
+// wings, N1 = e x ac and N2 = ad x e the normals of its left face (a, b, c) and
+// right face (b, a, d), r1 and r2 their inverse lengths.  (n1 x n2).e/|e| =
+// -|e| (ad.N1)/(|N1||N2|), the force on b is what makes the four sum to zero,
+// and energies are formed only where they are used.
+__device__ __forceinline__ void spring_forward(const Vec<float>& e, float l0, float ks, float& l,
+                                               float& inv_l, Vec<float>& fa, float& e_spring) {
   const float l2 = vdot(e, e);
-  const float inv_l = rsqrtf(l2);
-  const float l = l2 * inv_l, dl = l - l0;
+  inv_l = rsqrtf(l2);
+  l = l2 * inv_l;
+  const float dl = l - l0;
   fa = vscale(e, ks * dl * inv_l);
-  fb = {-fa.x, -fa.y, -fa.z};
-  fc = fd = {0.f, 0.f, 0.f};
   e_spring = 0.5f * ks * dl * dl;
-  e_bend = 0.f;
-  if (!has_hinge) return;
-  const Vec<float> ac = vsub(pc, pa), ad = vsub(pd, pa);
-  const Vec<float> N1 = vcross(e, ac), N2 = vcross(ad, e);
-  const float r1 = rsqrtf(vdot(N1, N1)), r2 = rsqrtf(vdot(N2, N2));
+}
+__device__ __forceinline__ void hinge_forward(const Vec<float>& e, float l, float inv_l,
+                                              const Vec<float>& ac, const Vec<float>& ad,
+                                              const Vec<float>& N1, const Vec<float>& N2, float r1,
+                                              float r2, float cos0, float sin0, float kb,
+                                              Vec<float>& fa, Vec<float>& fb, Vec<float>& fc,
+                                              Vec<float>& fd, float& e_bend) {
   const float r12 = r1 * r2;
   const float cth = vdot(N1, N2) * r12, sth = -l * vdot(ad, N1) * r12;
   const float s = kb * l * (sth * cos0 - cth * sin0);   // k_b |e| sin(theta - theta0)
@@ -83,27 +80,28 @@ __device__ __forceinline__ void edge_forward(const Vec<float>& pa, const Vec<flo
   e_bend = kb * (1.f - (cth * cos0 + sth * sin0));
 }
 
-// Local area, global area and volume forces of one face, values only.  The
-// area part is (m x (c - b), m x (a - c), minus their sum) with
-// m = -(c_A + k_a strain) n / 2.  The volume part gives every corner a third of
-// the face's normal, -c_V N / 6: grad_a V = b x c / 6 differs from N / 6 by
-// a x (c - b) / 6, whose sum over the closed fan of faces around a vertex is
-// zero (c_V is zero on open sheets), and N carries no products of the
-// body-frame coordinates.
-__device__ __forceinline__ void face_forward(const Vec<float>& pa, const Vec<float>& pb,
-                                             const Vec<float>& pc, float A0f, float ka, float cA,
-                                             float cV, Vec<float> (&f)[3], float& e_area) {
-  const Vec<float> ab = vsub(pb, pa), ac = vsub(pc, pa), bc = vsub(ac, ab);
-  const Vec<float> N = vcross(ab, ac);
-  const float q = vdot(N, N);
-  const float rn = rsqrtf(q);
-  const float da = 0.5f * q * rn - A0f;
-  const Vec<float> m = vscale(N, -0.5f * rn * (cA + ka * __fdividef(da, A0f)));
-  const Vec<float> v = vscale(N, cV * (-1.f / 6.f));
-  const Vec<float> fa = vcross(m, bc), fb = vcross(ac, m);   // m x (a - c) = ac x m
-  f[0] = vadd(fa, v);
-  f[1] = vadd(fb, v);
-  f[2] = {v.x - (fa.x + fb.x), v.y - (fa.y + fb.y), v.z - (fa.z + fb.z)};
+// Local area, global area and volume forces of the face on one side of an edge:
+// N its normal, rn = 1/|N|, w the vector from a to its third vertex, side = 1
+// (left face) or -1 (right face, which runs from b to a).  fa, fb, fw are added
+// to.  The area part is m x (w - e), -m x w and m x e with m = -side (c_A + k_a
+// strain) n / 2.  The volume part gives every corner a third of the face's
+// normal, -c_V N / 6: grad_a V = b x c / 6 differs from N / 6 by a x (c - b) / 6,
+// whose sum over the closed fan of faces around a vertex is zero (c_V is zero on
+// open sheets), and N carries no products of the body-frame coordinates.  t: a
+// load every corner gets besides.
+__device__ __forceinline__ void face_forward(const Vec<float>& e, const Vec<float>& w,
+                                             const Vec<float>& N, float rn, float side, float A0f,
+                                             float ka, float cA, float cV, const Vec<float>& t,
+                                             Vec<float>& fa, Vec<float>& fb, Vec<float>& fw,
+                                             float& e_area) {
+  const float da = 0.5f * vdot(N, N) * rn - A0f;
+  const float k = -0.5f * side * rn * (cA + ka * __fdividef(da, A0f)), kv = cV * (-1.f / 6.f);
+  const Vec<float> m = vscale(N, k);
+  const Vec<float> X = vcross(m, w), Y = vcross(m, e);
+  const Vec<float> v = {fmaf(kv, N.x, t.x), fmaf(kv, N.y, t.y), fmaf(kv, N.z, t.z)};
+  fa = vadd(fa, vadd(vsub(X, Y), v));
+  fb = vadd(fb, vsub(v, X));
+  fw = vadd(fw, vadd(Y, v));
   e_area = 0.5f * ka * da * da / A0f;
 }
 
@@ -113,34 +111,31 @@ __device__ __forceinline__ Vec<float> vmad(float k, const Vec<float>& u, float l
   return {fmaf(k, u.x, l * v.x), fmaf(k, u.y, l * v.y), fmaf(k, u.z, l * v.z)};
 }
 
-// Derivatives (suffix d) of an edge's forces along the tangents: e, ac, ad with
-// their tangents ed, acd, add (differences of the vertices').  fa..fd receive
-// the derivatives of the forces on a, b, c, d.  uk_s and uk_b receive y . dF/dk_s
-// and y . dF/dk_b, the forces per unit constant against the same tangents, which
+// Derivatives (suffix d) of the same along the tangents: e, ac, ad, w with their
+// tangents ed, acd, add, wd (differences of the vertices').  fa..fd receive the
+// derivatives of the forces.  uk_s, uk_b and uk_a receive y . dF/dk_s, y . dF/dk_b
+// and y . dF/dk_a, the forces per unit constant against the same tangents, which
 // are the force cotangents: sums of products already at hand.
-__device__ __forceinline__ void edge_tangent(const Vec<float>& e, const Vec<float>& ed,
-                                             const Vec<float>& ac, const Vec<float>& acd,
-                                             const Vec<float>& ad, const Vec<float>& add,
-                                             bool has_hinge, float l0, float cos0, float sin0,
-                                             float ks, float kb, Vec<float>& fa, Vec<float>& fb,
-                                             Vec<float>& fc, Vec<float>& fd, float& uk_s,
-                                             float& uk_b) {
+__device__ __forceinline__ void spring_tangent(const Vec<float>& e, const Vec<float>& ed, float l0,
+                                               float ks, float& l, float& ld, float& il, float& ild,
+                                               Vec<float>& fa, float& uk_s) {
   const float l2 = vdot(e, e), eed = vdot(e, ed);
-  const float il = rsqrtf(l2), l = l2 * il, ld = eed * il;
-  const float il2 = il * il, ild = -il2 * ld;            // (1/l)' = -l'/l^2
+  il = rsqrtf(l2);
+  l = l2 * il;
+  ld = eed * il;
+  ild = -il * il * ld;                                   // (1/l)' = -l'/l^2
   const float st = (l - l0) * il, std_ = ld * il + (l - l0) * ild;
   fa = vmad(ks * std_, e, ks * st, ed);
-  fb = {-fa.x, -fa.y, -fa.z};
-  fc = fd = {0.f, 0.f, 0.f};
   uk_s = -st * eed;
-  uk_b = 0.f;
-  if (!has_hinge) return;
-  const Vec<float> N1 = vcross(e, ac), N2 = vcross(ad, e);
-  const Vec<float> N1d = vadd(vcross(ed, ac), vcross(e, acd));
-  const Vec<float> N2d = vadd(vcross(add, e), vcross(ad, ed));
-  const float r1 = rsqrtf(vdot(N1, N1)), r2 = rsqrtf(vdot(N2, N2));
+}
+// N1d, N2d: the normals' tangents; h1, h2: |N|'/|N|
+__device__ __forceinline__ void hinge_tangent(
+    const Vec<float>& e, const Vec<float>& ed, float l, float ld, float il, float ild,
+    const Vec<float>& ac, const Vec<float>& acd, const Vec<float>& ad, const Vec<float>& add,
+    const Vec<float>& N1, const Vec<float>& N1d, const Vec<float>& N2, const Vec<float>& N2d,
+    float r1, float r2, float h1, float h2, float cos0, float sin0, float kb, Vec<float>& fa,
+    Vec<float>& fb, Vec<float>& fc, Vec<float>& fd, float& uk_b) {
   const float R1 = r1 * r1, R2 = r2 * r2, r12 = r1 * r2;
-  const float h1 = R1 * vdot(N1, N1d), h2 = R2 * vdot(N2, N2d);   // |N|'/|N|
   const float r12d = -r12 * (h1 + h2);
   const float D = vdot(N1, N2), Dd = vdot(N1d, N2) + vdot(N1, N2d);
   const float t = vdot(ad, N1), td = vdot(add, N1) + vdot(ad, N1d);
@@ -152,7 +147,7 @@ __device__ __forceinline__ void edge_tangent(const Vec<float>& e, const Vec<floa
   const float a2 = s * R2, a2d = sd_ * R2 - 2.f * a2 * h2;
   const Vec<float> uc = vscale(N1, a1), ucd = vmad(a1d, N1, a1, N1d);   // per unit k_b
   const Vec<float> ud = vscale(N2, a2), udd = vmad(a2d, N2, a2, N2d);
-  const float il2d = 2.f * il * ild;
+  const float il2 = il * il, il2d = 2.f * il * ild;
   const float pc = vdot(ac, e), pd = vdot(ad, e);
   const float sc = pc * il2, scd = (vdot(acd, e) + vdot(ac, ed)) * il2 + pc * il2d;
   const float sd = pd * il2, sdd = (vdot(add, e) + vdot(ad, ed)) * il2 + pd * il2d;
@@ -164,29 +159,25 @@ __device__ __forceinline__ void edge_tangent(const Vec<float>& e, const Vec<floa
   fd = vscale(udd, kb);
   uk_b = vdot(uc, acd) + vdot(ud, add) - vdot(g, ed);
 }
-
-// The same for a face: ab, ac with their tangents; cA, cV and their derivatives
-// cAd, cVd; uk_a receives y . dF/dk_a = -strain A'.
-__device__ __forceinline__ void face_tangent(const Vec<float>& ab, const Vec<float>& abd,
-                                             const Vec<float>& ac, const Vec<float>& acd,
-                                             float A0f, float ka, float cA, float cAd, float cV,
-                                             float cVd, Vec<float> (&f)[3], float& uk_a) {
-  const Vec<float> bc = vsub(ac, ab), bcd = vsub(acd, abd);
-  const Vec<float> N = vcross(ab, ac), Nd = vadd(vcross(abd, ac), vcross(ab, acd));
-  const float q = vdot(N, N);
-  const float rn = rsqrtf(q);
-  const float Afd = 0.5f * vdot(N, Nd) * rn;
-  const float strain = __fdividef(0.5f * q * rn - A0f, A0f);
+// h = |N|'/|N|; cA, cV and their derivatives cAd, cVd
+__device__ __forceinline__ void face_tangent(const Vec<float>& e, const Vec<float>& ed,
+                                             const Vec<float>& w, const Vec<float>& wd,
+                                             const Vec<float>& N, const Vec<float>& Nd, float rn,
+                                             float h, float side, float A0f, float ka, float cA,
+                                             float cAd, float cV, float cVd, Vec<float>& fa,
+                                             Vec<float>& fb, Vec<float>& fw, float& uk_a) {
+  const float Af = 0.5f * vdot(N, N) * rn, Afd = Af * h;
+  const float strain = __fdividef(Af - A0f, A0f);
   const float gA = cA + ka * strain, gAd = cAd + __fdividef(ka * Afd, A0f);
-  const float rnd = -2.f * rn * rn * Afd;                  // (1/|N|)' = -|N|'/|N|^2
-  const float k = -0.5f * rn * gA, kd = -0.5f * fmaf(rnd, gA, rn * gAd);
+  const float k0 = -0.5f * side * rn;
+  const float k = k0 * gA, kd = k0 * (gAd - h * gA);     // (1/|N|)' = -h/|N|
   const Vec<float> m = vscale(N, k), md = vmad(kd, N, k, Nd);
   const Vec<float> v = vmad(cVd * (-1.f / 6.f), N, cV * (-1.f / 6.f), Nd);
-  const Vec<float> fa = vadd(vcross(md, bc), vcross(m, bcd));
-  const Vec<float> fb = vadd(vcross(acd, m), vcross(ac, md));
-  f[0] = vadd(fa, v);
-  f[1] = vadd(fb, v);
-  f[2] = vsub(v, vadd(fa, fb));
+  const Vec<float> X = vadd(vcross(md, w), vcross(m, wd));
+  const Vec<float> Y = vadd(vcross(md, e), vcross(m, ed));
+  fa = vadd(fa, vadd(vsub(X, Y), v));
+  fb = vadd(fb, vsub(v, X));
+  fw = vadd(fw, vadd(Y, v));
   uk_a = -strain * Afd;
 }
 

@@ -34,9 +34,6 @@ struct Smem<true> {
   __device__ __forceinline__ void put(int s, const Vec<float>& f) const {
     if (s != kNone) c[s] = make_float4(f.x, f.y, f.z, 0.f);
   }
-  __device__ __forceinline__ void add(int s, const Vec<float>& f) const {
-    if (s != kNone) put(s, vadd(slot(s), f));
-  }
 };
 template <>
 struct Smem<false> {
@@ -61,10 +58,23 @@ struct Smem<false> {
     c[nc + s] = f.y;
     c[2 * nc + s] = f.z;
   }
-  __device__ __forceinline__ void add(int s, const Vec<float>& f) const {
-    if (s != kNone) put(s, vadd(slot(s), f));
-  }
 };
+
+// Sum of own vertex i's slots [s0, s1) in a fixed order.  A vertex of a regular
+// mesh has 12 slots, so eight neighbours reading their first, second, ... slots
+// together would meet two of the eight 16-byte banks; each starts elsewhere in
+// its run instead.
+template <class S>
+__device__ __forceinline__ Vec<float> slot_sum(const S& sm, int i, int s0, int s1) {
+  Vec<float> f = {0.f, 0.f, 0.f};
+  int s = s0 + (i & 7);
+  if (s >= s1) s = s0;
+  for (int k = s0; k < s1; ++k) {
+    f = vadd(f, sm.slot(s));
+    if (++s == s1) s = s0;
+  }
+  return f;
+}
 
 }  // namespace
 }  // namespace ibm

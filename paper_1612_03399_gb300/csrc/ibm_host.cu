@@ -248,6 +248,22 @@ void build_topology(HostTopo& T, const int32_t* tri, int nv, int nf, int P) {
     }
     std::sort(es.begin(), es.end());
     std::sort(fs.begin(), fs.end());
+    // edge i is the edge face i is attached to (distinct edges); the edges
+    // without a face follow
+    {
+      std::vector<int> at;
+      at.reserve(es.size());
+      for (const int f : fs) {
+        const int e = T.fatt[f] >> 1;
+        if (e_stamp[e] != p) fail(IBM_ERR_MESH, "face attached to an edge outside its patch");
+        e_stamp[e] = -2 - p;   // taken
+        at.push_back(e);
+      }
+      for (const int e : es)
+        if (e_stamp[e] == p) at.push_back(e);
+      for (const int e : es) e_stamp[e] = p;
+      es.swap(at);
+    }
     H.edge_off = (int32_t)T.pedge.size();
     H.n_edge = (int32_t)es.size();
     for (size_t i = 0; i < es.size(); ++i) {
@@ -300,7 +316,8 @@ void build_topology(HostTopo& T, const int32_t* tri, int nv, int nf, int P) {
     // has one slot per edge role it plays, contiguous and in the order of its
     // edge list above.  Per edge 4 words (a | b << 16, c | d << 16, slot of a |
     // slot of b << 16, slot of c | slot of d << 16; kNone for halo vertices);
-    // per face 2 words (edge | side << 30 | owned << 31, face id); then the
+    // per face 2 words (edge, the face's own position | corner of the edge's
+    // start as the face runs << 28 | side << 30 | owned << 31, face id); then the
     // first slot of every own vertex (n_own + 1 16-bit entries).
     {
       std::vector<uint16_t> dE(4 * es.size(), kNone);
@@ -327,10 +344,11 @@ void build_topology(HostTopo& T, const int32_t* tri, int nv, int nf, int P) {
       // faces in the patch's order; their rest data follows the same order
       const std::vector<int32_t>& fo = fs;
       for (const int f : fo) {
-        const int e = T.fatt[f] >> 1;
-        if (e_stamp[e] != p) fail(IBM_ERR_MESH, "face attached to an edge outside its patch");
         const bool owned = tri[3 * f] >= o0 && tri[3 * f] < o1;
-        T.fblob.push_back((uint32_t)e_loc[e] | (uint32_t)(T.fatt[f] & 1) << 30 |
+        const int e = T.fatt[f] >> 1, side = T.fatt[f] & 1;
+        const int v0 = side ? T.edge[e].y : T.edge[e].x;   // the face is (v0, v1, wing)
+        const int rot = tri[3 * f] == v0 ? 0 : (tri[3 * f + 1] == v0 ? 1 : 2);
+        T.fblob.push_back((uint32_t)e_loc[e] | (uint32_t)rot << 28 | (uint32_t)side << 30 |
                           (owned ? 0x80000000u : 0u));
         T.fblob.push_back((uint32_t)f);
       }
@@ -645,10 +663,10 @@ void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
 }
 
 // Threads per force-kernel block: the least thread-iterations over the work
-// items (edges, then faces at about half an edge's work, then own vertices at
-// a third).  Patches of 128 vertices of the icosphere drops have 522 edges: 256
-// threads would take three passes for them, 192 or 288 take the same three or
-// two with few idle threads.
+// items (edges with their faces, then own vertices at a third of the work).
+// Patches of 128 vertices of the icosphere drops have 522 edges: three passes of
+// 192 threads, 87 us against 91 with 128 threads and 99 with 256 (1000 drops,
+// with the marker kernel's tail).
 int choose_force_threads(const std::vector<FWork>& work) {
   int best = kForceThreads;
   double least = 1e300;
@@ -657,8 +675,7 @@ int choose_force_threads(const std::vector<FWork>& work) {
     const size_t step = std::max<size_t>(1, work.size() / 4096);
     for (size_t k = 0; k < work.size(); k += step) {
       const FWork& w = work[k];
-      cost += t * ((w.n_edge + t - 1) / t + 0.5 * ((w.n_face + t - 1) / t) +
-                   0.33 * ((w.n_own + t - 1) / t));
+      cost += t * ((w.n_edge + t - 1) / t + 0.33 * ((w.n_own + t - 1) / t));
     }
     if (cost < least) {
       least = cost;

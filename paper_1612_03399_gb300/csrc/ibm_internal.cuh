@@ -187,7 +187,8 @@ __device__ __forceinline__ int tiles_along(int f, int n, int T, int (&out)[3]) {
   }
   return k;
 }
-constexpr int kForceThreads = 256;   // threads per block of the advance kernel; most of the adjoint's
+constexpr int kForceThreads = 256;   // threads per block of the advance kernel
+constexpr int kAdjointThreads = 160; // most threads of a force-adjoint-kernel block
 constexpr int kForceThreadsMax = 288;   // most threads of a force-kernel block
 // host mirror of the node update's outputs (ibm_step_host): the force kernel
 // writes x', v' to device arrays and the last block to complete each chunk of

@@ -423,21 +423,23 @@ __global__ void __launch_bounds__(kMT, 3) ext_adjoint_kernel(
 
 constexpr size_t kExtBytes = 30 * sizeof(float) * kMT;   // ext_adjoint_kernel's values per thread
 
-// What bounds it: issue, and latency between its barriers, as the force kernel;
-// float64 instructions issue at a sixteenth of a warp per cycle and SM, so only
-// what must be float64 is, once per block where it can be.  48 bodies (246 k
-// faces, 960 patches): 64.9 us with generic forward-mode numbers, narrow slots
-// and a float64 division per thread; 48.1 us with the derivatives written out
-// (edge_tangent, face_tangent) and float4 slots; 41.9 us with the division per
-// block and the packed warp sums.  Three blocks on an SM (80 registers): 43.7 us.
-// The layout goes by the same rule as the force kernel's: float4 where it fits.
+// What bounds it: latency (record -> index -> position, tractions' cotangents)
+// and its barriers, as the force kernel; float64 instructions issue at a
+// sixteenth of a warp per cycle and SM, so only what must be float64 is, once
+// per block where it can be.  48 bodies (246 k faces, 960 patches): 64.9 us with
+// generic forward-mode numbers, narrow slots and a float64 division per thread;
+// 48.1 us with the derivatives written out (*_tangent) and float4 slots; 41.9 us
+// with the division per block and the packed warp sums; 36.1 us with the faces
+// and their corners' cotangents on the edges instead of a chain of loads per
+// vertex.  Three blocks of at most 160 threads fit an SM's registers: 35.7 us,
+// 40.6 with 192.  The layout goes by the force kernel's rule: float4 where it fits.
 template <bool WIDE>
-__global__ void __launch_bounds__(kForceThreads, 2) force_adjoint_kernel(
+__global__ void __launch_bounds__(kAdjointThreads, 3) force_adjoint_kernel(
     DeviceTables T, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ gxn, const float* __restrict__ gvn, float* __restrict__ gx,
     float* __restrict__ gvo, double* __restrict__ gparams, const float* __restrict__ gve) {
   extern __shared__ __align__(16) float sm[];
-  __shared__ double s_red[3][kForceThreads / 32];
+  __shared__ double s_red[3][kAdjointThreads / 32];
   __shared__ int s_last;
   __shared__ __align__(8) unsigned long long bar;
   const FWork P = T.fwork[blockIdx.x];
@@ -494,24 +496,69 @@ __global__ void __launch_bounds__(kForceThreads, 2) force_adjoint_kernel(
     return;
   }
   const float cAd = (float)s_red[0][0], cVd = (float)s_red[0][1];   // before the barriers below
+  // edges: spring, bending and the face attached to the edge (edge k's face is
+  // face k)
   for (int k = threadIdx.x; k < P.n_edge; k += blockDim.x) {
     const uint4 r = rec[k];
+    const bool face = k < P.n_face;
+    uint2 fr = make_uint2(0u, 0u);
+    Vec<float> tc[3] = {};
+    if (face) {
+      fr = frec[k];
+      const float* t = T.gxe + P.f_off + fr.y;
+      int corner = (fr.x >> 28) & 3;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const float* tj = t + 3 * (size_t)corner * F;
+        tc[j] = {__ldg(tj), __ldg(tj + F), __ldg(tj + 2 * (size_t)F)};
+        corner = corner == 2 ? 0 : corner + 1;
+      }
+    }
     const int la = r.x & 0xFFFF, lb = r.x >> 16, lc = r.y & 0xFFFF, ld = r.y >> 16;
     const bool hinge = ld != kNone;
+    const int wd = hinge ? ld : la;
     const Vec<float> pa = S.pos(la), ya = Y.pos(la);
     const Vec<float> e = vsub(S.pos(lb), pa), ed = vsub(Y.pos(lb), ya);
-    const int wc = hinge ? lc : la, wd = hinge ? ld : lb;
-    const Vec<float> ac = vsub(S.pos(wc), pa), acd = vsub(Y.pos(wc), ya);
+    const Vec<float> ac = vsub(S.pos(lc), pa), acd = vsub(Y.pos(lc), ya);
     const Vec<float> ad = vsub(S.pos(wd), pa), add = vsub(Y.pos(wd), ya);
-    const float c0 = hinge ? rest[pe + k] : 1.f, s0 = hinge ? rest[2 * pe + k] : 0.f;
-    // per-edge multipliers m: the forces use m k, the constants' cotangents
+    // per-element multipliers m: the forces use m k, the constants' cotangents
     // scale the per-unit-k forces by m
     const float ms = P.varied ? rest[3 * pe + pf + k] : 1.f;
     const float mb = P.varied ? rest[4 * pe + pf + k] : 1.f;
-    Vec<float> fa, fb, fc, fd;
-    float us, ub;
-    edge_tangent(e, ed, ac, acd, ad, add, hinge, rest[k], c0, s0, Bks * ms, Bkb * mb, fa, fb, fc,
-                 fd, us, ub);
+    Vec<float> fa, fb, fc = {0.f, 0.f, 0.f}, fd = {0.f, 0.f, 0.f};
+    float l, ld_, il, ild, us, ub = 0.f;
+    spring_tangent(e, ed, rest[k], Bks * ms, l, ld_, il, ild, fa, us);
+    fb = {-fa.x, -fa.y, -fa.z};
+    const Vec<float> N1 = vcross(e, ac), N2 = vcross(ad, e);
+    const Vec<float> N1d = vadd(vcross(ed, ac), vcross(e, acd));
+    const Vec<float> N2d = vadd(vcross(add, e), vcross(ad, ed));
+    const float r1 = rsqrtf(vdot(N1, N1)), r2 = rsqrtf(vdot(N2, N2));
+    const float h1 = r1 * r1 * vdot(N1, N1d), h2 = r2 * r2 * vdot(N2, N2d);
+    if (hinge)
+      hinge_tangent(e, ed, l, ld_, il, ild, ac, acd, ad, add, N1, N1d, N2, N2d, r1, r2, h1, h2,
+                    rest[pe + k], rest[2 * pe + k], Bkb * mb, fa, fb, fc, fd, ub);
+    if (face) {
+      const bool right = (fr.x >> 30) & 1u;
+      const float ma = P.varied ? rest[5 * pe + pf + k] : 1.f;
+      Vec<float> fw = right ? fd : fc;
+      float ua;
+      face_tangent(e, ed, right ? ad : ac, right ? add : acd, right ? N2 : N1, right ? N2d : N1d,
+                   right ? r2 : r1, right ? h2 : h1, right ? -1.f : 1.f, rest[3 * pe + k], Bka * ma,
+                   cf.x, cAd, cf.y, cVd, fa, fb, fw, ua);
+      if (right)
+        fd = fw;
+      else
+        fc = fw;
+      if (fr.x >> 31) gka += ma * ua;
+      // traction part: the cotangents the face left for its corners
+      const Vec<float>&t0 = right ? tc[1] : tc[0], &t1 = right ? tc[0] : tc[1];
+      fa = vadd(fa, t0);
+      fb = vadd(fb, t1);
+      if (right)
+        fd = vadd(fd, tc[2]);
+      else
+        fc = vadd(fc, tc[2]);
+    }
     S.put(r.z & 0xFFFF, fa);
     S.put(r.z >> 16, fb);
     S.put(r.w & 0xFFFF, fc);
@@ -521,51 +568,15 @@ __global__ void __launch_bounds__(kForceThreads, 2) force_adjoint_kernel(
       gkb += mb * ub;
     }
   }
-  __syncthreads();   // every edge slot written
-  // faces, added to the slots of the edge each is attached to (an edge per
-  // face: no two threads touch the same slot)
-  for (int k = threadIdx.x; k < P.n_face; k += blockDim.x) {
-    const uint2 fr = frec[k];
-    const uint4 r = rec[fr.x & 0x3FFFFFFFu];
-    const bool right = (fr.x >> 30) & 1u;
-    const int la = r.x & 0xFFFF, lb = r.x >> 16;
-    const int v0 = right ? lb : la, v1 = right ? la : lb;
-    const int v2 = right ? (int)(r.y >> 16) : (int)(r.y & 0xFFFF);
-    const int d0 = right ? (int)(r.z >> 16) : (int)(r.z & 0xFFFF);
-    const int d1 = right ? (int)(r.z & 0xFFFF) : (int)(r.z >> 16);
-    const int d2 = right ? (int)(r.w >> 16) : (int)(r.w & 0xFFFF);
-    Vec<float> f[3];
-    float ua;
-    const float ma = P.varied ? rest[5 * pe + pf + k] : 1.f;
-    const Vec<float> pa = S.pos(v0), ya = Y.pos(v0);
-    face_tangent(vsub(S.pos(v1), pa), vsub(Y.pos(v1), ya), vsub(S.pos(v2), pa), vsub(Y.pos(v2), ya),
-                 rest[3 * pe + k], Bka * ma, cf.x, cAd, cf.y, cVd, f, ua);
-    S.add(d0, f[0]);
-    S.add(d1, f[1]);
-    S.add(d2, f[2]);
-    if (fr.x >> 31) gka += ma * ua;
-  }
   __syncthreads();
   for (int i = threadIdx.x; i < P.n_own; i += blockDim.x) {
-    const int s0 = ptr[i], s1 = ptr[i + 1];
-    float jx = 0.f, jy = 0.f, jz = 0.f;
-    for (int s = s0; s < s1; ++s) {
-      const Vec<float> t = S.slot(s);
-      jx += t.x;
-      jy += t.y;
-      jz += t.z;
-    }
+    const Vec<float> js = slot_sum(S, i, ptr[i], ptr[i + 1]);
+    const float jx = js.x, jy = js.y, jz = js.z;
     const int gvx = P.v_off + P.own0 + i;
-    // traction part: the cotangents the faces left for this corner
     float wx = 0.f, wy = 0.f, wz = 0.f;   // the spread's velocity cotangent
-    for (int q = vptr[i]; q < vptr[i + 1]; ++q) {
-      const uint32_t e = vent[q];
-      const int corner = (int)(e >> 30);
-      const size_t gf = (size_t)P.f_off + (e & 0x3FFFFFFFu);
-      jx += __ldg(T.gxe + (corner * 3 + 0) * (size_t)F + gf);
-      jy += __ldg(T.gxe + (corner * 3 + 1) * (size_t)F + gf);
-      jz += __ldg(T.gxe + (corner * 3 + 2) * (size_t)F + gf);
-      if (gve) {
+    if (gve) {
+      for (int q = vptr[i]; q < vptr[i + 1]; ++q) {
+        const size_t gf = (size_t)P.f_off + (vent[q] & 0x3FFFFFFFu);
         wx += __ldg(gve + gf);
         wy += __ldg(gve + (size_t)F + gf);
         wz += __ldg(gve + 2 * (size_t)F + gf);
@@ -649,7 +660,7 @@ cudaError_t launch_backward(ibm_ctx* c, const float* x, const float* v, const fl
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   auto kernel = c->adjoint_wide ? force_adjoint_kernel<true> : force_adjoint_kernel<false>;
-  kernel<<<c->n_work, std::min(c->force_threads, kForceThreads), c->adjoint_smem, c->stream>>>(
+  kernel<<<c->n_work, std::min(c->force_threads, kAdjointThreads), c->adjoint_smem, c->stream>>>(
       c->d, c->sc, (int32_t)c->V, (int32_t)c->F, x, gx_next, gv_next, gx, gv, gparams, gve);
   return cudaGetLastError();
 }

@@ -90,14 +90,18 @@ __device__ __noinline__ void mirror_chunks(Mirror m, const float* x_out, const f
 // acceleration (F_int + F_ext^v)/m, zero on clamped nodes, into Fint.
 // ENERGY: the body's energies as well (MODE 0).
 //
-// What bounds it: instruction issue while its blocks compute, and between that
-// the latency of the chain record -> index -> position and of the barriers; its
-// 117 bytes per vertex take 11 us of HBM for 642 k vertices.  Hence one record
-// per block (a load instead of a chain of four), forces without the parts only
-// the adjoint uses, float4 positions and slots, and a block size whose whole
-// warps fit the patches' element counts (force_threads).  Measured with patches
-// of 128 vertices: 107 -> 84 us for 642 k vertices after the coupled step's
-// marker kernel, 28.5 -> 23.4 us for 160 k vertices on its own.
+// What bounds it: the shared-memory pipe while its blocks compute (two thirds
+// of its peak before, half now), and the latency of the chain record -> index ->
+// position; its 117 bytes per vertex take 11 us of HBM for 642 k vertices.
+// Hence one record per block (a load instead of a chain of four), forces
+// without the parts only the adjoint uses, float4 positions and slots, each
+// face computed with the edge it is attached to, from a normal that edge has
+// (no second pass over indices, positions and slots: 2650 -> 2150 shared
+// wavefronts a block), slots read from staggered starts (-> 1680), and a block
+// size whose whole warps fit the patches' edge counts (force_threads; 128 to
+// 288 threads differ by 5 %).  Patches of 128 vertices, 642 k vertices after
+// the marker kernel: 107 us at first, 84 with the record and the layouts, 72
+// with the faces on their edges.
 template <int MODE, bool ENERGY, bool WIDE>
 __global__ void __launch_bounds__(kForceThreadsMax, 3) force_kernel(
     DeviceTables T, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
@@ -157,95 +161,78 @@ __global__ void __launch_bounds__(kForceThreadsMax, 3) force_kernel(
     return;
   }
 
-  // edges: spring + bending, from shared memory only
+  // Everything above reads only static tables and positions written two
+  // launches back; the marker kernel launched just before (it lets this grid
+  // start once all its blocks run) produces the body sums and F_ext, so the
+  // rest waits for it to complete (a no-op without that launch mode).
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // per-body global-term coefficients from the marker kernel's exact
+  // fixed-point area / volume sums
+  const float2 cf = body_coef(B, __ldg(T.qsum + 2 * P.body), __ldg(T.qsum + 2 * P.body + 1));
+  const float cA = cf.x, cV = cf.y, Bka = B.ka, inv_mass = B.inv_mass;
+  // edges: spring, bending, and the face attached to the edge (edge k's face
+  // is face k), whose normal the hinge has at hand
   for (int k = threadIdx.x; k < P.n_edge; k += blockDim.x) {
     const uint4 r = rec[k];
+    const bool face = k < P.n_face;
+    uint2 fr = make_uint2(0u, 0u);
+    Vec<float> fe = {0.f, 0.f, 0.f};
+    if (face) {
+      fr = frec[k];
+      if (MODE != 0) {
+        // F_ext^v = sum over the vertex's faces of F_ext / 3: each face adds a
+        // third of its load to its corners, gathered with the forces
+        const int g = P.f_off + (int)fr.y;
+        fe = {__ldg(Fext + g), __ldg(Fext + F + g), __ldg(Fext + 2 * F + g)};
+      }
+    }
     const int la = r.x & 0xFFFF, lb = r.x >> 16, lc = r.y & 0xFFFF, ld = r.y >> 16;
     const bool hinge = ld != kNone;
-    const Vec<float> pa = S.pos(la), pb = S.pos(lb);
-    const Vec<float> pc = hinge ? S.pos(lc) : pa, pd = hinge ? S.pos(ld) : pb;
-    const float c0 = hinge ? rest[pe + k] : 1.f, s0 = hinge ? rest[2 * pe + k] : 0.f;
-    Vec<float> fa, fb, fc, fd;
-    float es, eb;
-    // per-edge constants (van Gelder springs, materials) where the body has them
+    const Vec<float> pa = S.pos(la), e = vsub(S.pos(lb), pa);
+    const Vec<float> ac = vsub(S.pos(lc), pa), ad = vsub(S.pos(hinge ? ld : la), pa);
+    // per-edge and per-face constants (van Gelder springs, materials) where
+    // the body has them
     const float ks = P.varied ? Bks * rest[3 * pe + pf + k] : Bks;
-    const float kb = P.varied ? Bkb * rest[4 * pe + pf + k] : Bkb;
-    edge_forward(pa, pb, pc, pd, hinge, rest[k], c0, s0, ks, kb, fa, fb, fc, fd, es, eb);
-    if (ENERGY && (r.z & 0xFFFF) != kNone) {   // the patch of vertex a owns the edge
-      eS += (double)es;
-      eB += (double)eb;
+    Vec<float> fa, fb, fc = {0.f, 0.f, 0.f}, fd = {0.f, 0.f, 0.f};
+    float l, inv_l, es, eb = 0.f, ea = 0.f;
+    spring_forward(e, rest[k], ks, l, inv_l, fa, es);
+    fb = {-fa.x, -fa.y, -fa.z};
+    const Vec<float> N1 = vcross(e, ac), N2 = vcross(ad, e);
+    const float r1 = rsqrtf(vdot(N1, N1)), r2 = rsqrtf(vdot(N2, N2));
+    if (hinge) {
+      const float kb = P.varied ? Bkb * rest[4 * pe + pf + k] : Bkb;
+      hinge_forward(e, l, inv_l, ac, ad, N1, N2, r1, r2, rest[pe + k], rest[2 * pe + k], kb, fa, fb,
+                    fc, fd, eb);
+    }
+    if (face) {
+      const bool right = (fr.x >> 30) & 1u;
+      const float ka = P.varied ? Bka * rest[5 * pe + pf + k] : Bka;
+      Vec<float> fw = right ? fd : fc;
+      face_forward(e, right ? ad : ac, right ? N2 : N1, right ? r2 : r1, right ? -1.f : 1.f,
+                   rest[3 * pe + k], ka, cA, cV, vscale(fe, 1.f / 3.f), fa, fb, fw, ea);
+      if (right)
+        fd = fw;
+      else
+        fc = fw;
+    }
+    if (ENERGY) {
+      if ((r.z & 0xFFFF) != kNone) {   // the patch of vertex a owns the edge
+        eS += (double)es;
+        eB += (double)eb;
+      }
+      if (fr.x >> 31) eA += (double)ea;
     }
     S.put(r.z & 0xFFFF, fa);
     S.put(r.z >> 16, fb);
     S.put(r.w & 0xFFFF, fc);
     S.put(r.w >> 16, fd);
   }
-  // Everything above reads only static tables and positions written two
-  // launches back; the marker kernel launched just before (it lets this grid
-  // start once all its blocks run) produces the body sums and F_ext, so the
-  // face part waits for it to complete (a no-op without that launch mode).
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  // per-body global-term coefficients from the marker kernel's exact
-  // fixed-point area / volume sums
-  const float2 cf = body_coef(B, __ldg(T.qsum + 2 * P.body), __ldg(T.qsum + 2 * P.body + 1));
-  const float cA = cf.x, cV = cf.y, Bka = B.ka, inv_mass = B.inv_mass;
-  __syncthreads();   // every edge slot written
-  // faces: local area, global area, volume, added to the slots of the edge
-  // each face is attached to (an edge per face: no two threads touch the same
-  // slot); two faces per thread with their tractions in flight
-  const float third = 1.f / 3.f;
-  for (int k0 = threadIdx.x; k0 < P.n_face; k0 += 2 * blockDim.x) {
-    const int k1 = k0 + blockDim.x;
-    const bool two = k1 < P.n_face;
-    const uint2 r0 = frec[k0];
-    const uint2 r1 = two ? frec[k1] : r0;
-    Vec<float> fe0 = {0.f, 0.f, 0.f}, fe1 = {0.f, 0.f, 0.f};
-    if (MODE != 0) {
-      // F_ext^v = sum over the vertex's faces of F_ext / 3: each face adds a
-      // third of its load to its corners, gathered with the forces
-      const int g0 = P.f_off + (int)r0.y, g1 = P.f_off + (int)r1.y;
-      fe0 = {__ldg(Fext + g0), __ldg(Fext + F + g0), __ldg(Fext + 2 * F + g0)};
-      fe1 = {__ldg(Fext + g1), __ldg(Fext + F + g1), __ldg(Fext + 2 * F + g1)};
-    }
-#pragma unroll 1
-    for (int h = 0; h < (two ? 2 : 1); ++h) {
-      const uint2 fr = h ? r1 : r0;
-      const int k = h ? k1 : k0;
-      const uint4 r = rec[fr.x & 0x3FFFFFFFu];
-      const bool right = (fr.x >> 30) & 1u;
-      const int la = r.x & 0xFFFF, lb = r.x >> 16;
-      const int v0 = right ? lb : la, v1 = right ? la : lb;
-      const int v2 = right ? (int)(r.y >> 16) : (int)(r.y & 0xFFFF);
-      const int d0 = right ? (int)(r.z >> 16) : (int)(r.z & 0xFFFF);
-      const int d1 = right ? (int)(r.z & 0xFFFF) : (int)(r.z >> 16);
-      const int d2 = right ? (int)(r.w >> 16) : (int)(r.w & 0xFFFF);
-      Vec<float> f[3];
-      float ea;
-      const float ka = P.varied ? Bka * rest[5 * pe + pf + k] : Bka;
-      face_forward(S.pos(v0), S.pos(v1), S.pos(v2), rest[3 * pe + k], ka, cA, cV, f, ea);
-      if (MODE != 0) {
-        const Vec<float> fe = vscale(h ? fe1 : fe0, third);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) f[c] = vadd(f[c], fe);
-      }
-      S.add(d0, f[0]);
-      S.add(d1, f[1]);
-      S.add(d2, f[2]);
-      if (ENERGY && (fr.x >> 31)) eA += (double)ea;
-    }
-  }
   __syncthreads();
 
   // own vertices: fixed-order sum of their contiguous slots
   for (int i = threadIdx.x; i < P.n_own; i += blockDim.x) {
-    const int s0 = ptr[i], s1 = ptr[i + 1];
-    float fx = 0.f, fy = 0.f, fz = 0.f;
-    for (int s = s0; s < s1; ++s) {
-      const Vec<float> t = S.slot(s);
-      fx += t.x;
-      fy += t.y;
-      fz += t.z;
-    }
+    const Vec<float> fs = slot_sum(S, i, ptr[i], ptr[i + 1]);
+    const float fx = fs.x, fy = fs.y, fz = fs.z;
     const int gv = P.v_off + P.own0 + i;
     if (MODE == 0) {
       Fint[gv] = fx;

@@ -58,6 +58,7 @@ struct ibm_flow {
   int solve_w[3] = {-1, -1, -1};
   float taps[3][3][9] = {};
   int rhs_planes = 16;          // planes per thread of the right-hand side kernel
+  int solve_planes[3] = {32, 32, 32};   // output planes per block of the real-space solves
   // per substep: solved by recursions along the lines; the powers of r they use
   bool lines[3] = {false, false, false};
   float* pw = nullptr;          // [3][pw_stride]
@@ -545,14 +546,14 @@ __global__ void __launch_bounds__(kQuadThreads)
   st4(p + o, val);
 }
 
-// asynchronous 4- and 8-byte global -> shared copies
+// asynchronous 4- and 16-byte global -> shared copies
 __device__ __forceinline__ void cp_async4(float* sdst, const float* gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
-__device__ __forceinline__ void cp_async8(float* sdst, const float* gsrc) {
+__device__ __forceinline__ void cp_async16(float* sdst, const float* gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -561,16 +562,23 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // The real-space factorised solve fused with u* = u + du.  A block owns a
-// 32 x 32 tile of (x, y) outputs of one component over kSolveZ planes; it
-// walks the kSolveZ + 2W planes that feed them (periodic wrap in every
-// direction), each staged with its x and y halo by asynchronous copies two
-// planes ahead.  Per plane: the x filter, four consecutive x per thread from
-// float4 windows; the y filter for two x and two y per thread and the z
-// filter in packed two-lane float arithmetic (pairs of x), from a register
-// ring of the last 2W + 1 filtered planes; the z filter gives the output
-// plane W planes back.  Taps are
-// symmetric: g[d][|m|].
-constexpr int kSolveT = 32, kSolveZ = 32, kMaxSolveW = 8;
+// 32 x 32 tile of (x, y) outputs of one component over `planes` planes; it
+// walks the planes + 2W that feed them (periodic wrap in every direction), each
+// staged with its x and y halo by asynchronous copies two planes ahead.  Per
+// plane the y filter, in packed two-lane float arithmetic, two rows of a quad of
+// x per thread, into a second buffer; from there each thread filters its own
+// quad in x and keeps the result in a register ring of 2W + 1 planes, whose z
+// filter gives the output W planes back.  Taps are symmetric: g[d][|m|].
+// What bounds it: instruction issue first (three filters of 2W + 1 taps; 95
+// instructions an output with x filtered first, 4-byte copies and a ring that
+// moved by one place a plane).  With y first, the ring's places fixed by
+// unrolling the walk 2W + 1 times and V4 (rows of whole float4s: 16-byte copies,
+// loads and stores; other rows and alignments go word by word) it is 38, and the
+// shared-memory pipe (70 %) and the barrier a plane remain.  256^3, 600 MB in
+// 90 us at the copy rate: W = 3 172 -> 130 us, W = 4 208 -> 136; 200 x 180 x 144,
+// W = 7: 144 -> 90; 64^3: 26 -> 8; word by word on 255 x 256 x 256 186 -> 161 and
+// 222 -> 178.
+constexpr int kSolveT = 32, kMaxSolveW = 8;
 
 struct SolveTaps {
   float g[3][kMaxSolveW + 1];
@@ -579,41 +587,34 @@ static_assert(sizeof(ibm_flow::taps[0]) == sizeof(SolveTaps), "tap table layout"
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
-// symmetric filter of half width W centred on win[c]: g0 w_c + sum_m g_m (w_{c-m} + w_{c+m})
-template <int W>
-__device__ __forceinline__ float2 sym_filter(const float2* win, int c, const float* g) {
-  float2 acc = __fmul2_rn(f2(g[0]), win[c]);
-#pragma unroll
-  for (int m = 1; m <= W; ++m) acc = __ffma2_rn(f2(g[m]), __fadd2_rn(win[c - m], win[c + m]), acc);
-  return acc;
+__host__ __device__ constexpr int solve_halo(int W) { return W <= 4 ? 4 : 8; }   // staged columns beside the tile
+__host__ __device__ constexpr int solve_blocks(int W) { return W <= 4 ? 3 : 2; } // resident blocks per SM
+constexpr size_t solve_smem(int W) {
+  return sizeof(float) * (size_t)(kSolveT + 2 * solve_halo(W)) * (3 * (kSolveT + 2 * W) + 2 * kSolveT);
 }
 
-template <int W>
-__global__ void __launch_bounds__(256, W <= 4 ? 3 : 2) cn_solve_kernel(FGrid G, const float* __restrict__ R,
-                                                          Vec3 u, SolveTaps T) {
-  constexpr int AY = kSolveT + 2 * W, AX = kSolveT + 2 * W;
-  constexpr int NW4 = (4 + 2 * W + 3) / 4;          // float4s in an x window
-  constexpr int AXP = kSolveT - 4 + 4 * NW4;        // row stride: windows stay in the row
-  constexpr int AN = AY * AX, SLOTS = (AN + 255) / 256, NB = 3, NU = 4;
-  static_assert(AXP >= AX && AXP % 4 == 0, "row stride");
-  // dynamic shared memory: A[NB][AY * AXP] raw planes with halo,
-  // Us[NU][32 * 32] u of the output planes, B[2][AY][32] x-filtered rows
+template <int W, bool V4>
+__global__ void __launch_bounds__(256, solve_blocks(W)) cn_solve_kernel(
+    FGrid G, const float* __restrict__ R, Vec3 u, SolveTaps T, int planes) {
+  constexpr int HX = solve_halo(W), AX = kSolveT + 2 * HX, QX = AX / 4, AY = kSolveT + 2 * W;
+  constexpr int NB = 3, RW = 2 * W + 1;
+  constexpr int CX = V4 ? QX : kSolveT + 2 * W;      // staged per row: quads, or single columns
+  constexpr int SLOTS = (AY * CX + 255) / 256;
+  // A[NB][AY][AX] raw planes with halo, Y[2][32][AX] y-filtered rows
   extern __shared__ __align__(16) float smem[];
-  float (*A)[AY * AXP] = reinterpret_cast<float (*)[AY * AXP]>(smem);
-  float (*Us)[kSolveT * kSolveT] = reinterpret_cast<float (*)[kSolveT * kSolveT]>(smem + NB * AY * AXP);
-  float (*B)[AY][kSolveT] =
-      reinterpret_cast<float (*)[AY][kSolveT]>(smem + NB * AY * AXP + NU * kSolveT * kSolveT);
+  float* const A = smem;
+  float* const Y = smem + NB * AY * AX;
   const int tid = threadIdx.x;
   const int nx = G.nx, ny = G.ny, nz = G.nz;
   const int ntx = (nx + kSolveT - 1) / kSolveT;
   const int x0 = (int)(blockIdx.y % ntx) * kSolveT, y0 = (int)(blockIdx.y / ntx) * kSolveT;
-  const int k0 = (int)blockIdx.x * kSolveZ;
-  const int nk = min(kSolveZ, nz - k0), nq = nk + 2 * W;
+  const int k0 = (int)blockIdx.x * planes;
+  const int nk = min(planes, nz - k0), nq = nk + 2 * W;
   const size_t plane = (size_t)nx * ny;
   const int c = blockIdx.z;
   const float* Rc = R + (size_t)c * plane * nz;
   float* uc = c == 0 ? u.c[0] : (c == 1 ? u.c[1] : u.c[2]);
-  // staging slots: shared index and wrapped in-plane offset (-1 past the tile)
+  // staging slots: wrapped in-plane offset (-1 past the tile)
   int off[SLOTS];
   short sdst[SLOTS];
 #pragma unroll
@@ -621,158 +622,168 @@ __global__ void __launch_bounds__(256, W <= 4 ? 3 : 2) cn_solve_kernel(FGrid G, 
     const int q = tid + 256 * s;
     off[s] = -1;
     sdst[s] = 0;
-    if (q < AN) {
-      const int r = q / AX, cc = q - r * AX;
-      const int x = ((x0 - W + cc) % nx + nx) % nx, y = ((y0 - W + r) % ny + ny) % ny;
-      off[s] = y * nx + x;
-      sdst[s] = (short)(r * AXP + cc);
+    if (q < AY * CX) {
+      const int r = q / CX, cc = q - r * CX;
+      const int xr = V4 ? 4 * cc - HX : cc - W;      // whole quads: x0 and nx are multiples of 4
+      const int xg = ((x0 + xr) % nx + nx) % nx, yg = ((y0 - W + r) % ny + ny) % ny;
+      off[s] = yg * nx + xg;
+      sdst[s] = (short)(r * AX + HX + xr);
     }
   }
-  // outputs: columns ox, ox + 1 of rows oy, oy + 1
-  const int lx = (tid & 15) * 2, ly = (tid >> 4) * 2;
-  const int ox = x0 + lx, oy = y0 + ly;
-  // 8-byte aligned column pairs: even rows and an 8-byte aligned field
-  const bool pair = (nx & 1) == 0 && (reinterpret_cast<uintptr_t>(uc) & 7) == 0;
-  auto stage = [&](int q) {
-    const int b = q % NB, bu = q % NU;
+  auto stage = [&](int q, int b) {
     int k = k0 - W + q;
     k = k < 0 ? k + nz : (k >= nz ? k - nz : k);
     const float* src = Rc + (size_t)k * plane;
+    float* dst = A + b * (AY * AX);
 #pragma unroll
-    for (int s = 0; s < SLOTS; ++s)
-      if (off[s] >= 0) cp_async4(&A[b][sdst[s]], src + off[s]);
-    const int ko = q - 2 * W;
-    if (ko >= 0) {
-      const float* us = uc + (size_t)(k0 + ko) * plane;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (oy + j >= ny) continue;
-        float* d = &Us[bu][(ly + j) * kSolveT + lx];
-        const float* g = us + (size_t)(oy + j) * nx + ox;
-        if (pair && ox + 1 < nx) {
-          cp_async8(d, g);
-        } else {
-          if (ox < nx) cp_async4(d, g);
-          if (ox + 1 < nx) cp_async4(d + 1, g + 1);
-        }
-      }
+    for (int s = 0; s < SLOTS; ++s) {
+      if (off[s] < 0) continue;
+      if (V4)
+        cp_async16(dst + sdst[s], src + off[s]);
+      else
+        cp_async4(dst + sdst[s], src + off[s]);
     }
     cp_async_commit();
   };
-  float2 ring[2][2 * W + 1];
+  // y filter: a quad of x in two rows; the first 128 threads take eight quads of
+  // a row pair each eight (no bank conflicts), the next the quads left over
+  constexpr int QR = QX - 8;
+  const int yr = 2 * (tid < 128 ? tid >> 3 : (tid - 128) / QR);
+  const int yc = 4 * (tid < 128 ? tid & 7 : 8 + (tid - 128) % QR);
+  auto yfilter = [&](int b, int t) {
+    if (tid >= 16 * QX) return;
+    const float* a = A + b * (AY * AX) + yr * AX + yc;
+    float2 o[2][2];
 #pragma unroll
-  for (int j = 0; j < 2; ++j)
+    for (int i = 0; i < RW + 1; ++i) {
+      const float4 v = *reinterpret_cast<const float4*>(a + i * AX);
+      const float2 lo = make_float2(v.x, v.y), hi = make_float2(v.z, v.w);
 #pragma unroll
-    for (int m = 0; m < 2 * W + 1; ++m) ring[j][m] = make_float2(0.f, 0.f);
-  // x filter of plane q into B[q & 1]: item = (row, quad of four x)
-  auto xfilter = [&](int q) {
-    const float* a = A[q % NB];
-    float (*Bq)[kSolveT] = B[q & 1];
-    for (int it = tid; it < AY * 8; it += 256) {
-      const int r = it >> 3, x4 = (it & 7) * 4;
-      float win[4 * NW4];
-      const float4* src = reinterpret_cast<const float4*>(a + r * AXP + x4);
-#pragma unroll
-      for (int v = 0; v < NW4; ++v) {
-        const float4 t = src[v];
-        win[4 * v] = t.x;
-        win[4 * v + 1] = t.y;
-        win[4 * v + 2] = t.z;
-        win[4 * v + 3] = t.w;
+      for (int j = 0; j < 2; ++j) {
+        if (i - j < 0 || i - j >= RW) continue;
+        const float2 g = f2(T.g[1][i - j < W ? W - i + j : i - j - W]);
+        o[j][0] = i == j ? __fmul2_rn(g, lo) : __ffma2_rn(g, lo, o[j][0]);
+        o[j][1] = i == j ? __fmul2_rn(g, hi) : __ffma2_rn(g, hi, o[j][1]);
       }
-      float o[4];
+    }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        float acc = T.g[0][0] * win[j + W];
+    for (int j = 0; j < 2; ++j)
+      *reinterpret_cast<float4*>(Y + (t * kSolveT + yr + j) * AX + yc) =
+          make_float4(o[j][0].x, o[j][0].y, o[j][1].x, o[j][1].y);
+  };
+  // outputs: columns ox .. ox + 3 of row oy
+  const int lx = 4 * (tid & 7), ly = tid >> 3;
+  const int ox = x0 + lx, oy = y0 + ly;
+  const bool mine = oy < ny && ox < nx;
+  const size_t oo = (size_t)oy * nx + ox;
+  float2 ring[RW][2];
 #pragma unroll
-        for (int m = 1; m <= W; ++m) acc += T.g[0][m] * (win[j + W - m] + win[j + W + m]);
-        o[j] = acc;
-      }
-      *reinterpret_cast<float4*>(&Bq[r][x4]) = make_float4(o[0], o[1], o[2], o[3]);
+  for (int m = 0; m < RW; ++m) ring[m][0] = ring[m][1] = make_float2(0.f, 0.f);
+
+  // one barrier per plane: between two of them the x and z filters of plane q
+  // and the y filter of plane q + 1
+  stage(0, 0);
+  if (nq > 1) {
+    stage(1, 1);
+    cp_async_wait<1>();
+  } else {
+    cp_async_wait<0>();
+  }
+  __syncthreads();
+  if (nq > 2) stage(2, 2);
+  yfilter(0, 0);
+  int b = 0;   // the buffer of plane q
+  // u of the output plane: V4 loads it a plane ahead (137 -> 130 us; without V4
+  // the registers are better spent on the offsets)
+  float un[4] = {0.f, 0.f, 0.f, 0.f};
+  auto load_u = [&](int ko) {
+    const float* ul = uc + (size_t)(k0 + ko) * plane + oo;
+    if (V4) {
+      const float4 t = *reinterpret_cast<const float4*>(ul);
+      un[0] = t.x; un[1] = t.y; un[2] = t.z; un[3] = t.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (ox + j < nx) un[j] = ul[j];
     }
   };
-  // one barrier per plane: the y and z filters of plane q and the x filter
-  // of plane q + 1 run between two barriers (B double-buffered, A three
-  // planes, Us four)
-  stage(0);
-  if (nq > 1) stage(1);
-  if (nq > 1)
-    cp_async_wait<1>();
-  else
-    cp_async_wait<0>();
-  __syncthreads();
-  if (nq > 2) stage(2);
-  xfilter(0);
-  for (int q = 0; q < nq; ++q) {
-    if (q + 2 < nq)
-      cp_async_wait<1>();
-    else
-      cp_async_wait<0>();
-    // B[q & 1] complete and plane q + 1 visible; every thread is past the x
-    // filter of plane q (A[q % NB] free) and the y filter of plane q - 1
-    // (B[(q + 1) & 1] and Us[(q - 1) % NU] free)
-    __syncthreads();
-    if (q + 3 < nq) stage(q + 3);
-    // y filter: rows ly, ly + 1 of columns lx, lx + 1
-    {
-      float2 col[2 + 2 * W];
+  if (V4 && W == 0 && mine) load_u(0);
+  for (int q0 = 0; q0 < nq; q0 += RW) {
 #pragma unroll
-      for (int i = 0; i < 2 + 2 * W; ++i)
-        col[i] = *reinterpret_cast<const float2*>(&B[q & 1][ly + i][lx]);
+    for (int s = 0; s < RW; ++s) {
+      const int q = q0 + s;
+      if (q >= nq) break;
+      if (q + 2 < nq)
+        cp_async_wait<1>();
+      else
+        cp_async_wait<0>();
+      // Y[q & 1] complete and plane q + 1 visible; every thread is past the y
+      // filter of plane q (its buffer is free) and the x filter of plane q - 1
+      // (Y[(q + 1) & 1] is free)
+      __syncthreads();
+      const int ko = q - 2 * W;
+      const float uu[4] = {un[0], un[1], un[2], un[3]};
+      if (mine && (V4 ? ko >= -1 && q + 1 < nq : ko >= 0)) load_u(V4 ? ko + 1 : ko);
+      if (q + 3 < nq) stage(q + 3, b);
+      b = b == NB - 1 ? 0 : b + 1;
+      if (q + 1 < nq) yfilter(b, (q + 1) & 1);
+      // x filter of the thread's quad: even distances on aligned pairs
+      {
+        float win[4 + 2 * HX];
+        const float* yq = Y + ((q & 1) * kSolveT + ly) * AX + lx;
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const float2 v = sym_filter<W>(col, j + W, T.g[1]);
+        for (int v = 0; v < 1 + HX / 2; ++v) {
+          const float4 t = *reinterpret_cast<const float4*>(yq + 4 * v);
+          win[4 * v] = t.x;
+          win[4 * v + 1] = t.y;
+          win[4 * v + 2] = t.z;
+          win[4 * v + 3] = t.w;
+        }
+        float2 o[2];
 #pragma unroll
-        for (int m = 0; m < 2 * W; ++m) ring[j][m] = ring[j][m + 1];
-        ring[j][2 * W] = v;
+        for (int j = 0; j < 2; ++j) {
+          const int w0 = HX + 2 * j;
+          o[j] = __fmul2_rn(f2(T.g[0][0]), make_float2(win[w0], win[w0 + 1]));
+#pragma unroll
+          for (int m = 2; m <= W; m += 2) {
+            o[j] = __ffma2_rn(f2(T.g[0][m]), make_float2(win[w0 - m], win[w0 - m + 1]), o[j]);
+            o[j] = __ffma2_rn(f2(T.g[0][m]), make_float2(win[w0 + m], win[w0 + m + 1]), o[j]);
+          }
+#pragma unroll
+          for (int m = 1; m <= W; m += 2) {
+            o[j].x = fmaf(T.g[0][m], win[w0 - m], o[j].x);
+            o[j].y = fmaf(T.g[0][m], win[w0 + 1 - m], o[j].y);
+            o[j].x = fmaf(T.g[0][m], win[w0 + m], o[j].x);
+            o[j].y = fmaf(T.g[0][m], win[w0 + 1 + m], o[j].y);
+          }
+          ring[s][j] = o[j];
+        }
       }
-    }
-    const int ko = q - 2 * W;
-    if (ko >= 0) {
-      float* uo = uc + (size_t)(k0 + ko) * plane;
-      const float* ub = Us[q % NU];
+      if (ko >= 0 && mine) {   // z filter: the newest plane is place s, the centre W before it
+        float2 r[2];
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (oy + j >= ny) continue;
-        const float2 d = sym_filter<W>(ring[j], W, T.g[2]);
-        const float2 uu = *reinterpret_cast<const float2*>(&ub[(ly + j) * kSolveT + lx]);
-        const float2 r = __fadd2_rn(uu, d);
-        float* g = uo + (size_t)(oy + j) * nx + ox;
-        if (pair && ox + 1 < nx) {
-          *reinterpret_cast<float2*>(g) = r;
+        for (int j = 0; j < 2; ++j) {
+          r[j] = V4 ? make_float2(uu[2 * j], uu[2 * j + 1]) : make_float2(un[2 * j], un[2 * j + 1]);
+          float2 d = __fmul2_rn(f2(T.g[2][0]), ring[(s + RW - W) % RW][j]);
+#pragma unroll
+          for (int m = 1; m <= W; ++m)
+            d = __ffma2_rn(f2(T.g[2][m]),
+                           __fadd2_rn(ring[(s + RW - W - m) % RW][j], ring[(s + RW - W + m) % RW][j]),
+                           d);
+          r[j] = __fadd2_rn(r[j], d);
+        }
+        float* uo = uc + (size_t)(k0 + ko) * plane + oo;
+        if (V4) {
+          *reinterpret_cast<float4*>(uo) = make_float4(r[0].x, r[0].y, r[1].x, r[1].y);
         } else {
-          if (ox < nx) g[0] = r.x;
-          if (ox + 1 < nx) g[1] = r.y;
+          const float o[4] = {r[0].x, r[0].y, r[1].x, r[1].y};
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if (ox + j < nx) uo[j] = o[j];
         }
       }
     }
-    if (q + 1 < nq) xfilter(q + 1);
   }
-}
-
-// dynamic shared memory of cn_solve_kernel<W>
-constexpr size_t solve_smem(int W) {
-  return sizeof(float) * (3 * (size_t)(kSolveT + 2 * W) * (kSolveT - 4 + 4 * ((4 + 2 * W + 3) / 4)) +
-                          4 * (size_t)kSolveT * kSolveT + 2 * (size_t)(kSolveT + 2 * W) * kSolveT);
-}
-
-// allow each real-space substep's kernel its dynamic shared memory
-cudaError_t set_solve_smem(const ibm_flow* fl) {
-  cudaError_t e = cudaSuccess;
-  for (int l = 0; l < 3 && e == cudaSuccess; ++l) {
-    switch (fl->solve_w[l]) {
-#define IBM_SOLVE_ATTR(WW)                                                                 \
-  case WW:                                                                                 \
-    e = cudaFuncSetAttribute(cn_solve_kernel<WW>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)solve_smem(WW));                                         \
-    break;
-      IBM_SOLVE_ATTR(0) IBM_SOLVE_ATTR(1) IBM_SOLVE_ATTR(2) IBM_SOLVE_ATTR(3) IBM_SOLVE_ATTR(4)
-      IBM_SOLVE_ATTR(5) IBM_SOLVE_ATTR(6) IBM_SOLVE_ATTR(7) IBM_SOLVE_ATTR(8)
-#undef IBM_SOLVE_ATTR
-      default: break;
-    }
-  }
-  return e;
 }
 
 // ---- the factorised solve by recursions along the lines ---------------------
@@ -879,19 +890,30 @@ __global__ void __launch_bounds__(32 * kSegs) line_yz_kernel(FGrid G, float* __r
 
 FGrid fgrid(const ibm_flow* fl);
 
+// every given field 16-byte aligned (null: not used) and rows of whole float4s
+template <class... P>
+bool quads(const ibm_flow* fl, P... f) {
+  const uintptr_t bits = (reinterpret_cast<uintptr_t>(f) | ...);
+  return fl->n[0] % 4 == 0 && (bits & 15u) == 0;
+}
 cudaError_t launch_cn_solve(const ibm_flow* fl, int l, float* u, float* v, float* w,
                             cudaStream_t s) {
   const FGrid G = fgrid(fl);
   SolveTaps T;
   for (int d = 0; d < 3; ++d)
     for (int m = 0; m <= kMaxSolveW; ++m) T.g[d][m] = fl->taps[l][d][m];
+  const int planes = fl->solve_planes[l];
   const unsigned tiles = (unsigned)(((fl->n[0] + kSolveT - 1) / kSolveT) *
                                     ((fl->n[1] + kSolveT - 1) / kSolveT));
-  const dim3 grid((unsigned)((fl->n[2] + kSolveZ - 1) / kSolveZ), tiles, 3), block(256);
+  const dim3 grid((unsigned)((fl->n[2] + planes - 1) / planes), tiles, 3), block(256);
   const Vec3 U{{u, v, w}};
+  const bool v4 = quads(fl, u, v, w);
   switch (fl->solve_w[l]) {
-#define IBM_SOLVE_CASE(WW) \
-  case WW: cn_solve_kernel<WW><<<grid, block, solve_smem(WW), s>>>(G, fl->R, U, T); break;
+#define IBM_SOLVE_CASE(WW)                                                            \
+  case WW:                                                                            \
+    (v4 ? cn_solve_kernel<WW, true> : cn_solve_kernel<WW, false>)<<<grid, block, solve_smem(WW), s>>>( \
+        G, fl->R, U, T, planes);                                                      \
+    break;
     IBM_SOLVE_CASE(0) IBM_SOLVE_CASE(1) IBM_SOLVE_CASE(2) IBM_SOLVE_CASE(3) IBM_SOLVE_CASE(4)
     IBM_SOLVE_CASE(5) IBM_SOLVE_CASE(6) IBM_SOLVE_CASE(7) IBM_SOLVE_CASE(8)
 #undef IBM_SOLVE_CASE
@@ -983,12 +1005,6 @@ dim3 cell_grid(const ibm_flow* fl) {
   return dim3((unsigned)((fl->n[0] + 31) / 32), (unsigned)((fl->n[1] + 7) / 8), (unsigned)fl->n[2]);
 }
 
-// every given field 16-byte aligned (null: not used) and rows of whole float4s
-template <class... P>
-bool quads(const ibm_flow* fl, P... f) {
-  const uintptr_t bits = (reinterpret_cast<uintptr_t>(f) | ...);
-  return fl->n[0] % 4 == 0 && (bits & 15u) == 0;
-}
 // blocks of the quad kernels: a plane's quads, and `planes` planes per block
 dim3 quad_grid(const ibm_flow* fl, int planes) {
   const int nq = fl->n[0] / 4 * fl->n[1];
@@ -1006,6 +1022,25 @@ int rhs_planes(const ibm_flow* fl, int n_sm) {
   for (int z = 4; z <= 32; ++z) {
     const long blocks = nb * ((fl->n[2] + z - 1) / z), waves = (blocks + 2 * n_sm - 1) / (2 * n_sm);
     const double cost = waves * (std::min(z, fl->n[2]) + 1.5);
+    if (cost < least) {
+      least = cost;
+      best = z;
+    }
+  }
+  return best;
+}
+
+// Output planes per block of cn_solve_kernel<W>: the whole waves of blocks times
+// the planes a block walks (its 2W planes of halo, and two to fill the pipeline)
+int solve_planes(const ibm_flow* fl, int W, int n_sm) {
+  const long tiles = 3l * ((fl->n[0] + kSolveT - 1) / kSolveT) * ((fl->n[1] + kSolveT - 1) / kSolveT);
+  const long slots = (long)solve_blocks(W) * n_sm;
+  int best = fl->n[2];
+  double least = 1e300;
+  for (int parts = 1; parts <= std::max(1, fl->n[2] / 8); ++parts) {
+    const int z = (fl->n[2] + parts - 1) / parts;
+    const long blocks = tiles * ((fl->n[2] + z - 1) / z);
+    const double cost = (double)((blocks + slots - 1) / slots) * (z + 2 * W + 2);
     if (cost < least) {
       least = cost;
       best = z;
@@ -1264,14 +1299,16 @@ extern "C" ibm_status ibm_flow_create(const ibm_grid_desc* grid, double nu, doub
   fl->dt = dt;
   ibm::choose_solves(fl);
   int n_sm = 0;
-  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, fl->device) == cudaSuccess)
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, fl->device) == cudaSuccess) {
     fl->rhs_planes = ibm::rhs_planes(fl, std::max(n_sm, 1));
+    for (int l = 0; l < 3; ++l)
+      if (fl->solve_w[l] >= 0) fl->solve_planes[l] = ibm::solve_planes(fl, fl->solve_w[l], std::max(n_sm, 1));
+  }
   const int nx = fl->n[0], ny = fl->n[1], nz = fl->n[2], nxh = nx / 2 + 1;
   fl->N = (size_t)nx * ny * nz;
   fl->NC = (size_t)nxh * ny * nz;
   cudaError_t e = cudaSuccess;
-  e = ibm::set_solve_smem(fl);
-  if (e == cudaSuccess) e = ibm::set_up_lines(fl);
+  e = ibm::set_up_lines(fl);
   for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMalloc(&fl->H[b], 3 * fl->N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fl->R, 3 * fl->N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fl->rp, fl->N * sizeof(float));

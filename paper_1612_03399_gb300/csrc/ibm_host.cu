@@ -659,6 +659,8 @@ void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
       if (cost[q] < cost[best]) best = q;
     }
     c->mshape[probe] = marker_shape(best, MT, probe != 0);
+    // at most 16 warps per SM: by the blocks there are, or by the shape
+    c->marker_few[probe] = (long long)n * MT <= 512ll * n_sm || best >= 2;
   }
 }
 

@@ -354,6 +354,7 @@ struct ibm_ctx {
   // launch shapes of the marker kernels without and with probes (chosen at
   // creation from the rest meshes)
   ibm::MarkerShape mshape[2] = {};
+  bool marker_few[2] = {false, false};   // their variants for few blocks per SM
   bool any_open = false;            // some body is an open sheet
   // coupled forcing (allocated by the first ibm_flow_step with this context):
   // the per-chunk tables and per-face geometry of substep 0, and the forcing's

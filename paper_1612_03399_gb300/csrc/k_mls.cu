@@ -45,20 +45,42 @@ namespace {
 // The global-memory path of a marker block whose footprint does not fit its
 // shared memory (rare): out of line, so that it does not crowd the
 // instruction cache of the staged path it sits beside.
-// (body cell G: read again here, so that it is not kept for this path)
+// (body cell G: read again here, so that it is not kept for this path; FEW: a
+// copy with the registers of the kernel's variant for few blocks)
 __device__ __forceinline__ GlobalRows global_rows(const Grid& g, const BodyDev* b) {
   return GlobalRows{g, {b->G[0], b->G[1], b->G[2]}};
 }
+// the 27 nodes of a support, all loads in flight
+struct Loaded {
+  float v[3][3][3];
+  __device__ __forceinline__ Loaded(const float* __restrict__ f, const GlobalAcc& A) {
+#pragma unroll
+    for (int sz = 0; sz < 3; ++sz)
+#pragma unroll
+      for (int sy = 0; sy < 3; ++sy) A.load(f, sy, sz, v[sz][sy]);
+  }
+  __device__ __forceinline__ void load(const float*, int sy, int sz, float (&u)[3]) const {
+#pragma unroll
+    for (int s = 0; s < 3; ++s) u[s] = v[sz][sy][s];
+  }
+};
+template <bool FEW>
 __device__ __noinline__ float value_global(const float* f, Grid g, const BodyDev* b, int c0, int c1,
                                           int c2, DirW X, DirW Y, DirW Z) {
   const int c[3] = {c0, c1, c2};
+  if (FEW) return mls_value(f, Loaded(f, global_rows(g, b).at(c)), X, Y, Z);
   return mls_value(f, global_rows(g, b).at(c), X, Y, Z);
 }
+template <bool FEW>
 __device__ __noinline__ float3 gradient_global(const float* f, Grid g, const BodyDev* b, ProbeW P) {
   float gr[3];
-  mls_grad(f, global_rows(g, b).at(P.cc), P.X, P.Y, P.Z, gr);
+  if (FEW)
+    mls_grad(f, Loaded(f, global_rows(g, b).at(P.cc)), P.X, P.Y, P.Z, gr);
+  else
+    mls_grad(f, global_rows(g, b).at(P.cc), P.X, P.Y, P.Z, gr);
   return make_float3(gr[0], gr[1], gr[2]);
 }
+template <bool FEW>
 __device__ __noinline__ void spread_global(float* f, Grid g, const BodyDev* b, int c0, int c1,
                                            int c2, DirW X, DirW Y, DirW Z, float coef) {
   const int c[3] = {c0, c1, c2};
@@ -81,8 +103,14 @@ __device__ __forceinline__ long long warp_sum_i64(long long q) {
 // for the second probe and the pressure the step's kernel needs no spills at
 // 80 registers (354 -> 339 us for the 1000 drops, 117 -> 111 us for the uneven
 // bodies).
-template <int MT, bool MEASURE, bool INTERP, bool PROBE, bool SPREAD, bool REC, bool PLAIN>
-__global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
+// FEW: 128 registers, 16 warps per SM, for launches that cannot use more: at most
+// two blocks of 256 faces per SM in all, or a shape of one or two blocks.  23 drops
+// with pressure (115 blocks): 26.4 -> 21.3 us; three large drops (15 blocks, every
+// footprint past its shape, all loads of a support in flight): a step 157 -> 139 us.
+// With more blocks the 24 warps are worth more: 500 drops 152 us against 177.
+enum MarkerVariant { kAll, kPlain, kFew };
+template <int MT, bool MEASURE, bool INTERP, bool PROBE, bool SPREAD, bool REC, int VAR>
+__global__ void __launch_bounds__(MT, (VAR == kFew ? 512 : 768) / MT) marker_kernel(
     DeviceTables T, Grid g, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
     const float* __restrict__ v, const float* __restrict__ u, const float* __restrict__ vv,
     const float* __restrict__ w, const float* __restrict__ pr, const float* __restrict__ accel,
@@ -90,6 +118,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
     float* __restrict__ Fext, float* __restrict__ fx, float* __restrict__ fy,
     float* __restrict__ fz, int record, int vec4, TileDev td, float phi_bound_all,
     int cache, int* __restrict__ cache_tab, float4* __restrict__ cache_face, MarkerShape shape) {
+  constexpr bool PLAIN = VAR == kPlain, FEW = VAR == kFew;
   constexpr bool FIELD = INTERP || PROBE || SPREAD;
   // the coupled forcing launch (interpolation and spread at the centroids)
   // may save its face geometry and row tables (cache 1) and, in the later
@@ -543,7 +572,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
             dir_weights(t3[1], sc.mk, Y);
             dir_weights(t3[2], sc.mk, Z);
             const float ps = fit ? mls_value((const float*)nullptr, SR.at(cc, obuf), X, Y, Z)
-                                 : value_global(pr, g, T.body + s_hdr[0], cc[0], cc[1], cc[2], X, Y, Z);
+                                 : value_global<FEW>(pr, g, T.body + s_hdr[0], cc[0], cc[1], cc[2], X, Y, Z);
             Pj += (l == 0 ? 1.f : -1.f) * ps + sc.probe_h * an;
           }
         }
@@ -562,7 +591,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
           if (fit) {
             mls_grad((const float*)nullptr, SR.at(P.cc, obuf), P.X, P.Y, P.Z, q);
           } else {
-            const float3 q3 = gradient_global(velc, g, T.body + s_hdr[0], P);
+            const float3 q3 = gradient_global<FEW>(velc, g, T.body + s_hdr[0], P);
             q[0] = q3.x;
             q[1] = q3.y;
             q[2] = q3.z;
@@ -597,7 +626,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
       if (mine) {
         if (INTERP) {
           const float Ul = fit ? mls_value((const float*)nullptr, SR.at(ccC, obuf), CX, CY, CZ)
-                               : value_global(velc, g, T.body + s_hdr[0], ccC[0], ccC[1], ccC[2], CX, CY, CZ);
+                               : value_global<FEW>(velc, g, T.body + s_hdr[0], ccC[0], ccC[1], ccC[2], CX, CY, CZ);
           const float Vb = PROBE ? s_own[(9 + comp) * MT]
                                  : (comp == 0 ? vb[0] : (comp == 1 ? vb[1] : vb[2]));
           Fc = (Vb - Ul) * sc.inv_dt;
@@ -664,7 +693,7 @@ __global__ void __launch_bounds__(MT, 768 / MT) marker_kernel(
         } else {
           asm volatile("griddepcontrol.wait;" ::: "memory");
           if (mine)
-            spread_global(fc, g, T.body + s_hdr[0], ccC[0], ccC[1], ccC[2], CX, CY, CZ, coef);
+            spread_global<FEW>(fc, g, T.body + s_hdr[0], ccC[0], ccC[1], ccC[2], CX, CY, CZ, coef);
         }
       }
       // the next component into the buffer that is free again (with the spread,
@@ -833,16 +862,24 @@ __global__ void __launch_bounds__(256) clear_kernel(DeviceTables T, Grid g, floa
   // float4 stores only for rows recorded in whole float4 groups
   vec4 = vec4 && lo.w == 2;
   if (lo.w == 1) {
-    const long long N = (long long)sz.x * sz.y * sz.z;
-    const int sxy = sz.x * sz.y;
-    for (long long idx = threadIdx.x; idx < N; idx += blockDim.x) {
-      const int k = (int)(idx / sxy), rem = (int)(idx - (long long)k * sxy), j = rem / sz.x,
-                i = rem - j * sz.x;
-      const size_t o = ((size_t)wrap(lo.z + k, g.n[2]) * g.n[1] + wrap(lo.y + j, g.n[1])) * nx +
-                       wrap(lo.x + i, nx);
-      fx[o] = 0.f;
-      fy[o] = 0.f;
-      fz[o] = 0.f;
+    // a warp per (y, z) row of the box (with 64-bit index divisions per node the
+    // 15 boxes of three large drops took the clear to 163 us; now 115, a step 139 -> 123)
+    const long long rows = (long long)sz.y * sz.z;
+    const int lane = threadIdx.x & 31;
+    int k = (int)((threadIdx.x >> 5) / sz.y), j = (int)(threadIdx.x >> 5) - k * sz.y;
+    for (long long r = threadIdx.x >> 5; r < rows; r += blockDim.x >> 5) {
+      const size_t base = ((size_t)wrap(lo.z + k, g.n[2]) * g.n[1] + wrap(lo.y + j, g.n[1])) * nx;
+      for (int i = lane; i < sz.x; i += 32) {
+        const size_t o = base + wrap(lo.x + i, nx);
+        fx[o] = 0.f;
+        fy[o] = 0.f;
+        fz[o] = 0.f;
+      }
+      j += blockDim.x >> 5;
+      while (j >= sz.y) {
+        j -= sz.y;
+        ++k;
+      }
     }
   } else {
     const int nrows = sz.w;
@@ -929,9 +966,11 @@ cudaError_t launch_mt(ibm_ctx* c, const float* x, const float* v, const float* u
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  auto kernel = marker_kernel<MT, M, I, P, S, R, true>;
+  auto kernel = marker_kernel<MT, M, I, P, S, R, kPlain>;
   if constexpr (P)
-    if (pr || c->any_open) kernel = marker_kernel<MT, M, I, P, S, R, false>;
+    if (pr || c->any_open) kernel = marker_kernel<MT, M, I, P, S, R, kAll>;
+  if constexpr (I || P || S)
+    if (c->marker_few[P ? 1 : 0]) kernel = marker_kernel<MT, M, I, P, S, R, kFew>;
   return cudaLaunchKernelEx(&cfg, kernel, tab ? *tab : c->d, c->grid,
                             c->sc, (int32_t)c->V, (int32_t)c->F, x, v, u, vv, w, pr, accel, U,
                             Fm, Fm_in, Fext, fx, fy, fz, record, vec4, c->td,
@@ -957,14 +996,14 @@ cudaError_t launch_t(ibm_ctx* c, const float* x, const float* v, const float* u,
 
 template <int MT, bool M, bool I, bool P, bool S, bool R>
 cudaError_t marker_smem_limit() {
-  cudaError_t e = cudaFuncSetAttribute(marker_kernel<MT, M, I, P, S, R, true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       marker_smem_max(MT, P));
+  auto set = [](auto kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                marker_smem_max(MT, P));
+  };
+  cudaError_t e = set(marker_kernel<MT, M, I, P, S, R, kPlain>);
   if constexpr (P)
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(marker_kernel<MT, M, I, P, S, R, false>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, marker_smem_max(MT, P));
-  return e;
+    if (e == cudaSuccess) e = set(marker_kernel<MT, M, I, P, S, R, kAll>);
+  return e == cudaSuccess ? set(marker_kernel<MT, M, I, P, S, R, kFew>) : e;
 }
 
 cudaError_t set_marker_smem_limit() {

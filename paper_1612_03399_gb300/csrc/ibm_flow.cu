@@ -1246,10 +1246,10 @@ void inverse_taps(double cc, int n, double* g) {
   }
 }
 
-// Picks each substep's solve: the smallest W <= kMaxSolveW, 2W + 1 <= n_d,
-// with the mass of the entries beyond |m| = W below 2^-26 in every
-// direction (real space), else the Fourier path (W = -1; also for planes of
-// more than 65535 tiles).
+// Picks each substep's solve: the smallest W <= kMaxSolveW with the mass of the
+// entries beyond |m| = W below 2^-26 in every direction and 2W + 1 <= n_d in every
+// direction (short filters), else W = -1 (line recursions or transforms; also for
+// planes of more than 65535 tiles).
 void choose_solves(ibm_flow* fl) {
   const long tiles = (long)((fl->n[0] + kSolveT - 1) / kSolveT) * ((fl->n[1] + kSolveT - 1) / kSolveT);
   for (int l = 0; l < 3; ++l) {
@@ -1273,6 +1273,10 @@ void choose_solves(ibm_flow* fl) {
       }
       wl = wd < 0 ? -1 : std::max(wl, wd);
     }
+    // every direction is filtered with the largest W: a short period that its own
+    // width already covers would count entries twice, and the walk wrap past it
+    for (int d = 0; d < 3; ++d)
+      if (2 * wl + 1 > fl->n[d]) wl = -1;
     fl->solve_w[l] = wl;
     for (int d = 0; d < 3; ++d)
       for (int m = 0; m <= kMaxSolveW; ++m)

@@ -59,7 +59,8 @@ struct ibm_flow {
   // its taps g[d][|m|] per direction, m = 0..W
   int solve_w[3] = {-1, -1, -1};
   float taps[3][3][9] = {};
-  bool z_lines = false;         // the Poisson solve's z direction by recursions
+  bool z_lines = false;         // the Poisson solve's z direction by recursions,
+  float4* zcol = nullptr;       // with their constants per column [ny][nx/2 + 1]
   int rhs_planes = 16;          // planes per thread of the right-hand side kernel
   int solve_planes[3] = {32, 32, 32};   // output planes per block of the real-space solves
   // per substep: solved by recursions along the lines; the powers of r they use
@@ -234,24 +235,50 @@ __global__ void __launch_bounds__(kRowThreads * kRowsPerBlock)
 // The Poisson solve's z direction without transforms: after the (x, y) transforms
 // each column (k_x, k_y) is a periodic tridiagonal system,
 //   (2 + d - E - E^-1) phi = -h_z^2 f,  d = -h_z^2 (lam_x + lam_y) > 0,
-// and 2 + d - E - E^-1 = (1 - r E^-1)(1 - r E)/r with r = exp(-theta), theta =
-// 2 asinh(sqrt(d)/2): one recursion up the column and one down.  They are run with
-// 1 - r, which keeps its relative precision where r is near 1.  A thread holds a
-// segment of at most kZSeg entries in registers and runs it twice, first from
-// zero for its end, then from the value that enters it: the segments' ends
-// combined, the column closing on itself (the sum over a turn / (1 - r^n)).
+// and 2 + d - E - E^-1 = (1 - r E^-1)(1 - r E)/r with, s = sqrt(d)/2 and
+// t = sqrt(1 + s^2), r = 1/(s + t)^2: one recursion up the column and one down.
+// Its constants come from a table in float64, each in the form that keeps it
+// to rounding: rho = 1 - r = 2s/(s + t) for the recursions (r near 1 for the long
+// waves), -h_z^2 r for the result (r near h_x^2/(8 h_z^2) for the short ones on
+// cells stretched in z), r^k from exp(-2k asinh(s)).  A recursion adds the small
+// f - rho y to y and carries what the addition loses, so a long wave's sum over a
+// column does not gather rounding.  A thread holds a segment of at most kZSeg
+// entries in registers and runs it twice, first from zero for its end, then from
+// the value that enters it: the segments' ends combined, the column closing on
+// itself (the sum over a turn / (1 - r^n)).
 // Column (0, 0), d = 0, is summed twice in float64 by one warp; its mean is 0.
 // What bounds it: HBM, 16 bytes per coefficient once; two z transforms with the
-// scaling between them moved three times that: 256^3 65 -> 25 us,
-// 200 x 180 x 144 29 -> 13.  The error of p against float64 over 40 x 36 x 20 ..
-// 128^3 and 30 x 40 x 500 is 0.2 .. 1.3 of the transforms', of u 0.4 .. 1.2.
+// scaling between them moved three times that: 256^3 65 -> 29 us,
+// 200 x 180 x 144 29 -> 12.
 constexpr int kZSeg = 16, kZMax = 512;   // entries of a segment, of a column (32 segments)
 
-__device__ __forceinline__ float2 step_line(float2 y, float2 f, float rho) {   // f + (1 - rho) y
-  return make_float2(fmaf(-rho, y.x, y.x) + f.x, fmaf(-rho, y.y, y.y) + f.y);
-}
+struct ZLine {   // y <- f + (1 - rho) y; c: what y is too large by
+  float2 y = {0.f, 0.f}, c = {0.f, 0.f};
+  __device__ __forceinline__ void add(float& v, float& e, float f, float rho) {
+    const float inc = fmaf(-rho, v, f) - e, n = v + inc;
+    e = (n - v) - inc;
+    v = n;
+  }
+  __device__ __forceinline__ float2 step(float2 f, float rho) {
+    add(y.x, c.x, f.x, rho);
+    add(y.y, c.y, f.y, rho);
+    return y;
+  }
+};
 __device__ __forceinline__ float2 axpy2(float a, float2 x, float2 y) {
   return make_float2(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y));
+}
+
+// per column (rho, -h_z^2 r, r^base, 1/(1 - r^n_z)), base the shorter segments' length
+__global__ void poisson_z_table_kernel(float4* __restrict__ table, int nx, int ny, int nz, int base,
+                                       double hx, double hy, double hz) {
+  const int nxh = nx / 2 + 1, col = blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= nxh * ny) return;
+  const int j = col / nxh;
+  const double kx = hz / hx * sinpi((double)(col - j * nxh) / nx), ky = hz / hy * sinpi((double)j / ny);
+  const double s = sqrt(kx * kx + ky * ky), q = 1.0 / (s + sqrt(1.0 + s * s)), theta = 2.0 * asinh(s);
+  table[col] = make_float4((float)(2.0 * s * q), (float)(-hz * hz * q * q), (float)exp(-theta * base),
+                           col ? (float)(-1.0 / expm1(-theta * nz)) : 0.f);
 }
 
 __device__ __noinline__ void poisson_z_mean_column(cufftComplex* __restrict__ S, size_t M, int n,
@@ -296,64 +323,68 @@ __device__ __noinline__ void poisson_z_mean_column(cufftComplex* __restrict__ S,
   }
 }
 
-// 32 columns per block, segment threadIdx.y; scale: what the forward and inverse
-// (x, y) transforms and the time step leave to divide by
+// 32 columns per block, segment threadIdx.y (the first block: column (0, 0));
+// scale: what the forward and inverse (x, y) transforms and the time step leave to
+// divide by
 __global__ void __launch_bounds__(32 * (kZMax / kZSeg))
     poisson_z_kernel(cufftComplex* __restrict__ S, int nxh, int ny, int nz,
-                     const float* __restrict__ lam, double h2, double scale) {
+                     const float4* __restrict__ table, double h2, double scale) {
   __shared__ float2 ends[2][kZMax / kZSeg][32];
-  const int M = nxh * ny, col = blockIdx.x * 32 + threadIdx.x, lane = threadIdx.x;
+  const int M = nxh * ny;
+  if (blockIdx.x == 0) {
+    if (threadIdx.y == 0) poisson_z_mean_column(S, (size_t)M, nz, h2, scale);
+    return;
+  }
+  const int col = (int)(blockIdx.x - 1) * 32 + threadIdx.x, lane = threadIdx.x;
   const bool in = col > 0 && col < M;
   const int g = threadIdx.y, segs = blockDim.y, n = nz;
   // the first n mod segs segments are one longer
   const int base = n / segs, rem = n - base * segs;
   const int k0 = g * base + min(g, rem), len = base + (g < rem ? 1 : 0);
   float2* at = reinterpret_cast<float2*>(S) + (size_t)k0 * M + col;
+  const float4 k = in ? __ldg(table + col) : make_float4(1.f, 0.f, 0.f, 0.f);
   float2 f[kZSeg];
 #pragma unroll
   for (int i = 0; i < kZSeg; ++i)
     f[i] = in && i < len ? at[(size_t)i * M] : make_float2(0.f, 0.f);
-  float rho = 1.f, theta = 1.f;
-  if (in) {
-    const int j = col / nxh;
-    const float d = -(float)h2 * (__ldg(lam + (col - j * nxh)) + __ldg(lam + nxh + j));
-    theta = 2.f * asinhf(0.5f * sqrtf(d));
-    rho = -expm1f(-theta);
-  }
-  const float close = -1.f / expm1f(-theta * (float)n);
-  const float turn = expf(-theta * (float)base), turn1 = turn * (1.f - rho);   // r^base, r^(base+1)
+  const float rho = k.x, turn = k.z, turn1 = fmaf(-turn, rho, turn), close = k.w;   // r^base, r^(base+1)
   auto across = [&](int h) { return h < rem ? turn1 : turn; };
-  float2 y = make_float2(0.f, 0.f);
+  {
+    ZLine a;
 #pragma unroll
-  for (int i = 0; i < kZSeg; ++i)
-    if (i < len) y = step_line(y, f[i], rho);
-  ends[0][g][lane] = y;
+    for (int i = 0; i < kZSeg; ++i)
+      if (i < len) a.step(f[i], rho);
+    ends[0][g][lane] = a.y;
+  }
   __syncthreads();
-  y = make_float2(0.f, 0.f);
-  for (int h = 0; h < segs; ++h) y = axpy2(across(h), y, ends[0][h][lane]);
-  y = make_float2(close * y.x, close * y.y);
-  for (int h = 0; h < g; ++h) y = axpy2(across(h), y, ends[0][h][lane]);
+  {
+    ZLine a;
+    for (int h = 0; h < segs; ++h) a.y = axpy2(across(h), a.y, ends[0][h][lane]);
+    a.y = make_float2(close * a.y.x, close * a.y.y);
+    for (int h = 0; h < g; ++h) a.y = axpy2(across(h), a.y, ends[0][h][lane]);
 #pragma unroll
-  for (int i = 0; i < kZSeg; ++i)
-    if (i < len) f[i] = y = step_line(y, f[i], rho);
-  float2 x = make_float2(0.f, 0.f);
+    for (int i = 0; i < kZSeg; ++i)
+      if (i < len) f[i] = a.step(f[i], rho);
+  }
+  {
+    ZLine a;
 #pragma unroll
-  for (int i = kZSeg - 1; i >= 0; --i)
-    if (i < len) x = step_line(x, f[i], rho);
-  ends[1][g][lane] = x;
+    for (int i = kZSeg - 1; i >= 0; --i)
+      if (i < len) a.step(f[i], rho);
+    ends[1][g][lane] = a.y;
+  }
   __syncthreads();
-  x = make_float2(0.f, 0.f);
-  for (int h = segs - 1; h >= 0; --h) x = axpy2(across(h), x, ends[1][h][lane]);
-  x = make_float2(close * x.x, close * x.y);
-  for (int h = segs - 1; h > g; --h) x = axpy2(across(h), x, ends[1][h][lane]);
-  const float s = (float)(-h2 * scale) * (1.f - rho);
+  ZLine a;
+  for (int h = segs - 1; h >= 0; --h) a.y = axpy2(across(h), a.y, ends[1][h][lane]);
+  a.y = make_float2(close * a.y.x, close * a.y.y);
+  for (int h = segs - 1; h > g; --h) a.y = axpy2(across(h), a.y, ends[1][h][lane]);
+  const float s = k.y * (float)scale;
 #pragma unroll
   for (int i = kZSeg - 1; i >= 0; --i)
     if (i < len) {
-      x = step_line(x, f[i], rho);
+      const float2 x = a.step(f[i], rho);
       if (in) at[(size_t)i * M] = make_float2(s * x.x, s * x.y);
     }
-  if (blockIdx.x == 0 && threadIdx.y == 0) poisson_z_mean_column(S, (size_t)M, n, h2, scale);
 }
 
 // u_c += du_c, du = [3][N]; the component in blockIdx.y
@@ -1093,9 +1124,11 @@ bool use_lines(const ibm_flow* fl, int l) {
 }
 
 // The Poisson solve takes the z direction by recursions where a column fits a
-// block's registers and its slowest recursion dies down to a half within a turn
-// (r^n <= 1/2; the largest of L_x, L_y at most nine times L_z): past that the
-// closing of the column amplifies its rounding.
+// block's registers and its slowest recursion dies down to e^-4 within a turn
+// (the larger of L_x, L_y at most 1.57 L_z): past that the closing of the column
+// amplifies its rounding.  Errors against float64 relative to the transforms', on
+// 9 x 5 x 15 .. 128^3 and cells 1 : 1 : 0.65 .. 1 : 1 : 16: p 0.3 .. 1.0, u 0.6 .. 1.0;
+// beyond the line, at L_x = 4 L_z, p up to 1.2.
 bool use_z_lines(const ibm_flow* fl) {
   if (fl->n[2] > kZMax || (long long)(fl->n[0] / 2 + 1) * fl->n[1] > 0x7fffffffll - 32) return false;
   double least = 1e300;
@@ -1104,7 +1137,20 @@ bool use_z_lines(const ibm_flow* fl) {
       const double k = 2.0 / fl->h[d] * std::sin(3.14159265358979323846 / fl->n[d]);
       least = std::min(least, 2.0 * std::asinh(0.5 * fl->h[2] * k));
     }
-  return least * fl->n[2] >= std::log(2.0);
+  return least * fl->n[2] >= 4.0;
+}
+
+int z_segments(const ibm_flow* fl) { return (fl->n[2] + kZSeg - 1) / kZSeg; }
+
+cudaError_t set_up_z_lines(ibm_flow* fl) {
+  fl->z_lines = use_z_lines(fl);
+  if (!fl->z_lines) return cudaSuccess;
+  const int M = (fl->n[0] / 2 + 1) * fl->n[1];
+  const cudaError_t e = cudaMalloc(&fl->zcol, sizeof(float4) * (size_t)M);
+  if (e != cudaSuccess) return e;
+  poisson_z_table_kernel<<<(unsigned)((M + 127) / 128), 128>>>(
+      fl->zcol, fl->n[0], fl->n[1], fl->n[2], fl->n[2] / z_segments(fl), fl->h[0], fl->h[1], fl->h[2]);
+  return cudaGetLastError();
 }
 
 // device table of the powers, and the kernels' shared memory
@@ -1222,7 +1268,7 @@ void release(ibm_flow* fl) {
     cufftDestroy(fl->c2r1);
   }
   for (void* q : {(void*)fl->H[0], (void*)fl->H[1], (void*)fl->R, (void*)fl->rp, (void*)fl->S,
-                  (void*)fl->lam, (void*)fl->pw})
+                  (void*)fl->lam, (void*)fl->pw, (void*)fl->zcol})
     if (q) cudaFree(q);
   for (auto& row : fl->ev)
     for (cudaEvent_t& ev : row)
@@ -1384,9 +1430,9 @@ cudaError_t flow_project(ibm_flow* fl, int l, float* u, float* v, float* w, floa
   if (e == cudaSuccess) {
     const int nxh = fl->n[0] / 2 + 1;
     if (fl->z_lines) {
-      const dim3 block(32, (unsigned)((fl->n[2] + kZSeg - 1) / kZSeg));
-      poisson_z_kernel<<<(unsigned)((nxh * fl->n[1] + 31) / 32), block, 0, s>>>(
-          fl->S, nxh, fl->n[1], fl->n[2], fl->lam, fl->h[2] * fl->h[2],
+      const dim3 block(32, (unsigned)z_segments(fl));
+      poisson_z_kernel<<<(unsigned)((nxh * fl->n[1] + 31) / 32) + 1, block, 0, s>>>(
+          fl->S, nxh, fl->n[1], fl->n[2], fl->zcol, fl->h[2] * fl->h[2],
           1.0 / ((double)fl->n[0] * fl->n[1] * alpha * fl->dt));
     } else {
       poisson_scale_kernel<<<row_blocks(fl), dim3(kRowThreads, kRowsPerBlock), 0, s>>>(
@@ -1463,6 +1509,7 @@ extern "C" ibm_status ibm_flow_create(const ibm_grid_desc* grid, double nu, doub
   fl->NC = (size_t)nxh * ny * nz;
   cudaError_t e = cudaSuccess;
   e = ibm::set_up_lines(fl);
+  if (e == cudaSuccess) e = ibm::set_up_z_lines(fl);
   for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMalloc(&fl->H[b], 3 * fl->N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fl->R, 3 * fl->N * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&fl->rp, fl->N * sizeof(float));
@@ -1478,6 +1525,8 @@ extern "C" ibm_status ibm_flow_create(const ibm_grid_desc* grid, double nu, doub
       }
     e = cudaMemcpy(fl->lam, lam.data(), lam.size() * sizeof(float), cudaMemcpyHostToDevice);
   }
+  // the tables are there whichever stream the flow runs on
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     ibm::release(fl);
     delete fl;
@@ -1490,7 +1539,6 @@ extern "C" ibm_status ibm_flow_create(const ibm_grid_desc* grid, double nu, doub
   bool ok = r == CUFFT_SUCCESS;
   if (ok) ok = cufftPlanMany(&fl->c2r3, 3, dims, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 3) == CUFFT_SUCCESS;
   // the Poisson solve's: all three directions, or (x, y) of every plane
-  fl->z_lines = ibm::use_z_lines(fl);
   const int rank = fl->z_lines ? 2 : 3, batch = fl->z_lines ? nz : 1;
   int* pd = dims + 3 - rank;
   if (ok) ok = cufftPlanMany(&fl->r2c1, rank, pd, nullptr, 1, 0, nullptr, 1, 0, CUFFT_R2C, batch) == CUFFT_SUCCESS;

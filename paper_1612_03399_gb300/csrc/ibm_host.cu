@@ -1103,14 +1103,15 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
       w.blob_off += topo_blob[body_topo[w.body]];
     }
     c->force_threads = choose_force_threads(fwork);
-    c->force_wide = force_smem_wide <= 227 * 1024;
+    size_t room = 0, adjoint_room = 0;
+    check_cuda(force_smem_room(&room), "cudaFuncGetAttributes");
+    check_cuda(adjoint_smem_room(&adjoint_room), "cudaFuncGetAttributes");
+    c->force_wide = force_smem_wide <= room;
     c->force_smem = c->force_wide ? force_smem_wide : force_smem;
-    if (c->force_smem > 227 * 1024)
-      fail(IBM_ERR_UNSUPPORTED, "force-kernel shared memory above 227 KB; lower patch_size");
-    c->adjoint_wide = adjoint_smem_wide <= 226 * 1024;   // 1 KB for the static part
+    c->adjoint_wide = adjoint_smem_wide <= adjoint_room;
     c->adjoint_smem = c->adjoint_wide ? adjoint_smem_wide : adjoint_smem;
     c->max_own = max_own;
-    if (c->adjoint_smem > 227 * 1024)
+    if (c->force_smem > room || c->adjoint_smem > adjoint_room)
       fail(IBM_ERR_UNSUPPORTED, "force-kernel shared memory above 227 KB; lower patch_size");
     check_cuda(set_force_smem_limit(c->force_smem), "cudaFuncSetAttribute");
     check_cuda(set_adjoint_smem_limit(c->adjoint_smem), "cudaFuncSetAttribute");

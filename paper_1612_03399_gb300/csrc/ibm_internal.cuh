@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -473,23 +474,33 @@ cudaError_t launch_taylor(ibm_ctx* c, const float* x, double* D);
 cudaError_t launch_interp64(ibm_ctx* c, const float* x, const float* v, const float* u,
                             const float* vv, const float* w, float* U, float* Fm, float* Fext);
 cudaError_t launch_taylor_backward(ibm_ctx* c, const float* x, const double* gD, float* gx);
-// Let a kernel be launched with as much dynamic shared memory as a block can
-// have beside its static part (the limit belongs to the function, not to a
-// context: a smaller one set for one context would fail another's launches);
-// cudaErrorInvalidValue when `bytes` is more than that.
+// The most dynamic shared memory a block of the kernel can have beside its static
+// part; *room is lowered to it.
 template <class... A>
-cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
+cudaError_t smem_room(void (*kernel)(A...), size_t* room) {
   cudaFuncAttributes at{};
   int dev = 0, most = 0;
   cudaError_t e = cudaFuncGetAttributes(&at, kernel);
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return e;
-  most -= (int)at.sharedSizeBytes;
-  if (bytes > (size_t)most) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) *room = std::min(*room, (size_t)most - at.sharedSizeBytes);
+  return e;
 }
+// Let a kernel be launched with that much (the limit belongs to the function, not
+// to a context: a smaller one set for one context would fail another's launches);
+// cudaErrorInvalidValue when `bytes` is more.
+template <class... A>
+cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
+  size_t room = SIZE_MAX;
+  const cudaError_t e = smem_room(kernel, &room);
+  if (e != cudaSuccess) return e;
+  if (bytes > room) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+}
+// the dynamic shared memory every force (adjoint) kernel can be launched with
+cudaError_t force_smem_room(size_t* room);
+cudaError_t adjoint_smem_room(size_t* room);
 cudaError_t set_force_smem_limit(size_t bytes);
 cudaError_t set_adjoint_smem_limit(size_t bytes);
 cudaError_t set_marker_smem_limit();

@@ -665,6 +665,11 @@ cudaError_t launch_backward(ibm_ctx* c, const float* x, const float* v, const fl
   return cudaGetLastError();
 }
 
+cudaError_t adjoint_smem_room(size_t* room) {
+  *room = SIZE_MAX;
+  const cudaError_t e = smem_room(force_adjoint_kernel<true>, room);
+  return e == cudaSuccess ? smem_room(force_adjoint_kernel<false>, room) : e;
+}
 cudaError_t set_adjoint_smem_limit(size_t bytes) {
   const cudaError_t e = allow_smem(force_adjoint_kernel<true>, bytes);
   return e == cudaSuccess ? allow_smem(force_adjoint_kernel<false>, bytes) : e;

@@ -396,14 +396,22 @@ cudaError_t launch_advance(ibm_ctx* c, const float* x, const float* v, const flo
   return cudaGetLastError();
 }
 
-cudaError_t set_force_smem_limit(size_t bytes) {
+template <class Fn>
+static cudaError_t each_force_kernel(Fn fn) {
   cudaError_t e = cudaSuccess;
   for (auto k : {force_kernel<0, false, true>, force_kernel<0, true, true>,
                  force_kernel<1, false, true>, force_kernel<2, false, true>,
                  force_kernel<0, false, false>, force_kernel<0, true, false>,
                  force_kernel<1, false, false>, force_kernel<2, false, false>})
-    if (e == cudaSuccess) e = allow_smem(k, bytes);
+    if (e == cudaSuccess) e = fn(k);
   return e;
+}
+cudaError_t force_smem_room(size_t* room) {
+  *room = SIZE_MAX;
+  return each_force_kernel([&](auto k) { return smem_room(k, room); });
+}
+cudaError_t set_force_smem_limit(size_t bytes) {
+  return each_force_kernel([&](auto k) { return allow_smem(k, bytes); });
 }
 
 }  // namespace ibm

@@ -95,7 +95,7 @@ __device__ __forceinline__ void face_forward(const Vec<float>& e, const Vec<floa
                                              Vec<float>& fa, Vec<float>& fb, Vec<float>& fw,
                                              float& e_area) {
   const float da = 0.5f * vdot(N, N) * rn - A0f;
-  const float k = -0.5f * side * rn * (cA + ka * __fdividef(da, A0f)), kv = cV * (-1.f / 6.f);
+  const float k = -0.5f * side * rn * (cA + ka * (da / A0f)), kv = cV * (-1.f / 6.f);
   const Vec<float> m = vscale(N, k);
   const Vec<float> X = vcross(m, w), Y = vcross(m, e);
   const Vec<float> v = {fmaf(kv, N.x, t.x), fmaf(kv, N.y, t.y), fmaf(kv, N.z, t.z)};
@@ -167,8 +167,8 @@ __device__ __forceinline__ void face_tangent(const Vec<float>& e, const Vec<floa
                                              float cAd, float cV, float cVd, Vec<float>& fa,
                                              Vec<float>& fb, Vec<float>& fw, float& uk_a) {
   const float Af = 0.5f * vdot(N, N) * rn, Afd = Af * h;
-  const float strain = __fdividef(Af - A0f, A0f);
-  const float gA = cA + ka * strain, gAd = cAd + __fdividef(ka * Afd, A0f);
+  const float iA = 1.f / A0f, strain = (Af - A0f) * iA;
+  const float gA = cA + ka * strain, gAd = cAd + ka * Afd * iA;
   const float k0 = -0.5f * side * rn;
   const float k = k0 * gA, kd = k0 * (gAd - h * gA);     // (1/|N|)' = -h/|N|
   const Vec<float> m = vscale(N, k), md = vmad(kd, N, k, Nd);

@@ -65,9 +65,9 @@ __device__ __forceinline__ void val_grad_at(const float* __restrict__ f, const G
   float t[3];
   locate(tau, comp, c, t);
   DirG X, Y, Z;
-  dir_grad(t[0], sc.mk, X);
-  dir_grad(t[1], sc.mk, Y);
-  dir_grad(t[2], sc.mk, Z);
+  dir_grad<true>(t[0], sc.mk, X);
+  dir_grad<true>(t[1], sc.mk, Y);
+  dir_grad<true>(t[2], sc.mk, Z);
   mls_val_grad(f, R.at(c), X, Y, Z, val, gr);
 #pragma unroll
   for (int j = 0; j < 3; ++j) gr[j] *= sc.kg[j];

@@ -40,10 +40,10 @@
 namespace ibm {
 namespace {
 
-// 2^x and 1/x by the special-function unit.  Arguments are in its full
-// precision range: |x| <= 2 kappa log2(e) / 2, and sums of weights or variances
-// of at least the smallest normal number (below it the closed form has no
-// float32 value).
+// 2^x and 1/x by the special-function unit (1/x: the marker and spread kernels).
+// Arguments are in its full precision range: |x| <= 2 kappa log2(e) / 2, and sums of
+// weights or variances of at least the smallest normal number (below it the closed
+// form has no float32 value).
 __device__ __forceinline__ float ex2_fast(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -81,15 +81,18 @@ __device__ __forceinline__ void dir_weights(float t, const MlsK& K, DirW& o) {
   o.b2 = r * fmaf(-o.a2, m, o.a2);
 }
 
-__device__ __forceinline__ void dir_grad(float t, const MlsK& K, DirG& o) {
+// IEEE: the reciprocals rounded correctly (the adjoint's); returns 1/s2
+template <bool IEEE = false>
+__device__ __forceinline__ float dir_grad(float t, const MlsK& K, DirG& o) {
+  auto rcp = [](float x) { return IEEE ? 1.f / x : rcp_fast(x); };
   const float z = K.z * t;
   const float rm = K.ek * ex2_fast(-z), rp = K.ek * ex2_fast(z);
-  const float i = rcp_fast(1.f + rm + rp);
+  const float i = rcp(1.f + rm + rp);
   o.a0 = rm * i;
   o.a2 = rp * i;
   const float m = o.a2 - o.a0, q = o.a0 + o.a2;
   const float s2 = fmaf(-m, m, q);
-  const float is2 = rcp_fast(s2);
+  const float is2 = rcp(s2);
   o.r = (m - t) * is2;
   o.c0 = -fmaf(o.a0, m, o.a0);
   o.c2 = fmaf(-o.a2, m, o.a2);
@@ -97,6 +100,7 @@ __device__ __forceinline__ void dir_grad(float t, const MlsK& K, DirG& o) {
   o.g2 = fmaf(o.c2, 1.f - m, -o.a2 * s2);
   const float mu3 = m * fmaf(-3.f, q, fmaf(2.f * m, m, 1.f));
   o.h = fmaf(o.r, mu3, K.hk) * is2;
+  return is2;
 }
 
 __device__ __forceinline__ int wrap(int i, int n) {
@@ -257,12 +261,12 @@ struct DirH : DirG {
   float k1, k2;   // the coefficients of gaa and daa above
 };
 __device__ __forceinline__ void dir_hess(float t, const MlsK& K, DirH& o) {
-  dir_grad(t, K, o);
+  const float is2 = dir_grad<true>(t, K, o);
   const float m = o.a2 - o.a0, q = o.a0 + o.a2, m2 = m * m;
   const float s2 = q - m2;
   const float mu3 = m * fmaf(-3.f, q, fmaf(2.f, m2, 1.f));
   const float mu4 = fmaf(-3.f * m, mu3, fmaf(-3.f, m2, 1.f) * s2);
-  const float dh = fmaf(fmaf(-2.f, o.h, 1.f), mu3, o.r * fmaf(-3.f * s2, s2, mu4)) * rcp_fast(s2);
+  const float dh = fmaf(fmaf(-2.f, o.h, 1.f), mu3, o.r * fmaf(-3.f * s2, s2, mu4)) * is2;
   o.k1 = fmaf(-o.r, fmaf(-3.f, q, 1.f), dh);
   o.k2 = fmaf(3.f * m, o.r, fmaf(2.f, o.h, -1.f));
 }

@@ -703,7 +703,8 @@ void make_consts(ibm_ctx* c) {
   c->sc.mu = (float)p.mu;
   c->sc.probe_h = (float)(p.probe_h > 0 ? p.probe_h : (h[0] + h[1] + h[2]) / 3.0);
   c->sc.kappa = (float)(1.0 / ((1.5 * alpha) * (1.5 * alpha)));
-  const double kappa = 1.0 / ((1.5 * alpha) * (1.5 * alpha));
+  // (below 1e-30 the weights are 1 to rounding, and 1/(2 kappa) would leave float32)
+  const double kappa = std::max(1.0 / ((1.5 * alpha) * (1.5 * alpha)), 1e-30);
   c->sc.mk.z = (float)(2.0 * kappa / std::log(2.0));
   c->sc.mk.ek = (float)std::exp(-kappa);
   c->sc.mk.hk = (float)(0.5 / kappa);

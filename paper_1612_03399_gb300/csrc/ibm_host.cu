@@ -625,12 +625,10 @@ PatchNodes patch_nodes(const ibm_ctx* c, const ibm_body_desc& B, const HostTopo&
 
 // The launch shapes of the marker kernels, from up to 64 patches spread over
 // the order of their areas (the largest among them).  A patch that does not
-// fit takes the global path, at about 4.4 times the time of a staged one;
-// against two buffers, one buffer measured the same with the spread in the
-// kernel and 1.05 .. 1.08 without, 16 warps per SM 1.2 .. 1.3, and where there is
-// at most one block per SM the warps per SM do not matter.  The shape with the
-// least expected time is taken; a tenth of the nodes and rows is kept for the
-// bodies' motion.
+// fit takes the global path, at about 4.4 times the time of a staged one; 16 warps
+// per SM measured 1.2 .. 1.3 times the time of 24, and where there is at most one
+// block per SM the warps per SM do not matter.  The shape with the least expected
+// time is taken; a tenth of the nodes and rows is kept for the bodies' motion.
 void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
                           const std::vector<HostTopo>& topos, const std::vector<int>& body_topo,
                           const std::vector<int4>& chunks, const std::vector<float>& area, int n_sm) {
@@ -651,7 +649,7 @@ void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
       }
     }
     const bool few = n <= n_sm;
-    const double rel[kMarkerShapes] = {1.0, 1.05, few ? 1.05 : 1.25, few ? 1.0 : 2.2};
+    const double rel[kMarkerShapes] = {1.0, few ? 1.0 : 1.25, few ? 1.0 : 2.2};
     int best = 0;
     double cost[kMarkerShapes];
     for (int q = 0; q < kMarkerShapes; ++q) {
@@ -660,7 +658,7 @@ void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
     }
     c->mshape[probe] = marker_shape(best, MT, probe != 0);
     // at most 16 warps per SM: by the blocks there are, or by the shape
-    c->marker_few[probe] = (long long)n * MT <= 512ll * n_sm || best >= 2;
+    c->marker_few[probe] = (long long)n * MT <= 512ll * n_sm || best >= 1;
   }
 }
 

@@ -266,41 +266,44 @@ struct DeviceTables {
 // marker-kernel dynamic shared memory: per (y, z) row the byte offset of its
 // staged start minus 4 x its first x, and its first group (16 bits); per
 // staged float4 group its global offset; a bit per group that received a
-// nonzero spread; then one or two staging buffers (velocity components, and in
-// place of a component once it is used its fixed-point spread accumulators),
-// and the probe kernels' per-thread values.  While the rows are being found,
-// the first buffer holds their x-ranges.
+// nonzero spread; then the staging room (a velocity component, and in place of a
+// component once it is used its fixed-point spread accumulators; two buffers of
+// half the room each where the patch's nodes fit one), and the probe kernels'
+// per-thread values.  While the rows are being found, the room holds their x-ranges.
 constexpr int kMaxRows = 4 * kMT;      // rows of a patch's footprint record
 __host__ __device__ constexpr int marker_mask_words(int nodes) {
   return ((nodes / 4 + 31) / 32 + 4) & ~3;
 }
 constexpr int kOwn = 19;               // per-thread values of the probe kernels
-// Launch shape of a marker kernel: (y, z) rows of its table, staged nodes of a
-// buffer, staging buffers
+// Launch shape of a marker kernel: (y, z) rows of its table, staged nodes
 struct MarkerShape {
-  int rows, nodes, buffers;
+  int rows, nodes;
 };
 __host__ __device__ constexpr int marker_smem_bytes(int MT, MarkerShape m, bool probe) {
   return 4 * m.rows + 2 * (m.rows + 8) + 4 * marker_mask_words(m.nodes) + 4 * (m.nodes / 4) +
-         4 * m.buffers * m.nodes + (probe ? 4 * kOwn * MT : 0);
+         4 * m.nodes + (probe ? 4 * kOwn * MT : 0);
 }
-// The shapes a launch may take: 24 warps per SM (three 256-face or six
-// 128-face blocks, 75 KB and 37 KB each) with two buffers; with one buffer (the
-// next component's copies then start only when the current one is used up);
-// 16 warps per SM; or 8 warps per SM
-constexpr int kMarkerShapes = 4;
+// The shapes a launch may take: 24 warps per SM (three 256-face or six 128-face
+// blocks, 75 KB and 37 KB each), 16 warps per SM, or 8 warps per SM.  A patch whose
+// nodes fit half of a shape's room copies the next component while it uses one;
+// the others use the room as one buffer (the next component's copies then start
+// only when the current one is used up).  Which of the two is each block's own
+// choice, so that bodies may stretch to twice the nodes before a patch leaves
+// shared memory: with two buffers or one fixed at creation, drops of 12 cells
+// stretched 2.0 times had 94 of 1000 patches outside and a step took 212 us; now 9
+// and 164.  1000 drops at rest on 512^3: 451 -> 442 us.
+constexpr int kMarkerShapes = 3;
 __host__ __device__ constexpr MarkerShape marker_shape(int k, int MT, bool probe) {
-  return k == 0   ? MarkerShape{4 * MT, (probe ? 21 : 29) * MT, 2}
-         : k == 1 ? MarkerShape{4 * MT, (probe ? 38 : 52) * MT, 1}
-         : k == 2 ? MarkerShape{6 * MT, (probe ? 64 : 80) * MT, 1}
-                  : MarkerShape{6 * MT, (probe ? 84 : 92) * MT, 2};
+  return k == 0   ? MarkerShape{4 * MT, (probe ? 38 : 52) * MT}
+         : k == 1 ? MarkerShape{6 * MT, (probe ? 64 : 80) * MT}
+                  : MarkerShape{6 * MT, (probe ? 156 : 172) * MT};
 }
 __host__ __device__ constexpr int marker_smem_max(int MT, bool probe) {
-  return marker_smem_bytes(MT, marker_shape(3, MT, probe), probe);
+  return marker_smem_bytes(MT, marker_shape(kMarkerShapes - 1, MT, probe), probe);
 }
 static_assert(marker_smem_max(kMT, true) <= 226 * 1024 && marker_smem_max(kMT, false) <= 226 * 1024,
               "a marker block's shared memory");
-constexpr int kTableRows = marker_shape(3, kMT, false).rows;     // of the largest shape
+constexpr int kTableRows = marker_shape(kMarkerShapes - 1, kMT, false).rows;     // of the largest shape
 // Per-chunk cache of the coupled forcing launch (the markers stay at x^n for
 // the three substeps of a coupled step): a 16-word header (x, y, z lo, x, y,
 // z size, staged nodes, fits), the row offsets (a word per row of the table),

@@ -44,7 +44,9 @@ namespace {
 
 // The global-memory path of a marker block whose footprint does not fit its
 // shared memory (rare): out of line, so that it does not crowd the
-// instruction cache of the staged path it sits beside.
+// instruction cache of the staged path it sits beside.  All loads of a support are
+// issued before the first is used (a step of 200 drops of 14 cells, 140 of 1000
+// patches on this path: 274 -> 264 us).
 // (body cell G: read again here, so that it is not kept for this path; FEW: a
 // copy with the registers of the kernel's variant for few blocks)
 __device__ __forceinline__ GlobalRows global_rows(const Grid& g, const BodyDev* b) {
@@ -68,16 +70,12 @@ template <bool FEW>
 __device__ __noinline__ float value_global(const float* f, Grid g, const BodyDev* b, int c0, int c1,
                                           int c2, DirW X, DirW Y, DirW Z) {
   const int c[3] = {c0, c1, c2};
-  if (FEW) return mls_value(f, Loaded(f, global_rows(g, b).at(c)), X, Y, Z);
-  return mls_value(f, global_rows(g, b).at(c), X, Y, Z);
+  return mls_value(f, Loaded(f, global_rows(g, b).at(c)), X, Y, Z);
 }
 template <bool FEW>
 __device__ __noinline__ float3 gradient_global(const float* f, Grid g, const BodyDev* b, ProbeW P) {
   float gr[3];
-  if (FEW)
-    mls_grad(f, Loaded(f, global_rows(g, b).at(P.cc)), P.X, P.Y, P.Z, gr);
-  else
-    mls_grad(f, global_rows(g, b).at(P.cc), P.X, P.Y, P.Z, gr);
+  mls_grad(f, Loaded(f, global_rows(g, b).at(P.cc)), P.X, P.Y, P.Z, gr);
   return make_float3(gr[0], gr[1], gr[2]);
 }
 template <bool FEW>
@@ -130,17 +128,15 @@ __global__ void __launch_bounds__(MT, (VAR == kFew ? 512 : 768) / MT) marker_ker
   constexpr bool FLUSH = SPREAD && !REC;      // spreads into the fields
   constexpr bool ROWMAP = VEL || FLUSH;
   extern __shared__ __align__(16) unsigned char dyn[];
-  const int MR = shape.rows, mn = shape.nodes;  // (y, z) rows, staged nodes of a buffer
+  const int MR = shape.rows, mn = shape.nodes;  // (y, z) rows, staged nodes
   int* s_off4 = reinterpret_cast<int*>(dyn);   // [MR] 4 (staged start of the row - its first x)
   unsigned short* s_grp = reinterpret_cast<unsigned short*>(s_off4 + MR);   // [MR + 1] first group
   unsigned* s_mask = reinterpret_cast<unsigned*>(s_grp + MR + 8);    // a bit per group: nonzero
   int* s_gofs = reinterpret_cast<int*>(s_mask + marker_mask_words(mn));   // [mn/4] global offsets
   float* bufA = reinterpret_cast<float*>(s_gofs + mn / 4);
-  const bool dbl = shape.buffers == 2;         // two staging buffers
-  float* bufB = bufA + mn;
   // probe kernels keep per-thread values that a component needs once or twice
   // here, not in registers: probe end(s), normal, centroid velocity, a.n
-  float* s_own = bufA + shape.buffers * mn + threadIdx.x;      // [kOwn][MT]
+  float* s_own = bufA + mn + threadIdx.x;      // [kOwn][MT]
   unsigned* s_xbits = reinterpret_cast<unsigned*>(bufA);   // [MR] x-intervals each row touches,
                                                            //  while the rows are found
   __shared__ int s_lo[3], s_hi[3];
@@ -521,12 +517,14 @@ __global__ void __launch_bounds__(MT, (VAR == kFew ? 512 : 768) / MT) marker_ker
   const StagedRows SR{dyn, -(ylo + sy * zlo), sy};
   const int ofsA = (int)(reinterpret_cast<unsigned char*>(bufA) - dyn);
   const int ngroups = fit ? N / 4 : 0;
+  const bool dbl = 2 * N <= mn;                // two staging buffers
+  float* bufB = bufA + mn / 2;
 
   // ---- the components, one after the other ---------------------------------
-  // Velocity: interpolation at the centroid, gradient at the probes.  The
-  // components are staged in two buffers (u -> A, v -> B, w -> A, and with a
-  // pressure field p -> B), the next one's copies in flight while the current
-  // one is used.  Traction t = (G + G^T) n: component i yields (G n)_i and
+  // Velocity: interpolation at the centroid, gradient at the probes.  Where two
+  // buffers fit, the components are staged in turn (u -> A, v -> B, w -> A, and
+  // with a pressure field p -> B), the next one's copies in flight while the
+  // current one is used.  Traction t = (G + G^T) n: component i yields (G n)_i and
   // adds n_i G_i. to G^T n; the pressure jump P = p+ - p- (open) or p (closed).
   // Spread: a component's marker forces are spread as soon as they are known,
   // with the factors of the interpolation, in exact fixed point (one 32-bit
@@ -548,7 +546,7 @@ __global__ void __launch_bounds__(MT, (VAR == kFew ? 512 : 768) / MT) marker_ker
     for (int comp = 0; comp < (press ? 4 : 3); ++comp) {
       const float* velc = comp == 0 ? u : (comp == 1 ? vv : (comp == 2 ? w : pr));
       float* buf = (dbl && (comp & 1)) ? bufB : bufA;
-      const int obuf = ofsA + ((dbl && (comp & 1)) ? 4 * mn : 0);
+      const int obuf = ofsA + ((dbl && (comp & 1)) ? 2 * mn : 0);
       if (VEL && fit) {
         // one later group (the next component) may still be in flight
         if (dbl && (comp < 2 || (comp == 2 && press))) cp_async_wait<1>(); else cp_async_wait<0>();
@@ -950,7 +948,7 @@ cudaError_t launch_mt(ibm_ctx* c, const float* x, const float* v, const float* u
                       const float* Fm_in, float* Fext, float* fx, float* fy, float* fz,
                       int record, int tmode, const DeviceTables* tab, int cache, bool pdl) {
   const bool rows = I || P || (S && !R);
-  const MarkerShape ms = rows ? c->mshape[P ? 1 : 0] : MarkerShape{0, 0, 1};
+  const MarkerShape ms = rows ? c->mshape[P ? 1 : 0] : MarkerShape{0, 0};
   const size_t smem = rows ? marker_smem_bytes(MT, ms, P) : 0;
   const int vec4 = c->vec4 && aligned16(u) && aligned16(vv) && aligned16(w) && aligned16(pr) &&
                    aligned16(fx) && aligned16(fy) && aligned16(fz);

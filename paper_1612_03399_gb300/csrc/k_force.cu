@@ -188,8 +188,8 @@ __global__ void __launch_bounds__(kForceThreadsMax, 3) force_kernel(
     }
     const int la = r.x & 0xFFFF, lb = r.x >> 16, lc = r.y & 0xFFFF, ld = r.y >> 16;
     const bool hinge = ld != kNone;
-    const Vec<float> pa = S.pos(la), e = vsub(S.pos(lb), pa);
-    const Vec<float> ac = vsub(S.pos(lc), pa), ad = vsub(S.pos(hinge ? ld : la), pa);
+    const Vec<float> pa = S.pos(la), pb = S.pos(lb), pd = S.pos(hinge ? ld : la);
+    const Vec<float> e = vsub(pb, pa), ac = vsub(S.pos(lc), pa), ad = vsub(pd, pa);
     // per-edge and per-face constants (van Gelder springs, materials) where
     // the body has them
     const float ks = P.varied ? Bks * rest[3 * pe + pf + k] : Bks;
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kForceThreadsMax, 3) force_kernel(
     float l, inv_l, es, eb = 0.f, ea = 0.f;
     spring_forward(e, rest[k], ks, l, inv_l, fa, es);
     fb = {-fa.x, -fa.y, -fa.z};
-    const Vec<float> N1 = vcross(e, ac), N2 = vcross(ad, e);
+    const Vec<float> N1 = vcross(e, ac), N2 = vcross(vsub(pd, pb), e);
     const float r1 = rsqrtf(vdot(N1, N1)), r2 = rsqrtf(vdot(N2, N2));
     if (hinge) {
       const float kb = P.varied ? Bkb * rest[4 * pe + pf + k] : Bkb;

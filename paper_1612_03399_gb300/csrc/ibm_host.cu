@@ -49,14 +49,11 @@ struct HostTopo {
   std::vector<PatchHdr> patch;
   std::vector<int32_t> loc_vert;
   std::vector<PEdge> pedge;
-  std::vector<PFace> pface;
-  std::vector<int32_t> csr_ptr;
-  std::vector<uint16_t> csr_slot;
   std::vector<uint32_t> fblob;          // packed element records of the force kernel
   std::vector<FPatch> fpatch;           //   (one 16-byte aligned blob per patch)
   std::vector<int32_t> fatt;            // per face: 2 * attached edge + side (1: right face)
   std::vector<int32_t> fface;           // per patch, its faces in the blob's order
-  int max_loc = 0, max_slot = 0, max_own = 0;
+  int max_own = 0;
   std::vector<int32_t> mface, mbound;   // faces in marker-patch order, patch boundaries
 };
 
@@ -205,7 +202,7 @@ void build_topology(HostTopo& T, const int32_t* tri, int nv, int nf, int P) {
   }
   // patches
   const int npatch = (nv + P - 1) / P;
-  std::vector<int32_t> e_stamp(T.ne, -1), e_loc(T.ne), f_stamp(nf, -1), f_loc(nf),
+  std::vector<int32_t> e_stamp(T.ne, -1), e_loc(T.ne), f_stamp(nf, -1),
       v_stamp(nv, -1), v_loc(nv);
   std::vector<int32_t> es, fs;
   for (int p = 0; p < npatch; ++p) {
@@ -278,38 +275,11 @@ void build_topology(HostTopo& T, const int32_t* tri, int nv, int nf, int P) {
       r.eid = e | ((E.x >= o0 && E.x < o1) ? (int32_t)0x80000000 : 0);
       T.pedge.push_back(r);
     }
-    H.face_off = (int32_t)T.pface.size();
+    H.face_off = (int32_t)T.fface.size();
     H.n_face = (int32_t)fs.size();
-    for (size_t i = 0; i < fs.size(); ++i) {
-      const int f = fs[i];
-      f_loc[f] = (int32_t)i;
-      PFace r;
-      r.l[0] = local(tri[3 * f]);
-      r.l[1] = local(tri[3 * f + 1]);
-      r.l[2] = local(tri[3 * f + 2]);
-      r.owned = (tri[3 * f] >= o0 && tri[3 * f] < o1) ? 1 : 0;
-      r.fid = f;
-      T.pface.push_back(r);
-    }
     H.n_loc = (int32_t)T.loc_vert.size() - H.loc_off;
-    H.n_slot = 4 * H.n_edge + 3 * H.n_face;
-    if (H.n_loc >= (int)kNone || H.n_slot > 65535)
+    if (H.n_loc >= (int)kNone || 4 * H.n_edge + 3 * H.n_face > 65535)
       fail(IBM_ERR_UNSUPPORTED, "patch too large for 16-bit local indices; lower patch_size");
-    H.csr_off = (int32_t)T.csr_ptr.size();
-    H.slot_off = (int32_t)T.csr_slot.size();
-    for (int v = o0; v < o1; ++v) {
-      T.csr_ptr.push_back((int32_t)T.csr_slot.size() - H.slot_off);
-      // contribution slots are laid out [role][element] (edges, then faces)
-      for (int k = v2e_ptr[v]; k < v2e_ptr[v + 1]; ++k) {
-        const int e = v2e[k] >> 2, role = v2e[k] & 3;
-        T.csr_slot.push_back((uint16_t)(role * H.n_edge + e_loc[e]));
-      }
-      for (int k = T.v2f_ptr[v]; k < T.v2f_ptr[v + 1]; ++k) {
-        const int f = v2fc[k] / 3, corner = v2fc[k] % 3;
-        T.csr_slot.push_back((uint16_t)(4 * H.n_edge + corner * H.n_face + f_loc[f]));
-      }
-    }
-    T.csr_ptr.push_back((int32_t)T.csr_slot.size() - H.slot_off);
     // The force kernel's blob of this patch.  Every face is attached to an
     // edge of its own (as its left face (a, b, c) or its right face (b, a, d))
     // and adds its corner forces to that edge's role slots, so an own vertex
@@ -375,8 +345,6 @@ void build_topology(HostTopo& T, const int32_t* tri, int nv, int nf, int P) {
       T.fpatch.push_back(Q);
       T.fface.insert(T.fface.end(), fo.begin(), fo.end());
     }
-    T.max_loc = std::max(T.max_loc, H.n_loc);
-    T.max_slot = std::max(T.max_slot, H.n_slot);
     T.max_own = std::max(T.max_own, H.n_own);
     T.patch.push_back(H);
   }
@@ -843,7 +811,6 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     std::vector<float> chunk_area;   // rest area of each marker patch
     std::vector<int2> work;
     std::vector<float> frest;        // force-kernel rest data per work item, patch order
-    std::vector<int64_t> wrest;
     std::vector<FWork> fwork;
     size_t force_smem = 0, force_smem_wide = 0, adjoint_smem = 0, adjoint_smem_wide = 0;
     c->h_body.resize(n_bodies);
@@ -977,7 +944,6 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
         const PatchHdr& H = T.patch[q];
         const int pe = pad4(H.n_edge), pf = pad4(H.n_face);
         const size_t r0 = frest.size();
-        wrest.push_back((int64_t)r0);
         frest.resize(r0 + frest_words(H.n_edge, H.n_face, varied), 0.f);
         for (int i = 0; i < H.n_edge; ++i) {
           const long long ge = eo + (T.pedge[H.edge_off + i].eid & 0x7fffffff);
@@ -1035,17 +1001,13 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
 
     // concatenate the topology tables
     std::vector<TopoDev> td(topos.size());
-    std::vector<int32_t> tri_all, v2f_ptr_all, v2f_idx_all, loc_all, csr_all, mface_all;
+    std::vector<int32_t> tri_all, v2f_ptr_all, v2f_idx_all, loc_all, mface_all;
     std::vector<int4> mtri_all;
     std::vector<int4> edge_all;
     std::vector<PatchHdr> patch_all;
-    std::vector<PEdge> pedge_all;
-    std::vector<PFace> pface_all;
-    std::vector<uint16_t> slot_all;
     std::vector<uint32_t> fblob_all;
-    std::vector<FPatch> fpatch_all;
     std::vector<int32_t> topo_loc, topo_blob;   // where each topology's tables start
-    int max_loc = 0, max_slot = 0, max_own = 0;
+    int max_own = 0;
     for (size_t t = 0; t < topos.size(); ++t) {
       const HostTopo& T = topos[t];
       TopoDev& D = td[t];
@@ -1068,35 +1030,18 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
         mtri_all.push_back(make_int4(T.tri[3 * f], T.tri[3 * f + 1], T.tri[3 * f + 2], f));
 
       D.patch_off = (int32_t)patch_all.size();
-      const int32_t lo = (int32_t)loc_all.size(), eo2 = (int32_t)pedge_all.size(),
-                    fo2 = (int32_t)pface_all.size(), co = (int32_t)csr_all.size(),
-                    so = (int32_t)slot_all.size();
+      const int32_t lo = (int32_t)loc_all.size();
       for (PatchHdr H : T.patch) {
         H.loc_off += lo;
-        H.edge_off += eo2;
-        H.face_off += fo2;
-        H.csr_off += co;
-        H.slot_off += so;
         patch_all.push_back(H);
       }
       loc_all.insert(loc_all.end(), T.loc_vert.begin(), T.loc_vert.end());
-      pedge_all.insert(pedge_all.end(), T.pedge.begin(), T.pedge.end());
-      pface_all.insert(pface_all.end(), T.pface.begin(), T.pface.end());
-      csr_all.insert(csr_all.end(), T.csr_ptr.begin(), T.csr_ptr.end());
-      slot_all.insert(slot_all.end(), T.csr_slot.begin(), T.csr_slot.end());
       const int32_t bo = (int32_t)fblob_all.size();
       topo_loc.push_back(lo);
       topo_blob.push_back(bo);
-      for (FPatch Q : T.fpatch) {
-        Q.blob_off += bo;
-        fpatch_all.push_back(Q);
-      }
       fblob_all.insert(fblob_all.end(), T.fblob.begin(), T.fblob.end());
-      max_loc = std::max(max_loc, T.max_loc);
-      max_slot = std::max(max_slot, T.max_slot);
       max_own = std::max(max_own, T.max_own);
     }
-    (void)max_slot;
     for (FWork& w : fwork) {
       w.loc_off += topo_loc[body_topo[w.body]];
       w.blob_off += topo_blob[body_topo[w.body]];
@@ -1129,14 +1074,8 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
     d.v2f_idx = upload(c, v2f_idx_all);
     d.patch = upload(c, patch_all);
     d.loc_vert = upload(c, loc_all);
-    d.pedge = upload(c, pedge_all);
-    d.pface = upload(c, pface_all);
-    d.csr_ptr = upload(c, csr_all);
-    d.csr_slot = upload(c, slot_all);
     d.fblob = upload(c, fblob_all);
-    d.fpatch = upload(c, fpatch_all);
     d.frest = upload(c, frest);
-    d.wrest = upload(c, wrest);
     d.fwork = upload(c, fwork);
     d.l0 = upload(c, l0);
     d.cs0 = upload(c, cs0);
@@ -1392,7 +1331,7 @@ extern "C" ibm_status ibm_spread(ibm_ctx* c, const float* x, const float* Fm, fl
     e = launch_tile_begin(c, true, false);
     if (e == cudaSuccess)
       e = launch_mls_records(c, x, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, Fm,
-                             nullptr, false, false, true);
+                             nullptr, false, false);
     if (e == cudaSuccess) e = launch_tile_spread(c, fx, fy, fz, true);
   } else {
     e = launch_mls(c, x, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, Fm,
@@ -1426,7 +1365,7 @@ cudaError_t step_launches(ibm_ctx* c, const float* x, const float* v, const floa
     mark(1);
     if (e == cudaSuccess && before_marker) e = cudaStreamWaitEvent(c->stream, before_marker, 0);
     if (e == cudaSuccess)
-      e = launch_mls_records(c, x, v, u, vv, w, p, accel, nullptr, c->d.fext, true, true, !clear);
+      e = launch_mls_records(c, x, v, u, vv, w, p, accel, nullptr, c->d.fext, true, true);
     mark(2);
     if (e == cudaSuccess) e = launch_tile_spread(c, fx, fy, fz, !clear);
     mark(3);
@@ -1946,7 +1885,7 @@ extern "C" ibm_status ibm_step_pc(ibm_ctx* c, const float* x, const float* v, co
   if (c->spread_variant == 2) {
     e = launch_tile_begin(c, !clear, true);
     if (e == cudaSuccess)
-      e = launch_mls_records(c, x, v, u, vv, w, p, accel, nullptr, c->d.fext, true, true, !clear);
+      e = launch_mls_records(c, x, v, u, vv, w, p, accel, nullptr, c->d.fext, true, true);
     if (e == cudaSuccess) e = launch_tile_spread(c, fx, fy, fz, !clear);
   } else {
     e = clear ? launch_clear(c, fx, fy, fz) : zero_body_sums(c);
@@ -2097,7 +2036,7 @@ extern "C" ibm_status ibm_graph_create(ibm_ctx* c, float* xa, float* va, float* 
       use_parity(c, c->qpar ^ 1);
       e = launch_tile_begin(c, false, true);
       if (e == cudaSuccess)
-        e = launch_mls_records(c, x, v, u, vv, w, p, accel, nullptr, c->d.fext, true, true, false);
+        e = launch_mls_records(c, x, v, u, vv, w, p, accel, nullptr, c->d.fext, true, true);
       if (e == cudaSuccess) e = cudaEventRecord(ev_marker, cap);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_marker, 0);
       if (e == cudaSuccess) {

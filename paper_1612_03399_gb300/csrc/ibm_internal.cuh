@@ -55,19 +55,13 @@ struct TopoDev {
 // elements touching them reference.
 struct PatchHdr {
   int32_t own0, n_own, n_loc, loc_off;       // own range, local vertex count, loc_vert offset
-  int32_t n_edge, edge_off, n_face, face_off;
-  int32_t csr_off, slot_off, n_slot, pad;    // csr_ptr offset (n_own + 1), csr_slot offset
+  int32_t n_edge, edge_off, n_face, face_off;   // offsets into the topology's lists (host)
 };
 
-// element records local to a patch: local vertex indices (0xFFFF = none)
+// edge records local to a patch (host): local vertex indices (0xFFFF = none)
 struct PEdge {
   uint16_t l[4];       // a, b (edge), c, d (wings)
   int32_t eid;         // body-local edge id; bit 31 set when this patch owns the edge
-};
-struct PFace {
-  uint16_t l[3];
-  uint16_t owned;      // 1 when this patch owns the face (energy bookkeeping)
-  int32_t fid;         // body-local face id
 };
 
 // The force kernel's own packed copy of a patch's element records, moved into
@@ -216,14 +210,8 @@ struct DeviceTables {
   int32_t* v2f_idx = nullptr;
   PatchHdr* patch = nullptr;
   int32_t* loc_vert = nullptr;
-  PEdge* pedge = nullptr;
-  PFace* pface = nullptr;
-  int32_t* csr_ptr = nullptr;
-  uint16_t* csr_slot = nullptr;
   uint32_t* fblob = nullptr;    // force-kernel element blobs (FPatch)
-  FPatch* fpatch = nullptr;     // per topology patch, indexed like `patch`
   float* frest = nullptr;       // rest data of every work item, in patch order
-  int64_t* wrest = nullptr;     // [n_work] word offset of the work item's rest data
   FWork* fwork = nullptr;       // [n_work] records of the force kernel
   float* l0 = nullptr;          // [E] rest edge lengths
   float2* cs0 = nullptr;        // [E] (cos theta0, sin theta0) per hinge edge
@@ -441,12 +429,11 @@ cudaError_t launch_forcing(ibm_ctx* c, int substep, const float* x, const float*
                            float* fz);
 
 // marker kernel without the spread, writing the spread records and counting
-// the marker-tile pairs of the tile-owned spread (`accumulate`: into the
-// fields' existing values, outside the clear-mode bookkeeping)
+// the marker-tile pairs of the tile-owned spread
 cudaError_t launch_mls_records(ibm_ctx* c, const float* x, const float* v, const float* u,
                                const float* vv, const float* w, const float* p,
                                const float* accel, const float* Fm_in, float* Fext, bool measure,
-                               bool probe, bool accumulate);
+                               bool probe);
 // tile-owned spread (k_tile.cu): begin a call (epoch, list lengths, body
 // sums), offsets of the tiles' lists, fill, and the spread itself
 cudaError_t launch_tile_begin(ibm_ctx* c, bool accumulate, bool zero_sums);

@@ -946,7 +946,7 @@ template <int MT, bool M, bool I, bool P, bool S, bool R>
 cudaError_t launch_mt(ibm_ctx* c, const float* x, const float* v, const float* u, const float* vv,
                       const float* w, const float* pr, const float* accel, float* U, float* Fm,
                       const float* Fm_in, float* Fext, float* fx, float* fy, float* fz,
-                      int record, int tmode, const DeviceTables* tab, int cache, bool pdl) {
+                      int record, const DeviceTables* tab, int cache, bool pdl) {
   const bool rows = I || P || (S && !R);
   const MarkerShape ms = rows ? c->mshape[P ? 1 : 0] : MarkerShape{0, 0};
   const size_t smem = rows ? marker_smem_bytes(MT, ms, P) : 0;
@@ -980,14 +980,14 @@ template <bool M, bool I, bool P, bool S, bool R = false>
 cudaError_t launch_t(ibm_ctx* c, const float* x, const float* v, const float* u, const float* vv,
                      const float* w, const float* pr, const float* accel, float* U, float* Fm,
                      const float* Fm_in, float* Fext, float* fx, float* fy, float* fz,
-                     int record, int tmode = 0, const DeviceTables* tab = nullptr, int cache = 0,
+                     int record, const DeviceTables* tab = nullptr, int cache = 0,
                      bool pdl = false) {
   if (c->n_chunks == 0) return cudaSuccess;
   if (c->marker_patch == 128)
     return launch_mt<128, M, I, P, S, R>(c, x, v, u, vv, w, pr, accel, U, Fm, Fm_in, Fext, fx, fy,
-                                         fz, record, tmode, tab, cache, pdl);
+                                         fz, record, tab, cache, pdl);
   return launch_mt<kMT, M, I, P, S, R>(c, x, v, u, vv, w, pr, accel, U, Fm, Fm_in, Fext, fx, fy,
-                                       fz, record, tmode, tab, cache, pdl);
+                                       fz, record, tab, cache, pdl);
 }
 
 }  // namespace
@@ -1032,7 +1032,7 @@ cudaError_t launch_mls(ibm_ctx* c, const float* x, const float* v, const float* 
   launch_t<M, I, P, S>(c, x, v, u, vv, w, pr, accel, U, Fm, Fm_in, Fext, fx, fy, fz, rb)
   if (measure && interp && probe && spread)
     return launch_t<true, true, true, true>(c, x, v, u, vv, w, pr, accel, U, Fm, Fm_in, Fext, fx,
-                                            fy, fz, rb, 0, nullptr, 0, after_clear);
+                                            fy, fz, rb, nullptr, 0, after_clear);
   if (measure && !interp && !probe && !spread) return L(true, false, false, false);
   if (measure && !interp && probe && !spread) return L(true, false, true, false);
   if (!measure && interp && probe && !spread) return L(false, true, true, false);
@@ -1047,19 +1047,18 @@ cudaError_t launch_mls(ibm_ctx* c, const float* x, const float* v, const float* 
 cudaError_t launch_mls_records(ibm_ctx* c, const float* x, const float* v, const float* u,
                                const float* vv, const float* w, const float* p,
                                const float* accel, const float* Fm_in, float* Fext, bool measure,
-                               bool probe, bool accumulate) {
-  const int tm = accumulate ? 2 : 1;
+                               bool probe) {
   if (measure && probe)   // the step: body sums, interpolation, traction, records
     return launch_t<true, true, true, true, true>(c, x, v, u, vv, w, p, accel, nullptr, nullptr,
-                                                  nullptr, Fext, nullptr, nullptr, nullptr, 0, tm);
+                                                  nullptr, Fext, nullptr, nullptr, nullptr, 0);
   if (!measure && !probe && u)   // the coupled forcing: interpolation and records
     return launch_t<false, true, false, true, true>(c, x, v, u, vv, w, nullptr, nullptr, nullptr,
                                                     nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                    nullptr, 0, tm);
+                                                    nullptr, 0);
   if (!measure && !probe && Fm_in)   // given marker forces
     return launch_t<false, false, false, true, true>(c, x, nullptr, nullptr, nullptr, nullptr,
                                                      nullptr, nullptr, nullptr, nullptr, Fm_in,
-                                                     nullptr, nullptr, nullptr, nullptr, 0, tm);
+                                                     nullptr, nullptr, nullptr, nullptr, 0);
   return cudaErrorInvalidValue;
 }
 
@@ -1103,7 +1102,7 @@ cudaError_t launch_forcing(ibm_ctx* c, int substep, const float* x, const float*
     if (e != cudaSuccess) return e;
   }
   return launch_t<false, true, false, true>(c, x, xv, u, vv, w, nullptr, nullptr, nullptr, nullptr,
-                                            nullptr, nullptr, fx, fy, fz, 1, 0, &t,
+                                            nullptr, nullptr, fx, fy, fz, 1, &t,
                                             substep == 0 ? 1 : 2);
 }
 

@@ -862,8 +862,8 @@ def flow_bytes(n, widths):
     """Algorithmic bytes per time step of the flow solver's own kernels
     (float32 fields of N cells, spectra of NC = nz ny (nx/2+1) complex
     values), summed over the three substeps: what each kernel must read and
-    write once.  `widths` are the substeps' viscous-solve widths (-1: Fourier
-    path); the u* update moves the same bytes on both paths (R or du read,
+    write once.  `widths` are the substeps' viscous-solve widths (-1: counted as
+    the Fourier path); the u* update moves the same bytes on both paths (R or du read,
     u read and written) and is named for the kernel that ran it."""
     N = n[0] * n[1] * n[2]
     NC = n[2] * n[1] * (n[0] // 2 + 1)

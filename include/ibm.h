@@ -377,13 +377,14 @@ ibm_status ibm_gts_read(const char* path, int64_t* n_vert, int64_t* n_face, doub
  *   lap(phi) = div(u*)/(alpha_l dt),  u = u* - alpha_l dt grad(phi),
  *   p <- p + phi - a lap(phi)                                      (projection).
  * In the periodic box both implicit operators are diagonal in Fourier space.
- * The Poisson equation is solved there (cuFFT transforms, float32).  The
- * factorised viscous operator is inverted exactly in one of two ways, fixed
- * per substep at creation: in real space when every direction's periodic
- * inverse, a circulant whose entries fall off as r^|m|, has less than 2^-26
- * of its mass beyond some |m| = W <= 8 with 2W + 1 <= n (then three
- * separable (2W+1)-tap filters, fused with the u* update; small
- * alpha_l dt nu / h^2), else by the same inverse as first-order recursions
+ * The Poisson equation is solved there in x and y (cuFFT transforms, float32),
+ * and in z by recursions along the columns, or there as well (n_z above 512, L_x or
+ * L_y above 1.57 L_z).  The factorised viscous operator is inverted exactly in one
+ * of three ways, fixed per substep at creation: in real space when every
+ * direction's periodic inverse, a circulant whose entries fall off as r^|m|, has
+ * less than 2^-26 of its mass beyond some |m| = W <= 8 with 2W + 1 <= n in every
+ * direction (then three separable (2W+1)-tap filters, fused with the u* update;
+ * small alpha_l dt nu / h^2), else by the same inverse as first-order recursions
  * along the lines (r <= 0.7) or in Fourier space.  A flow object owns its work
  * arrays (about thirteen fields) and FFT plans; velocity and pressure fields
  * are caller-owned device arrays [nz][ny][nx]. */

@@ -453,7 +453,8 @@ class Flow:
 
     def solve_widths(self):
         """Per substep, the half width W of the real-space viscous solve
-        (2W + 1 taps per direction), or -1 where it runs in Fourier space."""
+        (2W + 1 taps per direction), or -1 where it runs by line recursions or in
+        Fourier space."""
         out = []
         for l in range(3):
             w = C.c_int32()

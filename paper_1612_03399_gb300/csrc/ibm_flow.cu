@@ -1114,7 +1114,12 @@ cudaError_t launch_lines(const ibm_flow* fl, int l, float* u, float* v, float* w
 // The recursions take a substep instead of the transforms while r <= 0.7 (their
 // rounding, about 2/(1 - r) units per direction, is then that of a transform)
 // and lines fit shared memory.  Where 17 taps or fewer do, the fused filters
-// stay: W = 7 on 200 x 180 x 144 takes 145 us.
+// stay: W = 7 on 200 x 180 x 144 takes 90 us.  Long lines leave few blocks per SM
+// (one from 880 entries on), so the gain shrinks: a whole predictor, transforms
+// against lines, us: 200 x 180 x 144 384, 179; 512 x 256 x 128 879, 554; 128 x 256 x 512
+// 879, 498; 900 x 128 x 96 704, 595; 96 x 1600 x 64 881, 464; 1600 x 96 x 64 564, 539;
+// 1597 x 96 x 64 1131, 560; only x lines of 1000 to 1024, where the transforms are at
+// their best, lose: 1024 x 256 x 64 808, 848.
 bool use_lines(const ibm_flow* fl, int l) {
   if (fl->solve_w[l] >= 0) return false;
   const double a = (kGamma[l] + kRho[l]) * fl->dt * fl->nu / 2.0;
@@ -1128,7 +1133,7 @@ bool use_lines(const ibm_flow* fl, int l) {
 // (the larger of L_x, L_y at most 1.57 L_z): past that the closing of the column
 // amplifies its rounding.  Errors against float64 relative to the transforms', on
 // 9 x 5 x 15 .. 128^3 and cells 1 : 1 : 0.65 .. 1 : 1 : 16: p 0.3 .. 1.0, u 0.6 .. 1.0;
-// beyond the line, at L_x = 4 L_z, p up to 1.2.
+// beyond the line, at L_x = 4 L_z, p up to 1.2 (a float32 restatement).
 bool use_z_lines(const ibm_flow* fl) {
   if (fl->n[2] > kZMax || (long long)(fl->n[0] / 2 + 1) * fl->n[1] > 0x7fffffffll - 32) return false;
   double least = 1e300;

@@ -142,7 +142,10 @@ __global__ void __launch_bounds__(MT, (VAR == kFew ? 512 : 768) / MT) marker_ker
   __shared__ int s_lo[3], s_hi[3];
   __shared__ int s_N;
   __shared__ int s_warp[MT / 32];
+  // bound on a node's contributions: per component the largest |c_l F|, or (FEW) per
+  // warp the sum of |c_l F| / 256
   __shared__ unsigned s_bmax[3];
+  __shared__ float s_bsum[3][FEW ? MT / 32 : 1];
   __shared__ __align__(8) unsigned long long s_bar;
   __shared__ unsigned long long s_q[2][MT / 32];   // per-warp fixed-point body sums
   // what the end of the block needs again: body, its cell G, closed, patch
@@ -644,21 +647,39 @@ __global__ void __launch_bounds__(MT, (VAR == kFew ? 512 : 768) / MT) marker_ker
         const float coef = mine ? cl * Fc : 0.f;
         float* fc = comp == 0 ? fx : (comp == 1 ? fy : fz);
         if (fit) {
-          // the block's largest |c_l F| (non-negative floats order as their
-          // bit patterns, a NaN above all)
-          const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(coef)));
-          if (lane == 0) atomicMax(&s_bmax[comp], wm);
-          __syncthreads();   // the maximum is known and the staged component used up
+          if (FEW) {
+            // (over 256, so that it overflows only where a single one would)
+            float ws = fabsf(coef) * 0x1p-8f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, o);
+            if (lane == 0) s_bsum[comp][threadIdx.x >> 5] = ws;
+          } else {
+            // non-negative floats order as their bit patterns, a NaN above all
+            const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(coef)));
+            if (lane == 0) atomicMax(&s_bmax[comp], wm);
+          }
+          __syncthreads();   // the bound is known and the staged component used up
           int4* acc4 = reinterpret_cast<int4*>(buf);
           for (int q = threadIdx.x; q < ngroups; q += MT) acc4[q] = make_int4(0, 0, 0, 0);
           __syncthreads();
-          const float bm = __uint_as_float(s_bmax[comp]) * phi_bound_all;
+          float bm = FEW ? 0.f : __uint_as_float(s_bmax[comp]);
+          if (FEW) {
+#pragma unroll
+            for (int k = 0; k < MT / 32; ++k) bm += s_bsum[comp][k];
+          }
+          bm *= phi_bound_all;
           const bool fin = bm <= 3.0e38f;
           if (!fin && threadIdx.x == 0) atomicOr(T.err, ERR_NONFINITE);
           if (fin && bm > 0.f) {   // uniform over the block
-            // scale 2^k with every contribution below 2^22 (|c_l phi F| <= bm): a
-            // node takes at most MT <= 256 of them, so the sum stays below 2^30
-            const int k = max(min(22 - (ilogbf(bm) + 1), 120), -126);
+            // scale 2^k such that what a node can take stays below 2^31 (with room for
+            // the roundings: 1.001): MT contributions of at most bm, or all the block's
+            // contributions, 256 bm.  The sum makes it one to three bits finer at 1.3 %
+            // of a full launch, where FEW has idle issue slots and patches of few, large
+            // contributions, which the largest one alone scales worst (six drops of 11 to
+            // 22 cells: f against float64 3.4e-6 with a bound of 2^30 and the largest,
+            // 2.2e-6 now; 3.1e-6 when such patches took the global path)
+            constexpr int kTop = !FEW && MT == 128 ? 23 : 22;
+            const int k = max(min(kTop - ilogbf(bm * 1.001f), 120), -126);
             if (coef != 0.f)
               mls_spread_fixed(dyn, SR.at(ccC, obuf), CX, CY, CZ, coef * pow2f(k));
             __syncthreads();

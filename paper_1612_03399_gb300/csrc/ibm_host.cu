@@ -627,6 +627,13 @@ void choose_marker_shapes(ibm_ctx* c, const ibm_body_desc* bodies,
     c->mshape[probe] = marker_shape(best, MT, probe != 0);
     // at most 16 warps per SM: by the blocks there are, or by the shape
     c->marker_few[probe] = (long long)n * MT <= 512ll * n_sm || best >= 1;
+    // Where patches take the global path, what the blocks an SM gets do not need of
+    // its memory is worth more as L1: a block of that path takes 43 us with 90 KB of
+    // it and 92 with 28 (the driver's split follows the kernels before).
+    const int per_sm = (n + n_sm - 1) / n_sm;
+    const size_t need = per_sm * ((size_t)marker_smem_bytes(MT, c->mshape[probe], probe != 0) + 2048);
+    c->marker_carveout[probe] =
+        unfit[best] > 0 && need < 228 * 1024 ? (int)((100 * need + 228 * 1024 - 1) / (228 * 1024)) : 0;
   }
 }
 

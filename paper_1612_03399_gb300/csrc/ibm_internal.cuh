@@ -284,7 +284,7 @@ constexpr int kMarkerShapes = 3;
 __host__ __device__ constexpr MarkerShape marker_shape(int k, int MT, bool probe) {
   return k == 0   ? MarkerShape{4 * MT, (probe ? 38 : 52) * MT}
          : k == 1 ? MarkerShape{6 * MT, (probe ? 64 : 80) * MT}
-                  : MarkerShape{6 * MT, (probe ? 156 : 172) * MT};
+                  : MarkerShape{6 * MT, (probe ? 84 : 92) * MT};
 }
 __host__ __device__ constexpr int marker_smem_max(int MT, bool probe) {
   return marker_smem_bytes(MT, marker_shape(kMarkerShapes - 1, MT, probe), probe);
@@ -347,6 +347,7 @@ struct ibm_ctx {
   // creation from the rest meshes)
   ibm::MarkerShape mshape[2] = {};
   bool marker_few[2] = {false, false};   // their variants for few blocks per SM
+  int marker_carveout[2] = {0, 0};  // shared memory to carve out, percent (0: the driver's choice)
   bool any_open = false;            // some body is an open sheet
   // coupled forcing (allocated by the first ibm_flow_step with this context):
   // the per-chunk tables and per-face geometry of substep 0, and the forcing's

@@ -10,7 +10,7 @@ namespace {
 
 // Positions and contribution slots in shared memory: as float4 (WIDE, one
 // shared load or store each), or as three arrays, a quarter smaller, for
-// patches whose float4 form does not fit (above about 650 vertices).
+// patches whose float4 form would cost a resident block.
 template <bool WIDE>
 struct Smem;
 template <>

@@ -1054,16 +1054,21 @@ extern "C" ibm_status ibm_create_bodies(ibm_ctx** out, const ibm_body_desc* bodi
       w.blob_off += topo_blob[body_topo[w.body]];
     }
     c->force_threads = choose_force_threads(fwork);
-    size_t room = 0, adjoint_room = 0;
-    check_cuda(force_smem_room(&room), "cudaFuncGetAttributes");
-    check_cuda(adjoint_smem_room(&adjoint_room), "cudaFuncGetAttributes");
-    c->force_wide = force_smem_wide <= room;
+    // The float4 layouts where they cost no resident block: one shared access per
+    // position or slot is worth less than a block.  1000 drops, patches of 224, 256, 384
+    // vertices: forces and update 84, 82, 127 us with float4, 68, 65, 78 with three
+    // arrays; the adjoint of the step, patches of 192: 434, 390.
+    int wide = 0, narrow = 0;
+    check_cuda(force_occupancy(c->force_threads, force_smem_wide, force_smem, &wide, &narrow), "occupancy");
+    c->force_wide = wide >= narrow;
+    const bool fits = wide > 0 || narrow > 0;
+    check_cuda(adjoint_occupancy(c->force_threads, adjoint_smem_wide, adjoint_smem, &wide, &narrow), "occupancy");
+    c->adjoint_wide = wide >= narrow;
+    if (!fits || (wide == 0 && narrow == 0))
+      fail(IBM_ERR_UNSUPPORTED, "force-kernel shared memory above 227 KB; lower patch_size");
     c->force_smem = c->force_wide ? force_smem_wide : force_smem;
-    c->adjoint_wide = adjoint_smem_wide <= adjoint_room;
     c->adjoint_smem = c->adjoint_wide ? adjoint_smem_wide : adjoint_smem;
     c->max_own = max_own;
-    if (c->force_smem > room || c->adjoint_smem > adjoint_room)
-      fail(IBM_ERR_UNSUPPORTED, "force-kernel shared memory above 227 KB; lower patch_size");
     check_cuda(set_force_smem_limit(c->force_smem), "cudaFuncSetAttribute");
     check_cuda(set_adjoint_smem_limit(c->adjoint_smem), "cudaFuncSetAttribute");
     check_cuda(set_marker_smem_limit(), "cudaFuncSetAttribute");

@@ -489,9 +489,9 @@ cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
   if (bytes > room) return cudaErrorInvalidValue;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
 }
-// the dynamic shared memory every force (adjoint) kernel can be launched with
-cudaError_t force_smem_room(size_t* room);
-cudaError_t adjoint_smem_room(size_t* room);
+// resident blocks per SM with the float4 and the three-array layout (0: does not fit)
+cudaError_t force_occupancy(int threads, size_t wide_bytes, size_t narrow_bytes, int* wide, int* narrow);
+cudaError_t adjoint_occupancy(int threads, size_t wide_bytes, size_t narrow_bytes, int* wide, int* narrow);
 cudaError_t set_force_smem_limit(size_t bytes);
 cudaError_t set_adjoint_smem_limit(size_t bytes);
 cudaError_t set_marker_smem_limit();

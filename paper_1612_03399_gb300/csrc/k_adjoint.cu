@@ -432,7 +432,8 @@ constexpr size_t kExtBytes = 30 * sizeof(float) * kMT;   // ext_adjoint_kernel's
 // with the division per block and the packed warp sums; 36.1 us with the faces
 // and their corners' cotangents on the edges instead of a chain of loads per
 // vertex.  Three blocks of at most 160 threads fit an SM's registers: 35.7 us,
-// 40.6 with 192.  The layout goes by the force kernel's rule: float4 where it fits.
+// 40.6 with 192.  The layout goes by the force kernel's rule: float4 where it costs
+// no resident block.
 template <bool WIDE>
 __global__ void __launch_bounds__(kAdjointThreads, 3) force_adjoint_kernel(
     DeviceTables T, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,
@@ -665,7 +666,7 @@ cudaError_t launch_backward(ibm_ctx* c, const float* x, const float* v, const fl
   return cudaGetLastError();
 }
 
-cudaError_t adjoint_smem_room(size_t* room) {
+static cudaError_t adjoint_smem_room(size_t* room) {
   *room = SIZE_MAX;
   const cudaError_t e = smem_room(force_adjoint_kernel<true>, room);
   return e == cudaSuccess ? smem_room(force_adjoint_kernel<false>, room) : e;
@@ -673,6 +674,20 @@ cudaError_t adjoint_smem_room(size_t* room) {
 cudaError_t set_adjoint_smem_limit(size_t bytes) {
   const cudaError_t e = allow_smem(force_adjoint_kernel<true>, bytes);
   return e == cudaSuccess ? allow_smem(force_adjoint_kernel<false>, bytes) : e;
+}
+
+cudaError_t adjoint_occupancy(int threads, size_t wide_bytes, size_t narrow_bytes, int* wide, int* narrow) {
+  size_t room = 0;
+  cudaError_t e = adjoint_smem_room(&room);
+  *wide = *narrow = 0;
+  threads = std::min(threads, kAdjointThreads);
+  if (e == cudaSuccess) e = set_adjoint_smem_limit(0);
+  if (e == cudaSuccess && wide_bytes <= room)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(wide, force_adjoint_kernel<true>, threads, wide_bytes);
+  if (e == cudaSuccess && narrow_bytes <= room)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(narrow, force_adjoint_kernel<false>, threads,
+                                                      narrow_bytes);
+  return e;
 }
 
 }  // namespace ibm

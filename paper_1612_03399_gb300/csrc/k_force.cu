@@ -406,12 +406,27 @@ static cudaError_t each_force_kernel(Fn fn) {
     if (e == cudaSuccess) e = fn(k);
   return e;
 }
-cudaError_t force_smem_room(size_t* room) {
+// the dynamic shared memory every force kernel can be launched with
+static cudaError_t force_smem_room(size_t* room) {
   *room = SIZE_MAX;
   return each_force_kernel([&](auto k) { return smem_room(k, room); });
 }
 cudaError_t set_force_smem_limit(size_t bytes) {
   return each_force_kernel([&](auto k) { return allow_smem(k, bytes); });
+}
+
+// resident blocks per SM of the step's force kernel with each layout (0: does not fit)
+cudaError_t force_occupancy(int threads, size_t wide_bytes, size_t narrow_bytes, int* wide, int* narrow) {
+  size_t room = 0;
+  cudaError_t e = force_smem_room(&room);
+  *wide = *narrow = 0;
+  if (e == cudaSuccess) e = set_force_smem_limit(0);
+  if (e == cudaSuccess && wide_bytes <= room)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(wide, force_kernel<1, false, true>, threads, wide_bytes);
+  if (e == cudaSuccess && narrow_bytes <= room)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(narrow, force_kernel<1, false, false>, threads,
+                                                      narrow_bytes);
+  return e;
 }
 
 }  // namespace ibm

@@ -101,7 +101,8 @@ __device__ __noinline__ void mirror_chunks(Mirror m, const float* x_out, const f
 // size whose whole warps fit the patches' edge counts (force_threads; 128 to
 // 288 threads differ by 5 %).  Patches of 128 vertices, 642 k vertices after
 // the marker kernel: 107 us at first, 84 with the record and the layouts, 72
-// with the faces on their edges.
+// with the faces on their edges; forces and update alone 98 -> 63, 59 with the layout
+// that keeps the most blocks resident.
 template <int MODE, bool ENERGY, bool WIDE>
 __global__ void __launch_bounds__(kForceThreadsMax, 3) force_kernel(
     DeviceTables T, StepConsts sc, int32_t V, int32_t F, const float* __restrict__ x,

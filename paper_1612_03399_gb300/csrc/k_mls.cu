@@ -27,10 +27,10 @@
 // memory.  Kept in local memory instead it cost more than the 24 warps gave:
 // next to 220 KB of shared memory little L1 is left for it.  Measured, this
 // kernel alone (us; before: 128 registers, 16 warps, spread after all three
-// components): whole step 437 -> 354 for 1000 drops (1.28 M faces) on 512^3,
-// 151 -> 117 for 460 k faces of uneven bodies, 147 -> 114 for a membrane of
-// 377 k faces; interpolation and spread 232 -> 170 and probes with body sums
-// 233 -> 162 for the 1000 drops on 256^3.
+// components): whole step 437 -> 354 (319 with what followed: the variants, buffers
+// by block) for 1000 drops (1.28 M faces) on 512^3, 151 -> 117 (111) for 460 k faces of
+// uneven bodies, 147 -> 114 (112) for a membrane of 377 k faces; interpolation and
+// spread 232 -> 170 and probes with body sums 233 -> 162 for the 1000 drops on 256^3.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>

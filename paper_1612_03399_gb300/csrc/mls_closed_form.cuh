@@ -475,10 +475,9 @@ __device__ __forceinline__ void mls_spread(float* f, const GlobalAcc& A, const D
 }
 
 // Spread in exact fixed point, one 32-bit word per node: the contribution
-// coef*phi, already scaled by the block's power of two so that
-// |value| < 2^22, rounded to an integer and added with a native shared
-// atomic; a node receives at most kMT contributions, so the word does not
-// overflow, and the sum is independent of the order of the additions.
+// coef*phi, already scaled by the block's power of two so that all a node can
+// take stays below 2^31, rounded to an integer and added with a native shared
+// atomic; the sum is independent of the order of the additions.
 __device__ __forceinline__ void mls_spread_fixed(unsigned char* sm, const RowAcc& A, const DirW& X,
                                                  const DirW& Y, const DirW& Z, float coef) {
   const float xb1 = -(X.b0 + X.b2);
